@@ -1699,12 +1699,12 @@ int zero_pistons(fewha_handle* H, T* v, cudaStream_t st) {
 }
 
 // The double-precision twin of a single-precision handle: the same geometry and
-// parameters, no flags.  It computes the true residuals b - M x of the single-precision
+// parameters, no flag but PDL.  It computes the true residuals b - M x of the single-precision
 // form's converged solves and holds their double iterates.
 int twin_params(fewha_handle* H) {
     fewha_params p = H->params;
     p.precision = 64;
-    p.flags = 0;
+    p.flags &= FEWHA_FLAG_PDL;
     const int rc = fewha_update_params(H->twin, &p, H->weights.data(), H->setup.wfs_sigma.data());
     if (rc) return fail(H, rc, std::string("double-precision twin: ") + fewha_last_error(H->twin));
     return FEWHA_OK;
@@ -1714,7 +1714,7 @@ int ensure_twin(fewha_handle* H) {
     if (H->twin) return FEWHA_OK;
     fewha_params p = H->params;
     p.precision = 64;
-    p.flags = 0;
+    p.flags &= FEWHA_FLAG_PDL;
     std::vector<fewha_layer> layers = H->layers_in;
     for (size_t l = 0; l < layers.size(); ++l) layers[l].cn2_weight = H->weights[l];
     std::vector<fewha_wfs> wfs = H->wfs_in;
@@ -1828,6 +1828,24 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
     return FEWHA_OK;
 }
 
+// The converged solve of a single-precision handle on the twin's double vectors.  The float
+// recurrence needs 1.6 to 2.9 times the double one's iterations, by how its rounding falls
+// (8 m and 4 m geometries at 1e-11: 12.7k to 21k against 7.1k to 8k).  An iteration of a
+// small instance is a chain of short kernels whose arithmetic hides behind the launches, so
+// a double iteration costs 1.65 times a float one at 1280 coefficients (43.6 against 26.5
+// us) and 1.8 times at 3072; at 16384 it costs 2.2 times, at 49152 3.8 times.  Up to
+// SOLVE_DOUBLE_NC coefficients the recurrence runs in double: 8 m forward and backward
+// 747 -> 646 ms.
+constexpr int SOLVE_DOUBLE_NC = 4096;
+int mixed_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* x64, bool warm, double tol,
+                int max_iters, cudaStream_t st, int* iters_out, double* rel_out) {
+    if (H->setup.n_c > SOLVE_DOUBLE_NC)
+        return reliable_solve(H, X, b64, x64, warm, tol, max_iters, st, iters_out, rel_out);
+    const int rc = solve_converged<double>(X, b64, x64, warm, tol, max_iters, st, iters_out, rel_out);
+    H->have_prev = false;
+    return rc ? fail(H, rc, X->err) : FEWHA_OK;
+}
+
 template <class T>
 int reconstruct_converged(fewha_handle* H, const T* s, T* dm, double tol, int max_iters, int* iters,
                           double* rel, cudaStream_t st) {
@@ -1844,8 +1862,8 @@ int reconstruct_converged(fewha_handle* H, const T* s, T* dm, double tol, int ma
         k_convert<double, float><<<(d.n_s + 255) / 256, 256, 0, st>>>(d.n_s, s, s64);
         CK(cudaGetLastError(), "k_convert launch");
         if ((rc = enqueue_rhs<double>(X, dx, s64, static_cast<double*>(X->b), st))) return fail(H, rc, X->err);
-        if ((rc = reliable_solve(H, X, static_cast<const double*>(X->b), static_cast<double*>(X->cgrad),
-                                 X->have_cgrad, tol, max_iters, st, iters, rel)))
+        if ((rc = mixed_solve(H, X, static_cast<const double*>(X->b), static_cast<double*>(X->cgrad),
+                              X->have_cgrad, tol, max_iters, st, iters, rel)))
             return rc;
         X->have_cgrad = true;
         double* dm64 = static_cast<double*>(X->dm_tmp);
@@ -1891,7 +1909,7 @@ int backward(fewha_handle* H, const T* g_a, T* g_s, double* g_alpha, double* g_w
         CK(cudaGetLastError(), "k_convert launch");
         if ((rc = launch_layer<double, LSRC_DM, LDST_COEF, false>(X, dx, layer_args<double>(X, ga64, b64), st)))
             return fail(H, rc, X->err);
-        if ((rc = reliable_solve(H, X, b64, lam, X->have_lam, H->grad_tol, H->grad_max_iters, st, &it, &rel)))
+        if ((rc = mixed_solve(H, X, b64, lam, X->have_lam, H->grad_tol, H->grad_max_iters, st, &it, &rel)))
             return rc;
         X->have_lam = true;
         if (g_s) {
@@ -1955,7 +1973,7 @@ int solve_entry(fewha_handle* H, const T* b, T* x, double tol, int max_iters, cu
         double* x64 = static_cast<double*>(X->c_tmp);
         k_convert<double, float><<<(n + 255) / 256, 256, 0, st>>>(n, b, b64);
         CK(cudaGetLastError(), "k_convert launch");
-        if ((rc = reliable_solve(H, X, b64, x64, false, tol, max_iters, st, iters, rel))) return rc;
+        if ((rc = mixed_solve(H, X, b64, x64, false, tol, max_iters, st, iters, rel))) return rc;
         k_convert<float, double><<<(n + 255) / 256, 256, 0, st>>>(n, x64, x);
         CK(cudaGetLastError(), "k_convert launch");
         CK(cudaStreamSynchronize(st), "solve");
