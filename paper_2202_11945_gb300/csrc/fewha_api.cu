@@ -97,7 +97,7 @@ struct fewha_handle {
     // typed device arrays (float or double per precision)
     void *pfy = nullptr, *pfx = nullptr, *dfw = nullptr, *D = nullptr, *Jinv = nullptr;
     void *c = nullptr, *b = nullptr, *b_prev = nullptr, *r = nullptr, *z = nullptr, *p = nullptr,
-         *q = nullptr, *phi = nullptr, *phic = nullptr, *u = nullptr, *a_prev = nullptr, *dm_tmp = nullptr,
+         *p2 = nullptr, *q = nullptr, *phi = nullptr, *phic = nullptr, *u = nullptr, *a_prev = nullptr, *dm_tmp = nullptr,
          *s_tmp = nullptr, *c_tmp = nullptr, *cgrad = nullptr, *lam = nullptr;
     double* gdot = nullptr;           // per-layer sums of the backward pass
     // closed loop (FEWHA_FLAG_CLOSED_LOOP): DM projection tables, pseudo-open-loop slopes
@@ -142,6 +142,12 @@ struct fewha_handle {
     void* ptw = nullptr;              // adjoint-projection weights (PairBufs::tw), T
     void* tailop = nullptr;           // the 8 x 8 tail levels as one matrix (Desc::tailop), T
     int* pti = nullptr;               // their first index and count (PairBufs::ti)
+    // tiles of the layers (Desc::tl, tunit, tslot) and the inverse tile kernel's shared memory
+    TileLayer* tl = nullptr;
+    int* tunit = nullptr;
+    unsigned* tslot = nullptr;
+    int n_units = 0;
+    size_t smem_tinv = 0;
     std::vector<int> box_host;
     void* pairV = nullptr;
     void* pairY = nullptr;
@@ -304,6 +310,10 @@ Desc<T> make_desc(const fewha_handle* H) {
     for (int l = 0; l < d.n_layers && !s.dlev.empty(); ++l)
         for (int k = 0; k <= MAXLEV; ++k) d.Dlev[l][k] = T(s.dlev[l * (MAXLEV + 1) + k]);
     d.tailop = static_cast<const T*>(H->tailop);
+    d.tl = H->tl;
+    d.tunit = H->tunit;
+    d.tslot = H->tslot;
+    d.n_units = H->n_units;
     for (int g = 0; g < d.n_wfs; ++g)
         for (int l = 0; l < d.n_layers; ++l)
             for (int k = 0; k < 4; ++k) d.box[g][l][k] = H->box_host[(g * MAXL + l) * 4 + k];
@@ -494,9 +504,7 @@ int launch_inv(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream
         record<T>(PUPD ? BK_INV_UPD : BK_INV).cl = a;
         return FEWHA_OK;
     }
-    CK(launch_k(H, k_cl_inv<T, PUPD>, dim3(CL, d.n_layers), dim3(cblk<T>()), H->smem_inv, st, d, a,
-                H->lay_inv),
-       "k_cl_inv launch");
+    CK(launch_k(H, k_tinv<T, PUPD>, dim3(d.n_units), dim3(TINV_NT), H->smem_tinv, st, d, a), "k_tinv launch");
     return FEWHA_OK;
 }
 
@@ -524,9 +532,10 @@ struct Defer {
 };
 
 // q = M x (Eq. 6); the p.q partials go to slot `slot` (PQ_SLOTS doubles per slot).
-// With pupdate, x is the CG direction p, first advanced to z + beta p (iteration `slot`).
+// With pold, x is the CG direction p = z + beta pold, formed first (iteration `slot`) in
+// another buffer than pold's.
 template <class T>
-int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int slot, bool pupdate,
+int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int slot, const T* pold,
                   cudaStream_t st, const Defer& df = Defer()) {
     T* phi = static_cast<T*>(H->phi);
     T* u = static_cast<T*>(H->u);
@@ -536,8 +545,9 @@ int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int sl
     a.rz_parts = df.rz_parts;
     a.rz_cnt = df.rz_cnt;
     a.rz_slot = df.rz_slot;
-    if (pupdate) {
-        a.pupd = static_cast<T*>(H->p);
+    if (pold) {
+        a.pupd = const_cast<T*>(pold);       // read only
+        a.pout = const_cast<T*>(x);
         a.zupd = static_cast<const T*>(H->z);
         a.iter = slot;
         rc = launch_inv<T, 1>(H, d, a, st);
@@ -601,21 +611,12 @@ template <class T>
 int enqueue_apply_init(fewha_handle* H, const Desc<T>& d, T* c, cudaStream_t st, bool defer = false) {
     const T* x = c;
     const int slot = PQ_SCRATCH_SLOT;
-    const bool pupdate = false;
     T* phi = static_cast<T*>(H->phi);
     T* u = static_cast<T*>(H->u);
     int rc;
     ClArgs<T> a = cl_args<T>(H, x, phi);
     a.zero_piston = 1;
-    if (pupdate) {
-        a.pupd = static_cast<T*>(H->p);
-        a.zupd = static_cast<const T*>(H->z);
-        a.iter = slot;
-        rc = launch_inv<T, 1>(H, d, a, st);
-    } else {
-        rc = launch_inv<T, 0>(H, d, a, st);
-    }
-    if (rc) return rc;
+    if ((rc = launch_inv<T, 0>(H, d, a, st))) return rc;
     if ((rc = launch_proj<T>(H, d, phi, st))) return rc;
     if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, u, st))) return rc;
     if ((rc = launch_projT<T>(H, d, u, st))) return rc;
@@ -719,6 +720,13 @@ int launch_pol(fewha_handle* H, const Desc<T>& d, const T* s, T* out, cudaStream
     return FEWHA_OK;
 }
 
+// Buffer of the CG direction of iteration k: two take turns, since the tiles that form p_k
+// read p_(k-1) in their halos.
+template <class T>
+T* dir_buf(fewha_handle* H, int k) {
+    return static_cast<T*>((k & 1) ? H->p2 : H->p);
+}
+
 // `iters` PCG iterations on M c = b (b in H->b), r0 explicit or warm.
 // With s_resid (the explicit residual, single instances), r0 comes from the slopes'
 // residual chain (enqueue_resid_init) and b is not formed.
@@ -749,7 +757,6 @@ int enqueue_pcg(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool warm, c
         } else {
             if ((rc = enqueue_apply_init<T>(H, d, c, st, defer))) return rc;
         }
-        T* p = static_cast<T*>(H->p);
         for (int k = 0; k < iters; ++k) {
             Defer df;
             df.pq = true;
@@ -762,8 +769,11 @@ int enqueue_pcg(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool warm, c
                 df.rz_cnt = d.n_layers * CL;
                 df.rz_slot = 0;
             }
-            if ((rc = enqueue_apply<T>(H, d, p, static_cast<T*>(H->q), k, k > 0, st, df))) return rc;
+            T* p = dir_buf<T>(H, k);
+            if ((rc = enqueue_apply<T>(H, d, p, static_cast<T*>(H->q), k, k > 0 ? dir_buf<T>(H, k - 1) : nullptr, st, df)))
+                return rc;
             VecArgs<T> v = vec_args<T>(H, c, k);
+            v.p = p;
             v.pq_cnt = d.n_layers * CL;
             v.defer_rz = k + 1 < iters ? 1 : 0;
             v.phic = phic;
@@ -777,13 +787,15 @@ int enqueue_pcg(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool warm, c
     } else if (s_resid) {
         if ((rc = enqueue_resid_init<T>(H, d, s_resid, c, st, false, nullptr, phic))) return rc;
     } else {
-        if ((rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, false, st))) return rc;
+        if ((rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, nullptr, st))) return rc;
         if ((rc = launch_vec<T, V_INIT>(H, d.n_c, vec_args<T>(H, c, 0), st))) return rc;
     }
-    T* p = static_cast<T*>(H->p);
     for (int k = 0; k < iters; ++k) {
-        if ((rc = enqueue_apply<T>(H, d, p, static_cast<T*>(H->q), k, k > 0, st))) return rc;
+        T* p = dir_buf<T>(H, k);
+        if ((rc = enqueue_apply<T>(H, d, p, static_cast<T*>(H->q), k, k > 0 ? dir_buf<T>(H, k - 1) : nullptr, st)))
+            return rc;
         VecArgs<T> v = vec_args<T>(H, c, k);
+        v.p = p;
         v.phic = phic;
         v.phip = static_cast<const T*>(H->phi);
         if ((rc = launch_vec<T, V_UPDATE>(H, d.n_c, v, st))) return rc;
@@ -845,7 +857,7 @@ int enqueue_pcg_aug(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool war
                       (rc = launch_aug<T, V_AUG_INIT>(H, d.n_c, v, a, st))))
             return rc;
     } else {
-        if (!warm && (rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, false, st)))
+        if (!warm && (rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, nullptr, st)))
             return rc;
         if (m > 0) {
             rc = warm ? launch_aug<T, V_AUG_R0_WARM>(H, d.n_c, v, a, st) : launch_aug<T, V_AUG_R0>(H, d.n_c, v, a, st);
@@ -877,7 +889,7 @@ int enqueue_pcg_aug(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool war
             rc = enqueue_apply_aug<T>(H, d, k > 0 ? Pn + (k - 1) * ld : nullptr, pk, static_cast<const T*>(H->z), qk,
                                       k, a, st, df, (defer && k > 0) ? H->npart : 0);
         } else {
-            rc = enqueue_apply<T>(H, d, pk, qk, k, false, st, df);   // p_0 = z_0 (no directions)
+            rc = enqueue_apply<T>(H, d, pk, qk, k, nullptr, st, df);   // p_0 = z_0 (no directions)
         }
         if (rc) return rc;
         v.p = pk;
@@ -1156,9 +1168,9 @@ int set_smem_limits(fewha_handle* H) {
         (rc = allow_smem(H, k_cl_fwd<T, LSRC_NODES, LDST_COEF>, H->smem_fwd)) ||
         (rc = allow_smem(H, k_cl_fwd<T, LSRC_NODES, LDST_APPLY_INIT>, H->smem_fwd)) ||
         (rc = allow_smem(H, k_cl_fwd<T, LSRC_NODES, LDST_RESID_INIT>, H->smem_fwd)) ||
-        (rc = allow_smem(H, k_cl_inv<T, 0>, H->smem_inv)) ||
-        (rc = allow_smem(H, k_cl_inv<T, 1>, H->smem_inv)) ||
-        (rc = allow_smem(H, k_cl_inv<T, 2>, H->smem_inv)) ||
+        (rc = allow_smem(H, k_tinv<T, 0>, H->smem_tinv)) ||
+        (rc = allow_smem(H, k_tinv<T, 1>, H->smem_tinv)) ||
+        (rc = allow_smem(H, k_tinv<T, 2>, H->smem_tinv)) ||
         (rc = allow_smem(H, k_cl_sensor<T, SSRC_PHI>, H->smem_sen)) ||
         (rc = allow_smem(H, k_cl_sensor<T, SSRC_SLOPES>, H->smem_sen)) ||
         (rc = allow_smem(H, k_cl_sensor<T, SSRC_RESID>, H->smem_sen)) ||
@@ -1181,6 +1193,91 @@ bool tail_used(const HostSetup& s) {
 // sensors, element counts in T units after a fixed header; every region starts on a
 // 16-byte boundary (cp.async targets).
 int round4(int x) { return (x + 3) & ~3; }
+
+// Tile side (log2) of layer l: 32 nodes, halved while the adjoint projection's tile with
+// its halo of 4 would touch more than 64 aperture nodes a side (a layer coarser than the
+// apertures), at least 8, at most the layer.
+int tile_log2(const HostSetup& s, size_t l) {
+    double rho = 0.0;                    // aperture nodes per layer node
+    for (size_t g = 0; g < s.G.size(); ++g) {
+        const size_t tp = (g * MAXL + l) * TAB;
+        const int N = s.G[g].N, span = std::max(1, s.pi0y[tp + N] - s.pi0y[tp]);
+        rho = std::max(rho, static_cast<double>(N) / span);
+    }
+    int lts = std::min(5, s.L[l].log2n);
+    while (lts > 3 && ((1 << lts) + 4) * rho > 64.0) --lts;
+    return lts;
+}
+
+// Tables of the tile kernels (TileLayer, the units and the coefficient slots of a tile).
+template <class T>
+int tile_tables(fewha_handle* H) {
+    const HostSetup& s = H->setup;
+    std::vector<TileLayer> tl(s.L.size());
+    std::vector<int> unit;
+    std::vector<unsigned> slot;
+    size_t smem = 0;
+    for (size_t l = 0; l < s.L.size(); ++l) {
+        const LayerInfo& L = s.L[l];
+        TileLayer& t = tl[l];
+        std::memset(&t, 0, sizeof(t));
+        t.lts = tile_log2(s, l);
+        t.side = L.n >> t.lts;
+        t.tail = H->tailop && (L.n >> (L.levels - 1)) == 2 && L.levels >= 4;
+        t.J = t.tail ? L.levels - 3 : L.levels;
+        t.w[0] = 1 << t.lts;
+        t.whole[0] = t.side == 1;
+        t.np[0] = t.w[0] / 2;
+        for (int j = 1; j <= t.J; ++j) {
+            const int m = L.n >> j;
+            t.w[j] = t.np[j - 1] + 2;
+            t.whole[j] = t.w[j] >= m || (t.tail && j == t.J);
+            if (t.whole[j]) t.w[j] = m;
+            // output pairs of level j's window, the most over the tiles
+            t.np[j] = m / 2;
+            if (!t.whole[j]) {
+                t.np[j] = 0;
+                for (int x = 0; x < t.side; ++x) {
+                    int st = x << t.lts;
+                    for (int k = 1; k <= j; ++k) st = (st >> 1) - 2;     // no whole level above j
+                    t.np[j] = std::max(t.np[j], ((st + t.w[j] - 1) >> 1) - (st >> 1) + 1);
+                }
+            }
+        }
+        int off = 0;
+        for (int j = 0; j <= t.J; ++j) {
+            t.magic[j] = t.np[j] > 0 ? (65536 + t.np[j] - 1) / t.np[j] : 0;
+            t.stride[j] = t.w[j] | 1;
+            t.base[j] = off;
+            if (j > 0) off += 4 * t.w[j] * t.stride[j];
+        }
+        t.tailb = off;
+        off += t.tail ? 64 : 0;
+        smem = std::max(smem, static_cast<size_t>((t.tail ? TAIL_N : 0) + off) * sizeof(T));
+        t.slot_off = static_cast<int>(slot.size());
+        auto put = [&](int j, int q, int w) {
+            for (int r = 0; r < w; ++r)
+                for (int c = 0; c < w; ++c)
+                    slot.push_back(static_cast<unsigned>(j | q << 4 | r << 6 | c << 12));
+        };
+        for (int j = 1; j <= t.J; ++j)
+            for (int q = 1; q < 4; ++q) put(j, q, t.w[j]);
+        if (t.tail)
+            put(0, 0, 8);
+        else
+            put(t.J, 0, t.w[t.J]);
+        t.slot_cnt = static_cast<int>(slot.size()) - t.slot_off;
+        for (int y = 0; y < t.side; ++y)
+            for (int x = 0; x < t.side; ++x) unit.push_back(static_cast<int>(l) | y << 8 | x << 16);
+    }
+    H->n_units = static_cast<int>(unit.size());
+    H->smem_tinv = smem;
+    int rc;
+    if ((rc = dalloc(H, &H->tl, tl.size())) || (rc = upload(H, H->tl, tl)) || (rc = dalloc(H, &H->tunit, unit.size())) ||
+        (rc = upload(H, H->tunit, unit)) || (rc = dalloc(H, &H->tslot, slot.size())) || (rc = upload(H, H->tslot, slot)))
+        return rc;
+    return FEWHA_OK;
+}
 
 template <class T>
 int cluster_layouts(fewha_handle* H) {
@@ -1483,7 +1580,7 @@ int typed_create(fewha_handle* H) {
         (rc = talloc(H, &H->Jinv, s.n_c)) || (rc = talloc(H, &H->c, s.n_c)) ||
         (rc = talloc(H, &H->b, s.n_c)) || (rc = talloc(H, &H->b_prev, s.n_c)) ||
         (rc = talloc(H, &H->r, s.n_c)) || (rc = talloc(H, &H->z, s.n_c)) ||
-        (rc = talloc(H, &H->p, s.n_c)) || (rc = talloc(H, &H->q, s.n_c)) ||
+        (rc = talloc(H, &H->p, s.n_c)) || (rc = talloc(H, &H->p2, s.n_c)) || (rc = talloc(H, &H->q, s.n_c)) ||
         (rc = talloc(H, &H->phi, s.n_c)) || (rc = talloc(H, &H->phic, s.n_c)) || (rc = talloc(H, &H->c_tmp, s.n_c)) ||
         (rc = talloc(H, &H->u, s.n_nodes)) || (rc = talloc(H, &H->a_prev, s.n_act)) ||
         (rc = talloc(H, &H->dm_tmp, s.n_act)) || (rc = talloc(H, &H->s_tmp, s.n_s)) ||
@@ -1507,7 +1604,7 @@ int typed_create(fewha_handle* H) {
     H->smem_layer = (2 * NWARP + 4) * sizeof(double) + static_cast<size_t>(s.max_n) * s.max_n * sizeof(T);
     H->smem_sensor = (2 * NWARP + 4 + 2 * MAXCOARSE) * sizeof(double) +
                      (static_cast<size_t>(s.max_N + 1) * (s.max_N + 1) + 2 * static_cast<size_t>(s.max_N) * s.max_N) * sizeof(T);
-    if ((rc = cluster_layouts<T>(H))) return rc;
+    if ((rc = cluster_layouts<T>(H)) || (rc = tile_tables<T>(H))) return rc;
     if ((rc = set_smem_limits<T>(H))) return rc;
     return setup_tables<T>(H);
 }
@@ -1652,8 +1749,8 @@ int solve_converged(fewha_handle* H, const T* b, T* x, bool warm, double tol, in
     double rzb = 0.0, rz = 0.0;
     CK(cudaMemcpyAsync(&rzb, H->gdot + MAXL, sizeof(double), cudaMemcpyDeviceToHost, st), "solve norm");
     int done = 0;
-    T* p = static_cast<T*>(H->p);
     T* q = static_cast<T*>(H->q);
+    int turn = 0;                                // direction of the newest iteration: dir_buf(turn)
     while (done < max_iters) {
         int last;                                // slot of the newest r.z total
         if (done == 0) {
@@ -1661,14 +1758,17 @@ int solve_converged(fewha_handle* H, const T* b, T* x, bool warm, double tol, in
             if ((rc = enqueue_pcg<T>(H, d, x, k, false, st))) return rc;
             done = k;
             last = k;
+            turn = k - 1;
         } else {
             // resume: slots (K-1, K) -> (0, 1), then iterations 1 .. k of the recurrence
             CK(cudaMemcpyAsync(H->rztot, H->rztot + FEWHA_MAX_ITERS - 1, 2 * sizeof(double),
                                cudaMemcpyDeviceToDevice, st), "solve resume");
             const int k = std::min(FEWHA_MAX_ITERS - 1, max_iters - done);
-            for (int j = 1; j <= k; ++j) {
-                if ((rc = enqueue_apply<T>(H, d, p, q, j, true, st))) return rc;
-                if ((rc = launch_vec<T, V_UPDATE>(H, d.n_c, vec_args<T>(H, x, j), st))) return rc;
+            for (int j = 1; j <= k; ++j, ++turn) {
+                VecArgs<T> v = vec_args<T>(H, x, j);
+                v.p = dir_buf<T>(H, turn + 1);
+                if ((rc = enqueue_apply<T>(H, d, v.p, q, j, dir_buf<T>(H, turn), st))) return rc;
+                if ((rc = launch_vec<T, V_UPDATE>(H, d.n_c, v, st))) return rc;
             }
             done += k;
             last = k + 1;
@@ -1757,7 +1857,6 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
     double* r64 = static_cast<double*>(X->r);
     double* q64 = static_cast<double*>(X->q);
     float* x32 = static_cast<float*>(H->c_tmp);
-    float* p = static_cast<float*>(H->p);
     float* q = static_cast<float*>(H->q);
     int rc;
     double bn2 = 0.0, rr2 = 0.0;
@@ -1766,7 +1865,7 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
     const int gl = std::min(4 * 152, (n + PBLK - 1) / PBLK);
     auto true_residual = [&]() -> int {
         int r2 = 0;
-        if ((r2 = enqueue_apply<double>(X, dx, x64, q64, PQ_SCRATCH_SLOT, false, st))) return fail(H, r2, X->err);
+        if ((r2 = enqueue_apply<double>(X, dx, x64, q64, PQ_SCRATCH_SLOT, nullptr, st))) return fail(H, r2, X->err);
         k_lin<double><<<gl, PBLK, 0, st>>>(n, 1.0, b64, -1.0, q64, 0.0, nullptr, nullptr, r64);
         CK(cudaGetLastError(), "k_lin launch");
         return twin_wnorm(H, X, r64, &rr2, st);
@@ -1785,11 +1884,15 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
         CK(cudaStreamSynchronize(st), "solve rz");
         double rz_upd = rz[0];
         int j0 = 0;
+        int turn = 0;                            // direction of the next iteration: dir_buf(turn)
         for (;;) {
             const int k = std::min(FEWHA_MAX_ITERS - j0, max_iters - done);
-            for (int j = j0; j < j0 + k; ++j) {
-                if ((rc = enqueue_apply<float>(H, d, p, q, j, j > 0, st))) return rc;
-                if ((rc = launch_vec<float, V_UPDATE>(H, n, vec_args<float>(H, x32, j), st))) return rc;
+            for (int j = j0; j < j0 + k; ++j, ++turn) {
+                VecArgs<float> vj = vec_args<float>(H, x32, j);
+                vj.p = dir_buf<float>(H, turn);
+                if ((rc = enqueue_apply<float>(H, d, vj.p, q, j, j > 0 ? dir_buf<float>(H, turn + 1) : nullptr, st)))
+                    return rc;
+                if ((rc = launch_vec<float, V_UPDATE>(H, n, vj, st))) return rc;
             }
             done += k;
             const int last = j0 + k;
@@ -1813,6 +1916,7 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
             if (!std::isfinite(rr2)) break;
             if (rel <= tol || done >= max_iters || !(rr2 > 0.0) || stopped) break;
             const double scn = std::sqrt(rr2), ratio = sc / scn;
+            v.p = dir_buf<float>(H, turn + 1);   // the newest direction
             k_refresh<float><<<H->npart, PBLK, 0, st>>>(n, r64, 1.0 / scn, ratio, 0, rz[0] * ratio * ratio, v);
             CK(cudaGetLastError(), "k_refresh launch");
             CK(cudaMemcpyAsync(&rz_upd, H->rztot + 1, sizeof(double), cudaMemcpyDeviceToHost, st), "solve rz");
@@ -2216,7 +2320,7 @@ int frame_vjp(fewha_handle* H, const T* s, const T* c0, const T* g_a, T* dm, T* 
     // ---- forward: b, r0 = b - M c0, then the iterations, every vector kept -------------
     if ((rc = enqueue_rhs<T>(H, d, s, static_cast<T*>(H->b), st))) return rc;
     CK(cudaMemcpyAsync(c, c0, n * sizeof(T), cudaMemcpyDeviceToDevice, st), "vjp c0");
-    if ((rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, false, st))) return rc;
+    if ((rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, nullptr, st))) return rc;
     VecArgs<T> v = vec_args<T>(H, c, 0);
     v.r = R;
     v.z = Z;
@@ -2230,7 +2334,7 @@ int frame_vjp(fewha_handle* H, const T* s, const T* c0, const T* g_a, T* dm, T* 
         if (i > 0)
             rc = enqueue_apply_aug<T>(H, d, P + (i - 1) * ld, P + i * ld, Z + i * ld, Q + i * ld, i, a, st);
         else
-            rc = enqueue_apply<T>(H, d, P, Q, 0, false, st);
+            rc = enqueue_apply<T>(H, d, P, Q, 0, nullptr, st);
         if (rc) return rc;
         CK(cudaMemcpyAsync(R + (i + 1) * ld, R + i * ld, n * sizeof(T), cudaMemcpyDeviceToDevice, st), "vjp r");
         VecArgs<T> w = vec_args<T>(H, c, i);
@@ -2277,7 +2381,7 @@ int frame_vjp(fewha_handle* H, const T* s, const T* c0, const T* g_a, T* dm, T* 
         k_vjp<T, VJ_C><<<gv, PBLK, 0, st>>>(n, va);
         CK(cudaGetLastError(), "k_vjp launch");
         // q_i = M p_i: p_bar_i += M q_bar (added by the next VJ_A, or VJ_E)
-        if ((rc = enqueue_apply<T>(H, d, qbar, scratch, PQ_SCRATCH_SLOT, false, st))) return rc;
+        if ((rc = enqueue_apply<T>(H, d, qbar, scratch, PQ_SCRATCH_SLOT, nullptr, st))) return rc;
     }
     // p_0 = z_0, rho_0 = r_0 . z_0, z_0 = J^-1 r_0, r_0 = b - M c0: b_bar = r_bar_0
     if (k > 0) {
@@ -2334,7 +2438,7 @@ size_t barg_size(int kind) {
 
 size_t bsmem(const fewha_handle* H, int kind) {
     switch (kind) {
-        case BK_INV: case BK_INV_UPD: return H->smem_inv;
+        case BK_INV: case BK_INV_UPD: return H->smem_tinv;
         case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return H->smem_fwd;
         case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return H->smem_sen;
         case BK_PROJ: return H->smem_proj;
@@ -2397,7 +2501,7 @@ void batch_pack(const std::vector<Recorder<T>>& recs, const std::vector<int>& np
             const BStep<T>& st = recs[i].steps[j];
             unsigned char* dst = out.data() + offs[j] + i * sz;
             switch (bkind_list(kind)) {
-                case BL_LAYER: std::memcpy(dst, &st.cl, sz); break;
+                case BL_LAYER: case BL_TILE: std::memcpy(dst, &st.cl, sz); break;
                 case BL_SENSOR: std::memcpy(dst, &st.sa, sz); break;
                 case BL_PAIR: std::memcpy(dst, &st.ptr, sz); break;
                 case BL_FIT: std::memcpy(dst, &st.fa, sz); break;
@@ -2449,6 +2553,7 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
         const fewha_handle* H = B->h[i];
         const int g = grp[i], nl = static_cast<int>(H->setup.L.size()), nw = static_cast<int>(H->setup.G.size());
         for (int l = 0; l < nl; ++l) lists[g * BL_COUNT + BL_LAYER].push_back({i, l});
+        for (int k = 0; k < H->n_units; ++k) lists[g * BL_COUNT + BL_TILE].push_back({i, k});
         for (int w = 0; w < nw; ++w) lists[g * BL_COUNT + BL_SENSOR].push_back({i, w});
         for (int w = 0; w < nw; ++w)
             for (int l = 0; l < nl; ++l) lists[g * BL_COUNT + BL_PAIR].push_back({i, w * MAXL + l});
@@ -2463,7 +2568,6 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
         std::memset(&I, 0, sizeof(I));
         I.d = make_desc<T>(H);
         I.lay_fwd = H->lay_fwd;
-        I.lay_inv = H->lay_inv;
         I.lay_sen = H->lay_sen;
         I.pb = pair_bufs<T>(H);
         I.desc_bytes = static_cast<int>(offsetof(Desc<T>, box) + static_cast<size_t>(I.d.n_wfs) * MAXL * 4 * sizeof(int));
@@ -2841,7 +2945,7 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
     int rc = 0;
     switch (op) {
         case 0:  // M
-            return enqueue_apply<T>(H, d, x, y, PQ_SCRATCH_SLOT, false, st);
+            return enqueue_apply<T>(H, d, x, y, PQ_SCRATCH_SLOT, nullptr, st);
         case 1:  // rhs
             return enqueue_rhs<T>(H, d, x, y, st);
         case 2:  // dwt
@@ -2891,6 +2995,7 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
             case FEWHA_STAGE_IDWT: {
                 ClArgs<T> a = cl_args<T>(H, p, phi);
                 a.pupd = p;
+                a.pout = static_cast<T*>(H->p2);
                 a.zupd = static_cast<const T*>(H->z);
                 a.iter = 1;
                 a.zero_piston = 1;

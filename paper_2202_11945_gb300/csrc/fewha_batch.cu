@@ -22,17 +22,15 @@ __device__ __forceinline__ void load_desc(Desc<T>& sd, const BInst<T>* __restric
 }
 
 template <class T, int PUPD>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(cblk<T>(), 1)
-    kb_cl_inv(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args,
-              const BItem* __restrict__ items) {
+__global__ void __launch_bounds__(TINV_NT)
+    kb_tinv(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
     __shared__ __align__(16) Desc<T> sd;
     pdl_enter();
-    const BItem it = items[blockIdx.y];
+    const BItem it = items[blockIdx.x];
     const BInst<T>* I = inst + it.inst;
     load_desc<T>(sd, I);
     const ClArgs<T> a = args[it.inst];
-    const ClLayout lay = I->lay_inv;
-    cl_inv_body<T, PUPD>(sd, a, lay, it.unit);
+    tinv_body<T, PUPD>(sd, a, it.unit);
 }
 
 template <class T, int DST>
@@ -122,8 +120,8 @@ const void* kernel_of(int kind, int v) {
     constexpr int NP = cblk<T>(), NH = cblk<T>() / 2;
     const bool half = (v & 1) != 0, t4 = (v & 2) != 0;
     switch (kind) {
-        case BK_INV: return reinterpret_cast<const void*>(kb_cl_inv<T, 0>);
-        case BK_INV_UPD: return reinterpret_cast<const void*>(kb_cl_inv<T, 1>);
+        case BK_INV: return reinterpret_cast<const void*>(kb_tinv<T, 0>);
+        case BK_INV_UPD: return reinterpret_cast<const void*>(kb_tinv<T, 1>);
         case BK_PROJ:
             return half ? reinterpret_cast<const void*>(kb_proj<T, NH>) : reinterpret_cast<const void*>(kb_proj<T, NP>);
         case BK_SEN_PHI: return reinterpret_cast<const void*>(kb_cl_sensor<T, SSRC_PHI>);
@@ -218,8 +216,8 @@ cudaError_t batch_launch(const BLaunch& L, cudaStream_t st) {
     const VecArgs<T>* va = static_cast<const VecArgs<T>*>(L.args);
     const FitArgs<T>* fa = static_cast<const FitArgs<T>*>(L.args);
     switch (L.kind) {
-        case BK_INV: return launch_b(L.pdl, kb_cl_inv<T, 0>, cg, nt, L.smem, st, I, ca, L.items);
-        case BK_INV_UPD: return launch_b(L.pdl, kb_cl_inv<T, 1>, cg, nt, L.smem, st, I, ca, L.items);
+        case BK_INV: return launch_b(L.pdl, kb_tinv<T, 0>, pg, dim3(TINV_NT), L.smem, st, I, ca, L.items);
+        case BK_INV_UPD: return launch_b(L.pdl, kb_tinv<T, 1>, pg, dim3(TINV_NT), L.smem, st, I, ca, L.items);
         case BK_FWD_APPLY: return launch_b(L.pdl, kb_cl_fwd<T, LDST_APPLY>, cg, nt, L.smem, st, I, ca, L.items);
         case BK_FWD_COEF: return launch_b(L.pdl, kb_cl_fwd<T, LDST_COEF>, cg, nt, L.smem, st, I, ca, L.items);
         case BK_FWD_RINIT: return launch_b(L.pdl, kb_cl_fwd<T, LDST_RESID_INIT>, cg, nt, L.smem, st, I, ca, L.items);

@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "fewha_pair.cuh"
+#include "fewha_tile.cuh"
 
 namespace fewha {
 
@@ -21,7 +22,7 @@ struct BItem {
 template <class T>
 struct alignas(16) BInst {
     Desc<T> d;
-    ClLayout lay_fwd, lay_inv;
+    ClLayout lay_fwd;
     SensorLayout lay_sen;
     PairBufs<T> pb;
     int desc_bytes;     // leading bytes of d that the kernels read (through the last sensor's boxes)
@@ -59,11 +60,12 @@ enum BKind {
 };
 
 // Which work list a step kind runs over.
-enum BList { BL_LAYER = 0, BL_SENSOR, BL_PAIR, BL_VEC, BL_FIT, BL_COUNT };
+enum BList { BL_LAYER = 0, BL_TILE, BL_SENSOR, BL_PAIR, BL_VEC, BL_FIT, BL_COUNT };
 
 inline int bkind_list(int kind) {
     switch (kind) {
-        case BK_INV: case BK_INV_UPD: case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return BL_LAYER;
+        case BK_INV: case BK_INV_UPD: return BL_TILE;
+        case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return BL_LAYER;
         case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return BL_SENSOR;
         case BK_PROJ: case BK_PROJT: return BL_PAIR;
         case BK_FIT: return BL_FIT;

@@ -1055,13 +1055,6 @@ __device__ __forceinline__ void cl_inv_body(const Desc<T>& d, const ClArgs<T>& a
     }
 }
 
-template <class T, int PUPD>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(cblk<T>(), 1)
-    k_cl_inv(__grid_constant__ const Desc<T> d, __grid_constant__ const ClArgs<T> a,
-             __grid_constant__ const ClLayout lay) {
-    cl_inv_body<T, PUPD>(d, a, lay, blockIdx.y);
-}
-
 // ---------------------------------------------------------------------------
 // Sensor kernel (cluster per sensor): P_g (Sec. 2), Gamma_g, C_hat_g^-1 (Eq. 2, Sec. 3.2)
 // and Gamma_g^T, each CTA on a band of subaperture rows.  SRC_PHI: slopes of the

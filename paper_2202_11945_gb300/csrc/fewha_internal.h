@@ -26,6 +26,19 @@ struct LayerInfo {
     int full;     // levels == log2n: the LL band is the single piston coefficient
 };
 
+// Tiles of a layer (fewha_tile.cuh): ts = 1 << lts nodes a side, `side` tiles a side.  Level j
+// = 1 .. J of the tile's synthesis holds a window of w[j] coefficients a side of each
+// sub-band (the whole sub-band where whole[j]); np[j] output pairs a side give level j's
+// window (j = 0: the tile itself).  Shared-memory offsets in elements.
+struct TileLayer {
+    int lts, side;
+    int J;                  // coarsest level with windows of its own
+    int tail;               // level J's LL block is the 8 x 8 block of the tail operator
+    int tailb;              // that operator's input block
+    int slot_off, slot_cnt; // the tile's coefficients in Desc::tslot
+    int w[8], np[8], magic[8], base[8], stride[8], whole[8];
+};
+
 struct WfsInfo {
     int N;          // fine subapertures per side (n_sub * nb)
     int nb;         // fine per coarse (1: ordinary sensor)
@@ -92,6 +105,12 @@ struct alignas(16) Desc {   // 16-byte multiple: batched kernels copy it in 16-b
     // D per (layer, level): detail level k = 1 .. levels (1 the finest), levels + 1 the LL band
     T Dlev[MAXL][9];
     const T* tailop;   // analysis of the 8 x 8 tail levels (64 x TAIL_LD), or null
+    // tiles of the layers (n_units in all): per layer, per unit (layer | tile row << 8 | tile
+    // column << 16), and the coefficient slots of a layer's tile (see tinv_body)
+    const TileLayer* tl;
+    const int* tunit;
+    const unsigned* tslot;
+    int n_units;
     // footprint box of each (sensor, layer) pair: row0, rows, col0, cols (16-byte aligned
     // column superset); kept in the descriptor so that warps read it from the constant bank
     int box[MAXG][MAXL][4];
