@@ -1109,16 +1109,8 @@ int setup_tables(fewha_handle* H) {
         return FEWHA_OK;
     };
     if ((rc = conv(H->pfy, s.pfy)) || (rc = conv(H->pfx, s.pfx)) || (rc = conv(H->dfw, s.dfw))) return rc;
-    // wavelet taps
-    float h32[6], g32[6];
-    for (int t = 0; t < 6; ++t) {
-        h32[t] = static_cast<float>(s.taps_h[t]);
-        g32[t] = static_cast<float>(s.taps_g[t]);
-    }
-    CK(cudaMemcpyToSymbol(c_h32, h32, sizeof(h32)), "taps");
-    CK(cudaMemcpyToSymbol(c_g32, g32, sizeof(g32)), "taps");
-    CK(cudaMemcpyToSymbol(c_h64, s.taps_h, sizeof(s.taps_h)), "taps");
-    CK(cudaMemcpyToSymbol(c_g64, s.taps_g, sizeof(s.taps_g)), "taps");
+    for (int t = 0; t < 6; ++t)
+        if (s.taps_h[t] != db3_h(t)) return fail(H, FEWHA_ERR_CUDA, "wavelet taps differ from the kernels'");
     return compute_diagonals<T>(H);
 }
 
@@ -2611,7 +2603,6 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
             if (bkind_list(kind) != BL_VEC && smem[g * BK_COUNT + kind] > lim)
                 return bfail(B, FEWHA_ERR_LIMIT, "batched tile above the per-CTA shared-memory limit");
     }
-    BCK(batch_set_taps(B->h[0]->setup.taps_h, B->h[0]->setup.taps_g), "batch taps");
     // launch shapes: projection CTA size, adjoint-projection taps, vector CTA size
     int kmax = 0;
     for (int i = 0; i < n; ++i) kmax = std::max(kmax, B->h[i]->kmax);

@@ -152,19 +152,6 @@ const void* kernel_of(int kind, int v) {
 
 }  // namespace
 
-cudaError_t batch_set_taps(const double* h, const double* g) {
-    float h32[6], g32[6];
-    for (int k = 0; k < 6; ++k) {
-        h32[k] = static_cast<float>(h[k]);
-        g32[k] = static_cast<float>(g[k]);
-    }
-    cudaError_t e = cudaMemcpyToSymbol(c_h32, h32, sizeof(h32));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_g32, g32, sizeof(g32));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_h64, h, 6 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_g64, g, 6 * sizeof(double));
-    return e;
-}
-
 template <class T>
 cudaError_t batch_smem_limit(int kind, size_t* bytes) {
     if (bkind_list(kind) == BL_VEC) {

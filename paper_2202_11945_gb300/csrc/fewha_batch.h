@@ -91,10 +91,6 @@ struct BLaunch {
 template <class T>
 cudaError_t batch_launch(const BLaunch& L, cudaStream_t st);
 
-// The db3 taps of the batched kernels: __constant__ memory is per translation unit, so
-// this unit's copy is filled separately (per device, before the first batched launch).
-cudaError_t batch_set_taps(const double* h, const double* g);
-
 // Largest dynamic shared memory a batched kernel of this kind accepts (over its launch
 // shapes); sets the kernels' attribute to it on first use (per device).
 template <class T>
