@@ -142,12 +142,25 @@ struct fewha_handle {
     void* ptw = nullptr;              // adjoint-projection weights (PairBufs::tw), T
     void* tailop = nullptr;           // the 8 x 8 tail levels as one matrix (Desc::tailop), T
     int* pti = nullptr;               // their first index and count (PairBufs::ti)
-    // tiles of the layers (Desc::tl, tunit, tslot) and the inverse tile kernel's shared memory
+    // tiles and bands of the layers (Desc::tl, tslot, brow, tcl and the tables beside them),
+    // the forward kernels' LL blocks and band shares, shared-memory layouts
     TileLayer* tl = nullptr;
-    int* tunit = nullptr;
-    unsigned* tslot = nullptr;
-    int n_units = 0;
-    size_t smem_tinv = 0;
+    TilePlace* tslot = nullptr;
+    void *brow = nullptr, *ll = nullptr;
+    int *tcl = nullptr, *bsrc = nullptr;
+    // sensor kernel's tables (Desc::txi ...)
+    WfsInfo* gdev = nullptr;
+    int *txi = nullptr, *tyi = nullptr, *tcin = nullptr, *tsco = nullptr, *tybox = nullptr;
+    void *txf = nullptr, *tyf = nullptr, *tcw = nullptr;
+    int tnp = 0, tcols = 0, tks = 0;
+    bool wide_cluster = false;        // the sensor kernel runs in clusters of 16 CTAs
+    double* tshare = nullptr;
+    int n_tu = 0, n_bu = 0, n_tcl = 0, tslot_ld = 0;
+    int tu0[MAXL + 1] = {}, bu0[MAXL + 1] = {}, tcnt[MAXL] = {}, broff[MAXL] = {}, bkt[MAXL] = {};
+    TfLayout lay_tf{};
+    TcLayout lay_tc{};
+    TsLayout lay_ts[2] = {};          // clusters of 16 and of 8
+    size_t smem_tinv = 0, smem_tf = 0, smem_tc = 0, smem_ts[2] = {0, 0};
     std::vector<int> box_host;
     void* pairV = nullptr;
     void* pairY = nullptr;
@@ -311,9 +324,29 @@ Desc<T> make_desc(const fewha_handle* H) {
         for (int k = 0; k <= MAXLEV; ++k) d.Dlev[l][k] = T(s.dlev[l * (MAXLEV + 1) + k]);
     d.tailop = static_cast<const T*>(H->tailop);
     d.tl = H->tl;
-    d.tunit = H->tunit;
     d.tslot = H->tslot;
-    d.n_units = H->n_units;
+    d.brow = static_cast<const T*>(H->brow);
+    d.tcl = H->tcl;
+    d.bsrc = H->bsrc;
+    d.txi = H->txi;
+    d.gdev = H->gdev;
+    d.tyi = H->tyi;
+    d.txf = static_cast<const T*>(H->txf);
+    d.tyf = static_cast<const T*>(H->tyf);
+    d.tcw = static_cast<const T*>(H->tcw);
+    d.tcin = H->tcin;
+    d.tsco = H->tsco;
+    d.tybox = H->tybox;
+    d.tnp = H->tnp;
+    d.tcols = H->tcols;
+    d.tks = H->tks;
+    d.tslot_ld = H->tslot_ld;
+    d.n_tcl = H->n_tcl;
+    std::copy(std::begin(H->tu0), std::end(H->tu0), d.tu0);
+    std::copy(std::begin(H->bu0), std::end(H->bu0), d.bu0);
+    std::copy(std::begin(H->tcnt), std::end(H->tcnt), d.tcnt);
+    std::copy(std::begin(H->broff), std::end(H->broff), d.broff);
+    std::copy(std::begin(H->bkt), std::end(H->bkt), d.bkt);
     for (int g = 0; g < d.n_wfs; ++g)
         for (int l = 0; l < d.n_layers; ++l)
             for (int k = 0; k < 4; ++k) d.box[g][l][k] = H->box_host[(g * MAXL + l) * 4 + k];
@@ -348,7 +381,6 @@ struct BStep {
     ClArgs<T> cl;
     SensorArgs<T> sa;
     VecArgs<T> va;
-    const T* ptr;
     FitArgs<T> fa;
 };
 
@@ -437,6 +469,8 @@ ClArgs<T> cl_args(fewha_handle* H, const T* in, T* out) {
     a.in = in;
     a.out = out;
     a.pcg = pcg_slots(H);
+    a.ll = static_cast<T*>(H->ll);
+    a.tshare = H->tshare;
     return a;
 }
 
@@ -455,46 +489,21 @@ PairBufs<T> pair_bufs(fewha_handle* H) {
     return pb;
 }
 
-template <class T>
-int launch_proj(fewha_handle* H, const Desc<T>& d, const T* phi, cudaStream_t st) {
-    if (recorder<T>()) {
-        record<T>(BK_PROJ).ptr = phi;
-        return FEWHA_OK;
-    }
-    CK(launch_k(H, k_proj<T>, dim3(d.n_wfs, d.n_layers), dim3(cblk<T>()), H->smem_proj, st, d, phi,
-                pair_bufs<T>(H)),
-       "k_proj launch");
-    return FEWHA_OK;
-}
-
-template <class T>
-int launch_projT(fewha_handle* H, const Desc<T>& d, const T* u, cudaStream_t st) {
-    if (recorder<T>()) {
-        record<T>(BK_PROJT).ptr = u;
-        return FEWHA_OK;
-    }
-    if (H->kmax <= 4)
-        CK(launch_k(H, k_projT<T, 4>, dim3(d.n_wfs, d.n_layers), dim3(cblk<T>()), H->smem_projT, st, d, u,
-                    pair_bufs<T>(H)),
-           "k_projT launch");
-    else
-        CK(launch_k(H, k_projT<T, KMAX>, dim3(d.n_wfs, d.n_layers), dim3(cblk<T>()), H->smem_projT, st, d, u,
-                    pair_bufs<T>(H)),
-           "k_projT launch");
-    return FEWHA_OK;
-}
-
-template <class T, int SRC, int DST>
+// c = W sum_g P_g^T u_g with the epilogue DST: the bands, then the coarse levels of the
+// layers of several bands.
+template <class T, int DST>
 int launch_fwd(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream_t st) {
     if (recorder<T>()) {
-        if (SRC != LSRC_NODES || (DST != LDST_APPLY && DST != LDST_COEF && DST != LDST_RESID_INIT))
-            return fail(H, FEWHA_ERR_INVALID_ARG, "step without a batched form");
+        if (DST == LDST_APPLY_INIT) return fail(H, FEWHA_ERR_INVALID_ARG, "step without a batched form");
         record<T>(DST == LDST_APPLY ? BK_FWD_APPLY : DST == LDST_RESID_INIT ? BK_FWD_RINIT : BK_FWD_COEF).cl = a;
+        record<T>(DST == LDST_APPLY ? BK_TC_APPLY : DST == LDST_RESID_INIT ? BK_TC_RINIT : BK_TC_COEF).cl = a;
         return FEWHA_OK;
     }
-    CK(launch_k(H, k_cl_fwd<T, SRC, DST>, dim3(CL, d.n_layers), dim3(cblk<T>()), H->smem_fwd, st, d, a,
-                H->lay_fwd, pair_bufs<T>(H)),
-       "k_cl_fwd launch");
+    CK(launch_k(H, k_tfwd<T, DST>, dim3(H->n_bu), dim3(cblk<T>()), H->smem_tf, st, d, a, H->lay_tf, pair_bufs<T>(H)),
+       "k_tfwd launch");
+    if (d.n_tcl > 0)
+        CK(launch_k(H, k_tcoarse<T, DST>, dim3(d.n_tcl), dim3(cblk<T>()), H->smem_tc, st, d, a, H->lay_tc),
+           "k_tcoarse launch");
     return FEWHA_OK;
 }
 
@@ -504,20 +513,26 @@ int launch_inv(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream
         record<T>(PUPD ? BK_INV_UPD : BK_INV).cl = a;
         return FEWHA_OK;
     }
-    CK(launch_k(H, k_tinv<T, PUPD>, dim3(d.n_units), dim3(TINV_NT), H->smem_tinv, st, d, a), "k_tinv launch");
+    CK(launch_k(H, k_tinv<T, PUPD>, dim3(H->n_tu), dim3(TINV_NT), H->smem_tinv, st, d, a), "k_tinv launch");
     return FEWHA_OK;
 }
 
+// The sensor kernel from layers phi (PHI), measured slopes s (SLOPES) or both (RESID).
 template <class T, int SRC>
-int launch_csensor(fewha_handle* H, const Desc<T>& d, const T* in, T* out, cudaStream_t st) {
-    SensorArgs<T> a{in, out, H->status};
+int launch_csensor(fewha_handle* H, const Desc<T>& d, const T* phi, const T* s, cudaStream_t st) {
+    SensorArgs<T> a{s, nullptr, H->status, phi};
     if (recorder<T>()) {
         record<T>(SRC == SSRC_PHI ? BK_SEN_PHI : SRC == SSRC_RESID ? BK_SEN_RESID : BK_SEN_SLOPES).sa = a;
         return FEWHA_OK;
     }
-    CK(launch_k(H, k_cl_sensor<T, SRC>, dim3(CL, d.n_wfs), dim3(cblk<T>()), H->smem_sen, st, d, a,
-                H->lay_sen, pair_bufs<T>(H)),
-       "k_cl_sensor launch");
+    if (H->wide_cluster)
+        CK(launch_k(H, k_tsen<T, SRC, 16>, dim3(16, d.n_wfs), dim3(tsnt<T>()), H->smem_ts[0], st, d, a, H->lay_ts[0],
+                    pair_bufs<T>(H)),
+           "k_tsen launch");
+    else
+        CK(launch_k(H, k_tsen<T, SRC, 8>, dim3(8, d.n_wfs), dim3(tsnt<T>()), H->smem_ts[1], st, d, a, H->lay_ts[1],
+                    pair_bufs<T>(H)),
+           "k_tsen launch");
     return FEWHA_OK;
 }
 
@@ -538,7 +553,6 @@ template <class T>
 int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int slot, const T* pold,
                   cudaStream_t st, const Defer& df = Defer()) {
     T* phi = static_cast<T*>(H->phi);
-    T* u = static_cast<T*>(H->u);
     int rc;
     ClArgs<T> a = cl_args<T>(H, x, phi);
     a.zero_piston = 1;                 // the data path's input leaves the piston out
@@ -555,15 +569,13 @@ int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int sl
         rc = launch_inv<T, 0>(H, d, a, st);
     }
     if (rc) return rc;
-    if ((rc = launch_proj<T>(H, d, phi, st))) return rc;
-    if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, u, st))) return rc;
-    if ((rc = launch_projT<T>(H, d, u, st))) return rc;
-    ClArgs<T> b = cl_args<T>(H, u, qout);
+    if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st))) return rc;
+    ClArgs<T> b = cl_args<T>(H, nullptr, qout);
     b.pin = x;
     b.iter = slot;
     b.zero_piston = 1;
     b.defer_total = df.pq ? 1 : 0;
-    return launch_fwd<T, LSRC_NODES, LDST_APPLY>(H, d, b, st);
+    return launch_fwd<T, LDST_APPLY>(H, d, b, st);
 }
 
 // q = M p_new with the direction update of the augmented PCG (Sec. 3.4) fused into the
@@ -574,7 +586,6 @@ int enqueue_apply_aug(fewha_handle* H, const Desc<T>& d, const T* pold, T* pnew,
                       const AugArgs<T>& aug, cudaStream_t st, const Defer& df = Defer(),
                       int aug_pcnt = 0) {
     T* phi = static_cast<T*>(H->phi);
-    T* u = static_cast<T*>(H->u);
     int rc;
     ClArgs<T> a = cl_args<T>(H, nullptr, phi);
     a.zero_piston = 1;
@@ -593,34 +604,29 @@ int enqueue_apply_aug(fewha_handle* H, const Desc<T>& d, const T* pold, T* pnew,
     a.rz_cnt = df.rz_cnt;
     a.rz_slot = df.rz_slot;
     if ((rc = launch_inv<T, 2>(H, d, a, st))) return rc;
-    if ((rc = launch_proj<T>(H, d, phi, st))) return rc;
-    if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, u, st))) return rc;
-    if ((rc = launch_projT<T>(H, d, u, st))) return rc;
-    ClArgs<T> b = cl_args<T>(H, u, qout);
+    if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st))) return rc;
+    ClArgs<T> b = cl_args<T>(H, nullptr, qout);
     b.pin = pnew;
     b.iter = slot;
     b.zero_piston = 1;
     b.defer_total = df.pq ? 1 : 0;
-    return launch_fwd<T, LSRC_NODES, LDST_APPLY>(H, d, b, st);
+    return launch_fwd<T, LDST_APPLY>(H, d, b, st);
 }
 
 // r = b - M c0 (as enqueue_apply, then V_INIT) with the initial residual's vector step fused
 // into the forward kernel's epilogue: r0, z0 = J^-1 r0, p0 = z0, b_prev = b, r.z into slot 0
-// (with `defer`, only its n_layers * CL shares, at the start of the r.z slots).
+// (with `defer`, only its n_layers shares, at the start of the r.z slots).
 template <class T>
 int enqueue_apply_init(fewha_handle* H, const Desc<T>& d, T* c, cudaStream_t st, bool defer = false) {
     const T* x = c;
     const int slot = PQ_SCRATCH_SLOT;
     T* phi = static_cast<T*>(H->phi);
-    T* u = static_cast<T*>(H->u);
     int rc;
     ClArgs<T> a = cl_args<T>(H, x, phi);
     a.zero_piston = 1;
     if ((rc = launch_inv<T, 0>(H, d, a, st))) return rc;
-    if ((rc = launch_proj<T>(H, d, phi, st))) return rc;
-    if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, u, st))) return rc;
-    if ((rc = launch_projT<T>(H, d, u, st))) return rc;
-    ClArgs<T> b = cl_args<T>(H, u, static_cast<T*>(H->q));
+    if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st))) return rc;
+    ClArgs<T> b = cl_args<T>(H, nullptr, static_cast<T*>(H->q));
     b.pin = x;
     b.iter = slot;
     b.zero_piston = 1;
@@ -633,7 +639,7 @@ int enqueue_apply_init(fewha_handle* H, const Desc<T>& d, T* c, cudaStream_t st,
     b.rzslot = 0;
     b.rzp = H->rzpart;
     b.defer_total = defer ? 1 : 0;
-    return launch_fwd<T, LSRC_NODES, LDST_APPLY_INIT>(H, d, b, st);
+    return launch_fwd<T, LDST_APPLY_INIT>(H, d, b, st);
 }
 
 // r0 = b - M c0 formed in one chain, from the slopes' residual: the sensor kernel takes
@@ -646,15 +652,12 @@ template <class T>
 int enqueue_resid_init(fewha_handle* H, const Desc<T>& d, const T* s, T* c, cudaStream_t st, bool defer,
                        T* p0 = nullptr, T* phi_out = nullptr) {
     T* phi = phi_out ? phi_out : static_cast<T*>(H->phi);
-    T* u = static_cast<T*>(H->u);
     int rc;
     ClArgs<T> a = cl_args<T>(H, c, phi);
     a.zero_piston = 1;
     if ((rc = launch_inv<T, 0>(H, d, a, st))) return rc;
-    if ((rc = launch_proj<T>(H, d, phi, st))) return rc;
-    if ((rc = launch_csensor<T, SSRC_RESID>(H, d, s, u, st))) return rc;
-    if ((rc = launch_projT<T>(H, d, u, st))) return rc;
-    ClArgs<T> b = cl_args<T>(H, u, static_cast<T*>(H->q));
+    if ((rc = launch_csensor<T, SSRC_RESID>(H, d, phi, s, st))) return rc;
+    ClArgs<T> b = cl_args<T>(H, nullptr, static_cast<T*>(H->q));
     b.pin = c;
     b.iter = PQ_SCRATCH_SLOT;
     b.zero_piston = 1;
@@ -665,18 +668,16 @@ int enqueue_resid_init(fewha_handle* H, const Desc<T>& d, const T* s, T* c, cuda
     b.rzslot = 0;
     b.rzp = H->rzpart;
     b.defer_total = defer ? 1 : 0;
-    return launch_fwd<T, LSRC_NODES, LDST_RESID_INIT>(H, d, b, st);
+    return launch_fwd<T, LDST_RESID_INIT>(H, d, b, st);
 }
 
 template <class T>
 int enqueue_rhs(fewha_handle* H, const Desc<T>& d, const T* s, T* bout, cudaStream_t st) {
-    T* u = static_cast<T*>(H->u);
     int rc;
-    if ((rc = launch_csensor<T, SSRC_SLOPES>(H, d, s, u, st))) return rc;
-    if ((rc = launch_projT<T>(H, d, u, st))) return rc;
-    ClArgs<T> a = cl_args<T>(H, u, bout);
+    if ((rc = launch_csensor<T, SSRC_SLOPES>(H, d, nullptr, s, st))) return rc;
+    ClArgs<T> a = cl_args<T>(H, nullptr, bout);
     a.zero_piston = 1;
-    return launch_fwd<T, LSRC_NODES, LDST_COEF>(H, d, a, st);
+    return launch_fwd<T, LDST_COEF>(H, d, a, st);
 }
 
 int vec_grid(const fewha_handle* H) { return H->npart; }
@@ -766,7 +767,7 @@ int enqueue_pcg(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool warm, c
                 df.rz_slot = k;
             } else if (!warm) {
                 df.rz_parts = H->rzpart;
-                df.rz_cnt = d.n_layers * CL;
+                df.rz_cnt = d.n_layers;
                 df.rz_slot = 0;
             }
             T* p = dir_buf<T>(H, k);
@@ -774,7 +775,7 @@ int enqueue_pcg(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool warm, c
                 return rc;
             VecArgs<T> v = vec_args<T>(H, c, k);
             v.p = p;
-            v.pq_cnt = d.n_layers * CL;
+            v.pq_cnt = d.n_layers;
             v.defer_rz = k + 1 < iters ? 1 : 0;
             v.phic = phic;
             v.phip = static_cast<const T*>(H->phi);
@@ -894,7 +895,7 @@ int enqueue_pcg_aug(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool war
         if (rc) return rc;
         v.p = pk;
         v.q = qk;
-        v.pq_cnt = defer ? d.n_layers * CL : 0;
+        v.pq_cnt = defer ? d.n_layers : 0;
         v.defer_rz = (defer && k + 1 < iters) ? 1 : 0;
         a.mu_next = (m > 0 && k + 1 < iters) ? 1 : 0;
         if ((rc = launch_aug<T, V_UPDATE_AUG>(H, d.n_c, v, a, st))) return rc;
@@ -1086,6 +1087,7 @@ int compute_diagonals(fewha_handle* H) {
         for (int k = 1; k <= L.levels; ++k) su.dlev[l * (MAXLEV + 1) + k] = D[L.off + (L.n >> k)];
         su.dlev[l * (MAXLEV + 1) + L.levels + 1] = D[L.off];
     }
+    if (upload(H, H->gdev, H->setup.G)) return FEWHA_ERR_CUDA;   // sigma and the elongation constants
     const Desc<T> d = make_desc<T>(H);
     DiagArgs a{H->basis, H->basis_off, H->pfy64, H->pfx64, H->Jdata};
     k_jdiag<T><<<(d.n_c + 3) / 4, 128>>>(d, a);
@@ -1127,6 +1129,28 @@ int allow_smem(fewha_handle* H, K kernel, size_t need) {
     return FEWHA_OK;
 }
 
+// The sensor kernel in both cluster sizes; clusters of 16 are above the portable size.  They
+// are used where the device can hold all of the instance's at once: the sensors' bands are
+// then half as high.
+template <class T, int SRC>
+int allow_sensor(fewha_handle* H) {
+    int rc;
+    if ((rc = allow_smem(H, k_tsen<T, SRC, 16>, H->smem_ts[0])) || (rc = allow_smem(H, k_tsen<T, SRC, 8>, H->smem_ts[1])))
+        return rc;
+    CK(cudaFuncSetAttribute(k_tsen<T, SRC, 16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "cluster attr");
+    if (SRC == SSRC_PHI) {
+        cudaLaunchConfig_t q = {};
+        q.gridDim = dim3(16, static_cast<unsigned>(H->setup.G.size()));
+        q.blockDim = dim3(tsnt<T>());
+        q.dynamicSmemBytes = H->smem_ts[0];
+        int fit = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, k_tsen<T, SRC, 16>, &q);
+        if (e != cudaSuccess) cudaGetLastError();
+        H->wide_cluster = e == cudaSuccess && fit >= static_cast<int>(H->setup.G.size());
+    }
+    return FEWHA_OK;
+}
+
 template <class T>
 int set_smem_limits(fewha_handle* H) {
     const int maxsm = 227 * 1024;
@@ -1156,18 +1180,18 @@ int set_smem_limits(fewha_handle* H) {
         H->smem_sen > static_cast<size_t>(maxsm))
         return fail(H, FEWHA_ERR_LIMIT, "cluster shared-memory tile above 227 KB");
     int rc = 0;
-    if ((rc = allow_smem(H, k_cl_fwd<T, LSRC_NODES, LDST_APPLY>, H->smem_fwd)) ||
-        (rc = allow_smem(H, k_cl_fwd<T, LSRC_NODES, LDST_COEF>, H->smem_fwd)) ||
-        (rc = allow_smem(H, k_cl_fwd<T, LSRC_NODES, LDST_APPLY_INIT>, H->smem_fwd)) ||
-        (rc = allow_smem(H, k_cl_fwd<T, LSRC_NODES, LDST_RESID_INIT>, H->smem_fwd)) ||
+    if ((rc = allow_smem(H, k_tfwd<T, LDST_APPLY>, H->smem_tf)) || (rc = allow_smem(H, k_tfwd<T, LDST_COEF>, H->smem_tf)) ||
+        (rc = allow_smem(H, k_tfwd<T, LDST_APPLY_INIT>, H->smem_tf)) ||
+        (rc = allow_smem(H, k_tfwd<T, LDST_RESID_INIT>, H->smem_tf)) ||
+        (rc = allow_smem(H, k_tcoarse<T, LDST_APPLY>, H->smem_tc)) ||
+        (rc = allow_smem(H, k_tcoarse<T, LDST_COEF>, H->smem_tc)) ||
+        (rc = allow_smem(H, k_tcoarse<T, LDST_APPLY_INIT>, H->smem_tc)) ||
+        (rc = allow_smem(H, k_tcoarse<T, LDST_RESID_INIT>, H->smem_tc)) ||
         (rc = allow_smem(H, k_tinv<T, 0>, H->smem_tinv)) ||
         (rc = allow_smem(H, k_tinv<T, 1>, H->smem_tinv)) ||
         (rc = allow_smem(H, k_tinv<T, 2>, H->smem_tinv)) ||
-        (rc = allow_smem(H, k_cl_sensor<T, SSRC_PHI>, H->smem_sen)) ||
-        (rc = allow_smem(H, k_cl_sensor<T, SSRC_SLOPES>, H->smem_sen)) ||
-        (rc = allow_smem(H, k_cl_sensor<T, SSRC_RESID>, H->smem_sen)) ||
-        (rc = allow_smem(H, k_proj<T>, H->smem_proj)) || (rc = allow_smem(H, k_projT<T, 4>, H->smem_projT)) ||
-        (rc = allow_smem(H, k_projT<T, KMAX>, H->smem_projT)))
+        (rc = allow_sensor<T, SSRC_PHI>(H)) || (rc = allow_sensor<T, SSRC_SLOPES>(H)) ||
+        (rc = allow_sensor<T, SSRC_RESID>(H)))
         return rc;
     return FEWHA_OK;
 }
@@ -1186,34 +1210,21 @@ bool tail_used(const HostSetup& s) {
 // 16-byte boundary (cp.async targets).
 int round4(int x) { return (x + 3) & ~3; }
 
-// Tile side (log2) of layer l: 32 nodes, halved while the adjoint projection's tile with
-// its halo of 4 would touch more than 64 aperture nodes a side (a layer coarser than the
-// apertures), at least 8, at most the layer.
-int tile_log2(const HostSetup& s, size_t l) {
-    double rho = 0.0;                    // aperture nodes per layer node
-    for (size_t g = 0; g < s.G.size(); ++g) {
-        const size_t tp = (g * MAXL + l) * TAB;
-        const int N = s.G[g].N, span = std::max(1, s.pi0y[tp + N] - s.pi0y[tp]);
-        rho = std::max(rho, static_cast<double>(N) / span);
-    }
-    int lts = std::min(5, s.L[l].log2n);
-    while (lts > 3 && ((1 << lts) + 4) * rho > 64.0) --lts;
-    return lts;
-}
-
-// Tables of the tile kernels (TileLayer, the units and the coefficient slots of a tile).
+// Tables and shared-memory layouts of the tile, band and sensor kernels (fewha_tile.cuh).
 template <class T>
 int tile_tables(fewha_handle* H) {
     const HostSetup& s = H->setup;
-    std::vector<TileLayer> tl(s.L.size());
-    std::vector<int> unit;
-    std::vector<unsigned> slot;
+    constexpr int IPT = sizeof(T) / sizeof(int);           // ints per T
+    const int nl = static_cast<int>(s.L.size()), ng = static_cast<int>(s.G.size());
+    // ---- inverse transform: tiles of 32 x 32 nodes (the layer, if smaller) ----------------
+    std::vector<TileLayer> tl(nl);
+    std::vector<std::vector<unsigned>> slot(nl);           // level | quadrant << 4 | row << 6 | column << 12
     size_t smem = 0;
-    for (size_t l = 0; l < s.L.size(); ++l) {
+    for (int l = 0; l < nl; ++l) {
         const LayerInfo& L = s.L[l];
         TileLayer& t = tl[l];
         std::memset(&t, 0, sizeof(t));
-        t.lts = tile_log2(s, l);
+        t.lts = std::min(5, L.log2n);
         t.side = L.n >> t.lts;
         t.tail = H->tailop && (L.n >> (L.levels - 1)) == 2 && L.levels >= 4;
         t.J = t.tail ? L.levels - 3 : L.levels;
@@ -1236,21 +1247,23 @@ int tile_tables(fewha_handle* H) {
                 }
             }
         }
-        int off = 0;
+        int off = 0, vmax = 0;
         for (int j = 0; j <= t.J; ++j) {
             t.magic[j] = t.np[j] > 0 ? (65536 + t.np[j] - 1) / t.np[j] : 0;
+            t.magicw[j] = (65536 + 2 * t.w[j] - 1) / (2 * t.w[j]);
             t.stride[j] = t.w[j] | 1;
             t.base[j] = off;
             if (j > 0) off += 4 * t.w[j] * t.stride[j];
         }
         t.tailb = off;
         off += t.tail ? 64 : 0;
-        smem = std::max(smem, static_cast<size_t>((t.tail ? TAIL_N : 0) + off) * sizeof(T));
-        t.slot_off = static_cast<int>(slot.size());
+        t.vbuf = off;
+        for (int j = 1; j <= t.J; ++j) vmax = std::max(vmax, t.w[j - 1] * (2 * t.w[j] + 1));
+        off += vmax;
+        smem = std::max(smem, static_cast<size_t>((H->tailop ? TAIL_N : 0) + off) * sizeof(T));
         auto put = [&](int j, int q, int w) {
             for (int r = 0; r < w; ++r)
-                for (int c = 0; c < w; ++c)
-                    slot.push_back(static_cast<unsigned>(j | q << 4 | r << 6 | c << 12));
+                for (int c = 0; c < w; ++c) slot[l].push_back(static_cast<unsigned>(j | q << 4 | r << 6 | c << 12));
         };
         for (int j = 1; j <= t.J; ++j)
             for (int q = 1; q < 4; ++q) put(j, q, t.w[j]);
@@ -1258,15 +1271,249 @@ int tile_tables(fewha_handle* H) {
             put(0, 0, 8);
         else
             put(t.J, 0, t.w[t.J]);
-        t.slot_cnt = static_cast<int>(slot.size()) - t.slot_off;
-        for (int y = 0; y < t.side; ++y)
-            for (int x = 0; x < t.side; ++x) unit.push_back(static_cast<int>(l) | y << 8 | x << 16);
+        H->tcnt[l] = static_cast<int>(slot[l].size());
+        H->tslot_ld = std::max(H->tslot_ld, H->tcnt[l]);
+        H->tu0[l + 1] = H->tu0[l] + t.side * t.side;
     }
-    H->n_units = static_cast<int>(unit.size());
+    H->n_tu = H->tu0[nl];
     H->smem_tinv = smem;
+    std::vector<TilePlace> place(static_cast<size_t>(H->n_tu) * H->tslot_ld, TilePlace{0, 0});
+    for (int l = 0; l < nl; ++l) {
+        const LayerInfo& L = s.L[l];
+        const TileLayer& t = tl[l];
+        for (int ty = 0; ty < t.side; ++ty)
+            for (int tx = 0; tx < t.side; ++tx) {
+                int ss[2][8] = {{ty << t.lts}, {tx << t.lts}};
+                for (int e = 0; e < 2; ++e)
+                    for (int j = 1; j <= t.J; ++j) ss[e][j] = t.whole[j] ? 0 : (ss[e][j - 1] >> 1) - 2;
+                TilePlace* p = &place[static_cast<size_t>(H->tu0[l] + ty * t.side + tx) * H->tslot_ld];
+                for (unsigned c : slot[l]) {
+                    const int j = c & 15, q = (c >> 4) & 3, row = (c >> 6) & 63, col = (c >> 12) & 63;
+                    int pos, dst;
+                    bool own;
+                    if (j == 0) {
+                        pos = L.off + row * L.n + col;
+                        own = ty == 0 && tx == 0;
+                        dst = t.tailb + row * 8 + col;
+                    } else {
+                        const int h = L.n >> j;
+                        const int y = (ss[0][j] + row) & (h - 1), x = (ss[1][j] + col) & (h - 1);
+                        own = ((y << j) >> t.lts) == ty && ((x << j) >> t.lts) == tx;
+                        pos = L.off + (y + (q >> 1) * h) * L.n + x + (q & 1) * h;
+                        dst = t.base[j] + (q * t.w[j] + row) * t.stride[j] + col;
+                    }
+                    *p++ = TilePlace{static_cast<int>(static_cast<unsigned>(pos) | (own ? 0x80000000u : 0u)), dst};
+                }
+            }
+    }
+    auto ints = [](int k) { return round4((k + IPT - 1) / IPT); };
+    // ---- forward transform: bands of rows, their row weights of the adjoint projection ------
+    std::vector<T> brow;
+    std::vector<int> tcl;
+    std::vector<int> bsrc, row0;                           // row0: first staged row per unit and sensor
+    const int nyslot = H->pyslot;
+    int rw = 0, yw = 0, lb1 = 0, lbc = 0;
+    std::vector<std::vector<int>> need;                    // staged elements per unit and sensor
+    bool tail1 = false;
+    for (int l = 0; l < nl; ++l) {
+        const LayerInfo& L = s.L[l];
+        const int n = L.n, h = n / 2, bands = n > TF_ONE ? n / TF_BAND : 1;
+        const int bh = n / bands, ry = bands > 1 ? bh + 4 : n;
+        int kt = 0;
+        for (int g = 0; g < ng; ++g)
+            for (int i = 0; i < n; ++i) {
+                const int k = (g * MAXL + l) * MAXN + i;
+                kt = std::max(kt, s.ry_hi[k] - s.ry_lo[k]);
+            }
+        kt = kt <= 3 ? 3 : kt <= 5 ? 5 : KMAX;
+        H->bkt[l] = kt | (tl[l].tail ? 16 : 0);
+        H->broff[l] = static_cast<int>(brow.size());
+        H->bu0[l + 1] = H->bu0[l] + bands;
+        for (int b = 0; b < bands; ++b) {
+            need.emplace_back();
+            for (int g = 0; g < ng; ++g) {
+                // aperture rows that touch the band and its halo
+                int a0 = 1 << 20, a1 = 0;
+                for (int i = 0; i < ry; ++i) {
+                    const int k = (g * MAXL + l) * MAXN + ((b * bh + i) & (n - 1));
+                    if (s.ry_hi[k] > s.ry_lo[k]) {
+                        a0 = std::min(a0, s.ry_lo[k]);
+                        a1 = std::max(a1, s.ry_hi[k]);
+                    }
+                }
+                if (a1 == 0) a0 = 0;
+                const int* bx = &H->box_host[(g * MAXL + l) * 4];
+                const int e[4] = {(g * nl + l) * nyslot + a0 * bx[3], (a1 - a0) * bx[3], 0, 0};
+                bsrc.insert(bsrc.end(), e, e + 4);
+                row0.push_back(a0);
+                need.back().push_back(round4(e[1]));
+            }
+            for (int i = 0; i < ry; ++i)
+                for (int g = 0; g < ng; ++g) {
+                    const int px = (b * bh + i) & (n - 1), k = (g * MAXL + l) * MAXN + px, tp = (g * MAXL + l) * TAB;
+                    const int lo = s.ry_lo[k], cnt = s.ry_hi[k] - lo;
+                    for (int q = 0; q < kt; ++q) {
+                        T w = T(0);
+                        if (q < cnt) {
+                            const T f = static_cast<T>(s.pfy[tp + lo + q]);
+                            w = s.pi0y[tp + lo + q] == px ? T(1) - f : f;
+                        }
+                        brow.push_back(w);
+                    }
+                    brow.push_back(static_cast<T>(cnt > 0 ? lo : 0));
+                }
+        }
+        rw = std::max(rw, ry * ng * (kt + 1));
+        yw = std::max(yw, ry * ((h + 1) & ~1));
+        if (bands == 1) {
+            lb1 = std::max(lb1, h * (h + 1));
+            tail1 = tail1 || tl[l].tail;
+        } else {
+            lbc = std::max(lbc, h * (h + 1));
+            tcl.push_back(l);
+        }
+    }
+    H->n_bu = H->bu0[nl];
+    H->n_tcl = static_cast<int>(tcl.size());
+    for (int l = nl; l < MAXL; ++l) H->tu0[l + 1] = H->bu0[l + 1] = 1 << 30;
+    const size_t hdr = CWMAX * sizeof(double);
+    TfLayout f{};
+    f.w = 0;
+    f.ye = round4(rw);
+    f.yo = f.ye + round4(yw);
+    f.src = f.yo + round4(yw);
+    f.lbuf = f.src + ints(6 * ng);
+    f.tail = f.lbuf + round4(2 * lb1);
+    f.st = f.tail + (tail1 ? round4(TAIL_N) : 0);
+    // the staged aperture rows: as many sensors a pass as fit (the batched kernels hold the
+    // descriptor beside)
+    const int room = static_cast<int>((160 * 1024 - hdr) / sizeof(T)) - f.st;
+    for (f.gb = ng; f.gb >= 1; --f.gb) {
+        int most = 0;
+        for (size_t u = 0; u < need.size(); ++u) {
+            int at = 0;
+            for (int g = 0; g < ng; ++g) {
+                if (g % f.gb == 0) at = 0;
+                    bsrc[(u * ng + g) * 4 + 2] = at;
+                at += need[u][g];
+                most = std::max(most, at);
+            }
+        }
+        f.total = f.st + most;
+        if (most <= room) break;
+    }
+    f.gb = std::max(f.gb, 1);
+    // the first rows of the weights' entries become stage offsets
+    for (int l = 0; l < nl; ++l) {
+        const int n = s.L[l].n, bands = H->bu0[l + 1] - H->bu0[l], ry = bands > 1 ? TF_BAND + 4 : n, kt = H->bkt[l] & 15;
+        for (int b = 0; b < bands; ++b)
+            for (int i = 0; i < ry; ++i)
+                for (int g = 0; g < ng; ++g) {
+                    const int u = H->bu0[l] + b;
+                    T& e = brow[H->broff[l] + ((static_cast<size_t>(b) * ry + i) * ng + g) * (kt + 1) + kt];
+                    const int lo = std::max(0, static_cast<int>(e) - row0[u * ng + g]);
+                    e = static_cast<T>(bsrc[(u * ng + g) * 4 + 2] + lo * H->box_host[(g * MAXL + l) * 4 + 3]);
+                }
+    }
+    H->lay_tf = f;
+    H->smem_tf = hdr + static_cast<size_t>(f.total) * sizeof(T);
+    TcLayout q{};
+    q.lbuf = 0;
+    q.tmp = round4(lbc);
+    q.st = 2 * round4(lbc);
+    q.total = q.st + (lbc ? 3 * (MAXN / 2) * (MAXN / 2) : 0);
+    if (H->tailop && lbc) {
+        q.tail = q.total;
+        q.total += round4(TAIL_N);
+    }
+    H->lay_tc = q;
+    H->smem_tc = hdr + static_cast<size_t>(q.total) * sizeof(T);
+    tcl.push_back(0);
+    // ---- sensor kernel ----------------------------------------------------------------------
+    std::vector<int> txi, tyi, tcin, tsco, tybox;
+    std::vector<T> txf, tyf, tcw;
+    H->tnp = round4(s.max_N + 1);
+    int kx = 0;
+    for (int g = 0; g < ng; ++g) {
+        int c = 0;
+        for (int l = 0; l < nl; ++l) {
+            c += round4(H->box_host[(g * MAXL + l) * 4 + 3]);
+            for (int j = 0; j < s.L[l].n; ++j) {
+                const int k = (g * MAXL + l) * MAXN + j;
+                kx = std::max(kx, s.rx_hi[k] - s.rx_lo[k]);
+            }
+        }
+        H->tcols = std::max(H->tcols, c);
+    }
+    H->tks = kx <= 4 ? 4 : KMAX;
+    for (int g = 0; g < ng; ++g) {
+        int c = 0;
+        for (int l = 0; l < nl; ++l) {
+            const int tp = (g * MAXL + l) * TAB, n = s.L[l].n, NP = s.G[g].N + 1;
+            for (int b = 0; b < H->tnp; ++b) {
+                txi.push_back(b < NP ? s.L[l].off + s.pi0x[tp + b] : 0);
+                txf.push_back(b < NP ? static_cast<T>(s.pfx[tp + b]) : T(0));
+                tyi.push_back(b < NP ? s.pi0y[tp + b] * n : 0);
+                tyi.push_back(n);
+                tyf.push_back(b < NP ? static_cast<T>(s.pfy[tp + b]) : T(0));
+            }
+            const int* bx = &H->box_host[(g * MAXL + l) * 4];
+            tsco.push_back(c);
+            tybox.push_back(bx[3]);
+            tybox.push_back((g * nl + l) * H->pyslot);
+            for (int k = 0; k < round4(bx[3]); ++k, ++c) {
+                const int j = bx[2] + k, e = (g * MAXL + l) * MAXN + j;
+                const int lo = k < bx[3] && j < n ? s.rx_lo[e] : 0, cnt = k < bx[3] && j < n ? s.rx_hi[e] - lo : 0;
+                tcin.push_back(lo);
+                tcin.push_back(cnt);
+                for (int q = 0; q < H->tks; ++q) {
+                    T w = T(0);
+                    if (q < cnt) {
+                        const T f = static_cast<T>(s.pfx[tp + lo + q]);
+                        w = s.pi0x[tp + lo + q] == j ? T(1) - f : f;
+                    }
+                    tcw.push_back(w);
+                }
+            }
+        }
+        tsco.push_back(c);
+        for (int l = nl; l < MAXL; ++l) {
+            tsco.push_back(c);
+            tybox.push_back(0);
+            tybox.push_back(0);
+        }
+        tcin.resize(static_cast<size_t>(g + 1) * H->tcols * 2, 0);
+        tcw.resize(static_cast<size_t>(g + 1) * H->tcols * H->tks, T(0));
+    }
+    for (int w = 0; w < 2; ++w) {
+        const int scl = w == 0 ? 16 : 8, sr = (s.max_N + scl - 1) / scl;
+        TsLayout v{};
+        v.V = 0;
+        v.SX = v.V + round4((sr + 2) * (s.max_N + 1));
+        v.SY = v.SX + round4((sr + 1) * s.max_N);
+        v.msk = v.SY + round4((sr + 1) * s.max_N);
+        v.xi = v.msk + ints((sr + 1) * s.max_N);
+        v.xf = v.xi + ints(nl * H->tnp);
+        v.yi = v.xf + round4(nl * H->tnp);
+        v.yf = v.yi + ints(2 * nl * (sr + 2));
+        v.cw = v.yf + round4(nl * (sr + 2));
+        v.ci = v.cw + H->tcols * H->tks;
+        v.total = v.ci + ints(2 * H->tcols);
+        H->lay_ts[w] = v;
+        H->smem_ts[w] = static_cast<size_t>(v.total) * sizeof(T);
+    }
     int rc;
-    if ((rc = dalloc(H, &H->tl, tl.size())) || (rc = upload(H, H->tl, tl)) || (rc = dalloc(H, &H->tunit, unit.size())) ||
-        (rc = upload(H, H->tunit, unit)) || (rc = dalloc(H, &H->tslot, slot.size())) || (rc = upload(H, H->tslot, slot)))
+    if ((rc = dalloc(H, &H->tl, tl.size())) || (rc = upload(H, H->tl, tl)) || (rc = dalloc(H, &H->tslot, place.size())) ||
+        (rc = upload(H, H->tslot, place)) || (rc = talloc(H, &H->brow, brow.size())) || (rc = dalloc(H, &H->bsrc, bsrc.size())) || (rc = upload(H, H->bsrc, bsrc)) ||
+        (rc = upload(H, static_cast<T*>(H->brow), brow)) || (rc = dalloc(H, &H->tcl, tcl.size())) ||
+        (rc = upload(H, H->tcl, tcl)) || (rc = dalloc(H, &H->gdev, s.G.size())) || (rc = dalloc(H, &H->txi, txi.size() + 4)) || (rc = upload(H, H->txi, txi)) ||
+        (rc = dalloc(H, &H->tyi, tyi.size())) || (rc = upload(H, H->tyi, tyi)) || (rc = talloc(H, &H->txf, txf.size())) ||
+        (rc = upload(H, static_cast<T*>(H->txf), txf)) || (rc = talloc(H, &H->tyf, tyf.size())) ||
+        (rc = upload(H, static_cast<T*>(H->tyf), tyf)) || (rc = talloc(H, &H->tcw, tcw.size())) ||
+        (rc = upload(H, static_cast<T*>(H->tcw), tcw)) || (rc = dalloc(H, &H->tcin, tcin.size())) ||
+        (rc = upload(H, H->tcin, tcin)) || (rc = dalloc(H, &H->tsco, tsco.size())) || (rc = upload(H, H->tsco, tsco)) ||
+        (rc = dalloc(H, &H->tybox, tybox.size())) || (rc = upload(H, H->tybox, tybox)) ||
+        (rc = talloc(H, &H->ll, s.n_c / 4)) || (rc = dalloc(H, &H->tshare, H->n_bu)))
         return rc;
     return FEWHA_OK;
 }
@@ -1359,7 +1606,8 @@ int cluster_layouts(fewha_handle* H) {
             bx[1] = rows;
             bx[2] = c0;
             bx[3] = c1 - c0;
-            yslot = std::max(yslot, round4(rows * (c1 - c0)));
+            // a term of P^T on the box, or its column half on every aperture row
+            yslot = std::max(yslot, round4(std::max(rows, NP) * (c1 - c0)));
             proj = std::max(proj, static_cast<size_t>(round4(rows * (c1 - c0)) + rows * NP + 4 * NP + 4));
             projT = std::max(projT, static_cast<size_t>(round4(2 * V + NP * NP) + round4(NP * (c1 - c0)) +
                                                         (c1 - c0 + rows + 2) * (KMAX + 2) + 8));
@@ -2420,9 +2668,9 @@ template <class T>
 size_t barg_size(int kind) {
     switch (kind) {
         case BK_INV: case BK_INV_UPD: case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT:
+        case BK_TC_APPLY: case BK_TC_COEF: case BK_TC_RINIT:
             return sizeof(ClArgs<T>);
         case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return sizeof(SensorArgs<T>);
-        case BK_PROJ: case BK_PROJT: return sizeof(const T*);
         case BK_FIT: return sizeof(FitArgs<T>);
         default: return sizeof(VecArgs<T>);
     }
@@ -2431,10 +2679,9 @@ size_t barg_size(int kind) {
 size_t bsmem(const fewha_handle* H, int kind) {
     switch (kind) {
         case BK_INV: case BK_INV_UPD: return H->smem_tinv;
-        case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return H->smem_fwd;
-        case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return H->smem_sen;
-        case BK_PROJ: return H->smem_proj;
-        case BK_PROJT: return H->smem_projT;
+        case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return H->smem_tf;
+        case BK_TC_APPLY: case BK_TC_COEF: case BK_TC_RINIT: return H->smem_tc;
+        case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return H->smem_ts[1];
         default: return 0;
     }
 }
@@ -2493,9 +2740,8 @@ void batch_pack(const std::vector<Recorder<T>>& recs, const std::vector<int>& np
             const BStep<T>& st = recs[i].steps[j];
             unsigned char* dst = out.data() + offs[j] + i * sz;
             switch (bkind_list(kind)) {
-                case BL_LAYER: case BL_TILE: std::memcpy(dst, &st.cl, sz); break;
+                case BL_LAYER: case BL_TILE: case BL_BAND: std::memcpy(dst, &st.cl, sz); break;
                 case BL_SENSOR: std::memcpy(dst, &st.sa, sz); break;
-                case BL_PAIR: std::memcpy(dst, &st.ptr, sz); break;
                 case BL_FIT: std::memcpy(dst, &st.fa, sz); break;
                 default: {
                     VecArgs<T> v = st.va;
@@ -2544,11 +2790,11 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
     for (int i : order) {
         const fewha_handle* H = B->h[i];
         const int g = grp[i], nl = static_cast<int>(H->setup.L.size()), nw = static_cast<int>(H->setup.G.size());
-        for (int l = 0; l < nl; ++l) lists[g * BL_COUNT + BL_LAYER].push_back({i, l});
-        for (int k = 0; k < H->n_units; ++k) lists[g * BL_COUNT + BL_TILE].push_back({i, k});
+        for (int k = 0; k < H->n_tu; ++k) lists[g * BL_COUNT + BL_TILE].push_back({i, k});
+        for (int k = 0; k < H->n_bu; ++k) lists[g * BL_COUNT + BL_BAND].push_back({i, k});
+        for (int l = 0; l < nl; ++l)
+            if (H->bu0[l + 1] - H->bu0[l] > 1) lists[g * BL_COUNT + BL_LAYER].push_back({i, l});
         for (int w = 0; w < nw; ++w) lists[g * BL_COUNT + BL_SENSOR].push_back({i, w});
-        for (int w = 0; w < nw; ++w)
-            for (int l = 0; l < nl; ++l) lists[g * BL_COUNT + BL_PAIR].push_back({i, w * MAXL + l});
         for (int k = 0; k < nparts[i]; ++k) lists[g * BL_COUNT + BL_VEC].push_back({i, k});
         for (int k = 0; k < (H->setup.n_act + PBLK - 1) / PBLK; ++k) lists[g * BL_COUNT + BL_FIT].push_back({i, k});
     }
@@ -2559,11 +2805,11 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
         BInst<T>& I = inst[i];
         std::memset(&I, 0, sizeof(I));
         I.d = make_desc<T>(H);
-        I.lay_fwd = H->lay_fwd;
-        I.lay_sen = H->lay_sen;
+        I.lay_tf = H->lay_tf;
+        I.lay_tc = H->lay_tc;
+        I.lay_ts = H->lay_ts[1];
         I.pb = pair_bufs<T>(H);
         I.desc_bytes = static_cast<int>(offsetof(Desc<T>, box) + static_cast<size_t>(I.d.n_wfs) * MAXL * 4 * sizeof(int));
-        I.ctas_layer = static_cast<unsigned>(CL * I.d.n_layers);
         I.nparts = nparts[i];
     }
     // device block
@@ -2632,8 +2878,6 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
             L.n_items = static_cast<int>(lists[li].size());
             L.smem = smem[g * BK_COUNT + kind];
             L.pdl = (B->h[0]->params.flags & FEWHA_FLAG_PDL) != 0;
-            L.pair_nt = pair_nt;
-            L.taps = taps;
             L.vec_nt = vec_nt;
             le = batch_launch<T>(L, st);
         }
@@ -2978,7 +3222,6 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
     const Desc<T> d = make_desc<T>(H);
     T* p = static_cast<T*>(H->p);
     T* phi = static_cast<T*>(H->phi);
-    T* u = static_cast<T*>(H->u);
     T* q = static_cast<T*>(H->q);
     int rc = 0;
     for (int i = 0; i < reps && rc == 0; ++i) {
@@ -2993,31 +3236,28 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
                 rc = launch_inv<T, 1>(H, d, a, st);
                 break;
             }
+            // P runs in the sensor kernel, P^T half there and half in the layer kernels
             case FEWHA_STAGE_SENSOR:
-                rc = launch_csensor<T, SSRC_PHI>(H, d, phi, u, st);
+            case FEWHA_STAGE_PROJ:
+                rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st);
                 break;
-            case FEWHA_STAGE_LAYER: {
-                ClArgs<T> a = cl_args<T>(H, u, q);
+            case FEWHA_STAGE_LAYER:
+            case FEWHA_STAGE_PROJT: {
+                ClArgs<T> a = cl_args<T>(H, nullptr, q);
                 a.pin = p;
                 a.iter = PQ_SCRATCH_SLOT;
                 a.zero_piston = 1;
-                rc = launch_fwd<T, LSRC_NODES, LDST_APPLY>(H, d, a, st);
+                rc = launch_fwd<T, LDST_APPLY>(H, d, a, st);
                 break;
             }
             case FEWHA_STAGE_VECTOR:
                 rc = launch_vec<T, V_UPDATE>(H, d.n_c, vec_args<T>(H, static_cast<T*>(H->c), 0), st);
                 break;
             case FEWHA_STAGE_RHS:
-                rc = launch_csensor<T, SSRC_SLOPES>(H, d, static_cast<const T*>(H->s_tmp), u, st);
+                rc = launch_csensor<T, SSRC_SLOPES>(H, d, nullptr, static_cast<const T*>(H->s_tmp), st);
                 break;
             case FEWHA_STAGE_FIT:
                 rc = launch_fit<T>(H, d, phi, static_cast<T*>(H->a_prev), static_cast<T*>(H->dm_tmp), 1, st);
-                break;
-            case FEWHA_STAGE_PROJ:
-                rc = launch_proj<T>(H, d, phi, st);
-                break;
-            case FEWHA_STAGE_PROJT:
-                rc = launch_projT<T>(H, d, u, st);
                 break;
         }
     }

@@ -34,59 +34,44 @@ __global__ void __launch_bounds__(TINV_NT)
 }
 
 template <class T, int DST>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(cblk<T>(), 1)
-    kb_cl_fwd(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args,
-              const BItem* __restrict__ items) {
+__global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
+    kb_tfwd(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
     __shared__ __align__(16) Desc<T> sd;
     pdl_enter();
-    const BItem it = items[blockIdx.y];
+    const BItem it = items[blockIdx.x];
     const BInst<T>* I = inst + it.inst;
     load_desc<T>(sd, I);
     const ClArgs<T> a = args[it.inst];
-    const ClLayout lay = I->lay_fwd;
+    const TfLayout lay = I->lay_tf;
     const PairBufs<T> pb = I->pb;
-    cl_fwd_body<T, LSRC_NODES, DST>(sd, a, lay, pb, it.unit, I->ctas_layer);
+    tfwd_body<T, DST>(sd, a, lay, pb, it.unit);
+}
+
+template <class T, int DST>
+__global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
+    kb_tcoarse(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
+    __shared__ __align__(16) Desc<T> sd;
+    pdl_enter();
+    const BItem it = items[blockIdx.x];
+    const BInst<T>* I = inst + it.inst;
+    load_desc<T>(sd, I);
+    const ClArgs<T> a = args[it.inst];
+    const TcLayout lay = I->lay_tc;
+    tcoarse_body<T, DST>(sd, a, lay, it.unit);
 }
 
 template <class T, int SRC>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(cblk<T>(), 1)
-    kb_cl_sensor(const BInst<T>* __restrict__ inst, const SensorArgs<T>* __restrict__ args,
-                 const BItem* __restrict__ items) {
+__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(tsnt<T>(), sizeof(T) == 4 ? 2 : 1)
+    kb_tsen(const BInst<T>* __restrict__ inst, const SensorArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
     __shared__ __align__(16) Desc<T> sd;
     pdl_enter();
     const BItem it = items[blockIdx.y];
     const BInst<T>* I = inst + it.inst;
     load_desc<T>(sd, I);
     const SensorArgs<T> a = args[it.inst];
-    const SensorLayout lay = I->lay_sen;
+    const TsLayout lay = I->lay_ts;
     const PairBufs<T> pb = I->pb;
-    cl_sensor_body<T, SRC>(sd, a, lay, pb, it.unit);
-}
-
-template <class T, int NTP>
-__global__ void __launch_bounds__(NTP, 1)
-    kb_proj(const BInst<T>* __restrict__ inst, const T* const* __restrict__ args,
-            const BItem* __restrict__ items) {
-    __shared__ __align__(16) Desc<T> sd;
-    pdl_enter();
-    const BItem it = items[blockIdx.x];
-    const BInst<T>* I = inst + it.inst;
-    load_desc<T>(sd, I);
-    const PairBufs<T> pb = I->pb;
-    proj_body<T, NTP>(sd, args[it.inst], pb, it.unit / MAXL, it.unit % MAXL);
-}
-
-template <class T, int KM, int NTP>
-__global__ void __launch_bounds__(NTP, 1)
-    kb_projT(const BInst<T>* __restrict__ inst, const T* const* __restrict__ args,
-             const BItem* __restrict__ items) {
-    __shared__ __align__(16) Desc<T> sd;
-    pdl_enter();
-    const BItem it = items[blockIdx.x];
-    const BInst<T>* I = inst + it.inst;
-    load_desc<T>(sd, I);
-    const PairBufs<T> pb = I->pb;
-    projT_body<T, KM, NTP>(sd, args[it.inst], pb, it.unit / MAXL, it.unit % MAXL);
+    tsen_body<T, SRC, 8>(sd, a, lay, pb, it.unit);
 }
 
 template <class T, int PHASE, int NTV>
@@ -113,29 +98,23 @@ __global__ void __launch_bounds__(PBLK)
     fit_body<T>(sd, f.phi, f.a_prev, f.out, f.apply_gain, it.unit, nullptr, f.cpist);
 }
 
-// The kernel of a step kind in one launch shape (variant v: bit 0 half-size projection
-// CTAs, bit 1 the 4-tap adjoint projection; for the vector kernels, bit 0 512 threads).
+// The kernel of a step kind in one launch shape (variant v: 1 = the vector kernels with 512
+// threads).
 template <class T>
 const void* kernel_of(int kind, int v) {
-    constexpr int NP = cblk<T>(), NH = cblk<T>() / 2;
-    const bool half = (v & 1) != 0, t4 = (v & 2) != 0;
+    const bool half = (v & 1) != 0;
     switch (kind) {
         case BK_INV: return reinterpret_cast<const void*>(kb_tinv<T, 0>);
         case BK_INV_UPD: return reinterpret_cast<const void*>(kb_tinv<T, 1>);
-        case BK_PROJ:
-            return half ? reinterpret_cast<const void*>(kb_proj<T, NH>) : reinterpret_cast<const void*>(kb_proj<T, NP>);
-        case BK_SEN_PHI: return reinterpret_cast<const void*>(kb_cl_sensor<T, SSRC_PHI>);
-        case BK_SEN_SLOPES: return reinterpret_cast<const void*>(kb_cl_sensor<T, SSRC_SLOPES>);
-        case BK_SEN_RESID: return reinterpret_cast<const void*>(kb_cl_sensor<T, SSRC_RESID>);
-        case BK_PROJT:
-            if (t4)
-                return half ? reinterpret_cast<const void*>(kb_projT<T, 4, NH>)
-                            : reinterpret_cast<const void*>(kb_projT<T, 4, NP>);
-            return half ? reinterpret_cast<const void*>(kb_projT<T, KMAX, NH>)
-                        : reinterpret_cast<const void*>(kb_projT<T, KMAX, NP>);
-        case BK_FWD_APPLY: return reinterpret_cast<const void*>(kb_cl_fwd<T, LDST_APPLY>);
-        case BK_FWD_COEF: return reinterpret_cast<const void*>(kb_cl_fwd<T, LDST_COEF>);
-        case BK_FWD_RINIT: return reinterpret_cast<const void*>(kb_cl_fwd<T, LDST_RESID_INIT>);
+        case BK_SEN_PHI: return reinterpret_cast<const void*>(kb_tsen<T, SSRC_PHI>);
+        case BK_SEN_SLOPES: return reinterpret_cast<const void*>(kb_tsen<T, SSRC_SLOPES>);
+        case BK_SEN_RESID: return reinterpret_cast<const void*>(kb_tsen<T, SSRC_RESID>);
+        case BK_FWD_APPLY: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_APPLY>);
+        case BK_TC_APPLY: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_APPLY>);
+        case BK_FWD_COEF: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_COEF>);
+        case BK_TC_COEF: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_COEF>);
+        case BK_FWD_RINIT: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_RESID_INIT>);
+        case BK_TC_RINIT: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_RESID_INIT>);
         case BK_VEC_INIT:
             return half ? reinterpret_cast<const void*>(kb_vec<T, V_INIT, 2 * PBLK>)
                         : reinterpret_cast<const void*>(kb_vec<T, V_INIT, PBLK>);
@@ -159,7 +138,7 @@ cudaError_t batch_smem_limit(int kind, size_t* bytes) {
         return cudaSuccess;
     }
     int lim = 227 * 1024;
-    for (int v = 0; v < 4; ++v) {
+    for (int v = 0; v < 2; ++v) {
         const void* k = kernel_of<T>(kind, v);
         if (!k) return cudaErrorInvalidValue;
         cudaFuncAttributes fa;
@@ -194,10 +173,8 @@ cudaError_t batch_launch(const BLaunch& L, cudaStream_t st) {
     if (L.n_items <= 0) return cudaSuccess;
     const BInst<T>* I = static_cast<const BInst<T>*>(L.inst);
     const int n = L.n_items;
-    const dim3 cg(CL, n), pg(n), nt(cblk<T>()), vt(L.vec_nt), pt(L.pair_nt);
-    const bool ph = L.pair_nt != cblk<T>(), t4 = L.taps == 4, v2 = L.vec_nt != PBLK;
-    const T* const* pa = static_cast<const T* const*>(L.args);
-    constexpr int NP = cblk<T>(), NH = cblk<T>() / 2;
+    const dim3 cg(8, n), sn(tsnt<T>()), pg(n), nt(cblk<T>()), vt(L.vec_nt);
+    const bool v2 = L.vec_nt != PBLK;
     const ClArgs<T>* ca = static_cast<const ClArgs<T>*>(L.args);
     const SensorArgs<T>* sa = static_cast<const SensorArgs<T>*>(L.args);
     const VecArgs<T>* va = static_cast<const VecArgs<T>*>(L.args);
@@ -205,21 +182,15 @@ cudaError_t batch_launch(const BLaunch& L, cudaStream_t st) {
     switch (L.kind) {
         case BK_INV: return launch_b(L.pdl, kb_tinv<T, 0>, pg, dim3(TINV_NT), L.smem, st, I, ca, L.items);
         case BK_INV_UPD: return launch_b(L.pdl, kb_tinv<T, 1>, pg, dim3(TINV_NT), L.smem, st, I, ca, L.items);
-        case BK_FWD_APPLY: return launch_b(L.pdl, kb_cl_fwd<T, LDST_APPLY>, cg, nt, L.smem, st, I, ca, L.items);
-        case BK_FWD_COEF: return launch_b(L.pdl, kb_cl_fwd<T, LDST_COEF>, cg, nt, L.smem, st, I, ca, L.items);
-        case BK_FWD_RINIT: return launch_b(L.pdl, kb_cl_fwd<T, LDST_RESID_INIT>, cg, nt, L.smem, st, I, ca, L.items);
-        case BK_SEN_PHI: return launch_b(L.pdl, kb_cl_sensor<T, SSRC_PHI>, cg, nt, L.smem, st, I, sa, L.items);
-        case BK_SEN_SLOPES: return launch_b(L.pdl, kb_cl_sensor<T, SSRC_SLOPES>, cg, nt, L.smem, st, I, sa, L.items);
-        case BK_SEN_RESID: return launch_b(L.pdl, kb_cl_sensor<T, SSRC_RESID>, cg, nt, L.smem, st, I, sa, L.items);
-        case BK_PROJ:
-            return ph ? launch_b(L.pdl, kb_proj<T, NH>, pg, pt, L.smem, st, I, pa, L.items)
-                      : launch_b(L.pdl, kb_proj<T, NP>, pg, pt, L.smem, st, I, pa, L.items);
-        case BK_PROJT:
-            if (t4)
-                return ph ? launch_b(L.pdl, kb_projT<T, 4, NH>, pg, pt, L.smem, st, I, pa, L.items)
-                          : launch_b(L.pdl, kb_projT<T, 4, NP>, pg, pt, L.smem, st, I, pa, L.items);
-            return ph ? launch_b(L.pdl, kb_projT<T, KMAX, NH>, pg, pt, L.smem, st, I, pa, L.items)
-                      : launch_b(L.pdl, kb_projT<T, KMAX, NP>, pg, pt, L.smem, st, I, pa, L.items);
+        case BK_FWD_APPLY: return launch_b(L.pdl, kb_tfwd<T, LDST_APPLY>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_TC_APPLY: return launch_b(L.pdl, kb_tcoarse<T, LDST_APPLY>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_FWD_COEF: return launch_b(L.pdl, kb_tfwd<T, LDST_COEF>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_TC_COEF: return launch_b(L.pdl, kb_tcoarse<T, LDST_COEF>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_FWD_RINIT: return launch_b(L.pdl, kb_tfwd<T, LDST_RESID_INIT>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_TC_RINIT: return launch_b(L.pdl, kb_tcoarse<T, LDST_RESID_INIT>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_SEN_PHI: return launch_b(L.pdl, kb_tsen<T, SSRC_PHI>, cg, sn, L.smem, st, I, sa, L.items);
+        case BK_SEN_SLOPES: return launch_b(L.pdl, kb_tsen<T, SSRC_SLOPES>, cg, sn, L.smem, st, I, sa, L.items);
+        case BK_SEN_RESID: return launch_b(L.pdl, kb_tsen<T, SSRC_RESID>, cg, sn, L.smem, st, I, sa, L.items);
         case BK_VEC_INIT:
             return v2 ? launch_b(L.pdl, kb_vec<T, V_INIT, 2 * PBLK>, pg, vt, 0, st, I, va, L.items)
                       : launch_b(L.pdl, kb_vec<T, V_INIT, PBLK>, pg, vt, 0, st, I, va, L.items);

@@ -12,7 +12,7 @@
 
 namespace fewha {
 
-// One work item: instance index and unit within the instance (a pair is g * MAXL + l).
+// One work item: instance index and unit within the instance.
 struct BItem {
     int inst;
     int unit;
@@ -22,11 +22,11 @@ struct BItem {
 template <class T>
 struct alignas(16) BInst {
     Desc<T> d;
-    ClLayout lay_fwd;
-    SensorLayout lay_sen;
+    TfLayout lay_tf;
+    TcLayout lay_tc;
+    TsLayout lay_ts;
     PairBufs<T> pb;
     int desc_bytes;     // leading bytes of d that the kernels read (through the last sensor's boxes)
-    unsigned ctas_layer;  // CTAs of the instance in a layer-cluster launch (CL * n_layers)
     int nparts;         // CTAs of the instance in a vector launch
 };
 
@@ -44,10 +44,8 @@ struct FitArgs {
 enum BKind {
     BK_INV = 0,        // phi = W^T c                       (ClArgs)
     BK_INV_UPD,        // p = z + beta p, phi = W^T p       (ClArgs)
-    BK_PROJ,           // pair terms of P phi               (const T*: phi)
     BK_SEN_PHI,        // Gamma, C^-1, Gamma^T of P phi     (SensorArgs)
     BK_SEN_SLOPES,     // C^-1, Gamma^T of measured slopes  (SensorArgs)
-    BK_PROJT,          // pair terms of P^T u               (const T*: u)
     BK_FWD_APPLY,      // q = W sum P^T u + alpha D p, p.q  (ClArgs)
     BK_FWD_COEF,       // b = W sum P^T u                   (ClArgs)
     BK_VEC_INIT,       // r0 = b - q, z, p, r.z             (VecArgs)
@@ -56,18 +54,21 @@ enum BKind {
     BK_FIT,            // DM fit and gain                   (FitArgs)
     BK_SEN_RESID,      // C^-1, Gamma^T of s - Gamma P phi  (SensorArgs)
     BK_FWD_RINIT,      // r0 = W sum P^T u - alpha D c0, z0, p0, r.z (ClArgs)
+    BK_TC_APPLY,       // the coarse levels of the same       (ClArgs)
+    BK_TC_COEF,
+    BK_TC_RINIT,
     BK_COUNT
 };
 
 // Which work list a step kind runs over.
-enum BList { BL_LAYER = 0, BL_TILE, BL_SENSOR, BL_PAIR, BL_VEC, BL_FIT, BL_COUNT };
+enum BList { BL_LAYER = 0, BL_TILE, BL_BAND, BL_SENSOR, BL_VEC, BL_FIT, BL_COUNT };
 
 inline int bkind_list(int kind) {
     switch (kind) {
         case BK_INV: case BK_INV_UPD: return BL_TILE;
-        case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return BL_LAYER;
+        case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return BL_BAND;
+        case BK_TC_APPLY: case BK_TC_COEF: case BK_TC_RINIT: return BL_LAYER;
         case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return BL_SENSOR;
-        case BK_PROJ: case BK_PROJT: return BL_PAIR;
         case BK_FIT: return BL_FIT;
         default: return BL_VEC;
     }
@@ -82,8 +83,6 @@ struct BLaunch {
     int n_items;
     size_t smem;           // dynamic shared memory (max over the instances present)
     bool pdl;              // programmatic stream serialization (see FEWHA_FLAG_PDL)
-    int pair_nt;           // threads of the projection kernels: cblk<T>() or half of it
-    int taps;              // unrolled taps of the adjoint projection: 4 or KMAX
     int vec_nt;            // threads of the vector kernel: PBLK or 2 PBLK
 };
 

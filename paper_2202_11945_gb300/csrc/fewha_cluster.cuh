@@ -35,6 +35,12 @@ __device__ __forceinline__ void cp_async(T* smem, const T* gmem) {
     else
         asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem));
 }
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+// All but the newest N groups are done.
+template <int N>
+__device__ __forceinline__ void cp_async_wait_group() {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 // 16-byte copy; both addresses 16-byte aligned.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
@@ -422,6 +428,9 @@ struct ClArgs {
     const double* rz_parts;
     int rz_cnt;
     int rz_slot;
+    // forward tile kernels: the finest level's LL blocks (layer offset / 4), the tiles' shares
+    T* ll;
+    double* tshare;
 };
 
 struct ClLayout {       // shared-memory offsets set by the host, in T units
@@ -806,13 +815,6 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
             }
         }
     }
-}
-
-template <class T, int SRC, int DST>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(cblk<T>(), 1)
-    k_cl_fwd(__grid_constant__ const Desc<T> d, __grid_constant__ const ClArgs<T> a,
-             __grid_constant__ const ClLayout lay, __grid_constant__ const PairBufs<T> pb) {
-    cl_fwd_body<T, SRC, DST>(d, a, lay, pb, blockIdx.y, gridDim.x * gridDim.y);
 }
 
 // ---------------------------------------------------------------------------
@@ -1387,13 +1389,6 @@ __device__ __forceinline__ void cl_sensor_body(const Desc<T>& d, const SensorArg
         }
     }
     cluster.sync();                                                       // neighbours done reading
-}
-
-template <class T, int SRC>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(cblk<T>(), 1)
-    k_cl_sensor(__grid_constant__ const Desc<T> d, __grid_constant__ const SensorArgs<T> a,
-                __grid_constant__ const SensorLayout lay, __grid_constant__ const PairBufs<T> pb) {
-    cl_sensor_body<T, SRC>(d, a, lay, pb, blockIdx.y);
 }
 
 }  // namespace fewha

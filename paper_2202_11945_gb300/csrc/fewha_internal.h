@@ -34,9 +34,15 @@ struct TileLayer {
     int lts, side;
     int J;                  // coarsest level with windows of its own
     int tail;               // level J's LL block is the 8 x 8 block of the tail operator
-    int tailb;              // that operator's input block
-    int slot_off, slot_cnt; // the tile's coefficients in Desc::tslot
-    int w[8], np[8], magic[8], base[8], stride[8], whole[8];
+    int tailb, vbuf;        // that operator's input block; a level's column pass
+    int w[8], np[8], base[8], stride[8], whole[8];
+    int magic[8], magicw[8];    // reciprocals of np and of 2 w (tdiv)
+};
+
+// One coefficient of a tile: place in the coefficient vector (sign bit: the tile owns it) and
+// in shared memory.
+struct alignas(8) TilePlace {
+    int pos, dst;
 };
 
 struct WfsInfo {
@@ -105,12 +111,34 @@ struct alignas(16) Desc {   // 16-byte multiple: batched kernels copy it in 16-b
     // D per (layer, level): detail level k = 1 .. levels (1 the finest), levels + 1 the LL band
     T Dlev[MAXL][9];
     const T* tailop;   // analysis of the 8 x 8 tail levels (64 x TAIL_LD), or null
-    // tiles of the layers (n_units in all): per layer, per unit (layer | tile row << 8 | tile
-    // column << 16), and the coefficient slots of a layer's tile (see tinv_body)
+    // tiles of the layers (inverse transform): layer l has units tu0[l] .. tu0[l + 1], row by
+    // row; unit u's tcnt[l] coefficients at tslot + u * tslot_ld, each {place in the
+    // coefficient vector, sign bit set if the tile owns it; place in shared memory}
     const TileLayer* tl;
-    const int* tunit;
-    const unsigned* tslot;
-    int n_units;
+    const TilePlace* tslot;
+    // bands of the layers (forward transform): units bu0[l] .. bu0[l + 1]; row weights of the
+    // adjoint projection at brow + broff[l], per band, row and sensor kt weights and the stage
+    // offset of the first; bkt[l] = kt | (the tail operator applies) << 4
+    const T* brow;
+    // per band unit and sensor: {offset in PairBufs::Y, elements, offset in the stage, 0}
+    const int* bsrc;
+    const int* tcl;         // layers of several bands (n_tcl)
+    int tslot_ld, n_tcl;
+    // sensor kernel, per sensor: place of node column b's (txi) and node row's (tyi: offset,
+    // row pitch) layer column / row and the weight of the next one, [layer][tnp]; columns of
+    // P^T's column half, layer by layer from tsco: weights [tcols][tks], {first aperture
+    // column, count}; per layer {box columns, offset in PairBufs::Y}
+    const int* txi;
+    const int* tyi;
+    const T* txf;
+    const T* tyf;
+    const T* tcw;
+    const int* tcin;
+    const int* tsco;
+    const int* tybox;
+    const WfsInfo* gdev;    // G in device memory
+    int tnp, tcols, tks;
+    int tu0[MAXL + 1], bu0[MAXL + 1], tcnt[MAXL], broff[MAXL], bkt[MAXL];
     // footprint box of each (sensor, layer) pair: row0, rows, col0, cols (16-byte aligned
     // column superset); kept in the descriptor so that warps read it from the constant bank
     int box[MAXG][MAXL][4];

@@ -618,6 +618,7 @@ struct SensorArgs {
     const T* in;
     T* out;
     unsigned* status;   // bit 0: a non-finite input slope was seen
+    const T* phi;       // layers (the sensor kernel's PHI and RESID forms)
 };
 
 template <class T, int SRC, bool WEIGHT, int DST>

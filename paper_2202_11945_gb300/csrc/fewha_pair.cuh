@@ -70,13 +70,6 @@ __device__ __forceinline__ void proj_body(const Desc<T>& d, const T* __restrict_
     }
 }
 
-template <class T>
-__global__ void __launch_bounds__(cblk<T>(), 1) k_proj(__grid_constant__ const Desc<T> d,
-                                                       const T* __restrict__ phi,
-                                                       __grid_constant__ const PairBufs<T> pb) {
-    proj_body<T>(d, phi, pb, blockIdx.x, blockIdx.y);
-}
-
 // Y_gl(i, j) = sum_{a,b} wy(a, i) wx(b, j) u_g(a, b) on the pair's footprint box.  KM >= the
 // largest number of aperture rows (columns) touching one layer row (column): the loops over
 // a row's taps are unrolled to KM (the weight tables keep the stride KMAX).  NT threads per
@@ -151,13 +144,6 @@ __device__ __forceinline__ void projT_body(const Desc<T>& d, const T* __restrict
             out[ii * cols + jj] = acc;
         }
     }
-}
-
-template <class T, int KM>
-__global__ void __launch_bounds__(cblk<T>(), 1) k_projT(__grid_constant__ const Desc<T> d,
-                                                        const T* __restrict__ u,
-                                                        __grid_constant__ const PairBufs<T> pb) {
-    projT_body<T, KM>(d, u, pb, blockIdx.x, blockIdx.y);
 }
 
 }  // namespace fewha
