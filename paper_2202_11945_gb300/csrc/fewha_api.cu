@@ -145,22 +145,34 @@ struct fewha_handle {
     // tiles and bands of the layers (Desc::tl, tslot, brow, tcl and the tables beside them),
     // the forward kernels' LL blocks and band shares, shared-memory layouts
     TileLayer* tl = nullptr;
+    std::vector<TileLayer> tl_host;
     TilePlace* tslot = nullptr;
     void *brow = nullptr, *ll = nullptr;
     int *tcl = nullptr, *bsrc = nullptr;
     // sensor kernel's tables (Desc::txi ...)
     WfsInfo* gdev = nullptr;
     int *txi = nullptr, *tyi = nullptr, *tcin = nullptr, *tsco = nullptr, *tybox = nullptr;
-    void *txf = nullptr, *tyf = nullptr, *tcw = nullptr;
-    int tnp = 0, tcols = 0, tks = 0;
-    bool wide_cluster = false;        // the sensor kernel runs in clusters of 16 CTAs
-    double* tshare = nullptr;
+    void *txf = nullptr, *tyf = nullptr;
+    int tnp = 0, tcols = 0;
+    int n_su = 0, su0[MAXG + 1] = {};
+    // functionals of the layers (Desc::foff, fent), the tiles' shares, the measured sums
+    int* foff = nullptr;
+    void* fent = nullptr;
+    double *fsh = nullptr, *msum = nullptr;
+    int n_fun = 0, fcap = 0, n_writers = 0, n_coarse = 0;
+    double *lshz = nullptr, *lshq = nullptr;   // the layers' shares of r.z and p.q, per slot
+    int f0[MAXG + 1] = {};
+    size_t foff_cap = 0, fent_cap = 0, fsh_cap = 0;
+    double fun_eta = -1.0;            // elongation parameter they were built for
+    size_t lay_inv_elems = 0;         // the inverse tile kernel's windows, in elements
+    double *tshare = nullptr, *pqs = nullptr;
+    void* alphas = nullptr;
     int n_tu = 0, n_bu = 0, n_tcl = 0, tslot_ld = 0;
     int tu0[MAXL + 1] = {}, bu0[MAXL + 1] = {}, tcnt[MAXL] = {}, broff[MAXL] = {}, bkt[MAXL] = {};
     TfLayout lay_tf{};
     TcLayout lay_tc{};
-    TsLayout lay_ts[2] = {};          // clusters of 16 and of 8
-    size_t smem_tinv = 0, smem_tf = 0, smem_tc = 0, smem_ts[2] = {0, 0};
+    TsLayout lay_ts{};
+    size_t smem_tinv = 0, smem_tf = 0, smem_tc = 0, smem_ts = 0;
     std::vector<int> box_host;
     void* pairV = nullptr;
     void* pairY = nullptr;
@@ -282,6 +294,8 @@ int upload(fewha_handle* H, X* dst, const std::vector<X>& src) {
     return FEWHA_OK;
 }
 
+int round4(int x) { return (x + 3) & ~3; }
+
 template <class T>
 Desc<T> make_desc(const fewha_handle* H) {
     const HostSetup& s = H->setup;
@@ -333,13 +347,20 @@ Desc<T> make_desc(const fewha_handle* H) {
     d.tyi = H->tyi;
     d.txf = static_cast<const T*>(H->txf);
     d.tyf = static_cast<const T*>(H->tyf);
-    d.tcw = static_cast<const T*>(H->tcw);
     d.tcin = H->tcin;
     d.tsco = H->tsco;
     d.tybox = H->tybox;
     d.tnp = H->tnp;
     d.tcols = H->tcols;
-    d.tks = H->tks;
+    std::copy(std::begin(H->su0), std::end(H->su0), d.su0);
+    std::copy(std::begin(H->f0), std::end(H->f0), d.f0);
+    d.foff = H->foff;
+    d.fent = static_cast<const T*>(H->fent);
+    d.n_tu = H->n_tu;
+    d.n_fun = H->n_fun;
+    d.fpad = round4(3 * H->n_fun + 3);
+    d.fcap = H->fcap;
+    d.n_writers = H->n_writers;
     d.tslot_ld = H->tslot_ld;
     d.n_tcl = H->n_tcl;
     std::copy(std::begin(H->tu0), std::end(H->tu0), d.tu0);
@@ -446,6 +467,7 @@ VecArgs<T> vec_args(fewha_handle* H, T* c, int iter) {
     v.pcg = pcg_slots(H);
     v.iter = iter;
     v.pq_cnt = 0;
+    v.pq_parts = nullptr;
     v.defer_rz = 0;
     v.phic = nullptr;
     v.phip = nullptr;
@@ -494,15 +516,19 @@ PairBufs<T> pair_bufs(fewha_handle* H) {
 template <class T, int DST>
 int launch_fwd(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream_t st) {
     if (recorder<T>()) {
-        if (DST == LDST_APPLY_INIT) return fail(H, FEWHA_ERR_INVALID_ARG, "step without a batched form");
-        record<T>(DST == LDST_APPLY ? BK_FWD_APPLY : DST == LDST_RESID_INIT ? BK_FWD_RINIT : BK_FWD_COEF).cl = a;
-        record<T>(DST == LDST_APPLY ? BK_TC_APPLY : DST == LDST_RESID_INIT ? BK_TC_RINIT : BK_TC_COEF).cl = a;
+        if (DST == LDST_APPLY) return fail(H, FEWHA_ERR_INVALID_ARG, "step without a batched form");
+        record<T>(DST == LDST_UPDATE ? BK_FWD_UPD : DST == LDST_RESID_INIT ? BK_FWD_RINIT
+                  : DST == LDST_APPLY_INIT ? BK_FWD_AINIT : BK_FWD_COEF).cl = a;
+        record<T>(DST == LDST_UPDATE ? BK_TC_UPD : DST == LDST_RESID_INIT ? BK_TC_RINIT
+                  : DST == LDST_APPLY_INIT ? BK_TC_AINIT : BK_TC_COEF).cl = a;
         return FEWHA_OK;
     }
     CK(launch_k(H, k_tfwd<T, DST>, dim3(H->n_bu), dim3(cblk<T>()), H->smem_tf, st, d, a, H->lay_tf, pair_bufs<T>(H)),
        "k_tfwd launch");
-    if (d.n_tcl > 0)
-        CK(launch_k(H, k_tcoarse<T, DST>, dim3(d.n_tcl), dim3(cblk<T>()), H->smem_tc, st, d, a, H->lay_tc),
+    // (the vector parts are the CG update's)
+    const int coarse = DST == LDST_UPDATE ? H->n_tcl : H->n_coarse;
+    if (coarse > 0)
+        CK(launch_k(H, k_tcoarse<T, DST>, dim3(coarse), dim3(cblk<T>()), H->smem_tc, st, d, a, H->lay_tc),
            "k_tcoarse launch");
     return FEWHA_OK;
 }
@@ -510,29 +536,38 @@ int launch_fwd(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream
 template <class T, int PUPD>
 int launch_inv(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream_t st) {
     if (recorder<T>()) {
-        record<T>(PUPD ? BK_INV_UPD : BK_INV).cl = a;
+        record<T>(PUPD ? BK_INV_UPD : a.ms ? BK_INV_MS : BK_INV).cl = a;
         return FEWHA_OK;
     }
-    CK(launch_k(H, k_tinv<T, PUPD>, dim3(H->n_tu), dim3(TINV_NT), H->smem_tinv, st, d, a), "k_tinv launch");
+    // with a.ms, a CTA per sensor behind the tiles sums the measured slopes
+    const int units = H->n_tu + (a.ms ? d.n_wfs : 0);
+    CK(launch_k(H, k_tinv<T, PUPD>, dim3(units), dim3(TINV_NT), H->smem_tinv, st, d, a), "k_tinv launch");
     return FEWHA_OK;
 }
 
-// The sensor kernel from layers phi (PHI), measured slopes s (SLOPES) or both (RESID).
+// The sensor kernel from layers phi (PHI), measured slopes s (SLOPES) or both (RESID); the
+// functionals' shares come from the inverse kernel before it (PHI, RESID), the measured
+// sums from it (RESID) or from a kernel of their own here (SLOPES).  With p, the shares of
+// p.q for the CG update.
 template <class T, int SRC>
-int launch_csensor(fewha_handle* H, const Desc<T>& d, const T* phi, const T* s, cudaStream_t st) {
-    SensorArgs<T> a{s, nullptr, H->status, phi};
+int launch_csensor(fewha_handle* H, const Desc<T>& d, const T* phi, const T* s, cudaStream_t st,
+                   const T* p = nullptr) {
+    SensorArgs<T> a{s, nullptr, H->status, phi, H->fsh, H->msum, p,
+                    p ? H->pqs : nullptr};
     if (recorder<T>()) {
+        if (SRC == SSRC_SLOPES) {
+            ClArgs<T> m = cl_args<T>(H, nullptr, nullptr);
+            m.ms = s;
+            m.msum = H->msum;
+            record<T>(BK_MSUM).cl = m;
+        }
         record<T>(SRC == SSRC_PHI ? BK_SEN_PHI : SRC == SSRC_RESID ? BK_SEN_RESID : BK_SEN_SLOPES).sa = a;
         return FEWHA_OK;
     }
-    if (H->wide_cluster)
-        CK(launch_k(H, k_tsen<T, SRC, 16>, dim3(16, d.n_wfs), dim3(tsnt<T>()), H->smem_ts[0], st, d, a, H->lay_ts[0],
-                    pair_bufs<T>(H)),
-           "k_tsen launch");
-    else
-        CK(launch_k(H, k_tsen<T, SRC, 8>, dim3(8, d.n_wfs), dim3(tsnt<T>()), H->smem_ts[1], st, d, a, H->lay_ts[1],
-                    pair_bufs<T>(H)),
-           "k_tsen launch");
+    if (SRC == SSRC_SLOPES)
+        CK(launch_k(H, k_msum<T>, dim3(d.n_wfs), dim3(TINV_NT), 0, st, d, s, H->msum), "k_msum launch");
+    CK(launch_k(H, k_tsen<T, SRC>, dim3(H->n_su), dim3(tsnt<T>()), H->smem_ts, st, d, a, H->lay_ts, pair_bufs<T>(H)),
+       "k_tsen launch");
     return FEWHA_OK;
 }
 
@@ -546,6 +581,11 @@ struct Defer {
     int rz_slot = 0;
 };
 
+// The layers' shares of r.z and p.q of a slot (the forward kernels write them, see
+// layer_slot), TC_SH a layer.
+double* rz_shares(fewha_handle* H, int k) { return H->lshz + static_cast<size_t>(k) * MAXL * TC_SH; }
+double* pq_shares(fewha_handle* H, int k) { return H->lshq + static_cast<size_t>(k) * MAXL * TC_SH; }
+
 // q = M x (Eq. 6); the p.q partials go to slot `slot` (PQ_SLOTS doubles per slot).
 // With pold, x is the CG direction p = z + beta pold, formed first (iteration `slot`) in
 // another buffer than pold's.
@@ -555,7 +595,8 @@ int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int sl
     T* phi = static_cast<T*>(H->phi);
     int rc;
     ClArgs<T> a = cl_args<T>(H, x, phi);
-    a.zero_piston = 1;                 // the data path's input leaves the piston out
+    a.zero_piston = 1;
+    a.fsh = H->fsh;                 // the data path's input leaves the piston out
     a.rz_parts = df.rz_parts;
     a.rz_cnt = df.rz_cnt;
     a.rz_slot = df.rz_slot;
@@ -573,6 +614,7 @@ int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int sl
     ClArgs<T> b = cl_args<T>(H, nullptr, qout);
     b.pin = x;
     b.iter = slot;
+    b.lsh = pq_shares(H, slot);
     b.zero_piston = 1;
     b.defer_total = df.pq ? 1 : 0;
     return launch_fwd<T, LDST_APPLY>(H, d, b, st);
@@ -589,6 +631,7 @@ int enqueue_apply_aug(fewha_handle* H, const Desc<T>& d, const T* pold, T* pnew,
     int rc;
     ClArgs<T> a = cl_args<T>(H, nullptr, phi);
     a.zero_piston = 1;
+    a.fsh = H->fsh;
     a.pupd = const_cast<T*>(pold);       // read only by the augmented update
     a.zupd = z;
     a.pout = pnew;
@@ -608,6 +651,7 @@ int enqueue_apply_aug(fewha_handle* H, const Desc<T>& d, const T* pold, T* pnew,
     ClArgs<T> b = cl_args<T>(H, nullptr, qout);
     b.pin = pnew;
     b.iter = slot;
+    b.lsh = pq_shares(H, slot);
     b.zero_piston = 1;
     b.defer_total = df.pq ? 1 : 0;
     return launch_fwd<T, LDST_APPLY>(H, d, b, st);
@@ -624,11 +668,13 @@ int enqueue_apply_init(fewha_handle* H, const Desc<T>& d, T* c, cudaStream_t st,
     int rc;
     ClArgs<T> a = cl_args<T>(H, x, phi);
     a.zero_piston = 1;
+    a.fsh = H->fsh;
     if ((rc = launch_inv<T, 0>(H, d, a, st))) return rc;
     if ((rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st))) return rc;
     ClArgs<T> b = cl_args<T>(H, nullptr, static_cast<T*>(H->q));
     b.pin = x;
     b.iter = slot;
+    b.lsh = rz_shares(H, 0);
     b.zero_piston = 1;
     b.vr = static_cast<T*>(H->r);
     b.vz = static_cast<T*>(H->z);
@@ -637,7 +683,6 @@ int enqueue_apply_init(fewha_handle* H, const Desc<T>& d, T* c, cudaStream_t st,
     b.vbprev = static_cast<T*>(H->b_prev);
     b.vj = static_cast<const T*>(H->Jinv);
     b.rzslot = 0;
-    b.rzp = H->rzpart;
     b.defer_total = defer ? 1 : 0;
     return launch_fwd<T, LDST_APPLY_INIT>(H, d, b, st);
 }
@@ -650,23 +695,26 @@ int enqueue_apply_init(fewha_handle* H, const Desc<T>& d, T* c, cudaStream_t st,
 // right-hand side's 3 plus the apply's 5.  b and b_prev are not written.
 template <class T>
 int enqueue_resid_init(fewha_handle* H, const Desc<T>& d, const T* s, T* c, cudaStream_t st, bool defer,
-                       T* p0 = nullptr, T* phi_out = nullptr) {
+                       T* p0 = nullptr, T* phi_out = nullptr, T* r0 = nullptr, T* z0 = nullptr) {
     T* phi = phi_out ? phi_out : static_cast<T*>(H->phi);
     int rc;
     ClArgs<T> a = cl_args<T>(H, c, phi);
     a.zero_piston = 1;
+    a.fsh = H->fsh;
+    a.ms = s;
+    a.msum = H->msum;
     if ((rc = launch_inv<T, 0>(H, d, a, st))) return rc;
     if ((rc = launch_csensor<T, SSRC_RESID>(H, d, phi, s, st))) return rc;
     ClArgs<T> b = cl_args<T>(H, nullptr, static_cast<T*>(H->q));
     b.pin = c;
     b.iter = PQ_SCRATCH_SLOT;
+    b.lsh = rz_shares(H, 0);
     b.zero_piston = 1;
-    b.vr = static_cast<T*>(H->r);
-    b.vz = static_cast<T*>(H->z);
+    b.vr = r0 ? r0 : static_cast<T*>(H->r);
+    b.vz = z0 ? z0 : static_cast<T*>(H->z);
     b.vp = p0 ? p0 : static_cast<T*>(H->p);
     b.vj = static_cast<const T*>(H->Jinv);
     b.rzslot = 0;
-    b.rzp = H->rzpart;
     b.defer_total = defer ? 1 : 0;
     return launch_fwd<T, LDST_RESID_INIT>(H, d, b, st);
 }
@@ -685,7 +733,7 @@ int vec_grid(const fewha_handle* H) { return H->npart; }
 template <class T, int PHASE>
 int launch_vec(fewha_handle* H, int n, const VecArgs<T>& v, cudaStream_t st) {
     if (recorder<T>()) {
-        record<T>(PHASE == V_INIT ? BK_VEC_INIT : PHASE == V_INIT_WARM ? BK_VEC_WARM : BK_VEC_UPDATE).va = v;
+        record<T>(PHASE == V_INIT ? BK_VEC_INIT : BK_VEC_WARM).va = v;
         return FEWHA_OK;
     }
     CK(launch_k(H, k_vec<T, PHASE>, dim3(vec_grid(H)), dim3(PBLK), 0, st, n, v), "k_vec launch");
@@ -728,80 +776,99 @@ T* dir_buf(fewha_handle* H, int k) {
     return static_cast<T*>((k & 1) ? H->p2 : H->p);
 }
 
+// The vectors of one CG iteration (enqueue_iteration).
+template <class T>
+struct CgVecs {
+    T* c;
+    T* p;               // direction of this iteration
+    const T* pold;      // the one before (another buffer); null: p is given
+    const T* z;         // z of the direction update
+    const T* r;         // r before and after, z after
+    T* rnew;
+    T* znew;
+    T* q;               // q = M p, if wanted
+    T* phic;            // layers of c carried along, if wanted
+};
+
+
+// Iteration k of the PCG (Sec. 3.3) in four kernels: p = z + beta p_old and W^T p, the
+// sensors, and the two forward kernels with the update c += alpha p, r -= alpha q,
+// z = J^-1 r in their epilogues (p.q is known before q, see ClArgs::pqs).  The r.z total of
+// slot k comes from `rz_cnt` shares at rz_shares(H, k), or (0) is there already; that of
+// slot k + 1 is left as shares (`last`: totalled).
+template <class T>
+int enqueue_iteration(fewha_handle* H, const Desc<T>& d, const CgVecs<T>& v, int k, int rz_cnt, bool last,
+                      cudaStream_t st) {
+    T* phi = static_cast<T*>(H->phi);
+    int rc;
+    ClArgs<T> a = cl_args<T>(H, v.p, phi);
+    a.zero_piston = 1;
+    a.fsh = H->fsh;
+    a.rz_parts = rz_shares(H, k);
+    a.rz_cnt = rz_cnt;
+    a.rz_slot = k;
+    a.iter = k;
+    if (v.pold) {
+        a.pupd = const_cast<T*>(v.pold);     // read only
+        a.pout = v.p;
+        a.zupd = v.z;
+        rc = launch_inv<T, 1>(H, d, a, st);
+    } else {
+        rc = launch_inv<T, 0>(H, d, a, st);
+    }
+    if (rc || (rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st, static_cast<const T*>(v.p)))) return rc;
+    ClArgs<T> b = cl_args<T>(H, nullptr, v.q);
+    b.pin = v.p;
+    b.iter = k;
+    b.lsh = rz_shares(H, k + 1);
+    b.zero_piston = 1;
+    b.pqs = H->pqs;
+    b.n_pqs = H->n_su;
+    b.alphas = static_cast<T*>(H->alphas);
+    b.vc = v.c;
+    b.phic = v.phic;
+    b.phip = phi;
+    b.rin = v.r;
+    b.vr = v.rnew;
+    b.vz = v.znew;
+    b.vj = static_cast<const T*>(H->Jinv);
+    b.rzslot = k + 1;
+    b.defer_total = last ? 0 : 1;
+    return launch_fwd<T, LDST_UPDATE>(H, d, b, st);
+}
+
+// The iteration on the handle's own vectors, the direction buffers in turn.
+template <class T>
+CgVecs<T> cg_vecs(fewha_handle* H, T* c, int turn, bool first, T* phic = nullptr) {
+    T* r = static_cast<T*>(H->r);
+    T* z = static_cast<T*>(H->z);
+    return CgVecs<T>{c, dir_buf<T>(H, turn), first ? nullptr : dir_buf<T>(H, turn + 1), z, r, r, z, nullptr, phic};
+}
+
 // `iters` PCG iterations on M c = b (b in H->b), r0 explicit or warm.
-// With s_resid (the explicit residual, single instances), r0 comes from the slopes'
-// residual chain (enqueue_resid_init) and b is not formed.
+// With s_resid (the explicit residual), r0 comes from the slopes' residual chain
+// (enqueue_resid_init) and b is not formed.
 template <class T>
 int enqueue_pcg(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool warm, cudaStream_t st,
-                const T* s_resid = nullptr, bool carry = false) {
+                const T* s_resid = nullptr, bool carry = false, bool total = true) {
     // carry (with s_resid): the layers of c are carried through the iterations in H->phic
     // (W^T c without the full layers' pistons; the fit adds them), so the fit needs no
     // inverse transform
     T* phic = (carry && s_resid) ? static_cast<T*>(H->phic) : nullptr;
     int rc;
-    // the initial residual's vector step fused into the forward kernel (single instances; the
-    // batched frame keeps the separate vector kernel).  The iterations' CG updates stay in
-    // their own kernel: fused behind a grid-wide wait for the p.q total (a cooperative
-    // launch) they measured slower on GB300 than the separate launch.
-    //
-    // Dot totals are deferred to their consumers: no kernel of an iteration waits for a
-    // grid-wide arrival count.  p.q of iteration k is totalled by the CG update of k; r.z of
-    // slot k (the initial residual's for k = 0, else the update of k - 1) by the inverse
-    // kernel that starts iteration k, which needs it for beta.  Every total still reaches
-    // its slot (rztot[iters] through the last update's own arrival count).
-    if (!recorder<T>()) {
-        const bool defer = iters > 0;
-        if (warm) {
-            if ((rc = launch_vec<T, V_INIT_WARM>(H, d.n_c, vec_args<T>(H, c, 0), st))) return rc;
-        } else if (s_resid) {
-            if ((rc = enqueue_resid_init<T>(H, d, s_resid, c, st, defer, nullptr, phic))) return rc;
-        } else {
-            if ((rc = enqueue_apply_init<T>(H, d, c, st, defer))) return rc;
-        }
-        for (int k = 0; k < iters; ++k) {
-            Defer df;
-            df.pq = true;
-            if (k > 0) {
-                df.rz_parts = H->rzpart + static_cast<size_t>(k) * H->npart;
-                df.rz_cnt = H->npart;
-                df.rz_slot = k;
-            } else if (!warm) {
-                df.rz_parts = H->rzpart;
-                df.rz_cnt = d.n_layers;
-                df.rz_slot = 0;
-            }
-            T* p = dir_buf<T>(H, k);
-            if ((rc = enqueue_apply<T>(H, d, p, static_cast<T*>(H->q), k, k > 0 ? dir_buf<T>(H, k - 1) : nullptr, st, df)))
-                return rc;
-            VecArgs<T> v = vec_args<T>(H, c, k);
-            v.p = p;
-            v.pq_cnt = d.n_layers;
-            v.defer_rz = k + 1 < iters ? 1 : 0;
-            v.phic = phic;
-            v.phip = static_cast<const T*>(H->phi);
-            if ((rc = launch_vec<T, V_UPDATE>(H, d.n_c, v, st))) return rc;
-        }
-        return FEWHA_OK;
-    }
-    if (warm) {
-        if ((rc = launch_vec<T, V_INIT_WARM>(H, d.n_c, vec_args<T>(H, c, 0), st))) return rc;
-    } else if (s_resid) {
-        if ((rc = enqueue_resid_init<T>(H, d, s_resid, c, st, false, nullptr, phic))) return rc;
-    } else {
-        if ((rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, nullptr, st))) return rc;
-        if ((rc = launch_vec<T, V_INIT>(H, d.n_c, vec_args<T>(H, c, 0), st))) return rc;
-    }
-    for (int k = 0; k < iters; ++k) {
-        T* p = dir_buf<T>(H, k);
-        if ((rc = enqueue_apply<T>(H, d, p, static_cast<T*>(H->q), k, k > 0 ? dir_buf<T>(H, k - 1) : nullptr, st)))
-            return rc;
-        VecArgs<T> v = vec_args<T>(H, c, k);
-        v.p = p;
-        v.phic = phic;
-        v.phip = static_cast<const T*>(H->phi);
-        if ((rc = launch_vec<T, V_UPDATE>(H, d.n_c, v, st))) return rc;
-    }
-    return FEWHA_OK;
+    // Dot totals are left to their consumers: no kernel of an iteration waits for a grid-wide
+    // arrival count.  Every total still reaches its slot; rztot[iters] through the last
+    // iteration's own arrival count, and only with `total`: a frame has no reader for it.
+    const bool defer = iters > 0;
+    if (warm)
+        rc = launch_vec<T, V_INIT_WARM>(H, d.n_c, vec_args<T>(H, c, 0), st);
+    else if (s_resid)
+        rc = enqueue_resid_init<T>(H, d, s_resid, c, st, defer, nullptr, phic);
+    else
+        rc = enqueue_apply_init<T>(H, d, c, st, defer);
+    for (int k = 0; k < iters && !rc; ++k)
+        rc = enqueue_iteration<T>(H, d, cg_vecs<T>(H, c, k, k == 0, phic), k, k > 0 || !warm ? d.n_layers * TC_SH : 0, total && k + 1 == iters, st);
+    return rc;
 }
 
 template <class T, int PHASE>
@@ -895,7 +962,8 @@ int enqueue_pcg_aug(fewha_handle* H, const Desc<T>& d, T* c, int iters, bool war
         if (rc) return rc;
         v.p = pk;
         v.q = qk;
-        v.pq_cnt = defer ? d.n_layers : 0;
+        v.pq_cnt = defer ? d.n_layers * TC_SH : 0;
+        v.pq_parts = pq_shares(H, k);
         v.defer_rz = (defer && k + 1 < iters) ? 1 : 0;
         a.mu_next = (m > 0 && k + 1 < iters) ? 1 : 0;
         if ((rc = launch_aug<T, V_UPDATE_AUG>(H, d.n_c, v, a, st))) return rc;
@@ -1005,7 +1073,7 @@ int enqueue_frame(fewha_handle* H, const T* s, T* c, T* dm, bool warm, cudaStrea
     if (H->params.flags & FEWHA_FLAG_AUGMENTED)
         rc = enqueue_pcg_aug<T>(H, d, c, H->params.iters, warm, H->aug_set, H->aug_m, st, resid ? s : nullptr);
     else
-        rc = enqueue_pcg<T>(H, d, c, H->params.iters, warm, st, resid ? s : nullptr, carry);
+        rc = enqueue_pcg<T>(H, d, c, H->params.iters, warm, st, resid ? s : nullptr, carry, false);
     if (rc) return rc;
     return enqueue_fit<T>(H, d, c, dm, true, st, carry);
 }
@@ -1074,6 +1142,9 @@ int run_frame(fewha_handle* H, const T* s, T* c, T* dm, cudaStream_t st) {
 
 // D, the exact data diagonal (GPU) and J^-1 for the current parameters.
 template <class T>
+int functional_tables(fewha_handle* H);
+
+template <class T>
 int compute_diagonals(fewha_handle* H) {
     std::vector<double> D;
     prior_diag(H->setup, H->weights, H->params.r0, H->params.L0, D);
@@ -1088,6 +1159,7 @@ int compute_diagonals(fewha_handle* H) {
         su.dlev[l * (MAXLEV + 1) + L.levels + 1] = D[L.off];
     }
     if (upload(H, H->gdev, H->setup.G)) return FEWHA_ERR_CUDA;   // sigma and the elongation constants
+    if (const int rc = functional_tables<T>(H)) return rc;
     const Desc<T> d = make_desc<T>(H);
     DiagArgs a{H->basis, H->basis_off, H->pfy64, H->pfx64, H->Jdata};
     k_jdiag<T><<<(d.n_c + 3) / 4, 128>>>(d, a);
@@ -1129,28 +1201,6 @@ int allow_smem(fewha_handle* H, K kernel, size_t need) {
     return FEWHA_OK;
 }
 
-// The sensor kernel in both cluster sizes; clusters of 16 are above the portable size.  They
-// are used where the device can hold all of the instance's at once: the sensors' bands are
-// then half as high.
-template <class T, int SRC>
-int allow_sensor(fewha_handle* H) {
-    int rc;
-    if ((rc = allow_smem(H, k_tsen<T, SRC, 16>, H->smem_ts[0])) || (rc = allow_smem(H, k_tsen<T, SRC, 8>, H->smem_ts[1])))
-        return rc;
-    CK(cudaFuncSetAttribute(k_tsen<T, SRC, 16>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1), "cluster attr");
-    if (SRC == SSRC_PHI) {
-        cudaLaunchConfig_t q = {};
-        q.gridDim = dim3(16, static_cast<unsigned>(H->setup.G.size()));
-        q.blockDim = dim3(tsnt<T>());
-        q.dynamicSmemBytes = H->smem_ts[0];
-        int fit = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveClusters(&fit, k_tsen<T, SRC, 16>, &q);
-        if (e != cudaSuccess) cudaGetLastError();
-        H->wide_cluster = e == cudaSuccess && fit >= static_cast<int>(H->setup.G.size());
-    }
-    return FEWHA_OK;
-}
-
 template <class T>
 int set_smem_limits(fewha_handle* H) {
     const int maxsm = 227 * 1024;
@@ -1183,6 +1233,7 @@ int set_smem_limits(fewha_handle* H) {
     if ((rc = allow_smem(H, k_tfwd<T, LDST_APPLY>, H->smem_tf)) || (rc = allow_smem(H, k_tfwd<T, LDST_COEF>, H->smem_tf)) ||
         (rc = allow_smem(H, k_tfwd<T, LDST_APPLY_INIT>, H->smem_tf)) ||
         (rc = allow_smem(H, k_tfwd<T, LDST_RESID_INIT>, H->smem_tf)) ||
+        (rc = allow_smem(H, k_tfwd<T, LDST_UPDATE>, H->smem_tf)) || (rc = allow_smem(H, k_tcoarse<T, LDST_UPDATE>, H->smem_tc)) ||
         (rc = allow_smem(H, k_tcoarse<T, LDST_APPLY>, H->smem_tc)) ||
         (rc = allow_smem(H, k_tcoarse<T, LDST_COEF>, H->smem_tc)) ||
         (rc = allow_smem(H, k_tcoarse<T, LDST_APPLY_INIT>, H->smem_tc)) ||
@@ -1190,8 +1241,8 @@ int set_smem_limits(fewha_handle* H) {
         (rc = allow_smem(H, k_tinv<T, 0>, H->smem_tinv)) ||
         (rc = allow_smem(H, k_tinv<T, 1>, H->smem_tinv)) ||
         (rc = allow_smem(H, k_tinv<T, 2>, H->smem_tinv)) ||
-        (rc = allow_sensor<T, SSRC_PHI>(H)) || (rc = allow_sensor<T, SSRC_SLOPES>(H)) ||
-        (rc = allow_sensor<T, SSRC_RESID>(H)))
+        (rc = allow_smem(H, k_tsen<T, SSRC_PHI>, H->smem_ts)) || (rc = allow_smem(H, k_tsen<T, SSRC_SLOPES>, H->smem_ts)) ||
+        (rc = allow_smem(H, k_tsen<T, SSRC_RESID>, H->smem_ts)))
         return rc;
     return FEWHA_OK;
 }
@@ -1208,7 +1259,6 @@ bool tail_used(const HostSetup& s) {
 // Shared-memory layouts of the cluster kernels: the largest band over all layers and
 // sensors, element counts in T units after a fixed header; every region starts on a
 // 16-byte boundary (cp.async targets).
-int round4(int x) { return (x + 3) & ~3; }
 
 // Tables and shared-memory layouts of the tile, band and sensor kernels (fewha_tile.cuh).
 template <class T>
@@ -1219,7 +1269,6 @@ int tile_tables(fewha_handle* H) {
     // ---- inverse transform: tiles of 32 x 32 nodes (the layer, if smaller) ----------------
     std::vector<TileLayer> tl(nl);
     std::vector<std::vector<unsigned>> slot(nl);           // level | quadrant << 4 | row << 6 | column << 12
-    size_t smem = 0;
     for (int l = 0; l < nl; ++l) {
         const LayerInfo& L = s.L[l];
         TileLayer& t = tl[l];
@@ -1260,7 +1309,7 @@ int tile_tables(fewha_handle* H) {
         t.vbuf = off;
         for (int j = 1; j <= t.J; ++j) vmax = std::max(vmax, t.w[j - 1] * (2 * t.w[j] + 1));
         off += vmax;
-        smem = std::max(smem, static_cast<size_t>((H->tailop ? TAIL_N : 0) + off) * sizeof(T));
+        H->lay_inv_elems = std::max(H->lay_inv_elems, static_cast<size_t>((H->tailop ? TAIL_N : 0) + std::max(off, t.w[0] * t.w[0])));
         auto put = [&](int j, int q, int w) {
             for (int r = 0; r < w; ++r)
                 for (int c = 0; c < w; ++c) slot[l].push_back(static_cast<unsigned>(j | q << 4 | r << 6 | c << 12));
@@ -1276,7 +1325,6 @@ int tile_tables(fewha_handle* H) {
         H->tu0[l + 1] = H->tu0[l] + t.side * t.side;
     }
     H->n_tu = H->tu0[nl];
-    H->smem_tinv = smem;
     std::vector<TilePlace> place(static_cast<size_t>(H->n_tu) * H->tslot_ld, TilePlace{0, 0});
     for (int l = 0; l < nl; ++l) {
         const LayerInfo& L = s.L[l];
@@ -1309,7 +1357,7 @@ int tile_tables(fewha_handle* H) {
     auto ints = [](int k) { return round4((k + IPT - 1) / IPT); };
     // ---- forward transform: bands of rows, their row weights of the adjoint projection ------
     std::vector<T> brow;
-    std::vector<int> tcl;
+    std::vector<int> tcl, vec;
     std::vector<int> bsrc, row0;                           // row0: first staged row per unit and sensor
     const int nyslot = H->pyslot;
     int rw = 0, yw = 0, lb1 = 0, lbc = 0;
@@ -1366,14 +1414,22 @@ int tile_tables(fewha_handle* H) {
         rw = std::max(rw, ry * ng * (kt + 1));
         yw = std::max(yw, ry * ((h + 1) & ~1));
         if (bands == 1) {
+            ++H->n_writers;
             lb1 = std::max(lb1, h * (h + 1));
             tail1 = tail1 || tl[l].tail;
         } else {
             lbc = std::max(lbc, h * (h + 1));
+            // the leader, the quadrants of the level below the finest, chunks of the layer's vectors
             tcl.push_back(l);
+            const int quads = n > 64 ? 4 : 1, chunks = (n * n + TC_VEC - 1) / TC_VEC;
+            for (int k = 0; k < quads; ++k) tcl.push_back(l | (1 + k) << 8);
+            H->n_writers += 1 + (L.levels >= 2 ? quads : 0);
+            for (int k = 0; k < chunks; ++k) vec.push_back(l | (TC_SH + k) << 8);
         }
     }
     H->n_bu = H->bu0[nl];
+    H->n_coarse = static_cast<int>(tcl.size());
+    tcl.insert(tcl.end(), vec.begin(), vec.end());
     H->n_tcl = static_cast<int>(tcl.size());
     for (int l = nl; l < MAXL; ++l) H->tu0[l + 1] = H->bu0[l + 1] = 1 << 30;
     const size_t hdr = CWMAX * sizeof(double);
@@ -1418,10 +1474,12 @@ int tile_tables(fewha_handle* H) {
     H->lay_tf = f;
     H->smem_tf = hdr + static_cast<size_t>(f.total) * sizeof(T);
     TcLayout q{};
+    // lbuf: h/2 x (h/2 + 1) (or the whole LL block of a layer of one level, or a quadrant's
+    // region); tmp: the LL block; st: its rows' scaling half
     q.lbuf = 0;
-    q.tmp = round4(lbc);
-    q.st = 2 * round4(lbc);
-    q.total = q.st + (lbc ? 3 * (MAXN / 2) * (MAXN / 2) : 0);
+    q.tmp = round4(std::max(lbc, 36 * 37));
+    q.st = q.tmp + round4(lbc);
+    q.total = q.st + round4(lbc);
     if (H->tailop && lbc) {
         q.tail = q.total;
         q.total += round4(TAIL_N);
@@ -1431,21 +1489,13 @@ int tile_tables(fewha_handle* H) {
     tcl.push_back(0);
     // ---- sensor kernel ----------------------------------------------------------------------
     std::vector<int> txi, tyi, tcin, tsco, tybox;
-    std::vector<T> txf, tyf, tcw;
+    std::vector<T> txf, tyf;
     H->tnp = round4(s.max_N + 1);
-    int kx = 0;
     for (int g = 0; g < ng; ++g) {
         int c = 0;
-        for (int l = 0; l < nl; ++l) {
-            c += round4(H->box_host[(g * MAXL + l) * 4 + 3]);
-            for (int j = 0; j < s.L[l].n; ++j) {
-                const int k = (g * MAXL + l) * MAXN + j;
-                kx = std::max(kx, s.rx_hi[k] - s.rx_lo[k]);
-            }
-        }
+        for (int l = 0; l < nl; ++l) c += round4(H->box_host[(g * MAXL + l) * 4 + 3]);
         H->tcols = std::max(H->tcols, c);
     }
-    H->tks = kx <= 4 ? 4 : KMAX;
     for (int g = 0; g < ng; ++g) {
         int c = 0;
         for (int l = 0; l < nl; ++l) {
@@ -1461,47 +1511,40 @@ int tile_tables(fewha_handle* H) {
             tsco.push_back(c);
             tybox.push_back(bx[3]);
             tybox.push_back((g * nl + l) * H->pyslot);
+            tybox.push_back(s.L[l].off + bx[2]);
+            tybox.push_back(0);
             for (int k = 0; k < round4(bx[3]); ++k, ++c) {
                 const int j = bx[2] + k, e = (g * MAXL + l) * MAXN + j;
                 const int lo = k < bx[3] && j < n ? s.rx_lo[e] : 0, cnt = k < bx[3] && j < n ? s.rx_hi[e] - lo : 0;
-                tcin.push_back(lo);
-                tcin.push_back(cnt);
-                for (int q = 0; q < H->tks; ++q) {
-                    T w = T(0);
-                    if (q < cnt) {
-                        const T f = static_cast<T>(s.pfx[tp + lo + q]);
-                        w = s.pi0x[tp + lo + q] == j ? T(1) - f : f;
-                    }
-                    tcw.push_back(w);
-                }
+                tcin.push_back(lo | cnt << 16);
             }
         }
         tsco.push_back(c);
         for (int l = nl; l < MAXL; ++l) {
             tsco.push_back(c);
-            tybox.push_back(0);
-            tybox.push_back(0);
+            tybox.insert(tybox.end(), 4, 0);
         }
-        tcin.resize(static_cast<size_t>(g + 1) * H->tcols * 2, 0);
-        tcw.resize(static_cast<size_t>(g + 1) * H->tcols * H->tks, T(0));
+        tcin.resize(static_cast<size_t>(g + 1) * H->tcols, 0);
     }
-    for (int w = 0; w < 2; ++w) {
-        const int scl = w == 0 ? 16 : 8, sr = (s.max_N + scl - 1) / scl;
-        TsLayout v{};
-        v.V = 0;
-        v.SX = v.V + round4((sr + 2) * (s.max_N + 1));
-        v.SY = v.SX + round4((sr + 1) * s.max_N);
-        v.msk = v.SY + round4((sr + 1) * s.max_N);
-        v.xi = v.msk + ints((sr + 1) * s.max_N);
-        v.xf = v.xi + ints(nl * H->tnp);
-        v.yi = v.xf + round4(nl * H->tnp);
-        v.yf = v.yi + ints(2 * nl * (sr + 2));
-        v.cw = v.yf + round4(nl * (sr + 2));
-        v.ci = v.cw + H->tcols * H->tks;
-        v.total = v.ci + ints(2 * H->tcols);
-        H->lay_ts[w] = v;
-        H->smem_ts[w] = static_cast<size_t>(v.total) * sizeof(T);
-    }
+    constexpr int SR = TS_ROWS;
+    for (int g = 0; g < ng; ++g) H->su0[g + 1] = H->su0[g] + (s.G[g].N + SR - 1) / SR;
+    H->n_su = H->su0[ng];
+    for (int g = ng; g < MAXG; ++g) H->su0[g + 1] = H->n_su;
+    TsLayout v{};
+    v.V = 0;
+    v.SX = v.V + round4((SR + 2) * (s.max_N + 1));
+    v.SY = v.SX + round4((SR + 1) * s.max_N);
+    v.msk = v.SY + round4((SR + 1) * s.max_N);
+    v.xi = v.msk + ints((SR + 1) * s.max_N);
+    v.xf = v.xi + ints(nl * H->tnp);
+    v.yi = v.xf + round4(nl * H->tnp);
+    v.yf = v.yi + ints(2 * nl * (SR + 2));
+    v.ci = v.yf + round4(nl * (SR + 2));
+    v.dot = v.ci + ints(H->tcols);
+    v.total = v.dot + tsnt<T>() * static_cast<int>(sizeof(double) / sizeof(T));
+    H->lay_ts = v;
+    H->smem_ts = static_cast<size_t>(v.total) * sizeof(T);
+    H->tl_host = tl;
     int rc;
     if ((rc = dalloc(H, &H->tl, tl.size())) || (rc = upload(H, H->tl, tl)) || (rc = dalloc(H, &H->tslot, place.size())) ||
         (rc = upload(H, H->tslot, place)) || (rc = talloc(H, &H->brow, brow.size())) || (rc = dalloc(H, &H->bsrc, bsrc.size())) || (rc = upload(H, H->bsrc, bsrc)) ||
@@ -1509,12 +1552,151 @@ int tile_tables(fewha_handle* H) {
         (rc = upload(H, H->tcl, tcl)) || (rc = dalloc(H, &H->gdev, s.G.size())) || (rc = dalloc(H, &H->txi, txi.size() + 4)) || (rc = upload(H, H->txi, txi)) ||
         (rc = dalloc(H, &H->tyi, tyi.size())) || (rc = upload(H, H->tyi, tyi)) || (rc = talloc(H, &H->txf, txf.size())) ||
         (rc = upload(H, static_cast<T*>(H->txf), txf)) || (rc = talloc(H, &H->tyf, tyf.size())) ||
-        (rc = upload(H, static_cast<T*>(H->tyf), tyf)) || (rc = talloc(H, &H->tcw, tcw.size())) ||
-        (rc = upload(H, static_cast<T*>(H->tcw), tcw)) || (rc = dalloc(H, &H->tcin, tcin.size())) ||
+        (rc = upload(H, static_cast<T*>(H->tyf), tyf)) || (rc = dalloc(H, &H->tcin, tcin.size() + 4)) ||
         (rc = upload(H, H->tcin, tcin)) || (rc = dalloc(H, &H->tsco, tsco.size())) || (rc = upload(H, H->tsco, tsco)) ||
         (rc = dalloc(H, &H->tybox, tybox.size())) || (rc = upload(H, H->tybox, tybox)) ||
+        (rc = dalloc(H, &H->pqs, H->n_su)) || (rc = dalloc(H, &H->lshz, static_cast<size_t>(FEWHA_MAX_ITERS + 2) * MAXL * TC_SH)) ||
+        (rc = dalloc(H, &H->lshq, static_cast<size_t>(FEWHA_MAX_ITERS + 2) * MAXL * TC_SH)) || (rc = talloc(H, &H->alphas, FEWHA_MAX_ITERS + 2)) ||
         (rc = talloc(H, &H->ll, s.n_c / 4)) || (rc = dalloc(H, &H->tshare, H->n_bu)))
         return rc;
+    return FEWHA_OK;
+}
+
+// The functionals of the layers that the sensors' weighting needs (Desc::foff): node fields
+// Gamma^T of the summed slopes' weights, through P^T to the layers (both exact transposes of
+// what the sensor kernel applies), cut into the tiles.  Rebuilt when the elongation changes.
+template <class T>
+int functional_tables(fewha_handle* H) {
+    const HostSetup& s = H->setup;
+    if (H->fun_eta == H->params.alpha_eta) return FEWHA_OK;
+    const int nl = static_cast<int>(s.L.size()), ng = static_cast<int>(s.G.size());
+    int nf = 0;
+    for (int g = 0; g < ng; ++g) {
+        H->f0[g] = nf;
+        nf += s.G[g].lgs ? (s.G[g].el ? 4 : 2) : s.G[g].nb > 1 ? 2 * s.G[g].n_sub * s.G[g].n_sub : 0;
+    }
+    for (int g = ng; g <= MAXG; ++g) H->f0[g] = nf;
+    std::vector<std::vector<std::pair<int, double>>> ent(static_cast<size_t>(H->n_tu) * std::max(nf, 1));
+    std::vector<double> v, dense(static_cast<size_t>(MAXN) * MAXN, 0.0);
+    std::vector<int> nodes, hit;
+    for (int g = 0; g < ng; ++g) {
+        const WfsInfo& W = s.G[g];
+        const int N = W.N, NP = N + 1;
+        for (int f = H->f0[g]; f < H->f0[g + 1]; ++f) {
+            const int e = f - H->f0[g];
+            // node field of sum over the active subapertures of ax s^x + ay s^y
+            v.assign(static_cast<size_t>(NP) * NP, 0.0);
+            for (int i = 0; i < N; ++i)
+                for (int j = 0; j < N; ++j) {
+                    if (s.sidx[W.mask_off + i * N + j] < 0) continue;
+                    double ax = e == 0 ? 1.0 : 0.0, ay = e == 1 ? 1.0 : 0.0;
+                    if (W.lgs && e >= 2) {
+                        const double b1 = W.el_k * ((W.el_x0 + j * W.el_d) - W.el_lx);
+                        const double b2 = W.el_k * ((W.el_x0 + i * W.el_d) - W.el_ly);
+                        const double gam = W.el_c / (1.0 + W.el_c * (b1 * b1 + b2 * b2)), b = e == 2 ? b1 : b2;
+                        ax = gam * b * b1;
+                        ay = gam * b * b2;
+                    } else if (!W.lgs) {
+                        const bool in = e >> 1 == (i / W.nb) * W.n_sub + j / W.nb;
+                        ax = in && !(e & 1) ? 1.0 : 0.0;
+                        ay = in && (e & 1) ? 1.0 : 0.0;
+                    }
+                    double* p = &v[static_cast<size_t>(i) * NP + j];
+                    p[0] += -0.5 * ax - 0.5 * ay;
+                    p[1] += 0.5 * ax - 0.5 * ay;
+                    p[NP] += -0.5 * ax + 0.5 * ay;
+                    p[NP + 1] += 0.5 * ax + 0.5 * ay;
+                }
+            nodes.clear();
+            for (int k = 0; k < NP * NP; ++k)
+                if (v[k] != 0.0) nodes.push_back(k);
+            for (int l = 0; l < nl; ++l) {
+                const int tp = (g * MAXL + l) * TAB, n = s.L[l].n;
+                hit.clear();
+                for (int k : nodes) {
+                    const int a = k / NP, b = k % NP, y = s.pi0y[tp + a], x = s.pi0x[tp + b];
+                    const double fy = s.pfy[tp + a], fx = s.pfx[tp + b];
+                    for (int c = 0; c < 4; ++c) {
+                        const int at = (y + (c >> 1)) * n + x + (c & 1);
+                        const double w = (c >> 1 ? fy : 1.0 - fy) * (c & 1 ? fx : 1.0 - fx) * v[k];
+                        if (w == 0.0) continue;
+                        if (dense[at] == 0.0) hit.push_back(at);
+                        dense[at] += w;
+                    }
+                }
+                std::sort(hit.begin(), hit.end());
+                const TileLayer& t = H->tl_host[l];
+                const int ts = t.w[0];
+                for (int at : hit) {
+                    if (dense[at] == 0.0) continue;          // (listed twice, or cancelled)
+                    const int y = at / n, x = at % n;
+                    const int u = H->tu0[l] + (y >> t.lts) * t.side + (x >> t.lts);
+                    ent[static_cast<size_t>(u) * nf + f].emplace_back((y & (ts - 1)) * ts + (x & (ts - 1)), dense[at]);
+                    dense[at] = 0.0;
+                }
+            }
+        }
+    }
+    std::vector<int> off;
+    std::vector<T> flat;
+    int most = 0;
+    const int pad = round4(3 * nf + 3);
+    for (int u = 0; u < H->n_tu; ++u) {
+        const int at = static_cast<int>(flat.size() / 2);
+        int l = 0, nd = 0;
+        while (u >= H->tu0[l + 1]) ++l;
+        const int nodes2 = H->tl_host[l].w[0] * H->tl_host[l].w[0];
+        std::vector<int> o(pad, 0);
+        for (int f = 0; f < nf; ++f) {
+            const auto& list = ent[static_cast<size_t>(u) * nf + f];
+            o[2 * f] = o[2 * f + 1] = static_cast<int>(flat.size() / 2) - at;
+            if (list.size() > TINV_FEW) {
+                o[2 * f + 1] = o[2 * f] - 1;                 // (among the functionals of many)
+                o[2 * nf + 3 + nd++] = f;
+                continue;
+            }
+            for (const auto& e : list) {
+                flat.push_back(static_cast<T>(e.first));
+                flat.push_back(static_cast<T>(e.second));
+            }
+            o[2 * f + 1] = static_cast<int>(flat.size() / 2) - at;
+        }
+        o[2 * nf] = at;
+        o[2 * nf + 1] = static_cast<int>(flat.size() / 2) - at;
+        o[2 * nf + 2] = nd;
+        for (int i = 0; i < nd; ++i) {
+            const size_t base = flat.size();
+            flat.resize(base + nodes2, T(0));
+            for (const auto& e : ent[static_cast<size_t>(u) * nf + o[2 * nf + 3 + i]])
+                flat[base + e.first] = static_cast<T>(e.second);
+        }
+        most = std::max(most, static_cast<int>(flat.size() / 2) - at);
+        off.insert(off.end(), o.begin(), o.end());
+    }
+    int rc;
+    auto grow = [&](void** p, size_t* cap, size_t need, bool typed) -> int {
+        if (*cap >= need) return FEWHA_OK;
+        int* ip = nullptr;
+        const int e = typed ? talloc(H, p, need) : dalloc(H, &ip, need);
+        if (e) return e;
+        if (!typed) *p = ip;
+        *cap = need;
+        return FEWHA_OK;
+    };
+    void* fo = H->foff;
+    if ((rc = grow(&fo, &H->foff_cap, off.size(), false))) return rc;
+    H->foff = static_cast<int*>(fo);
+    const size_t shares = static_cast<size_t>(std::max(nf, 1)) * H->n_tu;
+    if ((rc = grow(&H->fent, &H->fent_cap, flat.size() + 2, true))) return rc;
+    if (H->fsh_cap < shares && (rc = dalloc(H, &H->fsh, shares))) return rc;
+    H->fsh_cap = std::max(H->fsh_cap, shares);
+    if (!H->msum && (rc = dalloc(H, &H->msum, MAXG * TS_FUN))) return rc;
+    if ((rc = upload(H, H->foff, off)) || (rc = upload(H, static_cast<T*>(H->fent), flat))) return rc;
+    H->n_fun = nf;
+    // staged entries: all of them, as far as 112 KB go
+    H->fcap = std::min(round4(most), static_cast<int>(112 * 1024 / (2 * sizeof(T))));
+    H->smem_tinv = pad * sizeof(int) + (2 * static_cast<size_t>(H->fcap) + H->lay_inv_elems) * sizeof(T);
+    H->fun_eta = H->params.alpha_eta;
     return FEWHA_OK;
 }
 
@@ -1844,7 +2026,7 @@ int typed_create(fewha_handle* H) {
     H->smem_layer = (2 * NWARP + 4) * sizeof(double) + static_cast<size_t>(s.max_n) * s.max_n * sizeof(T);
     H->smem_sensor = (2 * NWARP + 4 + 2 * MAXCOARSE) * sizeof(double) +
                      (static_cast<size_t>(s.max_N + 1) * (s.max_N + 1) + 2 * static_cast<size_t>(s.max_N) * s.max_N) * sizeof(T);
-    if ((rc = cluster_layouts<T>(H)) || (rc = tile_tables<T>(H))) return rc;
+    if ((rc = cluster_layouts<T>(H)) || (rc = tile_tables<T>(H)) || (rc = functional_tables<T>(H))) return rc;
     if ((rc = set_smem_limits<T>(H))) return rc;
     return setup_tables<T>(H);
 }
@@ -1989,7 +2171,6 @@ int solve_converged(fewha_handle* H, const T* b, T* x, bool warm, double tol, in
     double rzb = 0.0, rz = 0.0;
     CK(cudaMemcpyAsync(&rzb, H->gdot + MAXL, sizeof(double), cudaMemcpyDeviceToHost, st), "solve norm");
     int done = 0;
-    T* q = static_cast<T*>(H->q);
     int turn = 0;                                // direction of the newest iteration: dir_buf(turn)
     while (done < max_iters) {
         int last;                                // slot of the newest r.z total
@@ -2004,12 +2185,9 @@ int solve_converged(fewha_handle* H, const T* b, T* x, bool warm, double tol, in
             CK(cudaMemcpyAsync(H->rztot, H->rztot + FEWHA_MAX_ITERS - 1, 2 * sizeof(double),
                                cudaMemcpyDeviceToDevice, st), "solve resume");
             const int k = std::min(FEWHA_MAX_ITERS - 1, max_iters - done);
-            for (int j = 1; j <= k; ++j, ++turn) {
-                VecArgs<T> v = vec_args<T>(H, x, j);
-                v.p = dir_buf<T>(H, turn + 1);
-                if ((rc = enqueue_apply<T>(H, d, v.p, q, j, dir_buf<T>(H, turn), st))) return rc;
-                if ((rc = launch_vec<T, V_UPDATE>(H, d.n_c, v, st))) return rc;
-            }
+            for (int j = 1; j <= k; ++j, ++turn)
+                if ((rc = enqueue_iteration<T>(H, d, cg_vecs<T>(H, x, turn + 1, false), j, j > 1 ? d.n_layers * TC_SH : 0, j == k, st)))
+                    return rc;
             done += k;
             last = k + 1;
         }
@@ -2097,7 +2275,6 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
     double* r64 = static_cast<double*>(X->r);
     double* q64 = static_cast<double*>(X->q);
     float* x32 = static_cast<float*>(H->c_tmp);
-    float* q = static_cast<float*>(H->q);
     int rc;
     double bn2 = 0.0, rr2 = 0.0;
     if ((rc = twin_wnorm(H, X, b64, &bn2, st))) return rc;
@@ -2127,13 +2304,10 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
         int turn = 0;                            // direction of the next iteration: dir_buf(turn)
         for (;;) {
             const int k = std::min(FEWHA_MAX_ITERS - j0, max_iters - done);
-            for (int j = j0; j < j0 + k; ++j, ++turn) {
-                VecArgs<float> vj = vec_args<float>(H, x32, j);
-                vj.p = dir_buf<float>(H, turn);
-                if ((rc = enqueue_apply<float>(H, d, vj.p, q, j, j > 0 ? dir_buf<float>(H, turn + 1) : nullptr, st)))
+            for (int j = j0; j < j0 + k; ++j, ++turn)
+                if ((rc = enqueue_iteration<float>(H, d, cg_vecs<float>(H, x32, turn, j == 0), j, j > j0 ? d.n_layers * TC_SH : 0,
+                                                   j + 1 == j0 + k, st)))
                     return rc;
-                if ((rc = launch_vec<float, V_UPDATE>(H, n, vj, st))) return rc;
-            }
             done += k;
             const int last = j0 + k;
             CK(cudaMemcpyAsync(rz, H->rztot + last - 1, 2 * sizeof(double), cudaMemcpyDeviceToHost, st),
@@ -2557,32 +2731,13 @@ int frame_vjp(fewha_handle* H, const T* s, const T* c0, const T* g_a, T* dm, T* 
     T* qbar = pbi + ld;
     const T* Jinv = static_cast<const T*>(H->Jinv);
     int rc;
-    // ---- forward: b, r0 = b - M c0, then the iterations, every vector kept -------------
-    if ((rc = enqueue_rhs<T>(H, d, s, static_cast<T*>(H->b), st))) return rc;
+    // ---- forward: r0 from the slopes' residual, then the iterations, every vector kept ----
     CK(cudaMemcpyAsync(c, c0, n * sizeof(T), cudaMemcpyDeviceToDevice, st), "vjp c0");
-    if ((rc = enqueue_apply<T>(H, d, c, static_cast<T*>(H->q), PQ_SCRATCH_SLOT, nullptr, st))) return rc;
-    VecArgs<T> v = vec_args<T>(H, c, 0);
-    v.r = R;
-    v.z = Z;
-    v.p = P;
-    v.b_prev = scratch;                            // the handle's b_prev stays untouched
-    if ((rc = launch_vec<T, V_INIT>(H, n, v, st))) return rc;
-    AugArgs<T> a{};
-    a.m = 0;
+    if ((rc = enqueue_resid_init<T>(H, d, s, c, st, k > 0, P, nullptr, R, Z))) return rc;
     for (int i = 0; i < k; ++i) {
-        // p_i = z_i + beta p_(i-1) into its own slot, fused into the apply's inverse kernel
-        if (i > 0)
-            rc = enqueue_apply_aug<T>(H, d, P + (i - 1) * ld, P + i * ld, Z + i * ld, Q + i * ld, i, a, st);
-        else
-            rc = enqueue_apply<T>(H, d, P, Q, 0, nullptr, st);
-        if (rc) return rc;
-        CK(cudaMemcpyAsync(R + (i + 1) * ld, R + i * ld, n * sizeof(T), cudaMemcpyDeviceToDevice, st), "vjp r");
-        VecArgs<T> w = vec_args<T>(H, c, i);
-        w.p = P + i * ld;
-        w.q = Q + i * ld;
-        w.r = R + (i + 1) * ld;
-        w.z = Z + (i + 1) * ld;
-        if ((rc = launch_vec<T, V_UPDATE>(H, n, w, st))) return rc;
+        const CgVecs<T> v{c, P + i * ld, i > 0 ? P + (i - 1) * ld : nullptr, Z + i * ld, R + i * ld, R + (i + 1) * ld,
+                          Z + (i + 1) * ld, Q + i * ld, nullptr};
+        if ((rc = enqueue_iteration<T>(H, d, v, i, d.n_layers * TC_SH, i + 1 == k, st))) return rc;
     }
     if (dm && (rc = enqueue_fit<T>(H, d, c, dm, false, st))) return rc;
     if (!g_a) {
@@ -2667,8 +2822,8 @@ size_t round16(size_t x) { return (x + 15) & ~static_cast<size_t>(15); }
 template <class T>
 size_t barg_size(int kind) {
     switch (kind) {
-        case BK_INV: case BK_INV_UPD: case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT:
-        case BK_TC_APPLY: case BK_TC_COEF: case BK_TC_RINIT:
+        case BK_INV: case BK_INV_UPD: case BK_INV_MS: case BK_MSUM: case BK_FWD_UPD: case BK_FWD_COEF: case BK_FWD_RINIT:
+        case BK_FWD_AINIT: case BK_TC_AINIT: case BK_TC_UPD: case BK_TC_COEF: case BK_TC_RINIT:
             return sizeof(ClArgs<T>);
         case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return sizeof(SensorArgs<T>);
         case BK_FIT: return sizeof(FitArgs<T>);
@@ -2678,10 +2833,10 @@ size_t barg_size(int kind) {
 
 size_t bsmem(const fewha_handle* H, int kind) {
     switch (kind) {
-        case BK_INV: case BK_INV_UPD: return H->smem_tinv;
-        case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return H->smem_tf;
-        case BK_TC_APPLY: case BK_TC_COEF: case BK_TC_RINIT: return H->smem_tc;
-        case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return H->smem_ts[1];
+        case BK_INV: case BK_INV_UPD: case BK_INV_MS: case BK_MSUM: return H->smem_tinv;
+        case BK_FWD_UPD: case BK_FWD_COEF: case BK_FWD_RINIT: case BK_FWD_AINIT: return H->smem_tf;
+        case BK_TC_AINIT: case BK_TC_UPD: case BK_TC_COEF: case BK_TC_RINIT: return H->smem_tc;
+        case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return H->smem_ts;
         default: return 0;
     }
 }
@@ -2740,7 +2895,7 @@ void batch_pack(const std::vector<Recorder<T>>& recs, const std::vector<int>& np
             const BStep<T>& st = recs[i].steps[j];
             unsigned char* dst = out.data() + offs[j] + i * sz;
             switch (bkind_list(kind)) {
-                case BL_LAYER: case BL_TILE: case BL_BAND: std::memcpy(dst, &st.cl, sz); break;
+                case BL_LAYER: case BL_LAYER_UPD: case BL_TILE: case BL_TILE_MS: case BL_MSUM: case BL_BAND: std::memcpy(dst, &st.cl, sz); break;
                 case BL_SENSOR: std::memcpy(dst, &st.sa, sz); break;
                 case BL_FIT: std::memcpy(dst, &st.fa, sz); break;
                 default: {
@@ -2792,9 +2947,11 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
         const int g = grp[i], nl = static_cast<int>(H->setup.L.size()), nw = static_cast<int>(H->setup.G.size());
         for (int k = 0; k < H->n_tu; ++k) lists[g * BL_COUNT + BL_TILE].push_back({i, k});
         for (int k = 0; k < H->n_bu; ++k) lists[g * BL_COUNT + BL_BAND].push_back({i, k});
-        for (int l = 0; l < nl; ++l)
-            if (H->bu0[l + 1] - H->bu0[l] > 1) lists[g * BL_COUNT + BL_LAYER].push_back({i, l});
-        for (int w = 0; w < nw; ++w) lists[g * BL_COUNT + BL_SENSOR].push_back({i, w});
+        for (int k = 0; k < H->n_coarse; ++k) lists[g * BL_COUNT + BL_LAYER].push_back({i, k});
+        for (int k = 0; k < H->n_tcl; ++k) lists[g * BL_COUNT + BL_LAYER_UPD].push_back({i, k});
+        for (int k = 0; k < H->n_su; ++k) lists[g * BL_COUNT + BL_SENSOR].push_back({i, k});
+        for (int k = 0; k < H->n_tu + nw; ++k) lists[g * BL_COUNT + BL_TILE_MS].push_back({i, k});
+        for (int k = 0; k < nw; ++k) lists[g * BL_COUNT + BL_MSUM].push_back({i, H->n_tu + k});
         for (int k = 0; k < nparts[i]; ++k) lists[g * BL_COUNT + BL_VEC].push_back({i, k});
         for (int k = 0; k < (H->setup.n_act + PBLK - 1) / PBLK; ++k) lists[g * BL_COUNT + BL_FIT].push_back({i, k});
     }
@@ -2807,7 +2964,7 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
         I.d = make_desc<T>(H);
         I.lay_tf = H->lay_tf;
         I.lay_tc = H->lay_tc;
-        I.lay_ts = H->lay_ts[1];
+        I.lay_ts = H->lay_ts;
         I.pb = pair_bufs<T>(H);
         I.desc_bytes = static_cast<int>(offsetof(Desc<T>, box) + static_cast<size_t>(I.d.n_wfs) * MAXL * 4 * sizeof(int));
         I.nparts = nparts[i];
@@ -3244,6 +3401,7 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
             case FEWHA_STAGE_LAYER:
             case FEWHA_STAGE_PROJT: {
                 ClArgs<T> a = cl_args<T>(H, nullptr, q);
+                a.lsh = pq_shares(H, PQ_SCRATCH_SLOT);
                 a.pin = p;
                 a.iter = PQ_SCRATCH_SLOT;
                 a.zero_piston = 1;

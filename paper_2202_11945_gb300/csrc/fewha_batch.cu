@@ -21,11 +21,12 @@ __device__ __forceinline__ void load_desc(Desc<T>& sd, const BInst<T>* __restric
     __syncthreads();
 }
 
+// The transform and sensor kernels copy the descriptor and read their tables before their
+// body's wait: none of it is written inside the graph.
 template <class T, int PUPD>
 __global__ void __launch_bounds__(TINV_NT)
     kb_tinv(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
     __shared__ __align__(16) Desc<T> sd;
-    pdl_enter();
     const BItem it = items[blockIdx.x];
     const BInst<T>* I = inst + it.inst;
     load_desc<T>(sd, I);
@@ -37,7 +38,6 @@ template <class T, int DST>
 __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
     kb_tfwd(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
     __shared__ __align__(16) Desc<T> sd;
-    pdl_enter();
     const BItem it = items[blockIdx.x];
     const BInst<T>* I = inst + it.inst;
     load_desc<T>(sd, I);
@@ -51,7 +51,6 @@ template <class T, int DST>
 __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
     kb_tcoarse(const BInst<T>* __restrict__ inst, const ClArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
     __shared__ __align__(16) Desc<T> sd;
-    pdl_enter();
     const BItem it = items[blockIdx.x];
     const BInst<T>* I = inst + it.inst;
     load_desc<T>(sd, I);
@@ -61,17 +60,16 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
 }
 
 template <class T, int SRC>
-__global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(tsnt<T>(), sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(tsnt<T>(), sizeof(T) == 4 ? 2 : 1)
     kb_tsen(const BInst<T>* __restrict__ inst, const SensorArgs<T>* __restrict__ args, const BItem* __restrict__ items) {
     __shared__ __align__(16) Desc<T> sd;
-    pdl_enter();
-    const BItem it = items[blockIdx.y];
+    const BItem it = items[blockIdx.x];
     const BInst<T>* I = inst + it.inst;
     load_desc<T>(sd, I);
     const SensorArgs<T> a = args[it.inst];
     const TsLayout lay = I->lay_ts;
     const PairBufs<T> pb = I->pb;
-    tsen_body<T, SRC, 8>(sd, a, lay, pb, it.unit);
+    tsen_body<T, SRC>(sd, a, lay, pb, it.unit);
 }
 
 template <class T, int PHASE, int NTV>
@@ -104,16 +102,18 @@ template <class T>
 const void* kernel_of(int kind, int v) {
     const bool half = (v & 1) != 0;
     switch (kind) {
-        case BK_INV: return reinterpret_cast<const void*>(kb_tinv<T, 0>);
+        case BK_INV: case BK_INV_MS: case BK_MSUM: return reinterpret_cast<const void*>(kb_tinv<T, 0>);
         case BK_INV_UPD: return reinterpret_cast<const void*>(kb_tinv<T, 1>);
         case BK_SEN_PHI: return reinterpret_cast<const void*>(kb_tsen<T, SSRC_PHI>);
         case BK_SEN_SLOPES: return reinterpret_cast<const void*>(kb_tsen<T, SSRC_SLOPES>);
         case BK_SEN_RESID: return reinterpret_cast<const void*>(kb_tsen<T, SSRC_RESID>);
-        case BK_FWD_APPLY: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_APPLY>);
-        case BK_TC_APPLY: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_APPLY>);
+        case BK_FWD_UPD: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_UPDATE>);
+        case BK_TC_UPD: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_UPDATE>);
         case BK_FWD_COEF: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_COEF>);
         case BK_TC_COEF: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_COEF>);
         case BK_FWD_RINIT: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_RESID_INIT>);
+        case BK_FWD_AINIT: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_APPLY_INIT>);
+        case BK_TC_AINIT: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_APPLY_INIT>);
         case BK_TC_RINIT: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_RESID_INIT>);
         case BK_VEC_INIT:
             return half ? reinterpret_cast<const void*>(kb_vec<T, V_INIT, 2 * PBLK>)
@@ -121,9 +121,6 @@ const void* kernel_of(int kind, int v) {
         case BK_VEC_WARM:
             return half ? reinterpret_cast<const void*>(kb_vec<T, V_INIT_WARM, 2 * PBLK>)
                         : reinterpret_cast<const void*>(kb_vec<T, V_INIT_WARM, PBLK>);
-        case BK_VEC_UPDATE:
-            return half ? reinterpret_cast<const void*>(kb_vec<T, V_UPDATE, 2 * PBLK>)
-                        : reinterpret_cast<const void*>(kb_vec<T, V_UPDATE, PBLK>);
         case BK_FIT: return reinterpret_cast<const void*>(kb_fit<T>);
         default: return nullptr;
     }
@@ -173,33 +170,32 @@ cudaError_t batch_launch(const BLaunch& L, cudaStream_t st) {
     if (L.n_items <= 0) return cudaSuccess;
     const BInst<T>* I = static_cast<const BInst<T>*>(L.inst);
     const int n = L.n_items;
-    const dim3 cg(8, n), sn(tsnt<T>()), pg(n), nt(cblk<T>()), vt(L.vec_nt);
+    const dim3 sn(tsnt<T>()), pg(n), nt(cblk<T>()), vt(L.vec_nt);
     const bool v2 = L.vec_nt != PBLK;
     const ClArgs<T>* ca = static_cast<const ClArgs<T>*>(L.args);
     const SensorArgs<T>* sa = static_cast<const SensorArgs<T>*>(L.args);
     const VecArgs<T>* va = static_cast<const VecArgs<T>*>(L.args);
     const FitArgs<T>* fa = static_cast<const FitArgs<T>*>(L.args);
     switch (L.kind) {
-        case BK_INV: return launch_b(L.pdl, kb_tinv<T, 0>, pg, dim3(TINV_NT), L.smem, st, I, ca, L.items);
+        case BK_INV: case BK_INV_MS: case BK_MSUM: return launch_b(L.pdl, kb_tinv<T, 0>, pg, dim3(TINV_NT), L.smem, st, I, ca, L.items);
         case BK_INV_UPD: return launch_b(L.pdl, kb_tinv<T, 1>, pg, dim3(TINV_NT), L.smem, st, I, ca, L.items);
-        case BK_FWD_APPLY: return launch_b(L.pdl, kb_tfwd<T, LDST_APPLY>, pg, nt, L.smem, st, I, ca, L.items);
-        case BK_TC_APPLY: return launch_b(L.pdl, kb_tcoarse<T, LDST_APPLY>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_FWD_UPD: return launch_b(L.pdl, kb_tfwd<T, LDST_UPDATE>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_TC_UPD: return launch_b(L.pdl, kb_tcoarse<T, LDST_UPDATE>, pg, nt, L.smem, st, I, ca, L.items);
         case BK_FWD_COEF: return launch_b(L.pdl, kb_tfwd<T, LDST_COEF>, pg, nt, L.smem, st, I, ca, L.items);
         case BK_TC_COEF: return launch_b(L.pdl, kb_tcoarse<T, LDST_COEF>, pg, nt, L.smem, st, I, ca, L.items);
         case BK_FWD_RINIT: return launch_b(L.pdl, kb_tfwd<T, LDST_RESID_INIT>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_FWD_AINIT: return launch_b(L.pdl, kb_tfwd<T, LDST_APPLY_INIT>, pg, nt, L.smem, st, I, ca, L.items);
+        case BK_TC_AINIT: return launch_b(L.pdl, kb_tcoarse<T, LDST_APPLY_INIT>, pg, nt, L.smem, st, I, ca, L.items);
         case BK_TC_RINIT: return launch_b(L.pdl, kb_tcoarse<T, LDST_RESID_INIT>, pg, nt, L.smem, st, I, ca, L.items);
-        case BK_SEN_PHI: return launch_b(L.pdl, kb_tsen<T, SSRC_PHI>, cg, sn, L.smem, st, I, sa, L.items);
-        case BK_SEN_SLOPES: return launch_b(L.pdl, kb_tsen<T, SSRC_SLOPES>, cg, sn, L.smem, st, I, sa, L.items);
-        case BK_SEN_RESID: return launch_b(L.pdl, kb_tsen<T, SSRC_RESID>, cg, sn, L.smem, st, I, sa, L.items);
+        case BK_SEN_PHI: return launch_b(L.pdl, kb_tsen<T, SSRC_PHI>, pg, sn, L.smem, st, I, sa, L.items);
+        case BK_SEN_SLOPES: return launch_b(L.pdl, kb_tsen<T, SSRC_SLOPES>, pg, sn, L.smem, st, I, sa, L.items);
+        case BK_SEN_RESID: return launch_b(L.pdl, kb_tsen<T, SSRC_RESID>, pg, sn, L.smem, st, I, sa, L.items);
         case BK_VEC_INIT:
             return v2 ? launch_b(L.pdl, kb_vec<T, V_INIT, 2 * PBLK>, pg, vt, 0, st, I, va, L.items)
                       : launch_b(L.pdl, kb_vec<T, V_INIT, PBLK>, pg, vt, 0, st, I, va, L.items);
         case BK_VEC_WARM:
             return v2 ? launch_b(L.pdl, kb_vec<T, V_INIT_WARM, 2 * PBLK>, pg, vt, 0, st, I, va, L.items)
                       : launch_b(L.pdl, kb_vec<T, V_INIT_WARM, PBLK>, pg, vt, 0, st, I, va, L.items);
-        case BK_VEC_UPDATE:
-            return v2 ? launch_b(L.pdl, kb_vec<T, V_UPDATE, 2 * PBLK>, pg, vt, 0, st, I, va, L.items)
-                      : launch_b(L.pdl, kb_vec<T, V_UPDATE, PBLK>, pg, vt, 0, st, I, va, L.items);
         case BK_FIT: return launch_b(L.pdl, kb_fit<T>, pg, dim3(PBLK), L.smem, st, I, fa, L.items);
         default: return cudaErrorInvalidValue;
     }

@@ -43,31 +43,37 @@ struct FitArgs {
 // Step kinds of the frame (each names one kernel template instance).
 enum BKind {
     BK_INV = 0,        // phi = W^T c                       (ClArgs)
+    BK_INV_MS,         // phi = W^T c and the measured slopes' sums (ClArgs)
+    BK_MSUM,           // those sums alone                  (ClArgs)
     BK_INV_UPD,        // p = z + beta p, phi = W^T p       (ClArgs)
     BK_SEN_PHI,        // Gamma, C^-1, Gamma^T of P phi     (SensorArgs)
     BK_SEN_SLOPES,     // C^-1, Gamma^T of measured slopes  (SensorArgs)
-    BK_FWD_APPLY,      // q = W sum P^T u + alpha D p, p.q  (ClArgs)
+    BK_FWD_UPD,        // W sum P^T u and the CG update    (ClArgs)
     BK_FWD_COEF,       // b = W sum P^T u                   (ClArgs)
     BK_VEC_INIT,       // r0 = b - q, z, p, r.z             (VecArgs)
     BK_VEC_WARM,       // r0 = (b - b_prev) + r_prev        (VecArgs)
-    BK_VEC_UPDATE,     // CG update                         (VecArgs)
     BK_FIT,            // DM fit and gain                   (FitArgs)
     BK_SEN_RESID,      // C^-1, Gamma^T of s - Gamma P phi  (SensorArgs)
     BK_FWD_RINIT,      // r0 = W sum P^T u - alpha D c0, z0, p0, r.z (ClArgs)
-    BK_TC_APPLY,       // the coarse levels of the same       (ClArgs)
+    BK_TC_UPD,         // the coarse levels of the same     (ClArgs)
     BK_TC_COEF,
     BK_TC_RINIT,
+    BK_FWD_AINIT,      // r0 = b - M c0, z0, p0, r.z        (ClArgs)
+    BK_TC_AINIT,
     BK_COUNT
 };
 
 // Which work list a step kind runs over.
-enum BList { BL_LAYER = 0, BL_TILE, BL_BAND, BL_SENSOR, BL_VEC, BL_FIT, BL_COUNT };
+enum BList { BL_LAYER = 0, BL_LAYER_UPD, BL_TILE, BL_TILE_MS, BL_MSUM, BL_BAND, BL_SENSOR, BL_VEC, BL_FIT, BL_COUNT };
 
 inline int bkind_list(int kind) {
     switch (kind) {
         case BK_INV: case BK_INV_UPD: return BL_TILE;
-        case BK_FWD_APPLY: case BK_FWD_COEF: case BK_FWD_RINIT: return BL_BAND;
-        case BK_TC_APPLY: case BK_TC_COEF: case BK_TC_RINIT: return BL_LAYER;
+        case BK_INV_MS: return BL_TILE_MS;
+        case BK_MSUM: return BL_MSUM;
+        case BK_FWD_UPD: case BK_FWD_COEF: case BK_FWD_RINIT: case BK_FWD_AINIT: return BL_BAND;
+        case BK_TC_UPD: return BL_LAYER_UPD;
+        case BK_TC_COEF: case BK_TC_RINIT: case BK_TC_AINIT: return BL_LAYER;
         case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return BL_SENSOR;
         case BK_FIT: return BL_FIT;
         default: return BL_VEC;

@@ -42,6 +42,10 @@ __device__ __forceinline__ void cp_async_wait_group() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
+    const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem));
+}
 // 16-byte copy; both addresses 16-byte aligned.
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = static_cast<unsigned>(__cvta_generic_to_shared(smem));
@@ -431,6 +435,24 @@ struct ClArgs {
     // forward tile kernels: the finest level's LL blocks (layer offset / 4), the tiles' shares
     T* ll;
     double* tshare;
+    double* lsh;        // the layers' shares of the epilogue's inner product (TC_SH a layer)
+    // Inverse tile kernel: the tiles' shares of the sensors' sums go to fsh (functional f of
+    // tile u at f * n_tiles + u); with ms, the CTAs behind the tiles form each sensor's sums
+    // of the measured slopes ms into msum.
+    double* fsh;
+    const T* ms;
+    double* msum;
+    // The CG update fused into the forward kernels (LDST_UPDATE).  p.q is known before q:
+    // p.q = alpha p.D p + sum_g s.C^-1 s (s = Gamma P W^T p), so every CTA of the sensor kernel
+    // stores its share of both at pqs, and every forward CTA totals the n_pqs shares in the
+    // same order.  alphas[iter]: the step length, for the coarse kernel.
+    const double* pqs;
+    int n_pqs;
+    T* alphas;
+    T* vc;
+    T* phic;            // the layers of c, advanced beside it (null: not carried)
+    const T* phip;
+    const T* rin;       // r before the update (r after it goes to vr)
 };
 
 struct ClLayout {       // shared-memory offsets set by the host, in T units

@@ -122,22 +122,34 @@ struct alignas(16) Desc {   // 16-byte multiple: batched kernels copy it in 16-b
     const T* brow;
     // per band unit and sensor: {offset in PairBufs::Y, elements, offset in the stage, 0}
     const int* bsrc;
-    const int* tcl;         // layers of several bands (n_tcl)
+    const int* tcl;         // CTAs of the coarse kernel (n_tcl): layer | part << 8
     int tslot_ld, n_tcl;
     // sensor kernel, per sensor: place of node column b's (txi) and node row's (tyi: offset,
     // row pitch) layer column / row and the weight of the next one, [layer][tnp]; columns of
-    // P^T's column half, layer by layer from tsco: weights [tcols][tks], {first aperture
-    // column, count}; per layer {box columns, offset in PairBufs::Y}
+    // P^T's column half, layer by layer from tsco: first aperture column | count << 16; per
+    // layer {box columns, offset in PairBufs::Y, place of box column 0, 0}
     const int* txi;
     const int* tyi;
     const T* txf;
     const T* tyf;
-    const T* tcw;
     const int* tcin;
     const int* tsco;
     const int* tybox;
     const WfsInfo* gdev;    // G in device memory
-    int tnp, tcols, tks;
+    int tnp, tcols;
+    int su0[MAXG + 1];      // the sensor kernel's bands: sensor g has units su0[g] .. su0[g + 1]
+    // functionals of the layers that the weighting of sensor g's slopes needs, f0[g] ..
+    // f0[g + 1] (n_fun in all): sums of its modelled slopes (x, y; with spot elongation of gamma
+    // beta (beta . s) too) of a laser star, or over each block of a coarse sensor.  Tile u
+    // (n_tu in all) has {first, end} of functional f at foff[u * fpad + 2 f], then the place of
+    // its entries in fent, their count, the number of functionals of many entries and which
+    // these are; an entry is {node of the tile, weight}, after them a weight for each node of
+    // the tile per functional of many.  fpad, fcap: shared-memory space of a tile's offsets and entries
+    const int* foff;
+    const T* fent;
+    int n_tu, n_fun, fpad, fcap;
+    int n_writers;          // CTAs that store a share of the forward kernels' inner product
+    int f0[MAXG + 1];
     int tu0[MAXL + 1], bu0[MAXL + 1], tcnt[MAXL], broff[MAXL], bkt[MAXL];
     // footprint box of each (sensor, layer) pair: row0, rows, col0, cols (16-byte aligned
     // column superset); kept in the descriptor so that warps read it from the constant bank

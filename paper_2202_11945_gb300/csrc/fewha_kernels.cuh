@@ -476,7 +476,8 @@ enum { LSRC_PHI = 0, LSRC_NODES = 1, LSRC_DM = 2, LSRC_COEF = 3 };
 // step fused into its epilogue
 // LDST_RESID_INIT: the same vector step with the data term already the residual's (the
 // sensor kernel's SSRC_RESID): r0 = W y - alpha D c0, with no b
-enum { LDST_PHI = 0, LDST_COEF = 1, LDST_APPLY = 2, LDST_APPLY_INIT = 3, LDST_RESID_INIT = 4 };
+// LDST_UPDATE: the CG update c += a p, r -= a q, z = J^-1 r with r.z
+enum { LDST_PHI = 0, LDST_COEF = 1, LDST_APPLY = 2, LDST_APPLY_INIT = 3, LDST_RESID_INIT = 4, LDST_UPDATE = 5 };
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
     unsigned v;
@@ -619,6 +620,10 @@ struct SensorArgs {
     T* out;
     unsigned* status;   // bit 0: a non-finite input slope was seen
     const T* phi;       // layers (the sensor kernel's PHI and RESID forms)
+    const double* fsh;       // the tiles' shares of the sensors' sums, and the measured slopes' sums
+    const double* msum;
+    const T* p;         // with pqs: each CTA's share of s.C^-1 s + alpha p.D p goes to pqs
+    double* pqs;
 };
 
 template <class T, int SRC, bool WEIGHT, int DST>
@@ -866,6 +871,7 @@ struct VecArgs {
     // here from the forward kernel's pq_cnt shares (fixed order) and stored by CTA 0;
     // defer_rz, the r.z shares are stored and their total is left to the next inverse kernel
     int pq_cnt;
+    const double* pq_parts;
     int defer_rz;
     // V_UPDATE with phic: phi_c += alpha phi_p, the layers of c carried through the
     // iterations (phi_p = W^T p of the iteration's apply, piston left out like the data
@@ -900,7 +906,7 @@ __device__ __forceinline__ void vec_body(const int n, const VecArgs<T>& v, const
         // (warp 0, fixed order: the same value in every CTA)
         double pq = 0.0;
         if (v.pq_cnt > 0) {
-            pq = warp_total(v.pcg.pqpart + static_cast<long long>(iter) * PQ_SLOTS, v.pq_cnt,
+            pq = warp_total(v.pq_parts, v.pq_cnt,
                             static_cast<const DotAcc<T>*>(nullptr));
             if (threadIdx.x == 0 && cta == 0) v.pcg.pqtot[iter] = pq;
         }
@@ -1086,7 +1092,7 @@ __device__ __forceinline__ void aug_body(const int n, const VecArgs<T>& v, const
         // alpha; a deferred p.q total first (v.pq_cnt > 0: warp 1, fixed order)
         double pq = 0.0;
         if (v.pq_cnt > 0) {
-            pq = warp_total(v.pcg.pqpart + static_cast<long long>(v.iter) * PQ_SLOTS, v.pq_cnt,
+            pq = warp_total(v.pq_parts, v.pq_cnt,
                             static_cast<const DotAcc<T>*>(nullptr));
         }
         if (lane == 0) {

@@ -18,6 +18,8 @@ namespace fewha {
 
 constexpr int TINV_NT = 512;     // threads of the inverse tile kernel
 constexpr int TINV_SL = 4;       // coefficient slots per thread and round
+constexpr int TINV_FEW = 160;    // entries of a functional that 8 lanes take
+constexpr int TINV_DN = 16;      // functionals of more entries taken together
 
 // ---------------------------------------------------------------------------
 // Sums in a fixed order, in the arithmetic of DotAcc.
@@ -26,6 +28,14 @@ __device__ __forceinline__ double acc_merge(double a, double b) { return a + b; 
 __device__ __forceinline__ DFloat acc_merge(DFloat a, DFloat b) { return df_merge(a, b); }
 __device__ __forceinline__ double acc_warp(double a) { return warp_sum(a); }
 __device__ __forceinline__ DFloat acc_warp(DFloat a) { return warp_df_sum(a); }
+__device__ __forceinline__ double acc_shfl_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ DFloat acc_shfl_xor(DFloat a, int o) {
+    return DFloat{__shfl_xor_sync(0xffffffffu, a.s, o), __shfl_xor_sync(0xffffffffu, a.c, o)};
+}
+__device__ __forceinline__ double acc_from(double x) { return x; }
+__device__ __forceinline__ DFloat acc_from(float x) { return DFloat{x, 0.f}; }
+__device__ __forceinline__ double acc_neg(double a) { return -a; }
+__device__ __forceinline__ DFloat acc_neg(DFloat a) { return DFloat{-a.s, -a.c}; }
 template <class T> struct AccOf;
 template <> struct AccOf<float> {
     using type = DFloat;
@@ -42,15 +52,16 @@ static_assert(sizeof(DFloat) == sizeof(double), "a share is 8 bytes in both prec
 __device__ __forceinline__ double warp_value(double x) { return x; }
 __device__ __forceinline__ double warp_value(DFloat x) { return double(x.s) + double(x.c); }
 
-// Total of `cnt` shares by one warp (lane 0), L2 loads first.
-template <class T>
+// Total of `cnt` shares by one warp (lane 0): rounds of up to 32 U loads in flight, merged as
+// a tree.
+template <class T, int U = 4>
 __device__ __forceinline__ typename AccOf<T>::type shares_total(const double* p, int cnt) {
     using A = typename AccOf<T>::type;
     A s = AccOf<T>::zero();
-    for (int k0 = 0; k0 < cnt; k0 += 128) {
-        A v[4];
+    for (int k0 = 0; k0 < cnt; k0 += 32 * U) {
+        A v[U];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < U; ++k) {
             const int i = k0 + 32 * k + (threadIdx.x & 31);
             v[k] = AccOf<T>::zero();
             if (i < cnt) {
@@ -59,8 +70,11 @@ __device__ __forceinline__ typename AccOf<T>::type shares_total(const double* p,
             }
         }
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-            if (k0 + 32 * k < cnt) s = acc_merge(s, v[k]);
+        for (int w = 1; w < U; w *= 2)
+#pragma unroll
+            for (int k = 0; k + w < U; k += 2 * w)
+                if (k0 + 32 * (k + w) < cnt) v[k] = acc_merge(v[k], v[k + w]);
+        s = k0 ? acc_merge(s, v[0]) : v[0];
     }
     return acc_warp(s);
 }
@@ -83,6 +97,12 @@ __device__ __forceinline__ void cta_share(const DotAcc<T>& d, double* sh, const 
         }
     }
 }
+
+template <class T> struct Vec2;
+template <> struct Vec2<float> { using type = float2; };
+template <> struct Vec2<double> { using type = double2; };
+__device__ __forceinline__ void cp_async_pair(float2* smem, const float2* gmem) { cp_async8(smem, gmem); }
+__device__ __forceinline__ void cp_async_pair(double2* smem, const double2* gmem) { cp_async16(smem, gmem); }
 
 // Quotient of t < 2048 by n <= 64 through the host's reciprocal ceil(65536 / n).
 __device__ __forceinline__ int tdiv(int t, int magic) { return (t * magic) >> 16; }
@@ -111,6 +131,52 @@ __device__ __forceinline__ void acc_of(double x, DFloat& a) {
     a.c = static_cast<float>(x - static_cast<double>(a.s));
 }
 
+// Sums over one sensor's measured slopes, as its functionals sum the modelled ones: tip and
+// tilt of a laser star and, with spot elongation (Eq. 3), gamma beta (beta . s).  Compensated: the
+// residual's sums are the difference of these and the modelled ones.
+template <class T, int NT>
+__device__ __forceinline__ void measured_sums(const Desc<T>& d, const T* s, double* out, int g) {
+    using A = typename AccOf<T>::type;
+    __shared__ A ws[4][CWMAX + 2];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    const WfsInfo& W = d.G[g];
+    const int N = W.N, K = W.n_active, el = W.el;
+    DotAcc<T> sum[4];
+    pdl_wait();
+    pdl_trigger();
+    if (!W.lgs) return;
+    for (int k = t; k < N * N; k += NT) {
+        const int id = d.sidx[W.mask_off + k];
+        if (id >= 0) {
+            const T sx = s[W.soff + id], sy = s[W.soff + K + id];
+            sum[0].add(sx, T(1));
+            sum[1].add(sy, T(1));
+            if (el) {
+                T b1, b2, gam;
+                elong(W, k / N, k % N, b1, b2, gam);
+                const T bs = b1 * sx + b2 * sy;
+                sum[2].add(gam * b1, bs);
+                sum[3].add(gam * b2, bs);
+            }
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const A x = acc_warp(AccOf<T>::of(sum[e]));
+        if (lane == 0) ws[e][warp] = x;
+    }
+    __syncthreads();
+    if (warp < (el ? 4 : 2)) {
+        const A x = acc_warp(lane < NT / 32 ? ws[warp][lane] : AccOf<T>::zero());
+        if (lane == 0) *reinterpret_cast<A*>(out + d.f0[g] + warp) = x;
+    }
+}
+
+template <class T>
+__global__ void __launch_bounds__(TINV_NT) k_msum(__grid_constant__ const Desc<T> d, const T* s, double* out) {
+    measured_sums<T, TINV_NT>(d, s, out, blockIdx.x);
+}
+
 // ---------------------------------------------------------------------------
 // Inverse tile kernel: phi = W^T c on tile `unit` (d.tunit), optionally advancing the CG
 // direction first (Sec. 3.3): PUPD = 0, phi = W^T a.in.  PUPD = 1, p = z + beta p_old into
@@ -127,18 +193,38 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
     __shared__ TileLayer tl;
     __shared__ int ss[2][8];                              // window starts per dimension and level
     __shared__ T sbeta;
+    __shared__ typename AccOf<T>::type fden_w[TINV_DN][NT / 32];
     __shared__ T smu[AUG_MAX];
     using A = typename AccOf<T>::type;
     const int t = threadIdx.x;
+    if (unit >= d.n_tu) {
+        measured_sums<T, NT>(d, a.ms, a.msum, unit - d.n_tu);
+        return;
+    }
     int l = 0;
     while (unit >= d.tu0[l + 1]) ++l;
     const LayerInfo L = d.L[l];
     const int n = L.n;
+    // the tile's functionals (see Desc::fidx): offsets and, as far as they fit, the entries
+    int* foff = reinterpret_cast<int*>(sop + (d.tailop ? TAIL_N : 0));
+    using V2 = typename Vec2<T>::type;
+    V2* fent = reinterpret_cast<V2*>(foff + d.fpad);
+    const V2* gent = reinterpret_cast<const V2*>(d.fent);
+    if (a.fsh) {
+        for (int k = t; k < d.fpad; k += NT) cp_async(foff + k, d.foff + unit * d.fpad + k);
+    }
     if (t < static_cast<int>(sizeof(TileLayer) / sizeof(int)))
         reinterpret_cast<int*>(&tl)[t] = reinterpret_cast<const int*>(d.tl + l)[t];
-    T* sc = sop + (d.tailop ? TAIL_N : 0);                // the levels' quadrants
+    T* sc = reinterpret_cast<T*>(fent + d.fcap);          // the levels' quadrants
     if (d.tailop) stage16(sop, d.tailop, TAIL_N, t, NT);
     __syncthreads();
+    cp_async_wait();
+    __syncthreads();
+    if (a.fsh) {
+        const int f0 = foff[2 * d.n_fun];
+        const int cnt = min(foff[2 * d.n_fun + 1] + foff[2 * d.n_fun + 2] * ((tl.w[0] * tl.w[0]) >> 1), d.fcap);
+        for (int k = t; k < cnt; k += NT) cp_async_pair(fent + k, gent + f0 + k);
+    }
     if (t < 2) {
         const int side = tl.side, u = unit - d.tu0[l];
         int w0 = (t ? u & (side - 1) : u / side) << tl.lts;
@@ -302,6 +388,10 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
                 T* dst = a.out + L.off + (s0y + row) * n + x;
                 dst[0] = e;
                 dst[1] = o;
+                // the tile in shared memory too (this level's quadrants have been read)
+                T* keep = sc + row * w0 + 2 * bx;
+                keep[0] = e;
+                keep[1] = o;
             } else {
                 T* dst = sc + tl.base[j - 1] + row * tl.stride[j - 1];
                 const int rx = x - s0x;
@@ -310,6 +400,81 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
             }
         }
         if (j > 1) __syncthreads();
+    }
+    if (!a.fsh) return;
+    // ---- the tile's share of every functional: a warp each, fixed order
+    __syncthreads();
+    // (8 lanes each for the few boundary nodes of a sum; the dense ones of the elongation by
+    // the whole CTA)
+    const int f0 = foff[2 * d.n_fun], lg = t & 7;
+    for (int f = t >> 3; f < ((d.n_fun + NT / 8 - 1) & ~(NT / 8 - 1)); f += NT / 8) {
+        DotAcc<T> s;
+        const int k0 = f < d.n_fun ? foff[2 * f] : 0, k1 = f < d.n_fun ? foff[2 * f + 1] : 0;
+        for (int k = k0 + lg; k < k1; k += 32) {
+            V2 e[4];
+            T x = T(0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (k + 8 * q < k1) e[q] = k + 8 * q < d.fcap ? fent[k + 8 * q] : gent[f0 + k + 8 * q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (k + 8 * q < k1) x += e[q].y * sc[static_cast<int>(e[q].x)];
+            s.add(x, T(1));
+        }
+        A x = AccOf<T>::of(s);
+#pragma unroll
+        for (int o = 4; o; o >>= 1) x = acc_merge(x, acc_shfl_xor(x, o));
+        if (f < d.n_fun && lg == 0 && k1 >= k0) *reinterpret_cast<A*>(a.fsh + f * d.n_tu + unit) = x;
+    }
+    // those of many entries (elongation): a weight per node, two nodes a thread for TINV_DN of
+    // them at a time; their sums go through the warp together, halving the set at each step
+    const int nd = foff[2 * d.n_fun + 2], w0 = tl.w[0], np2 = (w0 * w0) >> 1, lane = t & 31;
+    const int* fden = foff + 2 * d.n_fun + 3;
+    for (int i0 = 0; i0 < nd; i0 += TINV_DN) {
+        T x[TINV_DN];
+        V2 v{T(0), T(0)};
+        if (t < np2) v = reinterpret_cast<const V2*>(sc)[t];
+#pragma unroll
+        for (int i = 0; i < TINV_DN; ++i) {
+            x[i] = T(0);
+            if (t < np2 && i0 + i < nd) {
+                const int k = foff[2 * d.n_fun + 1] + (i0 + i) * np2 + t;
+                const V2 e = k < d.fcap ? fent[k] : gent[f0 + k];
+                x[i] = e.x * v.x + e.y * v.y;
+            }
+        }
+        // after the step at width w a lane holds w of the sums, over 32 w / TINV_DN lanes; the
+        // first two, up to eight products, in T
+        A y[TINV_DN / 4];
+#pragma unroll
+        for (int w = TINV_DN / 2; w >= 1; w >>= 1) {
+            const int o = w * (32 / TINV_DN);
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int i = 0; i < w; ++i) {
+                if (w >= TINV_DN / 4) {
+                    const T send = up ? x[i] : x[i + w], mine = up ? x[i + w] : x[i];
+                    x[i] = mine + __shfl_xor_sync(0xffffffffu, send, o);
+                    if (w == TINV_DN / 4) y[i] = acc_from(x[i]);
+                } else {
+                    const A send = up ? y[i] : y[i + w], mine = up ? y[i + w] : y[i];
+                    y[i] = acc_merge(mine, acc_shfl_xor(send, o));
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 16 / TINV_DN; o; o >>= 1) y[0] = acc_merge(y[0], acc_shfl_xor(y[0], o));
+        if ((lane & (32 / TINV_DN - 1)) == 0) fden_w[lane / (32 / TINV_DN)][t >> 5] = y[0];
+        __syncthreads();
+        if (t < TINV_DN * (NT / 32)) {
+            // TINV_DN x NT / 32 partial sums: NT / 32 neighbouring lanes a sum
+            A z = (&fden_w[0][0])[t];
+#pragma unroll
+            for (int o = NT / 64; o; o >>= 1) z = acc_merge(z, acc_shfl_xor(z, o));
+            const int i = i0 + t / (NT / 32);
+            if (t % (NT / 32) == 0 && i < nd) *reinterpret_cast<A*>(a.fsh + fden[i] * d.n_tu + unit) = z;
+        }
+        if (i0 + TINV_DN < nd) __syncthreads();
     }
 }
 
@@ -431,28 +596,42 @@ template <> struct Quad<double> {
 // Operands of the epilogue at one coefficient.
 template <class T>
 struct EpiOp {
-    T p, b, j;
+    T p, b, j, r;
 };
 
 // The epilogue at one coefficient: v = (W y)(pos), dl its D.
 //   APPLY: q = v + alpha D p, written, p.q;  COEF: v written;
 //   RESID_INIT: r0 = v - alpha D c0 (v is the residual's data term), z = J^-1 r, p = z, r.z;
-//   APPLY_INIT: r0 = b - q, the same, and b_prev = b.
+//   APPLY_INIT: r0 = b - q, the same, and b_prev = b;
+//   UPDATE: r -= a q (q written to a.out too, if given), z = J^-1 r, r.z and, with upc,
+//   c += a p (step a).
 template <class T, int DST>
 __device__ __forceinline__ void epi_load(const ClArgs<T>& a, int pos, EpiOp<T>& o) {
     if (DST != LDST_COEF) o.p = a.pin[pos];
     if (DST == LDST_APPLY_INIT) o.b = a.vb[pos];
-    if (DST == LDST_APPLY_INIT || DST == LDST_RESID_INIT) o.j = a.vj[pos];
+    if (DST == LDST_APPLY_INIT || DST == LDST_RESID_INIT || DST == LDST_UPDATE) o.j = a.vj[pos];
+    if (DST == LDST_UPDATE) {
+        o.r = a.rin[pos];
+    }
 }
 template <class T, int DST>
 __device__ __forceinline__ void epi_apply(const ClArgs<T>& a, T alpha, T dl, int pos, T v, const EpiOp<T>& o,
-                                          DotAcc<T>& dot) {
+                                          DotAcc<T>& dot, T step = T(0), bool upc = false) {
     if (DST == LDST_COEF) {
         a.out[pos] = v;
     } else if (DST == LDST_APPLY) {
         const T q = v + alpha * dl * o.p;
         a.out[pos] = q;
         dot.add(o.p, q);
+    } else if (DST == LDST_UPDATE) {
+        const T q = v + alpha * dl * o.p;
+        if (a.out) a.out[pos] = q;
+        const T rr = o.r - step * q;
+        const T z = o.j * rr;
+        if (upc) a.vc[pos] = a.vc[pos] + step * o.p;
+        a.vr[pos] = rr;
+        a.vz[pos] = z;
+        dot.add(rr, z);
     } else {
         const T rr = DST == LDST_RESID_INIT ? v - alpha * dl * o.p : o.b - (v + alpha * dl * o.p);
         const T z = o.j * rr;
@@ -464,19 +643,21 @@ __device__ __forceinline__ void epi_apply(const ClArgs<T>& a, T alpha, T dl, int
     }
 }
 
-// Where a layer's share of the epilogue's inner product goes, and, unless it is left to the
-// next kernel, the total by the last of the instance's layers (fixed order).
+// Shares of the epilogue's inner product: TC_SH slots a layer (the bands' and the coarse
+// levels', then one per quadrant CTA of k_tcoarse), in the instance's slot row.  Unless the
+// total is left to the next kernel, the last of the `writers` CTAs forms it (fixed order).
+constexpr int TC_SH = 5;
 template <class T, int DST>
 __device__ __forceinline__ double* layer_slot(const ClArgs<T>& a, int l) {
-    return DST == LDST_APPLY ? a.pcg.pqpart + a.iter * PQ_SLOTS + l : a.rzp + l;
+    return a.lsh + l * TC_SH;
 }
 template <class T, int DST>
-__device__ __forceinline__ void layer_total(const ClArgs<T>& a, int n_layers) {
+__device__ __forceinline__ void layer_total(const ClArgs<T>& a, int n_layers, int writers) {
     if (DST == LDST_COEF || a.defer_total) return;
     __shared__ bool last;
     unsigned* count = a.pcg.count + (DST == LDST_APPLY ? 1 : 0);
-    if (last_arrival(count, static_cast<unsigned>(n_layers), &last) && threadIdx.x < 32) {
-        const typename AccOf<T>::type x = shares_total<T>(layer_slot<T, DST>(a, 0), n_layers);
+    if (last_arrival(count, static_cast<unsigned>(writers), &last) && threadIdx.x < 32) {
+        const typename AccOf<T>::type x = shares_total<T>(layer_slot<T, DST>(a, 0), n_layers * TC_SH);
         const double tot = warp_value(x);
         if (threadIdx.x == 0) {
             if (DST == LDST_APPLY)
@@ -566,6 +747,26 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
 #pragma unroll
         for (int e = 0; e < 3; ++e) epi_load<T, DST>(a, pos[e], op[e]);
     }
+    constexpr bool UPD = DST == LDST_UPDATE;
+    using A = typename AccOf<T>::type;
+    __shared__ A spq[2];
+    __shared__ T sstep;
+    // a layer of one band: its LL quadrant's operands, one per thread, and its layers of c
+    const bool one = bands == 1, cll = one && t < h * h;
+    const int pll = L.off + (t >> lh) * n + (t & (h - 1));
+    EpiOp<T> oll;
+    if (cll) epi_load<T, DST>(a, pll, oll);
+    constexpr int CPT = TF_ONE * TF_ONE / NT;             // the layers of c and of p, n <= TF_ONE
+    T cph[CPT], pph[CPT];
+    const bool carry = UPD && one && a.phic;
+#pragma unroll
+    for (int k = 0; k < CPT; ++k)
+        if (carry && t + k * NT < n * n) {
+            cph[k] = a.phic[L.off + t + k * NT];
+            pph[k] = a.phip[L.off + t + k * NT];
+        }
+    A rz = AccOf<T>::zero();
+    if (UPD && t == NT - 1) acc_of(a.pcg.rztot[a.iter], rz);
     cp_async_wait();
     __syncthreads();
     pdl_wait();
@@ -585,8 +786,24 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
             const int4 e = src[g];
             for (int k = t * V; k < e.y; k += NT * V) cp_async16(st + e.z + k, pb.Y + e.x + k);
         }
+        if (UPD && g0 == 0 && t >= NT - 64) {
+            // beside the copies, p.q from its shares: two warps, fixed order
+            const int w = (t - (NT - 64)) >> 5, half = (a.n_pqs + 1) >> 1;
+            const A x = shares_total<T>(a.pqs + w * half, w ? a.n_pqs - half : half);
+            if ((t & 31) == 0) spq[w] = x;
+        }
         cp_async_wait();
         __syncthreads();
+        if (UPD && g0 == 0 && t == NT - 1) {
+            // alpha = rz_k / (p . q)_k; zero if rz vanished (the iterate is final)
+            const A pq = acc_merge(spq[0], spq[1]);
+            const double pqv = warp_value(pq);
+            sstep = pqv > 0.0 && warp_value(rz) != 0.0 ? T(acc_ratio(rz, pq)) : T(0);
+            if (unit == 0) {
+                a.alphas[a.iter] = sstep;
+                a.pcg.pqtot[a.iter] = pqv;
+            }
+        }
 #pragma unroll
         for (int k = 0; k < TF_K; ++k) {
             const int task = t + k * NT;
@@ -626,6 +843,10 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
         }
     }
     __syncthreads();
+    const T step = UPD ? sstep : T(0);
+#pragma unroll
+    for (int k = 0; k < CPT; ++k)
+        if (carry && t + k * NT < n * n) a.phic[L.off + t + k * NT] = cph[k] + step * pph[k];
     // ---- the finest analysis level: rows, then columns ---------------------------------------
     DotAcc<T> dot;
     for (int b = t; b < nblk; b += NT) {                  // one block per thread, but for wide layers in double
@@ -660,7 +881,7 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
         else
             lbuf[rk * lsd + kx] = ll;
 #pragma unroll
-        for (int e = 0; e < 3; ++e) epi_apply<T, DST>(a, salpha, sD[1], pos[e], v[e], op[e], dot);
+        for (int e = 0; e < 3; ++e) epi_apply<T, DST>(a, salpha, sD[1], pos[e], v[e], op[e], dot, step, one);
     }
     if (bands == 1) {
         // ---- the other levels of a layer of one band ------------------------------------------
@@ -672,16 +893,14 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
         // by 1 / (alpha D_LL).
         if (a.zero_piston && L.full && t == 0) lbuf[0] = T(0);
         __syncthreads();
-        for (int k = t; k < h * h; k += NT) {
-            const int i = k >> lh, j = k & (h - 1), p = L.off + i * n + j;
-            EpiOp<T> o;
-            epi_load<T, DST>(a, p, o);
-            epi_apply<T, DST>(a, salpha, sD[level_of(i, j, L)], p, lbuf[i * lsd + j], o, dot);
+        if (cll) {
+            const int i = t >> lh, j = t & (h - 1);
+            epi_apply<T, DST>(a, salpha, sD[level_of(i, j, L)], pll, lbuf[i * lsd + j], oll, dot, step, true);
         }
     }
     if (DST != LDST_COEF) {
         cta_share<T>(dot, red, nullptr, bands > 1 ? a.tshare + unit : layer_slot<T, DST>(a, l));
-        if (bands == 1) layer_total<T, DST>(a, d.n_layers);
+        if (bands == 1) layer_total<T, DST>(a, d.n_layers, d.n_writers);
     }
 }
 
@@ -692,154 +911,231 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
     tfwd_body<T, DST>(d, a, lay, pb, blockIdx.x);
 }
 
-// The levels below the finest of layer l (of several bands) and their epilogue.  The LL
-// block (a.ll) comes from k_tfwd; the epilogue's operands are staged before the wait.
+// The levels below the finest of a layer of several bands and their epilogue, CTA `unit` of
+// d.tcl = {layer, part}: part 0, the leader, the level below the finest (its scaling half only)
+// and all coarser ones; parts 1 .. 4 the detail bands of the level below the finest, a
+// quadrant of 16 x 16 coefficients each; parts above, c += alpha p and the layers of c, a
+// chunk of TC_VEC each (they hide behind the leader).  The LL block (a.ll) comes from k_tfwd;
+// operands are read before the wait.
+//
+// Bound: the leader's chain of passes, latency of one CTA: 5.0 us of a MAORY iteration in
+// single precision.  The quadrants and the vector chunks on CTAs of their own keep it at that
+// with the updates of c, of its layers, of r and z inside, which were a kernel of 3 us before.
+constexpr int TC_VEC = 2048;
 struct TcLayout {
-    int lbuf, tmp, tail, st, total;  // T units after RED_DBL doubles; st: staged operands
+    int lbuf, tmp, tail, st, total;  // T units after the reduction scratch; st: staged operands
 };
 
 template <class T, int DST>
-__device__ __forceinline__ void tcoarse_body(const Desc<T>& d, const ClArgs<T>& a, const TcLayout& lay, const int l) {
-    constexpr int NT = cblk<T>(), V = vec16<T>();
-    constexpr bool QP = DST != LDST_COEF, QB = DST == LDST_APPLY_INIT;
-    constexpr bool QJ = DST == LDST_APPLY_INIT || DST == LDST_RESID_INIT;
+__device__ __forceinline__ void tcoarse_body(const Desc<T>& d, const ClArgs<T>& a, const TcLayout& lay, const int unit) {
+    constexpr int NT = cblk<T>();
+    constexpr bool QP = DST != LDST_COEF, UPD = DST == LDST_UPDATE;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* red = reinterpret_cast<double*>(smem_raw);
     T* sm = reinterpret_cast<T*>(red + CWMAX);
     const int t = threadIdx.x;
+    const int code = d.tcl[unit], l = code & 255, part = code >> 8;
     const LayerInfo L = d.L[l];
-    const int n = L.n, h = n >> 1, lh = L.log2n - 1, lsd = h + 1;
-    T* lbuf = sm + lay.lbuf;
-    T* sp = sm + lay.st;
-    T* sb = sp + (MAXN / 2) * (MAXN / 2);
-    T* sj = sb + (QB ? (MAXN / 2) * (MAXN / 2) : 0);
+    const int n = L.n, h = n >> 1, lh = L.log2n - 1, hh = h >> 1, lhh = lh - 1;
     __shared__ T sD[MAXLEV + 1];
-    __shared__ T salpha;
-    __shared__ double tiles;             // the bands' share of the inner product
+    __shared__ T salpha, sstep;
+    __shared__ double bands;             // the bands' share of the inner product
+    if (part > TC_SH - 1) {
+        // ---- c += alpha p, phi_c += alpha phi_p --------------------------------------------
+        pdl_wait();
+        pdl_trigger();
+        if (!UPD) return;
+        const T step = a.alphas[a.iter];
+        const int k0 = (part - TC_SH) * TC_VEC, k1 = min(k0 + TC_VEC, n * n);
+        for (int k = k0 + t; k < k1; k += NT) {
+            a.vc[L.off + k] += step * a.pin[L.off + k];
+            if (a.phic) a.phic[L.off + k] += step * a.phip[L.off + k];
+        }
+        return;
+    }
     if (t <= MAXLEV) sD[t] = d.Dlev[l][t];
     if (t == 0) salpha = d.alpha;
+    const T* src = a.ll + (L.off >> 2);
+    DotAcc<T> dot;
+    if (part > 0) {
+        // ---- detail bands of the level below the finest: 16 x 16 coefficients each ------------
+        constexpr int R = 36, RS = 37;   // region of the LL block, its row stride
+        T* buf = sm + lay.lbuf;
+        const bool has = L.levels >= 2;
+        const int ky0 = hh > 16 ? ((part - 1) >> 1) * 16 : 0, kx0 = hh > 16 ? ((part - 1) & 1) * 16 : 0;
+        const int ck = ky0 + ((t >> 4) & 15), cl = kx0 + (t & 15);
+        const int pos[3] = {L.off + ck * n + hh + cl, L.off + (hh + ck) * n + cl, L.off + (hh + ck) * n + hh + cl};
+        EpiOp<T> op[3];
+        if (t < 256 && has) {
+#pragma unroll
+            for (int e = 0; e < 3; ++e) epi_load<T, DST>(a, pos[e], op[e]);
+        }
+        __syncthreads();
+        pdl_wait();
+        pdl_trigger();
+        if (!has) return;
+        if (UPD && t == 0) sstep = a.alphas[a.iter];
+        for (int k = t; k < R * R; k += NT) {
+            const int i = k / R, j = k - i * R;
+            buf[i * RS + j] = src[((2 * ky0 + i) & (h - 1)) * h + ((2 * kx0 + j) & (h - 1))];
+        }
+        __syncthreads();
+        if (t < 256) {
+            const int ky = 2 * (t >> 4), kx = 2 * (t & 15);
+            T v[3] = {T(0), T(0), T(0)};
+#pragma unroll
+            for (int r = 0; r < 6; ++r) {
+                const T* x = buf + (ky + r) * RS + kx;
+                T av = T(0), dv = T(0);
+#pragma unroll
+                for (int q = 0; q < 6; ++q) {
+                    av += tap_h<T>(q) * x[q];
+                    dv += tap_g<T>(q) * x[q];
+                }
+                v[0] += tap_h<T>(r) * dv;
+                v[1] += tap_g<T>(r) * av;
+                v[2] += tap_g<T>(r) * dv;
+            }
+#pragma unroll
+            for (int e = 0; e < 3; ++e) epi_apply<T, DST>(a, salpha, sD[2], pos[e], v[e], op[e], dot, sstep);
+        }
+        if (QP) {
+            cta_share<T>(dot, red, nullptr, layer_slot<T, DST>(a, l) + part);
+            layer_total<T, DST>(a, d.n_layers, d.n_writers);
+        }
+        return;
+    }
+    // ---- the leader: LL of the level below the finest, the coarser levels -----------------------
+    T* lbuf = sm + lay.lbuf;
+    T* tmp = sm + lay.tmp;
+    const bool two = L.levels >= 2;      // else the LL block is the layer's LL band
+    const int m = two ? hh : h, lm = two ? lhh : lh, ld = m + 1, hs = h + 1;
     const bool tail_on = lay.tail > 0 && (d.bkt[l] >> 4);
     const int unit0 = d.bu0[l], units = d.bu0[l + 1] - d.bu0[l];
     if (tail_on) stage16(sm + lay.tail, d.tailop, TAIL_N, t, NT);
-    if (QP) {
-        // a caller's vector (the apply's input) may start off a 16-byte boundary
-        const bool wide = ((reinterpret_cast<size_t>(a.pin) | reinterpret_cast<size_t>(QB ? a.vb : a.pin)) & 15) == 0;
-        const int lc = wide ? lh - (V == 4 ? 2 : 1) : lh;    // log2 of the copies per row
-        for (int k = t; k < (h << lc); k += NT) {
-            const int i = k >> lc, c = (k & ((1 << lc) - 1)) * (wide ? V : 1), pos = L.off + i * n + c;
-            if (wide) {
-                cp_async16(sp + i * h + c, a.pin + pos);
-                if (QB) cp_async16(sb + i * h + c, a.vb + pos);
-                if (QJ) cp_async16(sj + i * h + c, a.vj + pos);
-            } else {
-                cp_async(sp + i * h + c, a.pin + pos);
-                if (QB) cp_async(sb + i * h + c, a.vb + pos);
-                if (QJ) cp_async(sj + i * h + c, a.vj + pos);
-            }
-        }
+    // operands of the epilogue at this thread's coefficients (two a thread at h = 64)
+    constexpr int TK = 4;
+    EpiOp<T> op[TK];
+#pragma unroll
+    for (int k = 0; k < TK; ++k) {
+        const int b = t + k * NT;
+        if (b < m << lm) epi_load<T, DST>(a, L.off + (b >> lm) * n + (b & (m - 1)), op[k]);
     }
+    __syncthreads();
     pdl_wait();
     pdl_trigger();
-    const T* src = a.ll + (L.off >> 2);
-    for (int k = t * V; k < h * h; k += NT * V) {
-        const Quad<T> v = *reinterpret_cast<const Quad<T>*>(src + k);
-        T* dst = lbuf + (k >> lh) * lsd + (k & (h - 1));
-#pragma unroll
-        for (int e = 0; e < V; ++e) dst[e] = reinterpret_cast<const T*>(&v)[e];
-    }
+    if (UPD && t == 0) sstep = a.alphas[a.iter];
     if (QP && t >= NT - 32) {
         const typename AccOf<T>::type x = shares_total<T>(a.tshare + unit0, units);
-        if (t == NT - 32) *reinterpret_cast<typename AccOf<T>::type*>(&tiles) = x;
+        if (t == NT - 32) *reinterpret_cast<typename AccOf<T>::type*>(&bands) = x;
     }
-    cp_async_wait();
-    __syncthreads();
-    if (L.levels >= 2) analyse<T>(lbuf, sm + lay.tmp, tail_on ? sm + lay.tail : nullptr, n, 1, L.levels, lsd);
+    if (two) {
+        // the scaling half of the level below the finest, rows then columns
+        T* raw = tmp;                                     // h x h, row stride h + 1
+        T* mid = sm + lay.st;                             // h x hh, row stride hh + 1
+        for (int k = t; k < h << lh; k += NT) raw[(k >> lh) * hs + (k & (h - 1))] = src[k];
+        cp_async_wait();
+        __syncthreads();
+        for (int b = t; b < h << lhh; b += NT) {
+            const int row = b >> lhh, k = b & (hh - 1);
+            const T* x = raw + row * hs;
+            T av = T(0);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) av += tap_h<T>(q) * x[(2 * k + q) & (h - 1)];
+            mid[row * ld + k] = av;
+        }
+        __syncthreads();
+        for (int b = t; b < hh << lhh; b += NT) {
+            const int k = b >> lhh, c = b & (hh - 1);
+            T av = T(0);
+#pragma unroll
+            for (int q = 0; q < 6; ++q) av += tap_h<T>(q) * mid[((2 * k + q) & (h - 1)) * ld + c];
+            lbuf[k * ld + c] = av;
+        }
+        __syncthreads();
+        if (L.levels >= 3) analyse<T>(lbuf, tmp, tail_on ? sm + lay.tail : nullptr, n, 2, L.levels, ld);
+    } else {
+        cp_async_wait();
+        for (int k = t; k < h << lh; k += NT) lbuf[(k >> lh) * ld + (k & (h - 1))] = src[k];
+        __syncthreads();
+    }
     if (a.zero_piston && L.full && t == 0) lbuf[0] = T(0);   // no piston in the data term (see tfwd_body)
     __syncthreads();
-    DotAcc<T> dot;
-    for (int k = t; k < h * h; k += NT) {
-        const int i = k >> lh, j = k & (h - 1);
+#pragma unroll
+    for (int k = 0; k < TK; ++k) {
+        const int b = t + k * NT, i = b >> lm, j = b & (m - 1);
+        if (b < m << lm)
+            epi_apply<T, DST>(a, salpha, sD[level_of(i, j, L)], L.off + i * n + j, lbuf[i * ld + j], op[k], dot,
+                              UPD ? sstep : T(0));
+    }
+    for (int b = t + TK * NT; b < m << lm; b += NT) {        // an LL band that is not transformed further
+        const int i = b >> lm, j = b & (m - 1), p = L.off + i * n + j;
         EpiOp<T> o;
-        if (QP) o.p = sp[k];
-        if (QB) o.b = sb[k];
-        if (QJ) o.j = sj[k];
-        epi_apply<T, DST>(a, salpha, sD[level_of(i, j, L)], L.off + i * n + j, lbuf[i * lsd + j], o, dot);
+        epi_load<T, DST>(a, p, o);
+        epi_apply<T, DST>(a, salpha, sD[level_of(i, j, L)], p, lbuf[i * ld + j], o, dot, UPD ? sstep : T(0));
     }
     if (QP) {
-        cta_share<T>(dot, red, &tiles, layer_slot<T, DST>(a, l));
-        layer_total<T, DST>(a, d.n_layers);
+        cta_share<T>(dot, red, &bands, layer_slot<T, DST>(a, l));
+        layer_total<T, DST>(a, d.n_layers, d.n_writers);
     }
 }
 
 template <class T, int DST>
 __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
     k_tcoarse(__grid_constant__ const Desc<T> d, __grid_constant__ const ClArgs<T> a, __grid_constant__ const TcLayout lay) {
-    tcoarse_body<T, DST>(d, a, lay, d.tcl[blockIdx.x]);
+    tcoarse_body<T, DST>(d, a, lay, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
-// Sensor kernel (cluster of SCL CTAs per sensor, a band of subaperture rows per CTA): P_g
-// (Sec. 2), Gamma_g, C_hat_g^-1 (Eq. 2, Sec. 3.2), Gamma_g^T and the column half of P_g^T.
-// SRC_PHI: slopes of the projected layers (the M-apply); SRC_RESID: measured minus modelled
-// slopes (the initial residual); SRC_SLOPES: measured slopes (the right-hand side).  The
-// layers are read by direct bilinear gathers; the result goes out per layer as the aperture
-// rows' values on the layer's columns (pb.Y, slot g * n_layers + l, rows of box[3]
-// columns), whose row half the band kernel applies.
+// Sensor kernel, a CTA per band of TS_ROWS subaperture rows of a sensor: P_g (Sec. 2),
+// Gamma_g, C_hat_g^-1 (Eq. 2, Sec. 3.2), Gamma_g^T and the column half of P_g^T.  SRC_PHI:
+// slopes of the projected layers (the M-apply); SRC_RESID: measured minus modelled slopes
+// (the initial residual); SRC_SLOPES: measured slopes (the right-hand side).  The layers are
+// read by direct bilinear gathers; the result goes out per layer as the aperture rows'
+// values on the layer's columns (pb.Y, slot g * n_layers + l, rows of box[3] columns), whose
+// row half the band kernel applies.
 //
-// Every CTA also forms the slopes of the row below its band, so that nothing but the
-// tip/tilt and coarse-block sums crosses the cluster: one barrier.  The sums are formed per
-// subaperture row and then over the rows, in an order that does not depend on SCL.
-//
-// Bound: latency (tables, one gather, one cluster barrier).  With the slopes of the row below
-// formed here too, two cluster barriers and a distributed-shared-memory read are gone; with
-// the projection and the column half of its adjoint in this kernel, so are the two kernels of
-// (sensor, layer) pairs.  Clusters of 16 CTAs halve the bands where the device holds all of
-// an instance's clusters at once (14 of them: the MAORY frame 156 us, with clusters of 8
-// 173); a batch fills the device with clusters of 8 (391 us a batch of 16 instances, with
-// clusters of 16 535).  Staging the layers' rows in shared memory first took 3 to 5 us more
-// than gathering from L2.  From the cluster kernels: frame of the 8 m system 91.3 -> 65.8 us,
-// paper's geometry 111 -> 77.7, MAORY 173.5 -> 156.4, in double 817 -> 664, closed loop
-// 200 -> 163, a batch of 16 uneven instances 566 -> 391.
+// No CTA waits for another.  What the weighting of one subaperture needs of all the others
+// (the tip/tilt means of a laser star, the block sums of a coarse sensor, the elongation's
+// sums) are linear functionals of the layers, whose shares the inverse kernel's tiles have
+// formed; the slopes of the row below the band are formed here once more.
 // ---------------------------------------------------------------------------
+constexpr int TS_ROWS = 4;       // 6 node rows of 81 nodes are one pass of 512 threads
 constexpr int TS_LG = 5;         // layers with their loads in flight together
-constexpr int TS_NV = 2 * FEWHA_MAX_COARSE;      // sums per subaperture row, at most
+constexpr int TS_FUN = 2 * MAXCOARSE;            // functionals of a sensor, at most
 
-// Threads: in single precision 7 node rows of 81 nodes in one pass.
+// 512 threads of at most 64 registers fit beside the CTAs of the kernels before and after
+// (each scheduler's registers hold four warps of each), so the prologue is hidden.
 template <class T>
 __host__ __device__ constexpr int tsnt() {
-    return sizeof(T) == 4 ? 576 : 288;
+    return sizeof(T) == 4 ? 512 : 256;
 }
-struct TsLayout {       // shared-memory offsets in T units, for clusters of 16 and 8
-    int V, SX, SY, msk, xi, xf, yi, yf, cw, ci, total;
+struct TsLayout {       // shared-memory offsets in T units
+    int V, SX, SY, msk, xi, xf, yi, yf, ci, dot, total;
 };
 
-template <class T, int SRC, int SCL>
+template <class T, int SRC>
 __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>& a, const TsLayout& lay,
-                                          const PairBufs<T>& pb, const int g) {
-    constexpr int NT = tsnt<T>();
+                                          const PairBufs<T>& pb, const int unit) {
+    constexpr int NT = tsnt<T>(), SR = TS_ROWS;
     constexpr bool FROM_PHI = SRC == SSRC_PHI || SRC == SSRC_RESID;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw);
-    cg::cluster_group cluster = cg::this_cluster();
-    const int r = static_cast<int>(cluster.block_rank());
     const int t = threadIdx.x, warp = t >> 5, lane = t & 31, nwarp = NT >> 5;
-    // peers' shared memory is written before the first full cluster barrier (the pushes
-    // below): arrive now, wait before the first push, so that every CTA has started
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
     // the sensor's constants in shared memory: the kernel-parameter bank is cold, and its
     // first reads would stand behind the dependency wait (a copy in device memory is read:
     // indexed reads of the parameters are slow)
     __shared__ WfsInfo sW;
     __shared__ int sco[MAXL + 1];                        // first column of each layer
-    __shared__ int2 ybox[MAXL];                          // each layer: box columns, offset in Y
-    __shared__ T rsum[MAXNF][TS_NV];                     // every subaperture row's sums (pushed)
-    __shared__ T tot[4];
-    __shared__ T cw[2 * MAXCOARSE];                      // weighted coarse slopes / nb
-    const int nl = d.n_layers, ks = d.tks;
-    const int N = d.G[g].N, NP = N + 1, NPs = d.tnp;
-    const int sr = (N + SCL - 1) / SCL;
-    const int s0 = min(r * sr, N), s1 = min((r + 1) * sr, N), rows = s1 - s0;
-    const int h0 = s0 > 0 && rows > 0 ? 1 : 0;           // the row below the band, if any
+    __shared__ int4 ybox[MAXL];                          // each layer: box columns, offset in Y, place of box column 0
+    __shared__ T tot[TS_FUN];                            // the sensor's functionals
+    __shared__ T cw[TS_FUN];                             // weighted coarse slopes / nb
+    int g = 0;
+    while (unit >= d.su0[g + 1]) ++g;
+    const int nl = d.n_layers, NPs = d.tnp, n_tu = d.n_tu;
+    const int N = d.G[g].N, NP = N + 1, f0 = d.f0[g], nf = d.f0[g + 1] - f0;
+    const int s0 = (unit - d.su0[g]) * SR, s1 = min(s0 + SR, N), rows = s1 - s0;
+    const int h0 = s0 > 0 ? 1 : 0;                       // the row below the band, if any
     const int q0 = s0 - h0, nrow = rows + h0;            // slope rows [q0, s1), node rows [q0, s1]
     T* Vb = sm + lay.V;         // (nrow + 1) x NP: node values, later the adjoint's
     T* SX = sm + lay.SX;        // nrow x N
@@ -849,45 +1145,56 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
     T* xf = sm + lay.xf;
     int2* yi = reinterpret_cast<int2*>(sm + lay.yi);     // [layer][node row]: offset of its layer row, row pitch
     T* yf = sm + lay.yf;
-    T* cwt = sm + lay.cw;                                // column weights of P^T: [column][ks]
-    int2* cin = reinterpret_cast<int2*>(sm + lay.ci);    // first aperture column, count
-    // ---- set-up tables, copied before the dependency wait; those of the column half of P^T
-    // in a group of their own, waited for where they are used ------------------------------
+    int* cin = reinterpret_cast<int*>(sm + lay.ci);      // per layer column: first aperture column | count << 16
+    using A = typename AccOf<T>::type;
+    A* dots = reinterpret_cast<A*>(sm + lay.dot);        // the threads' shares of p.q
+    // ---- set-up tables, copied before the dependency wait ---------------------------------
     for (int k = t; k < static_cast<int>(sizeof(WfsInfo) / sizeof(int)); k += NT)
         reinterpret_cast<int*>(&sW)[k] = reinterpret_cast<const int*>(d.gdev + g)[k];
     {
         const int* src = d.sidx + d.G[g].mask_off + q0 * N;
         for (int k = t; k < nrow * N; k += NT) cp_async(msk + k, src + k);
     }
+    const int nx = nl * NPs;
+    stage16(xi, d.txi + g * nx, nx, t, NT);
+    stage16(xf, d.txf + g * nx, nx, t, NT);
     if (FROM_PHI) {
-        const int nx = nl * NPs;
-        stage16(xi, d.txi + g * nx, nx, t, NT);
-        stage16(xf, d.txf + g * nx, nx, t, NT);
-        for (int k = t; k < nl * 16; k += NT) {
-            const int l = k >> 4;
-            for (int i = k & 15; i <= nrow; i += 16) {
-                yi[l * (sr + 2) + i] = reinterpret_cast<const int2*>(d.tyi)[g * nx + l * NPs + q0 + i];
-                yf[l * (sr + 2) + i] = d.tyf[g * nx + l * NPs + q0 + i];
+        for (int k = t; k < nl * 8; k += NT) {
+            const int l = k >> 3, i = k & 7;
+            if (i <= nrow) {
+                yi[l * (SR + 2) + i] = reinterpret_cast<const int2*>(d.tyi)[g * nx + l * NPs + q0 + i];
+                yf[l * (SR + 2) + i] = d.tyf[g * nx + l * NPs + q0 + i];
             }
         }
     }
     if (t < 32) {
         for (int k = t; k <= nl; k += 32) sco[k] = d.tsco[g * (MAXL + 1) + k];
-        for (int k = t; k < nl; k += 32) ybox[k] = reinterpret_cast<const int2*>(d.tybox)[g * MAXL + k];
+        for (int k = t; k < nl; k += 32) ybox[k] = reinterpret_cast<const int4*>(d.tybox)[g * MAXL + k];
     }
-    cp_async_commit();
-    stage16(cwt, d.tcw + static_cast<size_t>(g) * d.tcols * ks, d.tcols * ks, t, NT);
-    stage16(reinterpret_cast<int*>(cin), d.tcin + g * d.tcols * 2, 2 * d.tcols, t, NT);
-    cp_async_commit();
-    cp_async_wait_group<1>();
+    stage16(cin, d.tcin + g * d.tcols, d.tcols, t, NT);
+    cp_async_wait();
     __syncthreads();
     const WfsInfo& W = sW;
     const T inv = T(W.sig2inv);
     const T nbinv = T(1) / T(W.nb);
+    const int nu = d.su0[d.n_wfs], np = (d.n_c + nu - 1) / nu;           // this CTA's part of p.D p
+    const T alpha = d.alpha;
     pdl_wait();
     pdl_trigger();
     bool bad = false;                          // a non-finite measured slope (SLOPES, RESID)
-    if (FROM_PHI && rows > 0) {
+    DotAcc<T> dot;
+    // ---- the sensor's functionals: the tiles' shares, a warp each, in flight beside the gather
+    for (int f = warp; f < nf; f += nwarp) {
+        A x = AccOf<T>::zero();
+        if (FROM_PHI) x = shares_total<T, 6>(a.fsh + (f0 + f) * n_tu, n_tu);
+        if (lane == 0) {
+            // the residual of a laser star: measured minus modelled
+            if (SRC != SSRC_PHI && W.lgs)
+                x = acc_merge(*reinterpret_cast<const A*>(a.msum + f0 + f), acc_neg(x));
+            tot[f] = T(warp_value(x));
+        }
+    }
+    if (FROM_PHI) {
         // ---- V = P_g phi on node rows [q0, s1]: a thread per node, the layers in order ----
         for (int k = t; k < (nrow + 1) * NP; k += NT) {
             const int ia = k / NP, b = k - ia * NP;
@@ -897,7 +1204,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
 #pragma unroll
                 for (int e = 0; e < TS_LG; ++e)
                     if (l0 + e < nl) {
-                        const int2 y = yi[(l0 + e) * (sr + 2) + ia];
+                        const int2 y = yi[(l0 + e) * (SR + 2) + ia];
                         const T* p = a.phi + xi[(l0 + e) * NPs + b] + y.x;
                         q[e][0] = p[0];
                         q[e][1] = p[1];
@@ -907,26 +1214,67 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
 #pragma unroll
                 for (int e = 0; e < TS_LG; ++e)
                     if (l0 + e < nl) {
-                        const T fx = xf[(l0 + e) * NPs + b], fy = yf[(l0 + e) * (sr + 2) + ia];
+                        const T fx = xf[(l0 + e) * NPs + b], fy = yf[(l0 + e) * (SR + 2) + ia];
                         const T h0 = (T(1) - fx) * q[e][0] + fx * q[e][1], h1 = (T(1) - fx) * q[e][2] + fx * q[e][3];
                         v += (T(1) - fy) * h0 + fy * h1;
                     }
             }
             Vb[k] = v;
         }
+    }
+    if (SRC == SSRC_PHI && a.pqs) {
+        // this CTA's part of alpha p.D p
+        for (int k = t; k < np; k += NT) {
+            const int i = unit * np + k;
+            if (i < d.n_c) {
+                const T p = a.p[i];
+                dot.add(alpha * d.D[i] * p, p);
+            }
+        }
+    }
+    __syncthreads();
+    const bool coarse = FROM_PHI && W.nb > 1;
+    if (coarse) {
+        // coarse slope = block sum / nb; Gamma_coarse^T spreads sigma^-2 slope / nb.  The
+        // residual form subtracts it from the block's measured slope.
+        const int ns = W.n_sub;
+        if (t < 2 * ns * ns) {
+            T x = tot[t] * nbinv;
+            if (SRC == SSRC_RESID) {
+                const int K = d.cidx[W.cmask_off + (t >> 1)];
+                T m = T(0);
+                if (K >= 0) {
+                    m = a.in[W.soff + (t & 1) * W.n_active + K];
+                    bad |= !isfinite(m);
+                }
+                x = m - x;
+            } else if (unit == d.su0[g] && a.pqs) {
+                dot.add(x, inv * x);                         // s . sigma^-2 s, once a sensor
+            }
+            cw[t] = x * inv * nbinv;
+        }
         __syncthreads();
     }
-    // ---- the slopes of rows [q0, s1) and each band row's sums: a warp per row ---------------
-    const bool need_tt = W.lgs;
-    const bool need_coarse = FROM_PHI && W.nb > 1;
-    asm volatile("barrier.cluster.wait.aligned;\n" ::: "memory");
-    for (int ii = warp; ii < nrow; ii += nwarp) {
-        T sum[4] = {T(0), T(0), T(0), T(0)};
-        for (int j = lane; j < N; j += 32) {
-            const int k = ii * N + j;
-            T sx = T(0), sy = T(0);
-            const int id = msk[k];
-            if (id >= 0) {
+    // ---- the weighted slopes of rows [q0, s1) ------------------------------------------------
+    T mx = T(0), my = T(0), g1 = T(0), g2 = T(0);
+    if (W.lgs) {
+        mx = tot[0] / T(W.n_active);
+        my = tot[1] / T(W.n_active);
+        if (W.el) {
+            g1 = (tot[2] - (el_K(W, 0, T()) * mx + el_K(W, 1, T()) * my)) / T(W.n_active);
+            g2 = (tot[3] - (el_K(W, 1, T()) * mx + el_K(W, 2, T()) * my)) / T(W.n_active);
+        }
+    }
+    for (int k = t; k < nrow * N; k += NT) {
+        const int ii = k / N, j = k - ii * N, id = msk[k];
+        T wx = T(0), wy = T(0);
+        if (id >= 0) {
+            if (coarse) {
+                const int blk = ((q0 + ii) / W.nb) * W.n_sub + j / W.nb;
+                wx = cw[2 * blk];
+                wy = cw[2 * blk + 1];
+            } else {
+                T sx = T(0), sy = T(0);
                 if (FROM_PHI) {
                     // Gamma_g on the modelled nodes
                     const T v00 = Vb[ii * NP + j], v01 = Vb[ii * NP + j + 1];
@@ -934,216 +1282,119 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
                     sx = T(0.5) * ((v01 - v00) + (v11 - v10));
                     sy = T(0.5) * ((v10 - v00) + (v11 - v01));
                 }
-                if ((SRC == SSRC_RESID && W.nb == 1) || SRC == SSRC_SLOPES) {
-                    // measured slopes; the residual of an ordinary sensor is measured minus
-                    // modelled (a coarse sensor's measurement enters after its block sums)
-                    const T mx = a.in[W.soff + id], my = a.in[W.soff + W.n_active + id];
-                    bad |= !(isfinite(mx) && isfinite(my));
-                    sx = SRC == SSRC_RESID ? mx - sx : mx;
-                    sy = SRC == SSRC_RESID ? my - sy : my;
-                    if (SRC == SSRC_SLOPES && W.nb > 1) {    // (1/nb) sigma^-2 s_K on each active fine one
-                        sx *= nbinv * inv;
-                        sy *= nbinv * inv;
-                    }
+                if (SRC != SSRC_PHI) {
+                    const T ax = a.in[W.soff + id], ay = a.in[W.soff + W.n_active + id];
+                    bad |= !(isfinite(ax) && isfinite(ay));
+                    sx = ax - sx;
+                    sy = ay - sy;
                 }
-                if (W.nb == 1 && !W.lgs) {                   // NGS: C^-1 = sigma^-2 I
-                    sx *= inv;
-                    sy *= inv;
-                }
-                if (need_tt) {
-                    sum[0] += sx;
-                    sum[1] += sy;
+                if (W.lgs) {
+                    // C_hat^-1 = (I - T) C^-1 (I - T): sigma^-2 (s - m) or, elongated,
+                    // sigma^-2 (u - gamma beta (beta . u) + g), u = s - m, g = (e - K m) / |M|
+                    // the mean of gamma beta (beta . u)
+                    T ux = sx - mx, uy = sy - my;
                     if (W.el) {
-                        // spot elongation (Eq. 3): the sums of gamma beta (beta . s) as well
                         T b1, b2, gam;
                         elong(W, q0 + ii, j, b1, b2, gam);
-                        const T bs = b1 * sx + b2 * sy;
-                        sum[2] += gam * b1 * bs;
-                        sum[3] += gam * b2 * bs;
+                        const T bu = b1 * ux + b2 * uy;
+                        ux = (ux - gam * b1 * bu) + g1;
+                        uy = (uy - gam * b2 * bu) + g2;
                     }
+                    wx = inv * ux;
+                    wy = inv * uy;
+                } else if (W.nb > 1) {
+                    wx = sx * (nbinv * inv);                 // SLOPES of a coarse sensor
+                    wy = sy * (nbinv * inv);
+                } else {
+                    wx = inv * sx;                           // NGS: C^-1 = sigma^-2 I
+                    wy = inv * sy;
                 }
-            }
-            SX[k] = sx;
-            SY[k] = sy;
-        }
-        // a row's sums go to every rank; the row below the band is its owner's
-        if (need_tt && ii >= h0) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (e < 2 || W.el) {
-                    sum[e] = warp_sum_t(sum[e]);
-                    sum[e] = __shfl_sync(0xffffffffu, sum[e], 0);
-                    if (lane < SCL) cluster.map_shared_rank(&rsum[0][0], static_cast<unsigned>(lane))[(q0 + ii) * TS_NV + e] = sum[e];
-                }
-        }
-        if (need_coarse && ii >= h0) {
-            // per block column: the row's fine-slope sums
-            __syncwarp();
-            for (int J = 0; J < W.n_sub; ++J) {
-                T sx = T(0), sy = T(0);
-                for (int j = J * W.nb + lane; j < (J + 1) * W.nb; j += 32) {
-                    sx += SX[ii * N + j];
-                    sy += SY[ii * N + j];
-                }
-                sx = __shfl_sync(0xffffffffu, warp_sum_t(sx), 0);
-                sy = __shfl_sync(0xffffffffu, warp_sum_t(sy), 0);
-                if (lane < SCL) {
-                    T* dst = cluster.map_shared_rank(&rsum[0][0], static_cast<unsigned>(lane)) + (q0 + ii) * TS_NV + 2 * J;
-                    dst[0] = sx;
-                    dst[1] = sy;
+                if (SRC == SSRC_PHI && a.pqs && ii >= h0) {
+                    dot.add(sx, wx);
+                    dot.add(sy, wy);
                 }
             }
         }
+        SX[k] = wx;
+        SY[k] = wy;
     }
+    if (SRC == SSRC_PHI && a.pqs) dots[t] = AccOf<T>::of(dot);
     if (bad && a.status) atomicOr(a.status, 1u);
-    if (need_tt || need_coarse)
-        cluster.sync();                        // every row's sums are here; no remote access after this
-    else
-        __syncthreads();
-    if (need_tt) {
-        // the sums over the rows (fixed order), then the weighting
-        if (warp < (W.el ? 4 : 2)) {
-            T x = T(0);
-            for (int i = lane; i < N; i += 32) x += rsum[i][warp];
-            x = warp_sum_t(x);
-            if (lane == 0) tot[warp] = x;
-        }
-        __syncthreads();
-        const T mx = tot[0] / T(W.n_active), my = tot[1] / T(W.n_active);
-        if (!W.el) {
-            // C_hat^-1 = (I - T) sigma^-2 (I - T) = sigma^-2 (I - T) for an LGS
-            for (int k = t; k < nrow * N; k += NT) {
-                if (msk[k] >= 0) {
-                    SX[k] = inv * (SX[k] - mx);
-                    SY[k] = inv * (SY[k] - my);
-                }
-            }
-        } else {
-            // elongated: C_hat^-1 s = sigma^-2 (u - gamma beta (beta . u) + g), u = s
-            // minus its means m, g = (e - K m) / |M| the mean of gamma beta (beta . u)
-            const T ex = tot[2], ey = tot[3];
-            const T g1 = (ex - (el_K(W, 0, T()) * mx + el_K(W, 1, T()) * my)) / T(W.n_active);
-            const T g2 = (ey - (el_K(W, 1, T()) * mx + el_K(W, 2, T()) * my)) / T(W.n_active);
-            for (int ii = warp; ii < nrow; ii += nwarp)
-            for (int j = lane; j < N; j += 32) {
-                const int k = ii * N + j;
-                if (msk[k] >= 0) {
-                    T b1, b2, gam;
-                    elong(W, q0 + ii, j, b1, b2, gam);
-                    const T ux = SX[k] - mx, uy = SY[k] - my;
-                    const T bu = b1 * ux + b2 * uy;
-                    SX[k] = inv * ((ux - gam * b1 * bu) + g1);
-                    SY[k] = inv * ((uy - gam * b2 * bu) + g2);
-                }
-            }
-        }
-        __syncthreads();
+    __syncthreads();
+    // ---- Gamma_g^T on node rows [s0, s1) (and row N on the last band) ------------------------
+    const int nout = (s1 == N) ? rows + 1 : rows;
+    for (int k = t; k < nout * NP; k += NT) {
+        const int ia = k / NP, b = k - ia * NP;
+        // subaperture row s0 + ia (below the node) and the one before (above)
+        const bool has0 = s0 + ia < N, has1 = s0 + ia > 0, c0 = b < N, c1 = b > 0;
+        const T* x0 = SX + (ia + h0) * N;
+        const T* y0 = SY + (ia + h0) * N;
+        const T* x1 = x0 - N;
+        const T* y1 = y0 - N;
+        const T x_ab = (has0 && c0) ? x0[b] : T(0);
+        const T x_ab1 = (has0 && c1) ? x0[b - 1] : T(0);
+        const T x_a1b = (has1 && c0) ? x1[b] : T(0);
+        const T x_a1b1 = (has1 && c1) ? x1[b - 1] : T(0);
+        const T y_ab = (has0 && c0) ? y0[b] : T(0);
+        const T y_ab1 = (has0 && c1) ? y0[b - 1] : T(0);
+        const T y_a1b = (has1 && c0) ? y1[b] : T(0);
+        const T y_a1b1 = (has1 && c1) ? y1[b - 1] : T(0);
+        Vb[k] = T(0.5) * ((x_ab1 - x_ab) + (x_a1b1 - x_a1b)) + T(0.5) * ((y_a1b - y_ab) + (y_a1b1 - y_ab1));
     }
-    if (need_coarse) {
-        // coarse slope = sum / nb; Gamma_coarse^T spreads sigma^-2 slope / nb.  The residual
-        // form subtracts it from the block's measured slope.
-        const int ns = W.n_sub, nb = W.nb;
-        for (int e = warp; e < 2 * ns * ns; e += nwarp) {
-            const int blk = e >> 1, xy = e & 1, I = blk / ns, J = blk - I * ns;
-            T x = T(0);
-            for (int i = I * nb + lane; i < (I + 1) * nb; i += 32) x += rsum[i][2 * J + xy];
-            x = warp_sum_t(x);
-            if (lane == 0) {
-                x *= nbinv;
-                if (SRC == SSRC_RESID) {
-                    const int K = d.cidx[W.cmask_off + blk];
-                    T m = T(0);
-                    if (K >= 0) {
-                        m = a.in[W.soff + xy * W.n_active + K];
-                        if (!isfinite(m) && a.status) atomicOr(a.status, 1u);
-                    }
-                    x = m - x;
-                }
-                cw[e] = x * inv * nbinv;
-            }
-        }
-        __syncthreads();
-        for (int ii = warp; ii < nrow; ii += nwarp)
-        for (int j = lane; j < N; j += 32) {
-            const int k = ii * N + j;
-            T sx = T(0), sy = T(0);
-            if (msk[k] >= 0) {
-                const int blk = ((q0 + ii) / nb) * ns + j / nb;
-                sx = cw[2 * blk];
-                sy = cw[2 * blk + 1];
-            }
-            SX[k] = sx;
-            SY[k] = sy;
-        }
-        __syncthreads();
+    __syncthreads();
+    if (SRC == SSRC_PHI && a.pqs && warp == nwarp - 1) {
+        // the CTA's share of p.q, by the warp with the fewest columns below
+        A x = dots[lane];
+        for (int k = lane + 32; k < NT; k += 32) x = acc_merge(x, dots[k]);
+        x = acc_warp(x);
+        if (lane == 0) *reinterpret_cast<A*>(a.pqs + unit) = x;
     }
-    cp_async_wait();
-    if (rows > 0) {
-        // ---- Gamma_g^T on node rows [s0, s1) (and row N on the last band) ------------------
-        const int nout = (s1 == N) ? rows + 1 : rows;
-        for (int ia = warp; ia < nout; ia += nwarp)
-        for (int b = lane; b < NP; b += 32) {
-            // subaperture row s0 + ia (below the node) and the one before (above)
-            const bool has0 = s0 + ia < N, has1 = s0 + ia > 0, c0 = b < N, c1 = b > 0;
-            const T* x0 = SX + (ia + h0) * N;
-            const T* y0 = SY + (ia + h0) * N;
-            const T* x1 = x0 - N;
-            const T* y1 = y0 - N;
-            const T x_ab = (has0 && c0) ? x0[b] : T(0);
-            const T x_ab1 = (has0 && c1) ? x0[b - 1] : T(0);
-            const T x_a1b = (has1 && c0) ? x1[b] : T(0);
-            const T x_a1b1 = (has1 && c1) ? x1[b - 1] : T(0);
-            const T y_ab = (has0 && c0) ? y0[b] : T(0);
-            const T y_ab1 = (has0 && c1) ? y0[b - 1] : T(0);
-            const T y_a1b = (has1 && c0) ? y1[b] : T(0);
-            const T y_a1b1 = (has1 && c1) ? y1[b - 1] : T(0);
-            Vb[ia * NP + b] =
-                T(0.5) * ((x_ab1 - x_ab) + (x_a1b1 - x_a1b)) + T(0.5) * ((y_a1b - y_ab) + (y_a1b1 - y_ab1));
-        }
-        __syncthreads();
-        // ---- the column half of P_g^T: a thread owns a layer column and takes every row -----
-        for (int k = t; k < sco[nl]; k += NT) {
-            int l = 0;
-            while (k >= sco[l + 1]) ++l;
-            const int2 yb = ybox[l], c = cin[k];
-            const int j = k - sco[l], cols = yb.x;
-            if (j >= cols) continue;
-            T* dst = pb.Y + yb.y + s0 * cols + j;
-            const T* src = Vb + c.x;
-            const T* wk = cwt + k * ks;
-            if (c.y <= 3) {
-                T w[3];
+    // ---- the column half of P_g^T: a thread owns a layer column and takes every row -----------
+    for (int k = t; k < sco[nl]; k += NT) {
+        int l = 0;
+        while (k >= sco[l + 1]) ++l;
+        const int4 yb = ybox[l];
+        const int j = k - sco[l], cols = yb.x, at = yb.z + j;    // at: the column's place, as in xi
+        if (j >= cols) continue;
+        const int2 c = make_int2(cin[k] & 0xffff, cin[k] >> 16);
+        T* dst = pb.Y + yb.y + s0 * cols + j;
+        const T* src = Vb + c.x;
+        // node column b has the weight 1 - f on its layer column and f on the next one
+        const int* bi = xi + l * NPs + c.x;
+        const T* bf = xf + l * NPs + c.x;
+        if (c.y <= 3) {
+            T w[3];
 #pragma unroll
-                for (int q = 0; q < 3; ++q) w[q] = q < c.y ? wk[q] : T(0);
-#pragma unroll 3
-                for (int ia = 0; ia < nout; ++ia) {
+            for (int q = 0; q < 3; ++q) w[q] = q < c.y ? (bi[q] == at ? T(1) - bf[q] : bf[q]) : T(0);
+#pragma unroll
+            for (int ia = 0; ia < SR + 1; ++ia)
+                if (ia < nout) {
                     T x = T(0);
 #pragma unroll
                     for (int q = 0; q < 3; ++q)
                         if (q < c.y) x += w[q] * src[ia * NP + q];
                     dst[ia * cols] = x;
                 }
-            } else {
-                T w[KMAX];
+        } else {
+            T w[KMAX];
 #pragma unroll
-                for (int q = 0; q < KMAX; ++q) w[q] = q < c.y ? wk[q] : T(0);
-                for (int ia = 0; ia < nout; ++ia) {
-                    T x = T(0);
+            for (int q = 0; q < KMAX; ++q) w[q] = q < c.y ? (bi[q] == at ? T(1) - bf[q] : bf[q]) : T(0);
+            for (int ia = 0; ia < nout; ++ia) {
+                T x = T(0);
 #pragma unroll
-                    for (int q = 0; q < KMAX; ++q)
-                        if (q < c.y) x += w[q] * src[ia * NP + q];
-                    dst[ia * cols] = x;
-                }
+                for (int q = 0; q < KMAX; ++q)
+                    if (q < c.y) x += w[q] * src[ia * NP + q];
+                dst[ia * cols] = x;
             }
         }
     }
 }
 
-template <class T, int SRC, int SCL>
-__global__ void __cluster_dims__(SCL, 1, 1) __launch_bounds__(tsnt<T>(), sizeof(T) == 4 ? 2 : 1)
+template <class T, int SRC>
+__global__ void __launch_bounds__(tsnt<T>(), sizeof(T) == 4 ? 2 : 1)
     k_tsen(__grid_constant__ const Desc<T> d, __grid_constant__ const SensorArgs<T> a,
            __grid_constant__ const TsLayout lay, __grid_constant__ const PairBufs<T> pb) {
-    tsen_body<T, SRC, SCL>(d, a, lay, pb, blockIdx.y);
+    tsen_body<T, SRC>(d, a, lay, pb, blockIdx.x);
 }
 
 }  // namespace fewha
