@@ -68,10 +68,8 @@ struct LsfitDev {
     int *ly0 = nullptr, *lx0 = nullptr, *my0 = nullptr, *mx0 = nullptr;
     int *ylo = nullptr, *yhi = nullptr, *xlo = nullptr, *xhi = nullptr;
     void *lfy = nullptr, *lfx = nullptr, *mfy = nullptr, *mfx = nullptr;
-    void *v = nullptr, *r = nullptr, *p = nullptr, *q = nullptr;
-    double* part = nullptr;
-    double* msum = nullptr;
-    double* sc = nullptr;
+    void *v = nullptr, *r = nullptr, *p[2] = {};
+    double *us = nullptr, *s2 = nullptr, *rs = nullptr, *sc = nullptr;
     int* state = nullptr;
     size_t cap_pix = 0, cap_l = 0, cap_lf = 0, cap_m = 0, cap_mf = 0, cap_rng = 0, cap_v = 0;
 };
@@ -2577,8 +2575,9 @@ int ensure_lsfit(fewha_handle* H, const fewha_lsfit& cfg) {
     const size_t n_a = static_cast<size_t>(H->setup.n_act);
     const size_t nb = (n_a + LSF_ABLK - 1) / LSF_ABLK;
     if (!F.state) {   // allocated last: all of them are there
-        if ((rc = talloc(H, &F.r, n_a)) || (rc = talloc(H, &F.p, n_a)) || (rc = talloc(H, &F.q, n_a)) ||
-            (rc = dalloc(H, &F.part, nb)) || (rc = dalloc(H, &F.msum, LSF_MAXSL)) || (rc = dalloc(H, &F.sc, 2)) ||
+        if ((rc = talloc(H, &F.r, n_a)) || (rc = talloc(H, &F.p[0], n_a)) || (rc = talloc(H, &F.p[1], n_a)) ||
+            (rc = dalloc(H, &F.rs, nb)) || (rc = dalloc(H, &F.us, LSF_MAXSL)) || (rc = dalloc(H, &F.s2, LSF_MAXSL)) ||
+            (rc = dalloc(H, &F.sc, 4)) ||
             (rc = dalloc(H, &F.state, 2)))
             return rc;
     }
@@ -2641,8 +2640,8 @@ LsDesc<T> lsf_desc(const fewha_handle* H, const fewha_lsfit& cfg) {
     return d;
 }
 
-// phi = W^T c, the right-hand side, then CG chunks of FEWHA_MAX_ITERS steps until the
-// device reports that the CG has stopped.
+// phi = W^T c, the right-hand side, then CG chunks of LSF_CHUNK steps until the device reports
+// that the CG has stopped.
 template <class T>
 int fit_ls(fewha_handle* H, const fewha_lsfit& cfg, const T* c, T* a, double tol, int max_iters, int* iters_out,
            double* rel_out, cudaStream_t st) {
@@ -2651,46 +2650,44 @@ int fit_ls(fewha_handle* H, const fewha_lsfit& cfg, const T* c, T* a, double tol
     LsfitDev& F = *H->lsf;
     const Desc<T> d = make_desc<T>(H);
     T* phi = static_cast<T*>(H->phi);
-    if ((rc = launch_layer<T, LSRC_COEF, LDST_PHI, false>(H, d, layer_args<T>(H, c, phi), st))) return rc;
+    if ((rc = launch_inv<T, 0>(H, d, cl_args<T>(H, c, phi), st))) return rc;
     const LsDesc<T> ld = lsf_desc<T>(H, cfg);
-    T* v = static_cast<T*>(F.v);
-    T* p = static_cast<T*>(F.p);
-    T* q = static_cast<T*>(F.q);
-    const int nb = (ld.n_a + LSF_ABLK - 1) / LSF_ABLK;
-    const dim3 sgrid(ld.n_slices, ld.n_dirs);
-    k_lsf_sample<T, true><<<sgrid, LSF_SBLK, 0, st>>>(ld, phi, v, F.msum, nullptr);
-    k_lsf_adj<T><<<nb, LSF_ABLK, 0, st>>>(ld, v, F.msum, nullptr, q, nullptr, nullptr);
     LsCg<T> g{};
     g.n = ld.n_a;
-    g.nparts = nb;
+    g.nparts = (ld.n_a + LSF_ABLK - 1) / LSF_ABLK;
     g.max_iters = max_iters;
     g.tol2 = tol * tol;
     g.a = a;
     g.r = static_cast<T*>(F.r);
-    g.p = p;
-    g.q = q;
-    g.part = F.part;
+    g.p[0] = static_cast<T*>(F.p[0]);
+    g.p[1] = static_cast<T*>(F.p[1]);
+    g.v = static_cast<T*>(F.v);
+    g.us = F.us;
+    g.s2 = F.s2;
+    g.rs = F.rs;
     g.sc = F.sc;
     g.state = F.state;
-    k_lsf_cg<T, true><<<1, LSF_CBLK, 0, st>>>(g);
-    CK(cudaGetLastError(), "fit_ls launch");
+    const dim3 sg(ld.n_slices, ld.n_dirs), sb(LSF_SBLK), ag(g.nparts), ab((std::min(ld.n_dirs, LSF_AW) + 1) * 32);
+    CK(launch_k(H, k_lsf_sample<T, true>, sg, sb, 0, st, ld, g, static_cast<const T*>(phi), 0), "fit_ls launch");
+    CK(launch_k(H, k_lsf_adj<T, true>, ag, ab, 0, st, ld, g, 0), "fit_ls launch");
     int hst[2] = {0, 0};
     double hsc[2] = {0.0, 0.0};
     int run = 0;
     for (;;) {
-        const int k = std::min(FEWHA_MAX_ITERS, max_iters - run);
+        const int k = std::min(LSF_CHUNK, max_iters - run);
         for (int j = 0; j < k; ++j) {
-            k_lsf_sample<T, false><<<sgrid, LSF_SBLK, 0, st>>>(ld, p, v, F.msum, F.state);
-            k_lsf_adj<T><<<nb, LSF_ABLK, 0, st>>>(ld, v, F.msum, p, q, F.part, F.state);
-            k_lsf_cg<T, false><<<1, LSF_CBLK, 0, st>>>(g);
+            CK(launch_k(H, k_lsf_sample<T, false>, sg, sb, 0, st, ld, g, static_cast<const T*>(nullptr), run + j),
+               "fit_ls launch");
+            CK(launch_k(H, k_lsf_adj<T, false>, ag, ab, 0, st, ld, g, run + j), "fit_ls launch");
         }
-        CK(cudaGetLastError(), "fit_ls launch");
-        run += k;
+        run += std::max(k, 0);
+        CK(launch_k(H, k_lsf_check<T>, dim3(1), dim3(32), 0, st, g, run), "fit_ls launch");
         CK(cudaMemcpyAsync(hst, F.state, sizeof hst, cudaMemcpyDeviceToHost, st), "fit_ls state");
-        CK(cudaMemcpyAsync(hsc, F.sc, sizeof hsc, cudaMemcpyDeviceToHost, st), "fit_ls state");
+        CK(cudaMemcpyAsync(hsc, F.sc + 2, sizeof hsc, cudaMemcpyDeviceToHost, st), "fit_ls state");
         CK(cudaStreamSynchronize(st), "fit_ls");
         if (hst[0] || run >= max_iters) break;
     }
+    std::swap(hsc[0], hsc[1]);                            // r.r now, and at the start
     if (iters_out) *iters_out = hst[1];
     if (rel_out) *rel_out = hsc[1] > 0.0 ? std::sqrt(std::max(hsc[0], 0.0) / hsc[1]) : 0.0;
     if (!std::isfinite(hsc[0]) || !std::isfinite(hsc[1]))
