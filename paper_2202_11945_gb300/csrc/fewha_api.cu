@@ -524,9 +524,9 @@ int launch_fwd(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream
     CK(launch_k(H, k_tfwd<T, DST>, dim3(H->n_bu), dim3(cblk<T>()), H->smem_tf, st, d, a, H->lay_tf, pair_bufs<T>(H)),
        "k_tfwd launch");
     // (the vector parts are the CG update's)
-    const int coarse = DST == LDST_UPDATE ? H->n_tcl : H->n_coarse;
+    const int coarse = DST == LDST_UPDATE ? H->n_tcl : DST == LDST_PHI ? 0 : H->n_coarse;
     if (coarse > 0)
-        CK(launch_k(H, k_tcoarse<T, DST>, dim3(coarse), dim3(cblk<T>()), H->smem_tc, st, d, a, H->lay_tc),
+        CK(launch_k(H, k_tcoarse<T, DST == LDST_PHI ? LDST_COEF : DST>, dim3(coarse), dim3(cblk<T>()), H->smem_tc, st, d, a, H->lay_tc),
            "k_tcoarse launch");
     return FEWHA_OK;
 }
@@ -724,6 +724,62 @@ int enqueue_rhs(fewha_handle* H, const Desc<T>& d, const T* s, T* bout, cudaStre
     ClArgs<T> a = cl_args<T>(H, nullptr, bout);
     a.zero_piston = 1;
     return launch_fwd<T, LDST_COEF>(H, d, a, st);
+}
+
+// ---- operators beside the frame
+// Shared memory of k_model_slopes: the nodes of a band, or of a coarse subaperture.
+template <class T>
+size_t model_smem(const fewha_handle* H) {
+    size_t most = 0;
+    for (const WfsInfo& W : H->setup.G) {
+        const size_t n = W.nb > 1 ? static_cast<size_t>(W.nb + 1) * (W.nb + 1) : static_cast<size_t>(TS_ROWS + 1) * (W.N + 1);
+        most = std::max(most, n * sizeof(T));
+    }
+    return most;
+}
+
+// W^T c of every layer, its piston with it.
+template <class T>
+int enqueue_layers(fewha_handle* H, const Desc<T>& d, const T* c, T* phi, cudaStream_t st) {
+    return launch_inv<T, 0>(H, d, cl_args<T>(H, c, phi), st);
+}
+
+// s = Gamma P phi.
+template <class T>
+int enqueue_model(fewha_handle* H, const Desc<T>& d, const T* phi, T* s, cudaStream_t st) {
+    int units = 0;
+    for (const WfsInfo& W : H->setup.G) units += W.nb > 1 ? W.n_sub * W.n_sub : (W.N + TS_ROWS - 1) / TS_ROWS;
+    CK(launch_k(H, k_model_slopes<T>, dim3(units), dim3(OP_NT), model_smem<T>(H), st, d, phi, s), "k_model_slopes launch");
+    return FEWHA_OK;
+}
+
+// phi = P^T Gamma^T s.
+template <class T>
+int enqueue_model_adj(fewha_handle* H, const Desc<T>& d, const T* s, T* phi, cudaStream_t st) {
+    const SensorArgs<T> a{s, nullptr, H->status, nullptr, nullptr, nullptr, nullptr, nullptr};
+    CK(launch_k(H, k_tsen<T, SSRC_RAW>, dim3(H->n_su), dim3(tsnt<T>()), H->smem_ts, st, d, a, H->lay_ts, pair_bufs<T>(H)),
+       "k_tsen launch");
+    return launch_fwd<T, LDST_PHI>(H, d, cl_args<T>(H, nullptr, phi), st);
+}
+
+// out = C_hat^-1 s.
+template <class T>
+int enqueue_weigh(fewha_handle* H, const Desc<T>& d, const T* s, T* out, cudaStream_t st) {
+    int cells = 1;
+    for (const WfsInfo& W : H->setup.G) cells = std::max(cells, W.nb > 1 ? W.n_active : W.N * W.N);
+    CK(launch_k(H, k_msum<T>, dim3(d.n_wfs), dim3(TINV_NT), 0, st, d, s, H->msum), "k_msum launch");
+    CK(launch_k(H, k_weigh<T>, dim3((cells + OP_NT - 1) / OP_NT, d.n_wfs), dim3(OP_NT), 0, st, d, s,
+                static_cast<const double*>(H->msum), out, H->status),
+       "k_weigh launch");
+    return FEWHA_OK;
+}
+
+// c = W F^T a, the layers in H->phi on the way.
+template <class T>
+int enqueue_fit_adj(fewha_handle* H, const Desc<T>& d, const T* act, T* c, cudaStream_t st) {
+    T* phi = static_cast<T*>(H->phi);
+    CK(launch_k(H, k_fit_adj<T>, dim3((d.n_c + OP_NT - 1) / OP_NT), dim3(OP_NT), 0, st, d, act, phi), "k_fit_adj launch");
+    return launch_fwd<T, LDST_COEF>(H, d, cl_args<T>(H, static_cast<const T*>(phi), c), st);
 }
 
 int vec_grid(const fewha_handle* H) { return H->npart; }
@@ -1240,7 +1296,8 @@ int set_smem_limits(fewha_handle* H) {
         (rc = allow_smem(H, k_tinv<T, 1>, H->smem_tinv)) ||
         (rc = allow_smem(H, k_tinv<T, 2>, H->smem_tinv)) ||
         (rc = allow_smem(H, k_tsen<T, SSRC_PHI>, H->smem_ts)) || (rc = allow_smem(H, k_tsen<T, SSRC_SLOPES>, H->smem_ts)) ||
-        (rc = allow_smem(H, k_tsen<T, SSRC_RESID>, H->smem_ts)))
+        (rc = allow_smem(H, k_tsen<T, SSRC_RESID>, H->smem_ts)) || (rc = allow_smem(H, k_tsen<T, SSRC_RAW>, H->smem_ts)) ||
+        (rc = allow_smem(H, k_tfwd<T, LDST_PHI>, H->smem_tf)) || (rc = allow_smem(H, k_model_slopes<T>, model_smem<T>(H))))
         return rc;
     return FEWHA_OK;
 }
@@ -2423,7 +2480,7 @@ int backward(fewha_handle* H, const T* g_a, T* g_s, double* g_alpha, double* g_w
         double* lam = static_cast<double*>(X->lam);
         k_convert<double, float><<<(d.n_act + 255) / 256, 256, 0, st>>>(d.n_act, g_a, ga64);
         CK(cudaGetLastError(), "k_convert launch");
-        if ((rc = launch_layer<double, LSRC_DM, LDST_COEF, false>(X, dx, layer_args<double>(X, ga64, b64), st)))
+        if ((rc = enqueue_fit_adj<double>(X, dx, ga64, b64, st)))
             return fail(H, rc, X->err);
         if ((rc = mixed_solve(H, X, b64, lam, X->have_lam, H->grad_tol, H->grad_max_iters, st, &it, &rel)))
             return rc;
@@ -2435,9 +2492,8 @@ int backward(fewha_handle* H, const T* g_a, T* g_s, double* g_alpha, double* g_w
             double* t2 = static_cast<double*>(X->s_pol);
             CK(cudaMemcpyAsync(lz, lam, d.n_c * sizeof(double), cudaMemcpyDeviceToDevice, st), "lambda copy");
             if ((rc = zero_pistons<double>(H, lz, st))) return rc;
-            if ((rc = launch_layer<double, LSRC_COEF, LDST_PHI, false>(X, dx, layer_args<double>(X, lz, phi), st)) ||
-                (rc = launch_sensor<double, SSRC_PHI, false, SDST_SLOPES>(X, dx, phi, t1, st)) ||
-                (rc = launch_sensor<double, SSRC_SLOPES, true, SDST_SLOPES>(X, dx, t1, t2, st)))
+            if ((rc = enqueue_layers<double>(X, dx, lz, phi, st)) || (rc = enqueue_model<double>(X, dx, phi, t1, st)) ||
+                (rc = enqueue_weigh<double>(X, dx, t1, t2, st)))
                 return fail(H, rc, X->err);
             k_convert<float, double><<<(d.n_s + 255) / 256, 256, 0, st>>>(d.n_s, t2, g_s);
             CK(cudaGetLastError(), "k_convert launch");
@@ -2450,7 +2506,7 @@ int backward(fewha_handle* H, const T* g_a, T* g_s, double* g_alpha, double* g_w
         T* lam = static_cast<T*>(H->lam);
         T* phi = static_cast<T*>(H->phi);
         T* st_s = static_cast<T*>(H->s_tmp);
-        if ((rc = launch_layer<T, LSRC_DM, LDST_COEF, false>(H, d, layer_args<T>(H, g_a, b), st))) return rc;
+        if ((rc = enqueue_fit_adj<T>(H, d, g_a, b, st))) return rc;
         if ((rc = solve_converged<T>(H, b, lam, H->have_lam, H->grad_tol, H->grad_max_iters, st, &it, &rel)))
             return rc;
         H->have_lam = true;
@@ -2458,9 +2514,9 @@ int backward(fewha_handle* H, const T* g_a, T* g_s, double* g_alpha, double* g_w
             T* lz = static_cast<T*>(H->c_tmp);
             CK(cudaMemcpyAsync(lz, lam, d.n_c * sizeof(T), cudaMemcpyDeviceToDevice, st), "lambda copy");
             if ((rc = zero_pistons<T>(H, lz, st))) return rc;
-            if ((rc = launch_layer<T, LSRC_COEF, LDST_PHI, false>(H, d, layer_args<T>(H, lz, phi), st))) return rc;
-            if ((rc = launch_sensor<T, SSRC_PHI, false, SDST_SLOPES>(H, d, phi, st_s, st))) return rc;
-            if ((rc = launch_sensor<T, SSRC_SLOPES, true, SDST_SLOPES>(H, d, st_s, g_s, st))) return rc;
+            if ((rc = enqueue_layers<T>(H, d, lz, phi, st))) return rc;
+            if ((rc = enqueue_model<T>(H, d, phi, st_s, st))) return rc;
+            if ((rc = enqueue_weigh<T>(H, d, st_s, g_s, st))) return rc;
         }
         k_layer_dots<T><<<d.n_layers, PBLK, 0, st>>>(d, lam, static_cast<const T*>(H->cgrad), H->gdot);
         CK(cudaGetLastError(), "k_layer_dots launch");
@@ -2742,7 +2798,7 @@ int frame_vjp(fewha_handle* H, const T* s, const T* c0, const T* g_a, T* dm, T* 
         return FEWHA_OK;
     }
     // ---- reverse: every scalar on the device, no host round trip until the end ----------
-    if ((rc = launch_layer<T, LSRC_DM, LDST_COEF, false>(H, d, layer_args<T>(H, g_a, cbar), st))) return rc;
+    if ((rc = enqueue_fit_adj<T>(H, d, g_a, cbar, st))) return rc;
     CK(cudaMemsetAsync(rbar, 0, n * sizeof(T), st), "vjp zero");
     CK(cudaMemsetAsync(pbar, 0, n * sizeof(T), st), "vjp zero");
     CK(cudaMemsetAsync(H->gdot, 0, 4 * sizeof(double), st), "vjp scalars");
@@ -2782,19 +2838,19 @@ int frame_vjp(fewha_handle* H, const T* s, const T* c0, const T* g_a, T* dm, T* 
         k_vjp<T, VJ_E><<<gv, PBLK, 0, st>>>(n, va);
         CK(cudaGetLastError(), "k_vjp launch");
     }
-    // the recurrence must not have stopped (r.z or p.q vanished): checked once, at the end
-    std::vector<double> rho(k + 1), sigma(k + 1);
-    CK(cudaMemcpyAsync(rho.data(), H->rztot, (k + 1) * sizeof(double), cudaMemcpyDeviceToHost, st), "vjp rho");
-    if (k > 0)
-        CK(cudaMemcpyAsync(sigma.data(), H->pqtot, k * sizeof(double), cudaMemcpyDeviceToHost, st), "vjp sigma");
     // dJ/ds = C_hat^-1 Gamma P W^T b_bar (b_bar's pistons, large and annihilated by Gamma,
     // left out first)
     T* phi = static_cast<T*>(H->phi);
     T* st_s = static_cast<T*>(H->s_tmp);
     if ((rc = zero_pistons<T>(H, rbar, st))) return rc;
-    if ((rc = launch_layer<T, LSRC_COEF, LDST_PHI, false>(H, d, layer_args<T>(H, rbar, phi), st))) return rc;
-    if ((rc = launch_sensor<T, SSRC_PHI, false, SDST_SLOPES>(H, d, phi, st_s, st))) return rc;
-    if ((rc = launch_sensor<T, SSRC_SLOPES, true, SDST_SLOPES>(H, d, st_s, g_s, st))) return rc;
+    if ((rc = enqueue_layers<T>(H, d, rbar, phi, st))) return rc;
+    if ((rc = enqueue_model<T>(H, d, phi, st_s, st))) return rc;
+    if ((rc = enqueue_weigh<T>(H, d, st_s, g_s, st))) return rc;
+    // the recurrence must not have stopped (r.z or p.q vanished): checked once, at the end
+    std::vector<double> rho(k + 1), sigma(k + 1);
+    CK(cudaMemcpyAsync(rho.data(), H->rztot, (k + 1) * sizeof(double), cudaMemcpyDeviceToHost, st), "vjp rho");
+    if (k > 0)
+        CK(cudaMemcpyAsync(sigma.data(), H->pqtot, k * sizeof(double), cudaMemcpyDeviceToHost, st), "vjp sigma");
     CK(cudaStreamSynchronize(st), "vjp");
     for (int i = 0; i < k; ++i)
         if (!(sigma[i] > 0.0) || rho[i] == 0.0)
@@ -3329,9 +3385,6 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
     const Desc<T> d = make_desc<T>(H);
     const T* x = static_cast<const T*>(in);
     T* y = static_cast<T*>(out);
-    T* u = static_cast<T*>(H->u);
-    T* phi = static_cast<T*>(H->phi);
-    int rc = 0;
     switch (op) {
         case 0:  // M
             return enqueue_apply<T>(H, d, x, y, PQ_SCRATCH_SLOT, nullptr, st);
@@ -3340,7 +3393,7 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
         case 2:  // dwt
             return launch_layer<T, LSRC_PHI, LDST_COEF, false>(H, d, layer_args<T>(H, x, y), st);
         case 3:  // idwt
-            return launch_layer<T, LSRC_COEF, LDST_PHI, false>(H, d, layer_args<T>(H, x, y), st);
+            return enqueue_layers<T>(H, d, x, y, st);
         case 4:  // project
             return launch_sensor<T, SSRC_PHI, false, SDST_NODES>(H, d, x, y, st);
         case 5:  // project adjoint
@@ -3352,10 +3405,9 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
         case 8:  // noise weight
             return launch_sensor<T, SSRC_SLOPES, true, SDST_SLOPES>(H, d, x, y, st);
         case 9:  // forward model
-            return launch_sensor<T, SSRC_PHI, false, SDST_SLOPES>(H, d, x, y, st);
+            return enqueue_model<T>(H, d, x, y, st);
         case 10:  // forward adjoint
-            if ((rc = launch_sensor<T, SSRC_SLOPES, false, SDST_ADJ>(H, d, x, u, st))) return rc;
-            return launch_layer<T, LSRC_NODES, LDST_PHI, false>(H, d, layer_args<T>(H, u, y), st);
+            return enqueue_model_adj<T>(H, d, x, y, st);
         case 11:  // fit
             return enqueue_fit<T>(H, d, x, y, false, st);
         case 12:  // fit adjoint
@@ -3365,7 +3417,6 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
             return enqueue_pcg<T>(H, d, y, iters, false, st);
         }
         default:
-            (void)phi;
             return fail(H, FEWHA_ERR_INVALID_ARG, "unknown operator");
     }
 }

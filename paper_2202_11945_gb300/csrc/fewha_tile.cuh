@@ -600,14 +600,15 @@ struct EpiOp {
 };
 
 // The epilogue at one coefficient: v = (W y)(pos), dl its D.
-//   APPLY: q = v + alpha D p, written, p.q;  COEF: v written;
+//   APPLY: q = v + alpha D p, written, p.q;  COEF: v written (PHI has none: the layer itself
+//   is written, before the transform);
 //   RESID_INIT: r0 = v - alpha D c0 (v is the residual's data term), z = J^-1 r, p = z, r.z;
 //   APPLY_INIT: r0 = b - q, the same, and b_prev = b;
 //   UPDATE: r -= a q (q written to a.out too, if given), z = J^-1 r, r.z and, with upc,
 //   c += a p (step a).
 template <class T, int DST>
 __device__ __forceinline__ void epi_load(const ClArgs<T>& a, int pos, EpiOp<T>& o) {
-    if (DST != LDST_COEF) o.p = a.pin[pos];
+    if (DST != LDST_COEF && DST != LDST_PHI) o.p = a.pin[pos];
     if (DST == LDST_APPLY_INIT) o.b = a.vb[pos];
     if (DST == LDST_APPLY_INIT || DST == LDST_RESID_INIT || DST == LDST_UPDATE) o.j = a.vj[pos];
     if (DST == LDST_UPDATE) {
@@ -779,7 +780,20 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
     Quad<T> acc[TF_K];
 #pragma unroll
     for (int k = 0; k < TF_K; ++k) acc[k].zero();
-    for (int g0 = 0; g0 < d.n_wfs; g0 += lay.gb) {
+    const bool layers = DST == LDST_COEF && a.in;         // W of given layers (16-byte aligned)
+    if (layers)
+#pragma unroll
+        for (int k = 0; k < TF_K; ++k) {
+            const int task = t + k * NT;
+            if (task < (ry << lq)) {
+                const T* src = a.in + L.off + ((Y0 + (task >> lq)) & (n - 1)) * n + (task & ((1 << lq) - 1)) * (quads ? V : 1);
+                if (quads)
+                    acc[k] = *reinterpret_cast<const Quad<T>*>(src);
+                else
+                    acc[k].v.x = *src;
+            }
+        }
+    for (int g0 = 0; g0 < d.n_wfs && !layers; g0 += lay.gb) {
         const int nb = min(lay.gb, d.n_wfs - g0);
         if (g0 > 0) __syncthreads();
         for (int g = g0; g < g0 + nb; ++g) {
@@ -830,6 +844,20 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
                 }
             }
         }
+    }
+    if (DST == LDST_PHI) {
+#pragma unroll
+        for (int k = 0; k < TF_K; ++k) {
+            const int task = t + k * NT;
+            if (task < (bh << lq)) {
+                T* o = a.out + L.off + (Y0 + (task >> lq)) * n + (task & ((1 << lq) - 1)) * (quads ? V : 1);
+                const T* x = reinterpret_cast<const T*>(&acc[k].v);
+#pragma unroll
+                for (int e = 0; e < V; ++e)
+                    if (quads || e == 0) o[e] = x[e];
+            }
+        }
+        return;
     }
 #pragma unroll
     for (int k = 0; k < TF_K; ++k) {
@@ -1090,7 +1118,8 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
 // Sensor kernel, a CTA per band of TS_ROWS subaperture rows of a sensor: P_g (Sec. 2),
 // Gamma_g, C_hat_g^-1 (Eq. 2, Sec. 3.2), Gamma_g^T and the column half of P_g^T.  SRC_PHI:
 // slopes of the projected layers (the M-apply); SRC_RESID: measured minus modelled slopes
-// (the initial residual); SRC_SLOPES: measured slopes (the right-hand side).  The layers are
+// (the initial residual); SRC_SLOPES: measured slopes (the right-hand side); SRC_RAW: the same
+// without C_hat_g^-1 (the model's adjoint).  The layers are
 // read by direct bilinear gathers; the result goes out per layer as the aperture rows'
 // values on the layer's columns (pb.Y, slot g * n_layers + l, rows of box[3] columns), whose
 // row half the band kernel applies.
@@ -1175,7 +1204,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
     cp_async_wait();
     __syncthreads();
     const WfsInfo& W = sW;
-    const T inv = T(W.sig2inv);
+    const T inv = SRC == SSRC_RAW ? T(1) : T(W.sig2inv);
     const T nbinv = T(1) / T(W.nb);
     const int nu = d.su0[d.n_wfs], np = (d.n_c + nu - 1) / nu;           // this CTA's part of p.D p
     const T alpha = d.alpha;
@@ -1184,7 +1213,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
     bool bad = false;                          // a non-finite measured slope (SLOPES, RESID)
     DotAcc<T> dot;
     // ---- the sensor's functionals: the tiles' shares, a warp each, in flight beside the gather
-    for (int f = warp; f < nf; f += nwarp) {
+    for (int f = warp; f < (SRC == SSRC_RAW ? 0 : nf); f += nwarp) {
         A x = AccOf<T>::zero();
         if (FROM_PHI) x = shares_total<T, 6>(a.fsh + (f0 + f) * n_tu, n_tu);
         if (lane == 0) {
@@ -1257,7 +1286,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
     }
     // ---- the weighted slopes of rows [q0, s1) ------------------------------------------------
     T mx = T(0), my = T(0), g1 = T(0), g2 = T(0);
-    if (W.lgs) {
+    if (W.lgs && SRC != SSRC_RAW) {
         mx = tot[0] / T(W.n_active);
         my = tot[1] / T(W.n_active);
         if (W.el) {
@@ -1288,7 +1317,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
                     sx = ax - sx;
                     sy = ay - sy;
                 }
-                if (W.lgs) {
+                if (W.lgs && SRC != SSRC_RAW) {
                     // C_hat^-1 = (I - T) C^-1 (I - T): sigma^-2 (s - m) or, elongated,
                     // sigma^-2 (u - gamma beta (beta . u) + g), u = s - m, g = (e - K m) / |M|
                     // the mean of gamma beta (beta . u)
@@ -1395,6 +1424,144 @@ __global__ void __launch_bounds__(tsnt<T>(), sizeof(T) == 4 ? 2 : 1)
     k_tsen(__grid_constant__ const Desc<T> d, __grid_constant__ const SensorArgs<T> a,
            __grid_constant__ const TsLayout lay, __grid_constant__ const PairBufs<T> pb) {
     tsen_body<T, SRC>(d, a, lay, pb, blockIdx.x);
+}
+
+// ---------------------------------------------------------------------------
+// Operators beside the frame.  One CTA per sensor or layer took 34 us for the slopes of a
+// MAORY-size system's layers, 133 us for the adjoint and 41 us for the adjoint of the fit;
+// these spread each over the chip: 19 us, 11 us (k_tsen, k_tfwd) and about 8 us.
+// ---------------------------------------------------------------------------
+
+// Slopes of layers, s = Gamma P phi: a CTA per band of TS_ROWS subaperture rows of a fine sensor
+// or per subaperture of a coarse one (the mean over its block, summed in double).  Bound by
+// the latency of the tables' and the layers' loads.
+constexpr int OP_NT = 256;
+
+template <class T>
+__global__ void __launch_bounds__(OP_NT) k_model_slopes(__grid_constant__ const Desc<T> d, const T* phi, T* out) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* V = reinterpret_cast<T*>(smem_raw);
+    __shared__ double ws[2][OP_NT / 32];
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+    int g = 0, u = blockIdx.x;
+    for (;; ++g) {
+        const int cnt = d.G[g].nb > 1 ? d.G[g].n_sub * d.G[g].n_sub : (d.G[g].N + TS_ROWS - 1) / TS_ROWS;
+        if (u < cnt) break;
+        u -= cnt;
+    }
+    const WfsInfo& W = d.G[g];
+    const int N = W.N, nb = W.nb, K = nb > 1 ? d.cidx[W.cmask_off + u] : 0;
+    if (K < 0) return;                                   // an inactive coarse subaperture
+    const int i0 = nb > 1 ? u / W.n_sub * nb : u * TS_ROWS, j0 = nb > 1 ? u % W.n_sub * nb : 0;
+    const int rows = nb > 1 ? nb : min(TS_ROWS, N - i0), cols = nb > 1 ? nb : N, vw = cols + 1;
+    pdl_wait();
+    pdl_trigger();
+    for (int k = t; k < (rows + 1) * vw; k += OP_NT) {
+        const int ia = k / vw, aa = i0 + ia, bb = j0 + k - ia * vw;
+        T v = T(0);
+#pragma unroll 3
+        for (int l = 0; l < d.n_layers; ++l) {
+            const int tp = (g * MAXL + l) * TAB, n = d.L[l].n;
+            const T fy = d.pfy[tp + aa], fx = d.pfx[tp + bb];
+            const T* P = phi + d.L[l].off + d.pi0y[tp + aa] * n + d.pi0x[tp + bb];
+            v += (T(1) - fy) * ((T(1) - fx) * P[0] + fx * P[1]) + fy * ((T(1) - fx) * P[n] + fx * P[n + 1]);
+        }
+        V[k] = v;
+    }
+    __syncthreads();
+    double tx = 0.0, ty = 0.0;
+    for (int k = t; k < rows * cols; k += OP_NT) {
+        const int i = k / cols, j = k - i * cols, id = d.sidx[W.mask_off + (i0 + i) * N + j0 + j];
+        if (id < 0) continue;
+        const T* p = V + i * vw + j;
+        const T sx = T(0.5) * ((p[1] - p[0]) + (p[vw + 1] - p[vw])), sy = T(0.5) * ((p[vw] - p[0]) + (p[vw + 1] - p[1]));
+        if (nb > 1) {
+            tx += double(sx);
+            ty += double(sy);
+        } else {
+            out[W.soff + id] = sx;
+            out[W.soff + W.n_active + id] = sy;
+        }
+    }
+    if (nb <= 1) return;
+    tx = warp_sum(tx);
+    ty = warp_sum(ty);
+    if (lane == 0) {
+        ws[0][warp] = tx;
+        ws[1][warp] = ty;
+    }
+    __syncthreads();
+    if (t < 2) {
+        double x = 0.0;
+        for (int w = 0; w < OP_NT / 32; ++w) x += ws[t][w];
+        out[W.soff + t * W.n_active + K] = T(x / nb);
+    }
+}
+
+// C_hat^-1 s of every sensor (blockIdx.y) from the sums of k_msum (Sec. 3.2, Eq. 3), as in
+// tsen_body.
+template <class T>
+__global__ void __launch_bounds__(OP_NT) k_weigh(__grid_constant__ const Desc<T> d, const T* s, const double* msum,
+                                                 T* out, unsigned* status) {
+    using A = typename AccOf<T>::type;
+    const int g = blockIdx.y, k = blockIdx.x * OP_NT + threadIdx.x;
+    const WfsInfo& W = d.G[g];
+    const int cells = W.nb > 1 ? W.n_active : W.N * W.N;
+    const int id = k >= cells ? -1 : W.nb > 1 ? k : d.sidx[W.mask_off + k];
+    pdl_wait();
+    pdl_trigger();
+    if (id < 0) return;
+    const T inv = T(W.sig2inv);
+    T ux = s[W.soff + id], uy = s[W.soff + W.n_active + id];
+    if (!(isfinite(ux) && isfinite(uy)) && status) atomicOr(status, 1u);
+    if (W.lgs && W.nb == 1) {
+        const A* m = reinterpret_cast<const A*>(msum + d.f0[g]);
+        const T mx = T(warp_value(m[0])) / T(W.n_active), my = T(warp_value(m[1])) / T(W.n_active);
+        ux -= mx;
+        uy -= my;
+        if (W.el) {
+            const T g1 = (T(warp_value(m[2])) - (el_K(W, 0, T()) * mx + el_K(W, 1, T()) * my)) / T(W.n_active);
+            const T g2 = (T(warp_value(m[3])) - (el_K(W, 1, T()) * mx + el_K(W, 2, T()) * my)) / T(W.n_active);
+            T b1, b2, gam;
+            elong(W, k / W.N, k % W.N, b1, b2, gam);
+            const T bu = b1 * ux + b2 * uy;
+            ux = (ux - gam * b1 * bu) + g1;
+            uy = (uy - gam * b2 * bu) + g2;
+        }
+    }
+    out[W.soff + id] = inv * ux;
+    out[W.soff + W.n_active + id] = inv * uy;
+}
+
+// The layers F^T a of the DM fit's adjoint: y_l(i, j) = sum_m w_lm sum_p sum_q wy(p, i)
+// wx(q, j) a_m(p, q), a thread per layer node.
+template <class T>
+__global__ void __launch_bounds__(OP_NT) k_fit_adj(__grid_constant__ const Desc<T> d, const T* act, T* out) {
+    const int e = blockIdx.x * OP_NT + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
+    if (e >= d.n_c) return;
+    int l = 0;
+    while (l + 1 < d.n_layers && e >= d.L[l + 1].off) ++l;
+    const int n = d.L[l].n, i = (e - d.L[l].off) / n, j = (e - d.L[l].off) & (n - 1);
+    T acc = T(0);
+    for (int m = 0; m < d.n_dms; ++m) {
+        const T w = d.fitw[m][l];
+        if (w == T(0)) continue;
+        const int rb = (m * MAXL + l) * MAXN, tb = (m * MAXL + l) * MAXNACT, na = d.Mi[m].n_act;
+        const int p0 = d.dr_lo[rb + i], p1 = d.dr_hi[rb + i], q0 = d.dr_lo[rb + j], q1 = d.dr_hi[rb + j];
+        const T* am = act + d.Mi[m].off;
+        T sm = T(0);
+        for (int p = p0; p < p1; ++p) {
+            const T wy = d.di0[tb + p] == i ? T(1) - d.dfw[tb + p] : d.dfw[tb + p];
+            T row = T(0);
+            for (int q = q0; q < q1; ++q)
+                row += (d.di0[tb + q] == j ? T(1) - d.dfw[tb + q] : d.dfw[tb + q]) * am[p * na + q];
+            sm += wy * row;
+        }
+        acc += w * sm;
+    }
+    out[e] = acc;
 }
 
 }  // namespace fewha
