@@ -40,9 +40,8 @@ N_FRAMES_INPUT = 8          # distinct seeded frames, cycled through the timed l
 FLUSH_BYTES = 512 << 20     # > 129 MB L2
 _CSRC = os.path.join(ROOT, "paper_2202_11945_gb300", "csrc")
 # source file of each stage's kernel (the traffic record is tied to its hash)
-STAGE_SRC = {"idwt": "fewha_cluster.cuh", "sensor": "fewha_cluster.cuh", "layer": "fewha_cluster.cuh",
-             "rhs": "fewha_cluster.cuh", "proj": "fewha_pair.cuh", "projT": "fewha_pair.cuh",
-             "vector": "fewha_kernels.cuh", "fit": "fewha_kernels.cuh"}
+STAGE_SRC = {"idwt": "fewha_tile.cuh", "sensor": "fewha_tile.cuh", "layer": "fewha_tile.cuh",
+             "rhs": "fewha_tile.cuh", "fit": "fewha_kernels.cuh"}
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic_maory_fp32.txt")
 
 
@@ -173,23 +172,19 @@ def stage_bytes(R, b):
     nc, nn, ns, na = R.n_coeffs, R.n_nodes, R.n_slopes, R.n_act
     return {
         "idwt": 4 * nc * b,               # read z, p; write p, phi
-        "proj": (nc + nn) * b,            # read phi; write P phi on the aperture nodes
-        "sensor": 2 * nn * b,             # read P phi; write the aperture-node adjoint u
-        "projT": (nn + nc) * b,           # read u; write P^T u on the layers
-        "layer": 3 * nc * b,              # read P^T u and p; write q (D: one value per level)
-        "vector": 11 * nc * b,            # read c, p, r, q, J^-1, phi_c, phi_p; write c, r, z, phi_c
+        "sensor": (nc + nn) * b,          # read phi; write the aperture-node adjoint u
+        "layer": (nn + 10 * nc) * b,      # read u and c, p, r, J^-1, phi_c, phi_p; write c, r, z, phi_c
         "rhs": (ns + nn) * b,             # read slopes; write u
         "fit": (nc + 3 * na) * b,         # read phi, a_prev; write a_prev, dm
     }
 
 
 def stage_launches(iters):
-    """Launches of each stage's kernel in one explicit-residual frame: the initial residual's
-    chain (inverse transform, P, the sensor kernel on the slopes' residual, P^T, the forward
-    kernel with the vector step) and one apply plus one CG update per iteration; the fit
-    reads the carried layers (no inverse transform) and no right-hand side is formed."""
-    return {"idwt": iters + 1, "proj": iters + 1, "sensor": iters + 1, "projT": iters + 1,
-            "layer": iters + 1, "vector": iters, "rhs": 0, "fit": 1}
+    """Launches of each stage in one explicit-residual frame: the initial residual's chain
+    (inverse transform, the sensor kernel on the slopes' residual, the forward kernels) and
+    one apply with the CG update in its forward kernels per iteration; the fit reads the
+    carried layers (no inverse transform) and no right-hand side is formed."""
+    return {"idwt": iters + 1, "sensor": iters + 1, "layer": iters + 1, "rhs": 0, "fit": 1}
 
 
 def time_stages(R, flush, reps=100):
@@ -197,7 +192,7 @@ def time_stages(R, flush, reps=100):
     captured in a CUDA graph (so the host launch rate does not pace them), after a flush."""
     out = {}
     cap = torch.cuda.Stream()
-    for st in ("idwt", "proj", "sensor", "projT", "layer", "vector", "rhs", "fit"):
+    for st in ("idwt", "sensor", "layer", "rhs", "fit"):
         R.bench_stage(st, 3)
         torch.cuda.synchronize()
         g = torch.cuda.CUDAGraph()

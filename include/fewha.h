@@ -84,8 +84,7 @@ extern "C" {
 #define FEWHA_FLAG_GRAPH 1u         /* replay each frame as a captured CUDA graph    */
 #define FEWHA_FLAG_WARM_RESIDUAL 2u /* r0 = (b - b_prev) + r_prev (Algorithm 1)     */
 #define FEWHA_FLAG_PDL 4u           /* programmatic dependent launch: each kernel lets
-                                       the next one launch its CTAs early (the cluster
-                                       kernels from a barrier in their middle), which
+                                       the next one launch its CTAs early, which
                                        wait on the device for it to finish; shortens
                                        the gap between dependent kernels (the Python
                                        binding sets it by default)                     */
@@ -369,14 +368,15 @@ int fewha_fit_ls(fewha_handle* h, const fewha_lsfit* cfg, const void* d_c, void*
 /* ---- measurement --------------------------------------------------------------- */
 
 /* Hot-path stages of one PCG iteration and of the frame, for timing one kernel alone. */
-#define FEWHA_STAGE_IDWT 0      /* p = z + beta p and phi = W^T p, one CTA per layer       */
-#define FEWHA_STAGE_SENSOR 1    /* sum of the pair terms, Gamma_g, C_hat_g^-1, Gamma_g^T    */
-#define FEWHA_STAGE_LAYER 2     /* sum of the pair terms, W, + alpha D p, p.q               */
-#define FEWHA_STAGE_VECTOR 3    /* x += a p, r -= a q, z = J^-1 r, r.z                     */
+#define FEWHA_STAGE_IDWT 0      /* p = z + beta p and phi = W^T p, a CTA per tile           */
+#define FEWHA_STAGE_SENSOR 1    /* P_g, Gamma_g, C_hat_g^-1, Gamma_g^T, columns of P_g^T    */
+#define FEWHA_STAGE_LAYER 2     /* rows of P^T, W, + alpha D p and the CG update: bands, then
+                                   the coarse levels                                        */
+#define FEWHA_STAGE_VECTOR 3    /* the update as a kernel of its own (persistent frame)     */
 #define FEWHA_STAGE_RHS 4       /* C_hat^-1 and Gamma^T of the measured slopes             */
 #define FEWHA_STAGE_FIT 5       /* DM fit and gain                                          */
-#define FEWHA_STAGE_PROJ 6      /* R_y phi_l R_x^T per (sensor, layer) pair                  */
-#define FEWHA_STAGE_PROJT 7     /* R_y^T u_g R_x per (sensor, layer) pair                    */
+#define FEWHA_STAGE_PROJ 6      /* the kernel of FEWHA_STAGE_SENSOR, which holds P           */
+#define FEWHA_STAGE_PROJT 7     /* the kernels of FEWHA_STAGE_LAYER, which hold P^T          */
 #define FEWHA_NUM_STAGES 8
 
 /* Enqueue `reps` back-to-back launches of one stage's kernel on `stream`, working on the
@@ -450,8 +450,8 @@ int fewha_backward(fewha_handle* h, const void* d_grad_dm, void* d_grad_slopes, 
  * frame each in one CUDA-graph replay.  The frame of Algorithm 1 is the same sequence of
  * steps for every instance (right-hand side, initial residual, `iters` PCG iterations,
  * fit), so each step runs as ONE kernel launch over a work list of (instance, unit)
- * items, a unit being a layer, a sensor, a (sensor, layer) pair or a CTA of the vector
- * and fit kernels.  Results are bit-identical to the instances' own fewha_reconstruct.
+ * items, a unit being a tile, a band or a part of a layer, a band of a sensor, or a CTA of
+ * the vector and fit kernels.  Results are bit-identical to the instances' own fewha_reconstruct.
  * All instances must share the device, precision, iteration count and warm-residual
  * mode; each runs on its own internal warm state (as fewha_reconstruct with
  * d_x_warm = NULL).  A handle may belong to several batches but not twice to one; a
@@ -465,11 +465,11 @@ typedef struct {
     int groups;      /* 1..FEWHA_BATCH_MAX_GROUPS: instances split (by balanced cost) into this
                         many independent launch chains that run concurrently */
     int vec_passes;  /* 1..8: passes of 4 elements per thread of the vector kernel's CTAs */
-    int pair_threads;/* threads per CTA of the (sensor, layer) projection kernels: 0 = the
-                        single-instance size (512 in single, 256 in double precision), or
-                        half of it */
-    int proj_taps;   /* unrolled taps of the adjoint projection: 0 = as few as every member's
-                        geometry allows, 4 (only if every member allows it) or 8 */
+    int pair_threads;/* 0, 512 or 256 in single and 256 or 128 in double precision; the
+                        projections are part of the sensor and layer kernels, whose shape
+                        is fixed: accepted, without effect */
+    int proj_taps;   /* 0, 8, or 4 if every member's geometry has at most 4 aperture rows per
+                        layer row: accepted, without effect */
     int vec_threads; /* threads per CTA of the vector kernel: 0 = 256, 256 or 512 */
 } fewha_batch_config;
 
@@ -492,9 +492,7 @@ int fewha_batch_reconstruct(fewha_batch* b, const void* const* d_slopes, void* c
 
 /* Autotuner: times the candidate configurations on `reps` batched frames of the given
  * slopes (CUDA events on `stream`): first every order x groups x vec_passes with the default
- * kernel shapes, then, from the best of those, every pair_threads x proj_taps x vec_threads
- * (the CTA sizes of the projection and vector kernels and the adjoint projection's tap
- * unroll, as far as the members' geometry allows), and keeps the fastest
+ * kernel shapes, then, from the best of those, every vec_threads, and keeps the fastest
  * in the batch and in a process-wide table keyed by the instances' shapes (a later batch
  * of the same shapes starts from it), and restores every member's warm state afterwards.
  * *best_us (nullable) receives the chosen configuration's mean frame time.  Synchronous. */

@@ -845,6 +845,29 @@ struct CgVecs {
 };
 
 
+// The forward kernels' arguments of CG update k.
+template <class T>
+ClArgs<T> update_args(fewha_handle* H, const CgVecs<T>& v, int k, bool last) {
+    ClArgs<T> b = cl_args<T>(H, nullptr, v.q);
+    b.pin = v.p;
+    b.iter = k;
+    b.lsh = rz_shares(H, k + 1);
+    b.zero_piston = 1;
+    b.pqs = H->pqs;
+    b.n_pqs = H->n_su;
+    b.alphas = static_cast<T*>(H->alphas);
+    b.vc = v.c;
+    b.phic = v.phic;
+    b.phip = static_cast<const T*>(H->phi);
+    b.rin = v.r;
+    b.vr = v.rnew;
+    b.vz = v.znew;
+    b.vj = static_cast<const T*>(H->Jinv);
+    b.rzslot = k + 1;
+    b.defer_total = last ? 0 : 1;
+    return b;
+}
+
 // Iteration k of the PCG (Sec. 3.3) in four kernels: p = z + beta p_old and W^T p, the
 // sensors, and the two forward kernels with the update c += alpha p, r -= alpha q,
 // z = J^-1 r in their epilogues (p.q is known before q, see ClArgs::pqs).  The r.z total of
@@ -871,24 +894,7 @@ int enqueue_iteration(fewha_handle* H, const Desc<T>& d, const CgVecs<T>& v, int
         rc = launch_inv<T, 0>(H, d, a, st);
     }
     if (rc || (rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st, static_cast<const T*>(v.p)))) return rc;
-    ClArgs<T> b = cl_args<T>(H, nullptr, v.q);
-    b.pin = v.p;
-    b.iter = k;
-    b.lsh = rz_shares(H, k + 1);
-    b.zero_piston = 1;
-    b.pqs = H->pqs;
-    b.n_pqs = H->n_su;
-    b.alphas = static_cast<T*>(H->alphas);
-    b.vc = v.c;
-    b.phic = v.phic;
-    b.phip = phi;
-    b.rin = v.r;
-    b.vr = v.rnew;
-    b.vz = v.znew;
-    b.vj = static_cast<const T*>(H->Jinv);
-    b.rzslot = k + 1;
-    b.defer_total = last ? 0 : 1;
-    return launch_fwd<T, LDST_UPDATE>(H, d, b, st);
+    return launch_fwd<T, LDST_UPDATE>(H, d, update_args<T>(H, v, k, last), st);
 }
 
 // The iteration on the handle's own vectors, the direction buffers in turn.
@@ -3244,21 +3250,14 @@ int batch_autotune(fewha_batch* B, const void* const* s, void* const* dm, int re
             if (groups[gi] > static_cast<int>(n)) continue;
             for (int vi = 0; vi < 2 && rc == FEWHA_OK; ++vi) trial(fewha_batch_config{order, groups[gi], vps[vi], 0, 0, 0});
         }
-    // stage 2: from the best of stage 1, the kernels' launch shapes
-    int kmax = 0;
-    for (const fewha_handle* H : B->h) kmax = std::max(kmax, H->kmax);
-    const int nt = cblk<T>();
+    // stage 2: from the best of stage 1, the vector kernel's launch shape
     const fewha_batch_config base = best;
-    for (int pt : {nt, nt / 2})
-        for (int tp : {4, KMAX})
-            for (int vt : {PBLK, 2 * PBLK}) {
-                if (rc != FEWHA_OK || tp < kmax) continue;
-                fewha_batch_config c = base;
-                c.pair_threads = pt;
-                c.proj_taps = tp;
-                c.vec_threads = vt;
-                trial(c);
-            }
+    for (int vt : {PBLK, 2 * PBLK}) {
+        if (rc != FEWHA_OK) continue;
+        fewha_batch_config c = base;
+        c.vec_threads = vt;
+        trial(c);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     copy_state(false);
@@ -3427,7 +3426,6 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
     const Desc<T> d = make_desc<T>(H);
     T* p = static_cast<T*>(H->p);
     T* phi = static_cast<T*>(H->phi);
-    T* q = static_cast<T*>(H->q);
     int rc = 0;
     for (int i = 0; i < reps && rc == 0; ++i) {
         switch (stage) {
@@ -3441,19 +3439,16 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
                 rc = launch_inv<T, 1>(H, d, a, st);
                 break;
             }
-            // P runs in the sensor kernel, P^T half there and half in the layer kernels
+            // P runs in the sensor kernel, P^T half there and half in the layer kernels; the CG
+            // update in these
             case FEWHA_STAGE_SENSOR:
             case FEWHA_STAGE_PROJ:
                 rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st);
                 break;
             case FEWHA_STAGE_LAYER:
             case FEWHA_STAGE_PROJT: {
-                ClArgs<T> a = cl_args<T>(H, nullptr, q);
-                a.lsh = pq_shares(H, PQ_SCRATCH_SLOT);
-                a.pin = p;
-                a.iter = PQ_SCRATCH_SLOT;
-                a.zero_piston = 1;
-                rc = launch_fwd<T, LDST_APPLY>(H, d, a, st);
+                const CgVecs<T> v = cg_vecs<T>(H, static_cast<T*>(H->c), 0, true, static_cast<T*>(H->phic));
+                rc = launch_fwd<T, LDST_UPDATE>(H, d, update_args<T>(H, v, 0, true), st);
                 break;
             }
             case FEWHA_STAGE_VECTOR:
@@ -3904,17 +3899,21 @@ int fewha_bench_stage(fewha_handle* H, int stage, int reps, void* stream) {
 int fewha_frame_launches(const fewha_handle* H, int* launches) {
     if (!H || !launches) return FEWHA_ERR_INVALID_ARG;
     const bool warm = (H->params.flags & FEWHA_FLAG_WARM_RESIDUAL) != 0;
-    // the plain explicit frame: r0 from the slopes' residual, 5 (the right-hand side is not
-    // formed); with the warm recurrence, RHS 3 and r0 1 (its explicit refresh frames: 3 + 5);
-    // augmented: r0 5 and one more start kernel (its direction update is fused into the
-    // inverse kernel of each apply); 6 per iteration
     const int aug = (H->params.flags & FEWHA_FLAG_AUGMENTED) ? 1 : 0;
     const int closed = (H->params.flags & FEWHA_FLAG_CLOSED_LOOP) ? 2 : 0;
+    // the bands, and the coarse levels where a layer has several bands
+    const int fwd = H->n_coarse > 0 ? 2 : 1;
+    // r0 from the slopes' residual: inverse, sensor, forward (the right-hand side is not
+    // formed), and two start kernels if augmented; with the warm recurrence the sums of the
+    // measured slopes, sensor and forward for b, and the vector kernel (its explicit refresh
+    // frames form r0 by an apply)
+    const int start = 2 + fwd + (warm ? 1 : aug ? 2 : 0);
+    // inverse, sensor, forward (with the CG update; augmented, the update is a kernel)
+    const int per_iter = 2 + fwd + aug;
     // fit: 2 (inverse transform, fit), or 1 where the plain explicit frame carries the
     // layers of c through its iterations
-    const int per_iter = 6, start = warm ? 3 + 1 : (aug ? 5 + 1 : 5);
     const int fit = (warm || aug) ? 2 : 1;
-    *launches = (H->params.flags & FEWHA_FLAG_PERSISTENT) ? 1 : closed + start + aug + per_iter * H->params.iters + fit;
+    *launches = (H->params.flags & FEWHA_FLAG_PERSISTENT) ? 1 : closed + start + per_iter * H->params.iters + fit;
     return FEWHA_OK;
 }
 
