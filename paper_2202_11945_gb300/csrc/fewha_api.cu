@@ -1421,7 +1421,7 @@ int tile_tables(fewha_handle* H) {
     std::vector<int> tcl, vec;
     std::vector<int> bsrc, row0;                           // row0: first staged row per unit and sensor
     const int nyslot = H->pyslot;
-    int rw = 0, yw = 0, lb1 = 0, lbc = 0;
+    int rw = 0, yw = 0, lb1 = 0, lbc = 0, mw = 0;
     std::vector<std::vector<int>> need;                    // staged elements per unit and sensor
     bool tail1 = false;
     for (int l = 0; l < nl; ++l) {
@@ -1474,6 +1474,7 @@ int tile_tables(fewha_handle* H) {
         }
         rw = std::max(rw, ry * ng * (kt + 1));
         yw = std::max(yw, ry * ((h + 1) & ~1));
+        if (sizeof(T) == 8) mw = std::max(mw, round4(ry * (n + 1)));   // the finest level's rows
         if (bands == 1) {
             ++H->n_writers;
             lb1 = std::max(lb1, h * (h + 1));
@@ -1516,7 +1517,7 @@ int tile_tables(fewha_handle* H) {
                 most = std::max(most, at);
             }
         }
-        f.total = f.st + most;
+        f.total = f.st + std::max(most, mw);
         if (most <= room) break;
     }
     f.gb = std::max(f.gb, 1);
