@@ -2410,20 +2410,30 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
 
 // The converged solve of a single-precision handle on the twin's double vectors.  The float
 // recurrence needs 1.6 to 2.9 times the double one's iterations, by how its rounding falls
-// (8 m and 4 m geometries at 1e-11: 12.7k to 21k against 7.1k to 8k).  An iteration of a
-// small instance is a chain of short kernels whose arithmetic hides behind the launches, so
-// a double iteration costs 1.65 times a float one at 1280 coefficients (43.6 against 26.5
-// us) and 1.8 times at 3072; at 16384 it costs 2.2 times, at 49152 3.8 times.  Up to
-// SOLVE_DOUBLE_NC coefficients the recurrence runs in double: 8 m forward and backward
-// 747 -> 646 ms.
+// (8 m and 4 m geometries at 1e-11: 12.7k to 21k for forward and backward against 7.1k to
+// 10.8k), at 13 us an iteration against 43: forward and backward take 384 ms in float and 470
+// in double at 8 m, 299 to 375 against 354 to 408 on four smaller systems.  So that a small
+// instance does not run out of iterations where the rounding falls badly, the last quarter of
+// them is kept for the double recurrence, from where the float one got to.  Above
+// SOLVE_DOUBLE_NC coefficients, where a double iteration costs 4 times a float one in
+// arithmetic (49152 coefficients: 3.8), all of them are the float one's.
 constexpr int SOLVE_DOUBLE_NC = 4096;
 int mixed_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* x64, bool warm, double tol,
                 int max_iters, cudaStream_t st, int* iters_out, double* rel_out) {
-    if (H->setup.n_c > SOLVE_DOUBLE_NC)
-        return reliable_solve(H, X, b64, x64, warm, tol, max_iters, st, iters_out, rel_out);
-    const int rc = solve_converged<double>(X, b64, x64, warm, tol, max_iters, st, iters_out, rel_out);
+    const int first = H->setup.n_c > SOLVE_DOUBLE_NC ? max_iters : max_iters - max_iters / 4;
+    int it = 0;
+    double rel = 0.0;
+    int rc = reliable_solve(H, X, b64, x64, warm, tol, first, st, &it, &rel);
+    if (!rc && it >= first && it < max_iters && rel > tol) {
+        int more = 0;
+        rc = solve_converged<double>(X, b64, x64, true, tol, max_iters - it, st, &more, &rel);
+        it += more;
+        if (rc) fail(H, rc, X->err);
+    }
     H->have_prev = false;
-    return rc ? fail(H, rc, X->err) : FEWHA_OK;
+    if (iters_out) *iters_out = it;
+    if (rel_out) *rel_out = rel;
+    return rc;
 }
 
 template <class T>
