@@ -18,7 +18,11 @@ namespace fewha {
 
 constexpr int TINV_NT = 512;     // threads of the inverse tile kernel
 constexpr int TINV_SL = 4;       // coefficient slots per thread and round
-constexpr int TINV_FEW = 160;    // entries of a functional that 8 lanes take
+// Entries of a functional on a tile that 8 lanes take; one of more has a weight per node, for
+// all threads.  Boundary sums have at most some 150 entries a tile and take 1 us beside one
+// another; the elongation's have up to 1024, and as lists they took 6 us a launch, as weights
+// reduced together 1.2 (37 m frame 86.7 against 75.8 us).
+constexpr int TINV_FEW = 160;
 constexpr int TINV_DN = 16;      // functionals of more entries taken together
 
 // ---------------------------------------------------------------------------
@@ -557,8 +561,8 @@ __device__ __forceinline__ void analyse(T* buf, T* tmp, const T* tail, int n, in
 // a cluster per layer summed the pairs, transformed and finished on one leader CTA (11 us).
 // Bands of 8 whole rows keep every global read a contiguous block and need a halo in one
 // direction only; square tiles with a halo on four sides read the aperture vectors 1.9 times
-// over and were slower (the frame 212 us).  Stamps inside a frame: 5.3 us for the bands, 4.8
-// for the coarse levels.
+// over and were slower (the frame 212 us).  Stamps inside a frame: 6.5 us for the bands and 5
+// for the coarse levels, with the CG update in both (5.3, 4.8 and 2.5 as a kernel of its own).
 // ---------------------------------------------------------------------------
 constexpr int TF_BAND = 8;       // rows of a band
 constexpr int TF_ONE = 32;       // a layer of this side or less is one band
@@ -1147,8 +1151,7 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
 // Gamma_g, C_hat_g^-1 (Eq. 2, Sec. 3.2), Gamma_g^T and the column half of P_g^T.  SRC_PHI:
 // slopes of the projected layers (the M-apply); SRC_RESID: measured minus modelled slopes
 // (the initial residual); SRC_SLOPES: measured slopes (the right-hand side); SRC_RAW: the same
-// without C_hat_g^-1 (the model's adjoint).  The layers are
-// read by direct bilinear gathers; the result goes out per layer as the aperture rows'
+// without C_hat_g^-1 (the model's adjoint).  The layers are read by direct bilinear gathers; the result goes out per layer as the aperture rows'
 // values on the layer's columns (pb.Y, slot g * n_layers + l, rows of box[3] columns), whose
 // row half the band kernel applies.
 //
@@ -1156,6 +1159,12 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
 // (the tip/tilt means of a laser star, the block sums of a coarse sensor, the elongation's
 // sums) are linear functionals of the layers, whose shares the inverse kernel's tiles have
 // formed; the slopes of the row below the band are formed here once more.
+//
+// Bound: latency (launch, the gather's L2 reads, two barriers): 6 us a launch on the MAORY
+// geometry, 180 CTAs.  With the sums inside clusters of 16 CTAs it took 8.5 us, 3 of them
+// before the clusters started: a cluster waits for a group of SMs to be free, so nothing of
+// its prologue hides behind the kernel before.  Bands of 4 rows instead of 5 keep a CTA at
+// 512 threads of 64 registers, which fit beside the neighbours'; 576 of 56 did not.
 // ---------------------------------------------------------------------------
 constexpr int TS_ROWS = 4;       // 6 node rows of 81 nodes are one pass of 512 threads
 constexpr int TS_LG = 5;         // layers with their loads in flight together
