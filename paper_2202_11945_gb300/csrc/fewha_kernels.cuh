@@ -207,17 +207,23 @@ __device__ __forceinline__ double warp_total(const double* p, int cnt, const Dot
     return double(s.s) + double(s.c);
 }
 
+// a b + c d with its roundings spelt out: fma(a, b, c d).  Left to the compiler either product
+// may be the fused one, and a body compiled into two kernels (the frame of one instance, the
+// batched frame) need not get the same choice in both: the commands would differ by a rounding.
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
+__device__ __forceinline__ double dot2(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
+
 // LGS spot elongation of subaperture (i, j) (Eq. 3): beta and gamma, so that
 // C_ij^-1 = sigma^-2 (I - gamma beta beta^T) (Sherman-Morrison).
 __device__ __forceinline__ void elong(const WfsInfo& W, int i, int j, double& b1, double& b2, double& gam) {
     b1 = W.el_k * ((W.el_x0 + j * W.el_d) - W.el_lx);
     b2 = W.el_k * ((W.el_x0 + i * W.el_d) - W.el_ly);
-    gam = W.el_c / (1.0 + W.el_c * (b1 * b1 + b2 * b2));
+    gam = W.el_c / (1.0 + W.el_c * dot2(b1, b1, b2, b2));
 }
 __device__ __forceinline__ void elong(const WfsInfo& W, int i, int j, float& b1, float& b2, float& gam) {
     b1 = W.el_f[0] * ((W.el_f[4] + float(j) * W.el_f[5]) - W.el_f[2]);
     b2 = W.el_f[0] * ((W.el_f[4] + float(i) * W.el_f[5]) - W.el_f[3]);
-    gam = W.el_f[1] / (1.f + W.el_f[1] * (b1 * b1 + b2 * b2));
+    gam = W.el_f[1] / (1.f + W.el_f[1] * dot2(b1, b1, b2, b2));
 }
 // K11, K12, K22 (q = 0, 1, 2) of the sensor in the kernel's precision.
 __device__ __forceinline__ double el_K(const WfsInfo& W, int q, double) {
@@ -1288,8 +1294,8 @@ __device__ __forceinline__ void fit_body(const Desc<T>& d, const T* __restrict__
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (w[u] != T(0))
-                acc += w[u] * ((T(1) - fy[u]) * ((T(1) - fx[u]) * v[u][0] + fx[u] * v[u][1]) +
-                               fy[u] * ((T(1) - fx[u]) * v[u][2] + fx[u] * v[u][3]));
+                acc += w[u] * dot2(T(1) - fy[u], dot2(T(1) - fx[u], v[u][0], fx[u], v[u][1]), fy[u],
+                                   dot2(T(1) - fx[u], v[u][2], fx[u], v[u][3]));
     }
     if (cpist) {
         // phi without the full layers' pistons (the carried layers): a unit piston coefficient
@@ -1307,7 +1313,7 @@ __device__ __forceinline__ void fit_body(const Desc<T>& d, const T* __restrict__
         a_prev[idx] = a;
         out[idx] = a;
     } else if (apply_gain) {
-        const T a = (T(1) - d.gain) * a_prev[idx] + d.gain * acc;
+        const T a = dot2(T(1) - d.gain, a_prev[idx], d.gain, acc);
         a_prev[idx] = a;
         out[idx] = a;
     } else {

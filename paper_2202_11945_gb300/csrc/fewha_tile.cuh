@@ -115,8 +115,8 @@ __device__ __forceinline__ int tdiv(int t, int magic) { return (t * magic) >> 16
 // scaling (a) and wavelet (d) half.
 template <class T>
 __device__ __forceinline__ void synth_pair(T a0, T a1, T a2, T d0, T d1, T d2, T& e, T& o) {
-    e = tap_h<T>(0) * a0 + tap_h<T>(2) * a1 + tap_h<T>(4) * a2 + tap_g<T>(0) * d0 + tap_g<T>(2) * d1 + tap_g<T>(4) * d2;
-    o = tap_h<T>(1) * a0 + tap_h<T>(3) * a1 + tap_h<T>(5) * a2 + tap_g<T>(1) * d0 + tap_g<T>(3) * d1 + tap_g<T>(5) * d2;
+    e = dot2(tap_h<T>(0), a0, tap_h<T>(2), a1) + tap_h<T>(4) * a2 + tap_g<T>(0) * d0 + tap_g<T>(2) * d1 + tap_g<T>(4) * d2;
+    o = dot2(tap_h<T>(1), a0, tap_h<T>(3), a1) + tap_h<T>(5) * a2 + tap_g<T>(1) * d0 + tap_g<T>(3) * d1 + tap_g<T>(5) * d2;
 }
 
 // Quotient of two inner products as an operand of the vector updates, rounded to T: double
@@ -158,7 +158,7 @@ __device__ __forceinline__ void measured_sums(const Desc<T>& d, const T* s, doub
             if (el) {
                 T b1, b2, gam;
                 elong(W, k / N, k % N, b1, b2, gam);
-                const T bs = b1 * sx + b2 * sy;
+                const T bs = dot2(b1, sx, b2, sy);
                 sum[2].add(gam * b1, bs);
                 sum[3].add(gam * b2, bs);
             }
@@ -444,7 +444,7 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
             if (t < np2 && i0 + i < nd) {
                 const int k = foff[2 * d.n_fun + 1] + (i0 + i) * np2 + t;
                 const V2 e = k < d.fcap ? fent[k] : gent[f0 + k];
-                x[i] = e.x * v.x + e.y * v.y;
+                x[i] = dot2(e.x, v.x, e.y, v.y);
             }
         }
         // after the step at width w a lane holds w of the sums, over 32 w / TINV_DN lanes; the
@@ -1281,8 +1281,8 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
                 for (int e = 0; e < TS_LG; ++e)
                     if (l0 + e < nl) {
                         const T fx = xf[(l0 + e) * NPs + b], fy = yf[(l0 + e) * (SR + 2) + ia];
-                        const T h0 = (T(1) - fx) * q[e][0] + fx * q[e][1], h1 = (T(1) - fx) * q[e][2] + fx * q[e][3];
-                        v += (T(1) - fy) * h0 + fy * h1;
+                        const T h0 = dot2(T(1) - fx, q[e][0], fx, q[e][1]), h1 = dot2(T(1) - fx, q[e][2], fx, q[e][3]);
+                        v += dot2(T(1) - fy, h0, fy, h1);
                     }
             }
             Vb[k] = v;
@@ -1327,8 +1327,8 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
         mx = tot[0] / T(W.n_active);
         my = tot[1] / T(W.n_active);
         if (W.el) {
-            g1 = (tot[2] - (el_K(W, 0, T()) * mx + el_K(W, 1, T()) * my)) / T(W.n_active);
-            g2 = (tot[3] - (el_K(W, 1, T()) * mx + el_K(W, 2, T()) * my)) / T(W.n_active);
+            g1 = (tot[2] - dot2(el_K(W, 0, T()), mx, el_K(W, 1, T()), my)) / T(W.n_active);
+            g2 = (tot[3] - dot2(el_K(W, 1, T()), mx, el_K(W, 2, T()), my)) / T(W.n_active);
         }
     }
     for (int k = t; k < nrow * N; k += NT) {
@@ -1362,7 +1362,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
                     if (W.el) {
                         T b1, b2, gam;
                         elong(W, q0 + ii, j, b1, b2, gam);
-                        const T bu = b1 * ux + b2 * uy;
+                        const T bu = dot2(b1, ux, b2, uy);
                         ux = (ux - gam * b1 * bu) + g1;
                         uy = (uy - gam * b2 * bu) + g2;
                     }
