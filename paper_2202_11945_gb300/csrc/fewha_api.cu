@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <algorithm>
@@ -3402,8 +3403,14 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
             return enqueue_rhs<T>(H, d, x, y, st);
         case 2:  // dwt
             return launch_layer<T, LSRC_PHI, LDST_COEF, false>(H, d, layer_args<T>(H, x, y), st);
-        case 3:  // idwt
+        case 3: {  // idwt
+            // the tiles read coefficients all over a layer while others store: where the output
+            // overlaps the input, a CTA per layer that has read it all before it writes
+            const std::uintptr_t a = reinterpret_cast<std::uintptr_t>(in), b = reinterpret_cast<std::uintptr_t>(out);
+            if ((a < b ? b - a : a - b) < static_cast<size_t>(d.n_c) * sizeof(T))
+                return launch_layer<T, LSRC_COEF, LDST_PHI, false>(H, d, layer_args<T>(H, x, y), st);
             return enqueue_layers<T>(H, d, x, y, st);
+        }
         case 4:  // project
             return launch_sensor<T, SSRC_PHI, false, SDST_NODES>(H, d, x, y, st);
         case 5:  // project adjoint
