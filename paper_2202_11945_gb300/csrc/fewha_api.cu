@@ -154,15 +154,19 @@ struct fewha_handle {
     void *txf = nullptr, *tyf = nullptr;
     int tnp = 0, tcols = 0;
     int n_su = 0, su0[MAXG + 1] = {};
-    // functionals of the layers (Desc::foff, fent), the tiles' shares, the measured sums
-    int* foff = nullptr;
-    void* fent = nullptr;
+    // functionals of the layers (Desc::foff, fent) without and with spot elongation, the one in
+    // use, the tiles' shares, the measured sums
+    struct FunTab {
+        int* foff = nullptr;
+        void* fent = nullptr;
+        int n_fun = 0, fcap = 0, f0[MAXG + 1] = {};
+        size_t n_ent = 0, smem = 0;   // elements of fent; shared memory of the inverse tile kernel
+        double eta = 0.0;             // elongation parameter of its entries
+    } fun[2];
+    int fun_at = 0;
     double *fsh = nullptr, *msum = nullptr;
-    int n_fun = 0, fcap = 0, n_writers = 0, n_coarse = 0;
+    int n_writers = 0, n_coarse = 0;
     double *lshz = nullptr, *lshq = nullptr;   // the layers' shares of r.z and p.q, per slot
-    int f0[MAXG + 1] = {};
-    size_t foff_cap = 0, fent_cap = 0, fsh_cap = 0;
-    double fun_eta = -1.0;            // elongation parameter they were built for
     size_t lay_inv_elems = 0;         // the inverse tile kernel's windows, in elements
     double *tshare = nullptr, *pqs = nullptr;
     void* alphas = nullptr;
@@ -171,7 +175,8 @@ struct fewha_handle {
     TfLayout lay_tf{};
     TcLayout lay_tc{};
     TsLayout lay_ts{};
-    size_t smem_tinv = 0, smem_tf = 0, smem_tc = 0, smem_ts = 0;
+    size_t smem_tf = 0, smem_tc = 0, smem_ts = 0;
+    size_t smem_tinv() const { return fun[fun_at].smem; }
     std::vector<int> box_host;
     void* pairV = nullptr;
     void* pairY = nullptr;
@@ -352,13 +357,14 @@ Desc<T> make_desc(const fewha_handle* H) {
     d.tnp = H->tnp;
     d.tcols = H->tcols;
     std::copy(std::begin(H->su0), std::end(H->su0), d.su0);
-    std::copy(std::begin(H->f0), std::end(H->f0), d.f0);
-    d.foff = H->foff;
-    d.fent = static_cast<const T*>(H->fent);
+    const auto& fun = H->fun[H->fun_at];
+    std::copy(std::begin(fun.f0), std::end(fun.f0), d.f0);
+    d.foff = fun.foff;
+    d.fent = static_cast<const T*>(fun.fent);
     d.n_tu = H->n_tu;
-    d.n_fun = H->n_fun;
-    d.fpad = round4(3 * H->n_fun + 3);
-    d.fcap = H->fcap;
+    d.n_fun = fun.n_fun;
+    d.fpad = round4(3 * fun.n_fun + 3);
+    d.fcap = fun.fcap;
     d.n_writers = H->n_writers;
     d.tslot_ld = H->tslot_ld;
     d.n_tcl = H->n_tcl;
@@ -540,7 +546,7 @@ int launch_inv(fewha_handle* H, const Desc<T>& d, const ClArgs<T>& a, cudaStream
     }
     // with a.ms, a CTA per sensor behind the tiles sums the measured slopes
     const int units = H->n_tu + (a.ms ? d.n_wfs : 0);
-    CK(launch_k(H, k_tinv<T, PUPD>, dim3(units), dim3(TINV_NT), H->smem_tinv, st, d, a), "k_tinv launch");
+    CK(launch_k(H, k_tinv<T, PUPD>, dim3(units), dim3(TINV_NT), H->smem_tinv(), st, d, a), "k_tinv launch");
     return FEWHA_OK;
 }
 
@@ -1291,6 +1297,7 @@ int set_smem_limits(fewha_handle* H) {
         H->smem_sen > static_cast<size_t>(maxsm))
         return fail(H, FEWHA_ERR_LIMIT, "cluster shared-memory tile above 227 KB");
     int rc = 0;
+    const size_t smem_tinv = std::max(H->fun[0].smem, H->fun[1].smem);
     if ((rc = allow_smem(H, k_tfwd<T, LDST_APPLY>, H->smem_tf)) || (rc = allow_smem(H, k_tfwd<T, LDST_COEF>, H->smem_tf)) ||
         (rc = allow_smem(H, k_tfwd<T, LDST_APPLY_INIT>, H->smem_tf)) ||
         (rc = allow_smem(H, k_tfwd<T, LDST_RESID_INIT>, H->smem_tf)) ||
@@ -1299,9 +1306,8 @@ int set_smem_limits(fewha_handle* H) {
         (rc = allow_smem(H, k_tcoarse<T, LDST_COEF>, H->smem_tc)) ||
         (rc = allow_smem(H, k_tcoarse<T, LDST_APPLY_INIT>, H->smem_tc)) ||
         (rc = allow_smem(H, k_tcoarse<T, LDST_RESID_INIT>, H->smem_tc)) ||
-        (rc = allow_smem(H, k_tinv<T, 0>, H->smem_tinv)) ||
-        (rc = allow_smem(H, k_tinv<T, 1>, H->smem_tinv)) ||
-        (rc = allow_smem(H, k_tinv<T, 2>, H->smem_tinv)) ||
+        (rc = allow_smem(H, k_tinv<T, 0>, smem_tinv)) || (rc = allow_smem(H, k_tinv<T, 1>, smem_tinv)) ||
+        (rc = allow_smem(H, k_tinv<T, 2>, smem_tinv)) ||
         (rc = allow_smem(H, k_tsen<T, SSRC_PHI>, H->smem_ts)) || (rc = allow_smem(H, k_tsen<T, SSRC_SLOPES>, H->smem_ts)) ||
         (rc = allow_smem(H, k_tsen<T, SSRC_RESID>, H->smem_ts)) || (rc = allow_smem(H, k_tsen<T, SSRC_RAW>, H->smem_ts)) ||
         (rc = allow_smem(H, k_tfwd<T, LDST_PHI>, H->smem_tf)) || (rc = allow_smem(H, k_model_slopes<T>, model_smem<T>(H))))
@@ -1625,35 +1631,48 @@ int tile_tables(fewha_handle* H) {
     return FEWHA_OK;
 }
 
-// The functionals of the layers that the sensors' weighting needs (Desc::foff): node fields
-// Gamma^T of the summed slopes' weights, through P^T to the layers (both exact transposes of
-// what the sensor kernel applies), cut into the tiles.  Rebuilt when the elongation changes.
+// Host form of one table of functionals: the node fields Gamma^T of the summed slopes' weights,
+// through P^T to the layers (both exact transposes of what the sensor kernel applies), cut into
+// the tiles.  The constants of the elongation are those in H->setup.G.
 template <class T>
-int functional_tables(fewha_handle* H) {
+struct FunHost {
+    int n_fun = 0, most = 0, f0[MAXG + 1] = {};
+    std::vector<int> off;
+    std::vector<T> flat;
+};
+
+template <class T>
+FunHost<T> functional_lists(const fewha_handle* H) {
     const HostSetup& s = H->setup;
-    if (H->fun_eta == H->params.alpha_eta) return FEWHA_OK;
+    FunHost<T> out;
     const int nl = static_cast<int>(s.L.size()), ng = static_cast<int>(s.G.size());
     int nf = 0;
     for (int g = 0; g < ng; ++g) {
-        H->f0[g] = nf;
+        out.f0[g] = nf;
         nf += s.G[g].lgs ? (s.G[g].el ? 4 : 2) : s.G[g].nb > 1 ? 2 * s.G[g].n_sub * s.G[g].n_sub : 0;
     }
-    for (int g = ng; g <= MAXG; ++g) H->f0[g] = nf;
+    for (int g = ng; g <= MAXG; ++g) out.f0[g] = nf;
+    out.n_fun = nf;
     std::vector<std::vector<std::pair<int, double>>> ent(static_cast<size_t>(H->n_tu) * std::max(nf, 1));
     std::vector<double> v, dense(static_cast<size_t>(MAXN) * MAXN, 0.0);
-    std::vector<int> nodes, hit;
+    std::vector<char> seen(static_cast<size_t>(MAXN) * MAXN, 0), touched;
+    std::vector<int> hit;
     for (int g = 0; g < ng; ++g) {
         const WfsInfo& W = s.G[g];
         const int N = W.N, NP = N + 1;
-        for (int f = H->f0[g]; f < H->f0[g + 1]; ++f) {
-            const int e = f - H->f0[g];
+        for (int f = out.f0[g]; f < out.f0[g + 1]; ++f) {
+            const int e = f - out.f0[g];
+            // the elongation's entries are kept by their place, zero or not: whatever the
+            // parameter's value, its table has the same places and the same size
+            const bool el = W.lgs && e >= 2;
             // node field of sum over the active subapertures of ax s^x + ay s^y
             v.assign(static_cast<size_t>(NP) * NP, 0.0);
+            touched.assign(static_cast<size_t>(NP) * NP, 0);
             for (int i = 0; i < N; ++i)
                 for (int j = 0; j < N; ++j) {
                     if (s.sidx[W.mask_off + i * N + j] < 0) continue;
                     double ax = e == 0 ? 1.0 : 0.0, ay = e == 1 ? 1.0 : 0.0;
-                    if (W.lgs && e >= 2) {
+                    if (el) {
                         const double b1 = W.el_k * ((W.el_x0 + j * W.el_d) - W.el_lx);
                         const double b2 = W.el_k * ((W.el_x0 + i * W.el_d) - W.el_ly);
                         const double gam = W.el_c / (1.0 + W.el_c * (b1 * b1 + b2 * b2)), b = e == 2 ? b1 : b2;
@@ -1664,102 +1683,127 @@ int functional_tables(fewha_handle* H) {
                         ax = in && !(e & 1) ? 1.0 : 0.0;
                         ay = in && (e & 1) ? 1.0 : 0.0;
                     }
-                    double* p = &v[static_cast<size_t>(i) * NP + j];
+                    const size_t at = static_cast<size_t>(i) * NP + j;
+                    double* p = &v[at];
                     p[0] += -0.5 * ax - 0.5 * ay;
                     p[1] += 0.5 * ax - 0.5 * ay;
                     p[NP] += -0.5 * ax + 0.5 * ay;
                     p[NP + 1] += 0.5 * ax + 0.5 * ay;
+                    touched[at] = touched[at + 1] = touched[at + NP] = touched[at + NP + 1] = 1;
                 }
-            nodes.clear();
-            for (int k = 0; k < NP * NP; ++k)
-                if (v[k] != 0.0) nodes.push_back(k);
             for (int l = 0; l < nl; ++l) {
                 const int tp = (g * MAXL + l) * TAB, n = s.L[l].n;
                 hit.clear();
-                for (int k : nodes) {
+                for (int k = 0; k < NP * NP; ++k) {
+                    if (!touched[k] || (!el && v[k] == 0.0)) continue;
                     const int a = k / NP, b = k % NP, y = s.pi0y[tp + a], x = s.pi0x[tp + b];
                     const double fy = s.pfy[tp + a], fx = s.pfx[tp + b];
                     for (int c = 0; c < 4; ++c) {
                         const int at = (y + (c >> 1)) * n + x + (c & 1);
-                        const double w = (c >> 1 ? fy : 1.0 - fy) * (c & 1 ? fx : 1.0 - fx) * v[k];
+                        const double w = (c >> 1 ? fy : 1.0 - fy) * (c & 1 ? fx : 1.0 - fx);
                         if (w == 0.0) continue;
-                        if (dense[at] == 0.0) hit.push_back(at);
-                        dense[at] += w;
+                        if (!seen[at]) hit.push_back(at);
+                        seen[at] = 1;
+                        dense[at] += w * v[k];
                     }
                 }
                 std::sort(hit.begin(), hit.end());
                 const TileLayer& t = H->tl_host[l];
                 const int ts = t.w[0];
                 for (int at : hit) {
-                    if (dense[at] == 0.0) continue;          // (listed twice, or cancelled)
+                    const double w = dense[at];
+                    dense[at] = 0.0;
+                    seen[at] = 0;
+                    if (w == 0.0 && !el) continue;           // (cancelled)
                     const int y = at / n, x = at % n;
                     const int u = H->tu0[l] + (y >> t.lts) * t.side + (x >> t.lts);
-                    ent[static_cast<size_t>(u) * nf + f].emplace_back((y & (ts - 1)) * ts + (x & (ts - 1)), dense[at]);
-                    dense[at] = 0.0;
+                    ent[static_cast<size_t>(u) * nf + f].emplace_back((y & (ts - 1)) * ts + (x & (ts - 1)), w);
                 }
             }
         }
     }
-    std::vector<int> off;
-    std::vector<T> flat;
-    int most = 0;
     const int pad = round4(3 * nf + 3);
     for (int u = 0; u < H->n_tu; ++u) {
-        const int at = static_cast<int>(flat.size() / 2);
+        const int at = static_cast<int>(out.flat.size() / 2);
         int l = 0, nd = 0;
         while (u >= H->tu0[l + 1]) ++l;
         const int nodes2 = H->tl_host[l].w[0] * H->tl_host[l].w[0];
         std::vector<int> o(pad, 0);
         for (int f = 0; f < nf; ++f) {
             const auto& list = ent[static_cast<size_t>(u) * nf + f];
-            o[2 * f] = o[2 * f + 1] = static_cast<int>(flat.size() / 2) - at;
+            o[2 * f] = o[2 * f + 1] = static_cast<int>(out.flat.size() / 2) - at;
             if (list.size() > TINV_FEW) {
                 o[2 * f + 1] = o[2 * f] - 1;                 // (among the functionals of many)
                 o[2 * nf + 3 + nd++] = f;
                 continue;
             }
             for (const auto& e : list) {
-                flat.push_back(static_cast<T>(e.first));
-                flat.push_back(static_cast<T>(e.second));
+                out.flat.push_back(static_cast<T>(e.first));
+                out.flat.push_back(static_cast<T>(e.second));
             }
-            o[2 * f + 1] = static_cast<int>(flat.size() / 2) - at;
+            o[2 * f + 1] = static_cast<int>(out.flat.size() / 2) - at;
         }
         o[2 * nf] = at;
-        o[2 * nf + 1] = static_cast<int>(flat.size() / 2) - at;
+        o[2 * nf + 1] = static_cast<int>(out.flat.size() / 2) - at;
         o[2 * nf + 2] = nd;
         for (int i = 0; i < nd; ++i) {
-            const size_t base = flat.size();
-            flat.resize(base + nodes2, T(0));
+            const size_t base = out.flat.size();
+            out.flat.resize(base + nodes2, T(0));
             for (const auto& e : ent[static_cast<size_t>(u) * nf + o[2 * nf + 3 + i]])
-                flat[base + e.first] = static_cast<T>(e.second);
+                out.flat[base + e.first] = static_cast<T>(e.second);
         }
-        most = std::max(most, static_cast<int>(flat.size() / 2) - at);
-        off.insert(off.end(), o.begin(), o.end());
+        out.most = std::max(out.most, static_cast<int>(out.flat.size() / 2) - at);
+        out.off.insert(out.off.end(), o.begin(), o.end());
     }
-    int rc;
-    auto grow = [&](void** p, size_t* cap, size_t need, bool typed) -> int {
-        if (*cap >= need) return FEWHA_OK;
-        int* ip = nullptr;
-        const int e = typed ? talloc(H, p, need) : dalloc(H, &ip, need);
-        if (e) return e;
-        if (!typed) *p = ip;
-        *cap = need;
-        return FEWHA_OK;
-    };
-    void* fo = H->foff;
-    if ((rc = grow(&fo, &H->foff_cap, off.size(), false))) return rc;
-    H->foff = static_cast<int*>(fo);
-    const size_t shares = static_cast<size_t>(std::max(nf, 1)) * H->n_tu;
-    if ((rc = grow(&H->fent, &H->fent_cap, flat.size() + 2, true))) return rc;
-    if (H->fsh_cap < shares && (rc = dalloc(H, &H->fsh, shares))) return rc;
-    H->fsh_cap = std::max(H->fsh_cap, shares);
-    if (!H->msum && (rc = dalloc(H, &H->msum, MAXG * TS_FUN))) return rc;
-    if ((rc = upload(H, H->foff, off)) || (rc = upload(H, static_cast<T*>(H->fent), flat))) return rc;
-    H->n_fun = nf;
-    // staged entries: all of them, as far as 112 KB go
-    H->fcap = std::min(round4(most), static_cast<int>(112 * 1024 / (2 * sizeof(T))));
-    H->smem_tinv = pad * sizeof(int) + (2 * static_cast<size_t>(H->fcap) + H->lay_inv_elems) * sizeof(T);
-    H->fun_eta = H->params.alpha_eta;
+    return out;
+}
+
+// The functionals of the layers that the sensors' weighting needs (Desc::foff), at creation:
+// one table for the plain noise model and, if a sensor can be elongated, one for the elongated
+// model, with the shares sized for both.  A change of the elongation parameter then allocates
+// nothing: it selects a table and, for another value, writes new weights into the same places.
+template <class T>
+int functional_alloc(fewha_handle* H) {
+    HostSetup& s = H->setup;
+    const std::vector<WfsInfo> keep = s.G;
+    int rc = FEWHA_OK, shares = 1;
+    for (int k = 0; k < 2 && !rc; ++k) {
+        auto& F = H->fun[k];
+        F.eta = k == 0 ? 0.0 : H->params.alpha_eta > 0.0 ? H->params.alpha_eta : 1.0;
+        set_elongation(s, F.eta);
+        if (k == 1 && std::none_of(s.G.begin(), s.G.end(), [](const WfsInfo& W) { return W.el != 0; })) break;
+        const FunHost<T> h = functional_lists<T>(H);
+        F.n_fun = h.n_fun;
+        std::copy(std::begin(h.f0), std::end(h.f0), F.f0);
+        F.n_ent = h.flat.size();
+        shares = std::max(shares, h.n_fun);
+        // staged entries: all of them, as far as 112 KB go
+        F.fcap = std::min(round4(h.most), static_cast<int>(112 * 1024 / (2 * sizeof(T))));
+        F.smem = round4(3 * h.n_fun + 3) * sizeof(int) + (2 * static_cast<size_t>(F.fcap) + H->lay_inv_elems) * sizeof(T);
+        if ((rc = dalloc(H, &F.foff, h.off.size())) || (rc = talloc(H, &F.fent, h.flat.size() + 2)) ||
+            (rc = upload(H, F.foff, h.off)) || (rc = upload(H, static_cast<T*>(F.fent), h.flat)))
+            break;
+    }
+    s.G = keep;
+    if (rc || (rc = dalloc(H, &H->fsh, static_cast<size_t>(shares) * H->n_tu)) || (rc = dalloc(H, &H->msum, MAXG * TS_FUN)))
+        return rc;
+    return FEWHA_OK;
+}
+
+// The table of the present parameters.
+template <class T>
+int functional_tables(fewha_handle* H) {
+    const bool el = std::any_of(H->setup.G.begin(), H->setup.G.end(), [](const WfsInfo& W) { return W.el != 0; });
+    auto& F = H->fun[el ? 1 : 0];
+    if (el && F.eta != H->params.alpha_eta) {
+        const FunHost<T> h = functional_lists<T>(H);
+        if (h.flat.size() != F.n_ent || h.n_fun != F.n_fun)
+            return fail(H, FEWHA_ERR_CUDA, "elongation table of another size");
+        int rc;
+        if ((rc = upload(H, F.foff, h.off)) || (rc = upload(H, static_cast<T*>(F.fent), h.flat))) return rc;
+        F.eta = H->params.alpha_eta;
+    }
+    H->fun_at = el ? 1 : 0;
     return FEWHA_OK;
 }
 
@@ -2089,7 +2133,7 @@ int typed_create(fewha_handle* H) {
     H->smem_layer = (2 * NWARP + 4) * sizeof(double) + static_cast<size_t>(s.max_n) * s.max_n * sizeof(T);
     H->smem_sensor = (2 * NWARP + 4 + 2 * MAXCOARSE) * sizeof(double) +
                      (static_cast<size_t>(s.max_N + 1) * (s.max_N + 1) + 2 * static_cast<size_t>(s.max_N) * s.max_N) * sizeof(T);
-    if ((rc = cluster_layouts<T>(H)) || (rc = tile_tables<T>(H)) || (rc = functional_tables<T>(H))) return rc;
+    if ((rc = cluster_layouts<T>(H)) || (rc = tile_tables<T>(H)) || (rc = functional_alloc<T>(H))) return rc;
     if ((rc = set_smem_limits<T>(H))) return rc;
     return setup_tables<T>(H);
 }
@@ -2904,7 +2948,7 @@ size_t barg_size(int kind) {
 
 size_t bsmem(const fewha_handle* H, int kind) {
     switch (kind) {
-        case BK_INV: case BK_INV_UPD: case BK_INV_MS: case BK_MSUM: return H->smem_tinv;
+        case BK_INV: case BK_INV_UPD: case BK_INV_MS: case BK_MSUM: return H->smem_tinv();
         case BK_FWD_UPD: case BK_FWD_COEF: case BK_FWD_RINIT: case BK_FWD_AINIT: return H->smem_tf;
         case BK_TC_AINIT: case BK_TC_UPD: case BK_TC_COEF: case BK_TC_RINIT: return H->smem_tc;
         case BK_SEN_PHI: case BK_SEN_SLOPES: case BK_SEN_RESID: return H->smem_ts;
