@@ -2453,34 +2453,6 @@ int reliable_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* 
     return FEWHA_OK;
 }
 
-// The converged solve of a single-precision handle on the twin's double vectors.  The float
-// recurrence needs 1.6 to 2.9 times the double one's iterations, by how its rounding falls
-// (8 m and 4 m geometries at 1e-11: 12.7k to 21k for forward and backward against 7.1k to
-// 10.8k), at 13 us an iteration against 43: forward and backward take 384 ms in float and 470
-// in double at 8 m, 299 to 375 against 354 to 408 on four smaller systems.  So that a small
-// instance does not run out of iterations where the rounding falls badly, the last quarter of
-// them is kept for the double recurrence, from where the float one got to.  Above
-// SOLVE_DOUBLE_NC coefficients, where a double iteration costs 4 times a float one in
-// arithmetic (49152 coefficients: 3.8), all of them are the float one's.
-constexpr int SOLVE_DOUBLE_NC = 4096;
-int mixed_solve(fewha_handle* H, fewha_handle* X, const double* b64, double* x64, bool warm, double tol,
-                int max_iters, cudaStream_t st, int* iters_out, double* rel_out) {
-    const int first = H->setup.n_c > SOLVE_DOUBLE_NC ? max_iters : max_iters - max_iters / 4;
-    int it = 0;
-    double rel = 0.0;
-    int rc = reliable_solve(H, X, b64, x64, warm, tol, first, st, &it, &rel);
-    if (!rc && it >= first && it < max_iters && rel > tol) {
-        int more = 0;
-        rc = solve_converged<double>(X, b64, x64, true, tol, max_iters - it, st, &more, &rel);
-        it += more;
-        if (rc) fail(H, rc, X->err);
-    }
-    H->have_prev = false;
-    if (iters_out) *iters_out = it;
-    if (rel_out) *rel_out = rel;
-    return rc;
-}
-
 template <class T>
 int reconstruct_converged(fewha_handle* H, const T* s, T* dm, double tol, int max_iters, int* iters,
                           double* rel, cudaStream_t st) {
@@ -2497,7 +2469,7 @@ int reconstruct_converged(fewha_handle* H, const T* s, T* dm, double tol, int ma
         k_convert<double, float><<<(d.n_s + 255) / 256, 256, 0, st>>>(d.n_s, s, s64);
         CK(cudaGetLastError(), "k_convert launch");
         if ((rc = enqueue_rhs<double>(X, dx, s64, static_cast<double*>(X->b), st))) return fail(H, rc, X->err);
-        if ((rc = mixed_solve(H, X, static_cast<const double*>(X->b), static_cast<double*>(X->cgrad),
+        if ((rc = reliable_solve(H, X, static_cast<const double*>(X->b), static_cast<double*>(X->cgrad),
                               X->have_cgrad, tol, max_iters, st, iters, rel)))
             return rc;
         X->have_cgrad = true;
@@ -2544,7 +2516,7 @@ int backward(fewha_handle* H, const T* g_a, T* g_s, double* g_alpha, double* g_w
         CK(cudaGetLastError(), "k_convert launch");
         if ((rc = enqueue_fit_adj<double>(X, dx, ga64, b64, st)))
             return fail(H, rc, X->err);
-        if ((rc = mixed_solve(H, X, b64, lam, X->have_lam, H->grad_tol, H->grad_max_iters, st, &it, &rel)))
+        if ((rc = reliable_solve(H, X, b64, lam, X->have_lam, H->grad_tol, H->grad_max_iters, st, &it, &rel)))
             return rc;
         X->have_lam = true;
         if (g_s) {
@@ -2607,7 +2579,7 @@ int solve_entry(fewha_handle* H, const T* b, T* x, double tol, int max_iters, cu
         double* x64 = static_cast<double*>(X->c_tmp);
         k_convert<double, float><<<(n + 255) / 256, 256, 0, st>>>(n, b, b64);
         CK(cudaGetLastError(), "k_convert launch");
-        if ((rc = mixed_solve(H, X, b64, x64, false, tol, max_iters, st, iters, rel))) return rc;
+        if ((rc = reliable_solve(H, X, b64, x64, false, tol, max_iters, st, iters, rel))) return rc;
         k_convert<float, double><<<(n + 255) / 256, 256, 0, st>>>(n, x64, x);
         CK(cudaGetLastError(), "k_convert launch");
         CK(cudaStreamSynchronize(st), "solve");
