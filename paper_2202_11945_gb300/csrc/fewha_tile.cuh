@@ -119,22 +119,6 @@ __device__ __forceinline__ void synth_pair(T a0, T a1, T a2, T d0, T d1, T d2, T
     o = dot2(tap_h<T>(1), a0, tap_h<T>(3), a1) + tap_h<T>(5) * a2 + tap_g<T>(1) * d0 + tap_g<T>(3) * d1 + tap_g<T>(5) * d2;
 }
 
-// Quotient of two inner products as an operand of the vector updates, rounded to T: double
-// totals, or double-float ones divided on the FP32 pipes (a double division is a chain of
-// ~10 instructions of ~64 cycles).  Zero if the divisor is zero.
-__device__ __forceinline__ double acc_ratio(double a, double b) { return b != 0.0 ? a / b : 0.0; }
-__device__ __forceinline__ float acc_ratio(DFloat a, DFloat b) {
-    if (b.s == 0.f) return 0.f;
-    const float q = __fdiv_rn(a.s, b.s);
-    const float rem = __fadd_rn(__fmaf_rn(-q, b.s, a.s), __fmaf_rn(-q, b.c, a.c));
-    return __fadd_rn(q, __fdiv_rn(rem, b.s));
-}
-__device__ __forceinline__ void acc_of(double x, double& a) { a = x; }
-__device__ __forceinline__ void acc_of(double x, DFloat& a) {
-    a.s = static_cast<float>(x);
-    a.c = static_cast<float>(x - static_cast<double>(a.s));
-}
-
 // Sums over one sensor's measured slopes, as its functionals sum the modelled ones: tip and
 // tilt of a laser star and, with spot elongation (Eq. 3), gamma beta (beta . s).  Compensated: the
 // residual's sums are the difference of these and the modelled ones.
@@ -244,8 +228,8 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
     // the unit's slots: place in the coefficient vector (its sign bit: this tile owns it) and
     // in shared memory
     const int cnt = d.tcnt[l];
-    A rz_old = AccOf<T>::zero();                          // rz of the iteration before: long written
-    if (PUPD && has_old && t == 0) acc_of(a.pcg.rztot[a.iter - 1], rz_old);
+    double rz_old = 0.0;                                  // rz of the iteration before: long written
+    if (PUPD && has_old && t == 0) rz_old = a.pcg.rztot[a.iter - 1];
     const int2* slots = reinterpret_cast<const int2*>(d.tslot + static_cast<size_t>(unit) * d.tslot_ld);
     for (int r0 = 0; r0 < cnt; r0 += NT * SL) {
         int dst[SL], pos[SL];
@@ -278,14 +262,14 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
             // beta and the mu_j while the loads are in flight; a deferred r.z total first
             // (warp 0, fixed order: the same value in every CTA)
             if (t < 32 && (PUPD || a.rz_cnt > 0)) {
-                A rz_new = AccOf<T>::zero();
+                double rz_new = 0.0;
                 if (a.rz_cnt > 0) {
-                    rz_new = shares_total<T>(a.rz_parts, a.rz_cnt);
-                    if (t == 0 && unit == 0) a.pcg.rztot[a.rz_slot] = warp_value(rz_new);
+                    rz_new = warp_value(shares_total<T>(a.rz_parts, a.rz_cnt));
+                    if (t == 0 && unit == 0) a.pcg.rztot[a.rz_slot] = rz_new;
                 } else if (has_old && t == 0) {
-                    acc_of(a.pcg.rztot[a.iter], rz_new);
+                    rz_new = a.pcg.rztot[a.iter];
                 }
-                if (PUPD && t == 0) sbeta = has_old ? acc_ratio(rz_new, rz_old) : T(0);
+                if (PUPD && t == 0) sbeta = T(has_old && rz_old != 0.0 ? rz_new / rz_old : 0.0);
             }
             if (PUPD == 2) {
                 if (a.aug_pcnt > 0) {
@@ -770,8 +754,8 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
             cph[k] = a.phic[L.off + t + k * NT];
             pph[k] = a.phip[L.off + t + k * NT];
         }
-    A rz = AccOf<T>::zero();
-    if (UPD && t == NT - 1) acc_of(a.pcg.rztot[a.iter], rz);
+    double rz = 0.0;
+    if (UPD && t == NT - 1) rz = a.pcg.rztot[a.iter];
     cp_async_wait();
     __syncthreads();
     pdl_wait();
@@ -814,12 +798,11 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
         __syncthreads();
         if (UPD && g0 == 0 && t == NT - 1) {
             // alpha = rz_k / (p . q)_k; zero if rz vanished (the iterate is final)
-            const A pq = acc_merge(spq[0], spq[1]);
-            const double pqv = warp_value(pq);
-            sstep = pqv > 0.0 && warp_value(rz) != 0.0 ? T(acc_ratio(rz, pq)) : T(0);
+            const double pq = warp_value(acc_merge(spq[0], spq[1]));
+            sstep = T(pq > 0.0 && rz != 0.0 ? rz / pq : 0.0);
             if (unit == 0) {
                 a.alphas[a.iter] = sstep;
-                a.pcg.pqtot[a.iter] = pqv;
+                a.pcg.pqtot[a.iter] = pq;
             }
         }
 #pragma unroll
