@@ -1519,7 +1519,7 @@ __global__ void __launch_bounds__(OP_NT) k_model_slopes(__grid_constant__ const 
 }
 
 // C_hat^-1 s of every sensor (blockIdx.y) from the sums of k_msum (Sec. 3.2, Eq. 3), as in
-// tsen_body.
+// tsen_body, but the means and e - K m, which cancels for an elongated star, in double.
 template <class T>
 __global__ void __launch_bounds__(OP_NT) k_weigh(__grid_constant__ const Desc<T> d, const T* s, const double* msum,
                                                  T* out, unsigned* status) {
@@ -1536,12 +1536,12 @@ __global__ void __launch_bounds__(OP_NT) k_weigh(__grid_constant__ const Desc<T>
     if (!(isfinite(ux) && isfinite(uy)) && status) atomicOr(status, 1u);
     if (W.lgs && W.nb == 1) {
         const A* m = reinterpret_cast<const A*>(msum + d.f0[g]);
-        const T mx = T(warp_value(m[0])) / T(W.n_active), my = T(warp_value(m[1])) / T(W.n_active);
+        const T mx = T(warp_value(m[0]) / W.n_active), my = T(warp_value(m[1]) / W.n_active);
         ux -= mx;
         uy -= my;
         if (W.el) {
-            const T g1 = (T(warp_value(m[2])) - (el_K(W, 0, T()) * mx + el_K(W, 1, T()) * my)) / T(W.n_active);
-            const T g2 = (T(warp_value(m[3])) - (el_K(W, 1, T()) * mx + el_K(W, 2, T()) * my)) / T(W.n_active);
+            const T g1 = T((warp_value(m[2]) - (W.el_K11 * double(mx) + W.el_K12 * double(my))) / W.n_active);
+            const T g2 = T((warp_value(m[3]) - (W.el_K12 * double(mx) + W.el_K22 * double(my))) / W.n_active);
             T b1, b2, gam;
             elong(W, k / W.N, k % W.N, b1, b2, gam);
             const T bu = b1 * ux + b2 * uy;
