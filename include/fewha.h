@@ -341,8 +341,9 @@ int fewha_get_diagonals(fewha_handle* h, void* d_D, void* d_J, void* stream);
  * the pupil nodes (piston is not fitted).  The normal equations
  * (sum_k w_k A_k^T Pi A_k + eps I) a = sum_k w_k A_k^T Pi L_k phi are solved by
  * (unpreconditioned) CG from a = 0 until the recurrence residual falls to tol times the
- * right-hand side's norm or max_iters iterations have run; the CG inner products and
- * scalars are double, the operators the handle's element type. */
+ * right-hand side's norm or max_iters iterations have run; the CG's inner products are
+ * formed to double accuracy, its scalars in double, the operators in the handle's element
+ * type. */
 #define FEWHA_MAX_FIT_DIRS 32
 #define FEWHA_MAX_FIT_NODES 256  /* largest n_fit                                      */
 typedef struct fewha_lsfit {
