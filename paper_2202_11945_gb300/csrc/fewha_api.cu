@@ -3455,9 +3455,20 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
 }
 
 // Back-to-back launches of one hot-path kernel on the internal buffers (timing only).
+// `reps` launches of one stage with the arguments it has in an iteration of the frame.
 template <class T>
 int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
     const Desc<T> d = make_desc<T>(H);
+    // The band kernel reads r and the layers of c ahead of its wait, which is right where a
+    // kernel stands between it and the one that wrote them.  Where no layer has coarse levels
+    // its repetitions follow one another: without dependent launch then.
+    const unsigned flags = H->params.flags;
+    struct Restore {
+        fewha_handle* H;
+        unsigned flags;
+        ~Restore() { H->params.flags = flags; }
+    } restore{H, flags};
+    if ((stage == FEWHA_STAGE_LAYER || stage == FEWHA_STAGE_PROJT) && H->n_coarse == 0) H->params.flags &= ~FEWHA_FLAG_PDL;
     T* p = static_cast<T*>(H->p);
     T* phi = static_cast<T*>(H->phi);
     int rc = 0;
@@ -3470,6 +3481,10 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
                 a.zupd = static_cast<const T*>(H->z);
                 a.iter = 1;
                 a.zero_piston = 1;
+                a.fsh = H->fsh;
+                a.rz_parts = rz_shares(H, 1);
+                a.rz_cnt = d.n_layers * TC_SH;
+                a.rz_slot = 1;
                 rc = launch_inv<T, 1>(H, d, a, st);
                 break;
             }
@@ -3477,7 +3492,7 @@ int bench_stage(fewha_handle* H, int stage, int reps, cudaStream_t st) {
             // update in these
             case FEWHA_STAGE_SENSOR:
             case FEWHA_STAGE_PROJ:
-                rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st);
+                rc = launch_csensor<T, SSRC_PHI>(H, d, phi, nullptr, st, static_cast<const T*>(p));
                 break;
             case FEWHA_STAGE_LAYER:
             case FEWHA_STAGE_PROJT: {
