@@ -492,8 +492,9 @@ int fewha_batch_reconstruct(fewha_batch* b, const void* const* d_slopes, void* c
                             void* stream);
 
 /* Autotuner: times the candidate configurations on `reps` batched frames of the given
- * slopes (CUDA events on `stream`): first every order x groups x vec_passes with the default
- * kernel shapes, then, from the best of those, every vec_threads, and keeps the fastest
+ * slopes (CUDA events on `stream`): every order x groups and, for the warm recurrence, whose
+ * frames start with the vector kernel, x vec_passes and then, from the best of those, every
+ * vec_threads (the explicit frame has no vector kernel: 1 and 0), and keeps the fastest
  * in the batch and in a process-wide table keyed by the instances' shapes (a later batch
  * of the same shapes starts from it), and restores every member's warm state afterwards.
  * *best_us (nullable) receives the chosen configuration's mean frame time.  Synchronous. */

@@ -3280,18 +3280,21 @@ int batch_autotune(fewha_batch* B, const void* const* s, void* const* dm, int re
             best = c;
         }
     };
+    // The vector kernel starts the frames of the warm recurrence; the explicit frame has none,
+    // and its shapes would be the same launches again, chosen between by noise.
+    const bool vec = (B->h[0]->params.flags & FEWHA_FLAG_WARM_RESIDUAL) != 0;
     // stage 1: work order, launch chains and vector passes with the default kernel shapes
     const int groups[] = {1, 2, 4, 8};
     const int vps[] = {1, 4};
     for (int order = 0; order < 2 && rc == FEWHA_OK; ++order)
         for (int gi = 0; gi < 4 && rc == FEWHA_OK; ++gi) {
             if (groups[gi] > static_cast<int>(n)) continue;
-            for (int vi = 0; vi < 2 && rc == FEWHA_OK; ++vi) trial(fewha_batch_config{order, groups[gi], vps[vi], 0, 0, 0});
+            for (int vi = 0; vi < (vec ? 2 : 1) && rc == FEWHA_OK; ++vi) trial(fewha_batch_config{order, groups[gi], vps[vi], 0, 0, 0});
         }
     // stage 2: from the best of stage 1, the vector kernel's launch shape
     const fewha_batch_config base = best;
     for (int vt : {PBLK, 2 * PBLK}) {
-        if (rc != FEWHA_OK) continue;
+        if (rc != FEWHA_OK || !vec) continue;
         fewha_batch_config c = base;
         c.vec_threads = vt;
         trial(c);
