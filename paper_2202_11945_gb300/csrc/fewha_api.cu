@@ -432,9 +432,9 @@ BStep<T>& record(int kind) {
 }
 
 // ---------------------------------------------------------------- launchers
-template <class T, int SRC, int DST, bool PUPD>
+template <class T, int SRC, int DST>
 int launch_layer(fewha_handle* H, const Desc<T>& d, const LayerArgs<T>& a, cudaStream_t st) {
-    k_layer<T, SRC, DST, PUPD><<<d.n_layers, BLK, H->smem_layer, st>>>(d, a);
+    k_layer<T, SRC, DST><<<d.n_layers, BLK, H->smem_layer, st>>>(d, a);
     CK(cudaGetLastError(), "k_layer launch");
     return FEWHA_OK;
 }
@@ -474,8 +474,6 @@ VecArgs<T> vec_args(fewha_handle* H, T* c, int iter) {
     v.pq_cnt = 0;
     v.pq_parts = nullptr;
     v.defer_rz = 0;
-    v.phic = nullptr;
-    v.phip = nullptr;
     return v;
 }
 
@@ -794,7 +792,8 @@ int vec_grid(const fewha_handle* H) { return H->npart; }
 template <class T, int PHASE>
 int launch_vec(fewha_handle* H, int n, const VecArgs<T>& v, cudaStream_t st) {
     if (recorder<T>()) {
-        record<T>(PHASE == V_INIT ? BK_VEC_INIT : BK_VEC_WARM).va = v;
+        if (PHASE != V_INIT_WARM) return fail(H, FEWHA_ERR_INVALID_ARG, "step without a batched form");
+        record<T>(BK_VEC_WARM).va = v;
         return FEWHA_OK;
     }
     CK(launch_k(H, k_vec<T, PHASE>, dim3(vec_grid(H)), dim3(PBLK), 0, st, n, v), "k_vec launch");
@@ -1273,25 +1272,21 @@ int set_smem_limits(fewha_handle* H) {
     const int maxsm = 227 * 1024;
     if (H->smem_layer > static_cast<size_t>(maxsm) || H->smem_sensor > static_cast<size_t>(maxsm))
         return fail(H, FEWHA_ERR_LIMIT, "shared-memory tile above 227 KB");
-#define SETL(S, D, P) \
-    CK(cudaFuncSetAttribute(k_layer<T, S, D, P>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm), "smem attr")
-    SETL(LSRC_COEF, LDST_PHI, false);
-    SETL(LSRC_COEF, LDST_PHI, true);
-    SETL(LSRC_NODES, LDST_APPLY, false);
-    SETL(LSRC_NODES, LDST_COEF, false);
-    SETL(LSRC_NODES, LDST_PHI, false);
-    SETL(LSRC_PHI, LDST_COEF, false);
-    SETL(LSRC_DM, LDST_COEF, false);
+#define SETL(S, D) \
+    CK(cudaFuncSetAttribute(k_layer<T, S, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm), "smem attr")
+    SETL(LSRC_COEF, LDST_PHI);
+    SETL(LSRC_NODES, LDST_APPLY);
+    SETL(LSRC_NODES, LDST_PHI);
+    SETL(LSRC_PHI, LDST_COEF);
+    SETL(LSRC_DM, LDST_COEF);
 #undef SETL
 #define SETS(S, W, D) \
     CK(cudaFuncSetAttribute(k_sensor<T, S, W, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, maxsm), "smem attr")
     SETS(SSRC_PHI, true, SDST_ADJ);
-    SETS(SSRC_SLOPES, true, SDST_ADJ);
     SETS(SSRC_PHI, false, SDST_NODES);
     SETS(SSRC_NODES, false, SDST_SLOPES);
     SETS(SSRC_SLOPES, false, SDST_ADJ);
     SETS(SSRC_SLOPES, true, SDST_SLOPES);
-    SETS(SSRC_PHI, false, SDST_SLOPES);
 #undef SETS
     if (H->smem_fwd > static_cast<size_t>(maxsm) || H->smem_inv > static_cast<size_t>(maxsm) ||
         H->smem_sen > static_cast<size_t>(maxsm))
@@ -3093,15 +3088,7 @@ int batch_build(fewha_batch* B, const std::vector<Recorder<T>>& recs, const std:
             if (bkind_list(kind) != BL_VEC && smem[g * BK_COUNT + kind] > lim)
                 return bfail(B, FEWHA_ERR_LIMIT, "batched tile above the per-CTA shared-memory limit");
     }
-    // launch shapes: projection CTA size, adjoint-projection taps, vector CTA size
-    int kmax = 0;
-    for (int i = 0; i < n; ++i) kmax = std::max(kmax, B->h[i]->kmax);
-    const int pair_nt = cfg.pair_threads ? cfg.pair_threads : cblk<T>();
-    const int taps = cfg.proj_taps ? cfg.proj_taps : (kmax <= 4 ? 4 : KMAX);
     const int vec_nt = cfg.vec_threads ? cfg.vec_threads : PBLK;
-    if ((pair_nt != cblk<T>() && pair_nt != cblk<T>() / 2) || (taps != 4 && taps != KMAX) || taps < kmax ||
-        (vec_nt != PBLK && vec_nt != 2 * PBLK))
-        return bfail(B, FEWHA_ERR_INVALID_ARG, "launch shape not available for these instances");
     // capture
     BCK(cudaStreamBeginCapture(B->cap, cudaStreamCaptureModeThreadLocal), "batch capture");
     cudaError_t le = cudaSuccess;
@@ -3431,19 +3418,19 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
         case 1:  // rhs
             return enqueue_rhs<T>(H, d, x, y, st);
         case 2:  // dwt
-            return launch_layer<T, LSRC_PHI, LDST_COEF, false>(H, d, layer_args<T>(H, x, y), st);
+            return launch_layer<T, LSRC_PHI, LDST_COEF>(H, d, layer_args<T>(H, x, y), st);
         case 3: {  // idwt
             // the tiles read coefficients all over a layer while others store: where the output
             // overlaps the input, a CTA per layer that has read it all before it writes
             const std::uintptr_t a = reinterpret_cast<std::uintptr_t>(in), b = reinterpret_cast<std::uintptr_t>(out);
             if ((a < b ? b - a : a - b) < static_cast<size_t>(d.n_c) * sizeof(T))
-                return launch_layer<T, LSRC_COEF, LDST_PHI, false>(H, d, layer_args<T>(H, x, y), st);
+                return launch_layer<T, LSRC_COEF, LDST_PHI>(H, d, layer_args<T>(H, x, y), st);
             return enqueue_layers<T>(H, d, x, y, st);
         }
         case 4:  // project
             return launch_sensor<T, SSRC_PHI, false, SDST_NODES>(H, d, x, y, st);
         case 5:  // project adjoint
-            return launch_layer<T, LSRC_NODES, LDST_PHI, false>(H, d, layer_args<T>(H, x, y), st);
+            return launch_layer<T, LSRC_NODES, LDST_PHI>(H, d, layer_args<T>(H, x, y), st);
         case 6:  // slopes
             return launch_sensor<T, SSRC_NODES, false, SDST_SLOPES>(H, d, x, y, st);
         case 7:  // slopes adjoint
@@ -3457,7 +3444,7 @@ int op_dispatch(fewha_handle* H, int op, const void* in, void* out, int iters, c
         case 11:  // fit
             return enqueue_fit<T>(H, d, x, y, false, st);
         case 12:  // fit adjoint
-            return launch_layer<T, LSRC_DM, LDST_COEF, false>(H, d, layer_args<T>(H, x, y), st);
+            return launch_layer<T, LSRC_DM, LDST_COEF>(H, d, layer_args<T>(H, x, y), st);
         case 13: {  // pcg on b = in, c = out (in/out)
             CK(cudaMemcpyAsync(H->b, x, d.n_c * sizeof(T), cudaMemcpyDeviceToDevice, st), "b copy");
             return enqueue_pcg<T>(H, d, y, iters, false, st);
@@ -3584,14 +3571,14 @@ int apply_M_noalloc(fewha_handle* H, const T* x, T* qout, cudaStream_t st) {
     // entry point, so these slots are write-only and need no clearing
     double* pq = reinterpret_cast<double*>(base + b_phi + b_u);
     const Desc<T> d = make_desc<T>(H);
-    if ((rc = launch_layer<T, LSRC_COEF, LDST_PHI, false>(H, d, layer_args<T>(H, x, phi), st))) return rc;
+    if ((rc = launch_layer<T, LSRC_COEF, LDST_PHI>(H, d, layer_args<T>(H, x, phi), st))) return rc;
     if ((rc = launch_sensor<T, SSRC_PHI, true, SDST_ADJ>(H, d, phi, u, st))) return rc;
     LayerArgs<T> a = layer_args<T>(H, u, qout);
     a.pin = x;
     a.iter = 0;
     a.zero_piston = 1;
     a.pcg.pqpart = pq;
-    return launch_layer<T, LSRC_NODES, LDST_APPLY, false>(H, d, a, st);
+    return launch_layer<T, LSRC_NODES, LDST_APPLY>(H, d, a, st);
 }
 
 }  // namespace

@@ -115,9 +115,6 @@ const void* kernel_of(int kind, int v) {
         case BK_FWD_AINIT: return reinterpret_cast<const void*>(kb_tfwd<T, LDST_APPLY_INIT>);
         case BK_TC_AINIT: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_APPLY_INIT>);
         case BK_TC_RINIT: return reinterpret_cast<const void*>(kb_tcoarse<T, LDST_RESID_INIT>);
-        case BK_VEC_INIT:
-            return half ? reinterpret_cast<const void*>(kb_vec<T, V_INIT, 2 * PBLK>)
-                        : reinterpret_cast<const void*>(kb_vec<T, V_INIT, PBLK>);
         case BK_VEC_WARM:
             return half ? reinterpret_cast<const void*>(kb_vec<T, V_INIT_WARM, 2 * PBLK>)
                         : reinterpret_cast<const void*>(kb_vec<T, V_INIT_WARM, PBLK>);
@@ -190,9 +187,6 @@ cudaError_t batch_launch(const BLaunch& L, cudaStream_t st) {
         case BK_SEN_PHI: return launch_b(L.pdl, kb_tsen<T, SSRC_PHI>, pg, sn, L.smem, st, I, sa, L.items);
         case BK_SEN_SLOPES: return launch_b(L.pdl, kb_tsen<T, SSRC_SLOPES>, pg, sn, L.smem, st, I, sa, L.items);
         case BK_SEN_RESID: return launch_b(L.pdl, kb_tsen<T, SSRC_RESID>, pg, sn, L.smem, st, I, sa, L.items);
-        case BK_VEC_INIT:
-            return v2 ? launch_b(L.pdl, kb_vec<T, V_INIT, 2 * PBLK>, pg, vt, 0, st, I, va, L.items)
-                      : launch_b(L.pdl, kb_vec<T, V_INIT, PBLK>, pg, vt, 0, st, I, va, L.items);
         case BK_VEC_WARM:
             return v2 ? launch_b(L.pdl, kb_vec<T, V_INIT_WARM, 2 * PBLK>, pg, vt, 0, st, I, va, L.items)
                       : launch_b(L.pdl, kb_vec<T, V_INIT_WARM, PBLK>, pg, vt, 0, st, I, va, L.items);

@@ -50,7 +50,6 @@ enum BKind {
     BK_SEN_SLOPES,     // C^-1, Gamma^T of measured slopes  (SensorArgs)
     BK_FWD_UPD,        // W sum P^T u and the CG update    (ClArgs)
     BK_FWD_COEF,       // b = W sum P^T u                   (ClArgs)
-    BK_VEC_INIT,       // r0 = b - q, z, p, r.z             (VecArgs)
     BK_VEC_WARM,       // r0 = (b - b_prev) + r_prev        (VecArgs)
     BK_FIT,            // DM fit and gain                   (FitArgs)
     BK_SEN_RESID,      // C^-1, Gamma^T of s - Gamma P phi  (SensorArgs)

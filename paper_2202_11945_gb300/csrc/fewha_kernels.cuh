@@ -473,16 +473,12 @@ __device__ __forceinline__ bool last_arrival(unsigned* count, unsigned ctas, boo
 // aperture-node vectors (SRC_NODES, P^T as a gather), or the adjoint DM fit
 // (SRC_DM).  Destination: layer values (DST_PHI), wavelet coefficients (DST_COEF),
 // or q = W y + alpha D p with the partial p.q (DST_APPLY).
-// PUPDATE: before use, the CG direction of this layer is advanced, p = z + beta p,
-// beta = rz_k / rz_(k-1) (Sec. 3.3; the update is fused into the first kernel of
-// iteration k).
 // ---------------------------------------------------------------------------
 enum { LSRC_PHI = 0, LSRC_NODES = 1, LSRC_DM = 2, LSRC_COEF = 3 };
-// LDST_APPLY_INIT: the forward cluster kernel's apply with the initial residual's vector
-// step fused into its epilogue
-// LDST_RESID_INIT: the same vector step with the data term already the residual's (the
-// sensor kernel's SSRC_RESID): r0 = W y - alpha D c0, with no b
-// LDST_UPDATE: the CG update c += a p, r -= a q, z = J^-1 r with r.z
+// of the forward band kernels beside these: LDST_APPLY_INIT, the apply with the initial
+// residual's vector step in its epilogue; LDST_RESID_INIT, the same vector step with the data term
+// already the residual's (the sensor kernel's SSRC_RESID), r0 = W y - alpha D c0, with no b;
+// LDST_UPDATE, the CG update c += a p, r -= a q, z = J^-1 r with r.z
 enum { LDST_PHI = 0, LDST_COEF = 1, LDST_APPLY = 2, LDST_APPLY_INIT = 3, LDST_RESID_INIT = 4, LDST_UPDATE = 5 };
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
@@ -496,14 +492,12 @@ struct LayerArgs {
     const T* in;      // source vector
     const T* pin;     // p of the apply (DST_APPLY)
     T* out;           // destination vector
-    T* pupd;          // p to advance (PUPDATE), updated in place
-    const T* zupd;    // z of the update
     PcgSlots pcg;
-    int iter;         // CG iteration of the apply / update
+    int iter;         // slot of the p.q partials
     int zero_piston;  // data term: the full-depth LL coefficient is exactly 0
 };
 
-template <class T, int SRC, int DST, bool PUPDATE>
+template <class T, int SRC, int DST>
 __global__ void __launch_bounds__(BLK) k_layer(const Desc<T> d, const LayerArgs<T> a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* red = reinterpret_cast<double*>(smem_raw);          // 2*NWARP + 4 doubles
@@ -512,16 +506,7 @@ __global__ void __launch_bounds__(BLK) k_layer(const Desc<T> d, const LayerArgs<
     const LayerInfo L = d.L[l];
     const int n = L.n, nn = n * n, off = L.off;
 
-    if (PUPDATE) {
-        const double rz_new = sum_partials(a.pcg.rzpart + a.iter * a.pcg.npart, a.pcg.npart, red);
-        const double rz_old = sum_partials(a.pcg.rzpart + (a.iter - 1) * a.pcg.npart, a.pcg.npart, red);
-        const T beta = rz_old != 0.0 ? T(rz_new / rz_old) : T(0);
-        for (int k = threadIdx.x; k < nn; k += BLK) {
-            const T p = a.zupd[off + k] + beta * a.pupd[off + k];
-            a.pupd[off + k] = p;
-            S[k] = p;
-        }
-    } else if (SRC == LSRC_PHI || SRC == LSRC_COEF) {
+    if (SRC == LSRC_PHI || SRC == LSRC_COEF) {
         for (int k = threadIdx.x; k < nn; k += BLK) S[k] = a.in[off + k];
     } else if (SRC == LSRC_NODES) {
         // y(i, j) = sum_g sum_a sum_b wy(a, i) wx(b, j) u_g(a, b): P_g^T as a gather over
@@ -582,7 +567,7 @@ __global__ void __launch_bounds__(BLK) k_layer(const Desc<T> d, const LayerArgs<
     __syncthreads();
 
     if (DST == LDST_PHI) {
-        if (SRC == LSRC_COEF || PUPDATE) dwt_inverse(S, L);
+        if (SRC == LSRC_COEF) dwt_inverse(S, L);
         for (int k = threadIdx.x; k < nn; k += BLK) a.out[off + k] = S[k];
         return;
     }
@@ -874,17 +859,12 @@ struct VecArgs {
     const T* Jinv;
     PcgSlots pcg;
     int iter;
-    // V_UPDATE with deferred totals: pq_cnt > 0, the p.q total of the iteration is formed
-    // here from the forward kernel's pq_cnt shares (fixed order) and stored by CTA 0;
+    // V_UPDATE_AUG with deferred totals: pq_cnt > 0, the p.q total of the iteration is formed
+    // there from the forward kernels' pq_cnt shares (fixed order) and stored by CTA 0;
     // defer_rz, the r.z shares are stored and their total is left to the next inverse kernel
     int pq_cnt;
     const double* pq_parts;
     int defer_rz;
-    // V_UPDATE with phic: phi_c += alpha phi_p, the layers of c carried through the
-    // iterations (phi_p = W^T p of the iteration's apply, piston left out like the data
-    // path), so that the fit needs no inverse transform of the final c
-    T* phic;
-    const T* phip;
 };
 
 enum { V_INIT = 0, V_INIT_WARM = 1, V_UPDATE = 2 };
@@ -906,19 +886,11 @@ __device__ __forceinline__ void vec_body(const int n, const VecArgs<T>& v, const
     // it without a wait of its own); the other phases were waited for by their caller.
     bool waited = PHASE != V_UPDATE;
     auto form_alpha = [&]() {
-        if (threadIdx.x >= 32) return;
         // alpha = rz_k / (p . q)_k; zero if rz vanished (the iterate is final).  Formed
         // once and broadcast (an FP64 division is ~10 instructions on GB300's slow FP64
-        // pipe), while the batch's vector loads are in flight; a deferred p.q total first
-        // (warp 0, fixed order: the same value in every CTA)
-        double pq = 0.0;
-        if (v.pq_cnt > 0) {
-            pq = warp_total(v.pq_parts, v.pq_cnt,
-                            static_cast<const DotAcc<T>*>(nullptr));
-            if (threadIdx.x == 0 && cta == 0) v.pcg.pqtot[iter] = pq;
-        }
+        // pipe), while the batch's vector loads are in flight
         if (threadIdx.x == 0) {
-            if (v.pq_cnt == 0) pq = v.pcg.pqtot[iter];
+            const double pq = v.pcg.pqtot[iter];
             const double rz = v.pcg.rztot[iter];
             salpha = T((rz != 0.0 && pq > 0.0) ? rz / pq : 0.0);
         }
@@ -926,8 +898,7 @@ __device__ __forceinline__ void vec_body(const int n, const VecArgs<T>& v, const
     DotAcc<T> dot;
     for (int base = cta * NTV * PVEC; base < n; base += nparts * NTV * PVEC) {
         // issue every load of the batch before the arithmetic
-        T b[PVEC], q[PVEC], r[PVEC], p[PVEC], c[PVEC], bp[PVEC], jv[PVEC], fc[PVEC], fp[PVEC];
-        const bool track = PHASE == V_UPDATE && v.phic != nullptr;
+        T b[PVEC], q[PVEC], r[PVEC], p[PVEC], c[PVEC], bp[PVEC], jv[PVEC];
 #pragma unroll
         for (int k = 0; k < PVEC; ++k) {
             const int i = base + k * NTV + threadIdx.x;
@@ -944,10 +915,6 @@ __device__ __forceinline__ void vec_body(const int n, const VecArgs<T>& v, const
                     c[k] = v.c[i];
                     p[k] = v.p[i];
                     r[k] = v.r[i];
-                    if (track) {
-                        fc[k] = v.phic[i];
-                        fp[k] = v.phip[i];
-                    }
                 }
             }
         }
@@ -982,7 +949,6 @@ __device__ __forceinline__ void vec_body(const int n, const VecArgs<T>& v, const
                     v.b_prev[i] = b[k];
                 } else {
                     v.c[i] = c[k] + ta * p[k];
-                    if (track) v.phic[i] = fc[k] + ta * fp[k];
                     rr = r[k] - ta * q[k];
                 }
                 v.r[i] = rr;
@@ -1002,7 +968,6 @@ __device__ __forceinline__ void vec_body(const int n, const VecArgs<T>& v, const
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int slot = (PHASE == V_UPDATE) ? iter + 1 : 0;
     cta_dot_store(dot, part, v.pcg.rzpart + slot * v.pcg.npart + cta);
-    if (PHASE == V_UPDATE && v.defer_rz) return;        // the next inverse kernel totals r.z
     if (last_arrival(v.pcg.count, nparts, &last) && w == 0) {
         const double tot = warp_total(v.pcg.rzpart + slot * v.pcg.npart, v.pcg.npart, &dot);
         if (lane == 0) {
@@ -1037,7 +1002,7 @@ enum {
     V_AUG_R0_RESID = 8,  // p_j.r0 of an r0 already formed (the slopes' residual chain)
     V_UPDATE_AUG = 7     // the CG update of V_UPDATE; keeps p.q; q_j.z for the next direction
                          // (the direction update p = z + beta p_old - P mu runs fused into the
-                         // inverse wavelet kernel, k_cl_inv with PUPD = 2)
+                         // inverse tile kernel, k_tinv with PUPD = 2)
 };
 
 template <class T>

@@ -886,7 +886,8 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
         __syncthreads();
     }
     DotAcc<T> dot;
-    for (int b = t; b < nblk; b += NT) {                  // one block per thread, but for wide layers in double
+    static_assert((TF_BAND / 2) * (MAXN / 2) <= NT && (TF_ONE / 2) * (TF_ONE / 2) <= NT, "a block per thread");
+    if (const int b = t; b < nblk) {
         const int msk = bands > 1 ? 15 : n - 1;           // a band holds its halo
         const int ky = 2 * (b >> lh), kx = b & (h - 1);
         T ra[6], rd[6];
