@@ -374,7 +374,7 @@ struct PairBufs {
 
 // ---------------------------------------------------------------------------
 // Forward layer kernel (cluster per layer).
-//   SRC_NODES: y = sum_g P_g^T u_g (Sec. 2, adjoint), then W y;  SRC_PHI: W phi.
+//   y = sum_g P_g^T u_g (Sec. 2, adjoint), then W y.
 //   DST_COEF:  write W y (b of Sec. 3.1 when u comes from the measured slopes);
 //   DST_APPLY: write q = W y + alpha D p and p.q (Eq. 6); the grid's last CTA forms
 //              the total p.q in a fixed order.
@@ -406,16 +406,14 @@ struct ClArgs {
     // here in the fixed order instead of read from aug_tot
     const double* aug_parts;
     int aug_pcnt;
-    // the initial residual's vector step fused into the forward kernel (DST_APPLY_INIT): the
-    // vectors r, z, p, b, b_prev, J^-1; r.z shares at rzp[l * CL + rank], total into rz slot
-    // rzslot
+    // the initial residual's vector step fused into the forward kernels (DST_APPLY_INIT): the
+    // vectors r, z, p, b, b_prev, J^-1; the r.z total into rz slot rzslot
     T* vr;
     T* vz;
     T* vp;
     const T* vb;
     T* vbprev;
     const T* vj;
-    double* rzp;
     int rzslot;
     // Deferred totals.  defer_total (forward kernel): the CTA shares of p.q (APPLY) or r.z
     // (APPLY_INIT) are stored and the total is left to the next kernel that needs it, so no
@@ -456,15 +454,15 @@ struct ClLayout {       // shared-memory offsets set by the host, in T units
     int umax;           // one staging buffer of the P^T pipeline
     int ystg;           // staged pair terms of the band (forward kernel), 0 = not staged
     int ydirect;        // the band's pair terms read straight from L2 in 16-byte groups
-    int lstage;         // the LL quadrant's epilogue operands, staged by the leader (3 x
-                        // (MAXN / 2)^2); 0 = the LL epilogue is shared out over the cluster
+    int lstage;         // the LL quadrant's p, staged by the leader ((MAXN / 2)^2); 0 = the LL
+                        // epilogue is shared out over the cluster
 };
 
 constexpr int KMAX = 8;      // aperture rows / columns touching one layer row / column
 
 // Body of the forward layer kernel for layer l; `ctas` = CTAs of the instance's grid
 // (the p.q total is formed by the last of them to arrive).
-template <class T, int SRC, int DST>
+template <class T, int DST>
 __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a, const ClLayout& lay,
                                             const PairBufs<T>& pb, const int l, const unsigned ctas) {
     constexpr int NT = cblk<T>();
@@ -505,39 +503,32 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
     if (threadIdx.x <= MAXLEV) sD[threadIdx.x] = d.Dlev[l][threadIdx.x];
     // the band-run table of the staged sum, loaded now so that its latency overlaps
     int4 ytv = make_int4(0, 0, 0, 0);
-    if (SRC == LSRC_NODES && (lay.ystg > 0 || lay.ydirect) && has_band && threadIdx.x < 2 * d.n_wfs)
+    if ((lay.ystg > 0 || lay.ydirect) && has_band && threadIdx.x < 2 * d.n_wfs)
         ytv = pb.ytab[(l * CL + r) * 2 * d.n_wfs + threadIdx.x];
     // this CTA's share of the LL quadrant's rows (coarse layers): [lr0, lr1), hb rows each.
     // A quadrant narrower than 32 stays with the leader: sharing it out costs a cluster
     // barrier, more than the leader's few positions take.
-    constexpr bool INIT = DST == LDST_APPLY_INIT || DST == LDST_RESID_INIT;   // fused r0 step
-    constexpr bool NEEDB = DST == LDST_APPLY_INIT;                              // b read
-    constexpr bool QAPPLY = DST == LDST_APPLY || INIT;                         // p read
+    constexpr bool QAPPLY = DST == LDST_APPLY;                         // p read
     constexpr int PL = ((MAXN / 2) * (MAXN / 2) / CL + NT - 1) / NT;   // LL-share positions per thread
-    // With lay.lstage (single precision), the leader stages the LL quadrant's operands in
-    // shared memory now and forms the whole LL epilogue itself after its coarse levels: no
+    // With lay.lstage (single precision), the leader stages the LL quadrant's p in shared
+    // memory now and forms the whole LL epilogue itself after its coarse levels: no
     // rows go back to the other ranks and no third cluster barrier is needed.
     const bool lstaged = lay.lstage > 0 && coarse;
     const bool ldist = !lstaged && h >= 32;
     const int hb = ldist ? h >> 3 : h;
     const int lr0 = coarse ? min(r * hb, h) : 0, lr1 = coarse ? min(lr0 + hb, h) : 0;
     const int lcnt = lstaged ? 0 : (lr1 - lr0) * h;     // LL positions prefetched to registers
-    T* lsp = sm + lay.lstage;                           // staged p, b, J^-1 of LL (stride h)
-    T* lsb = lsp + (MAXN / 2) * (MAXN / 2);
-    T* lsj = lsb + (MAXN / 2) * (MAXN / 2);
+    T* lsp = sm + lay.lstage;                           // staged p of LL (stride h)
     if (lstaged && r == 0 && QAPPLY) {
         constexpr int V = vec16<T>();
         const int lc = lh - (V == 4 ? 2 : 1);           // log2 of the 16-byte chunks per row
         for (int k = threadIdx.x; k < (h << lc); k += NT) {
             const int i = k >> lc, c = (k & ((1 << lc) - 1)) * V, pos = off + i * n + c;
             cp_async16(lsp + i * h + c, a.pin + pos);
-            if (NEEDB) cp_async16(lsb + i * h + c, a.vb + pos);
-            if (INIT) cp_async16(lsj + i * h + c, a.vj + pos);
         }
     }
-    // operands of the epilogue at this CTA's positions (band, then LL share), loaded now so
-    // that their latency overlaps: p; with the fused initial residual also b and J^-1
-    T pl[PL], xb[PF], xl[PL], jb[PF], jl[PL];
+    // p at this CTA's positions (band, then LL share), loaded now so that its latency overlaps
+    T pl[PL];
     if (QAPPLY) {
 #pragma unroll
         for (int s = 0; s < PF; ++s) {
@@ -545,8 +536,6 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
             if (k < ecnt) {
                 const int pos = off + (row_start + (k >> lrb)) * n + r0 + (k & (rb - 1));
                 pre_p[s] = a.pin[pos];
-                if (NEEDB) xb[s] = a.vb[pos];
-                if (INIT) jb[s] = a.vj[pos];
             }
         }
 #pragma unroll
@@ -555,8 +544,6 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
             if (k < lcnt) {
                 const int pos = off + (lr0 + (k >> lh)) * n + (k & (h - 1));
                 pl[s] = a.pin[pos];
-                if (NEEDB) xl[s] = a.vb[pos];
-                if (INIT) jl[s] = a.vj[pos];
             }
         }
     }
@@ -567,14 +554,7 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
     pdl_wait();
     // ---- 1. the row band of y ---------------------------------------------------
     if (has_band) {
-        if (SRC == LSRC_PHI) {
-            for (int k = threadIdx.x; k < rb * n; k += NT) {
-                const int i = (k >> L.log2n), j = k - i * n;
-                cp_async(ybuf + i * ys + j, a.in + off + (r0 + i) * n + j);
-            }
-            cp_async_wait();
-            __syncthreads();
-        } else if (lay.ydirect) {
+        if (lay.ydirect) {
             // y = sum_g R_y,gl^T u_g R_x,gl over this band, read straight from the pair slots:
             // the boxes' columns are 16-byte groups of the layer grid (host-checked), so a
             // thread owns one group and issues one 16-byte L2 read per sensor, all in flight
@@ -713,38 +693,16 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
     }
     cluster.sync();                                                       // #1: column tiles complete
     DotAcc<T> dot;                 // p.q share of this CTA (double accuracy)
-    DotAcc<T> drz;                 // r.z share (fused initial residual)
-    // The epilogue at one position: v = (W y)(i, j), p and the prefetched operands.
-    //   APPLY: q = v + alpha D p, written, p.q;  COEF: v written;
-    //   APPLY_INIT (initial residual, Algorithm 1): r = b - q, z = J^-1 r, p = z, b_prev = b, r.z.
-    auto epi = [&](int i, int j, int pos, T v, T p, T x, T jv) {
+    // The epilogue at one position: v = (W y)(i, j).  APPLY: q = v + alpha D p, written, p.q;
+    // COEF: v written.
+    auto epi = [&](int i, int j, int pos, T v, T p) {
         if (!QAPPLY) {
             a.out[pos] = v;
             return;
         }
-        if (DST == LDST_RESID_INIT) {
-            // v is the residual's data term: r0 = v - alpha D c0
-            const T rr = v - d.alpha * sD[level_of(i, j, L)] * p;
-            const T z = jv * rr;
-            a.vr[pos] = rr;
-            a.vz[pos] = z;
-            a.vp[pos] = z;
-            drz.add(rr, z);
-            return;
-        }
         const T q = v + d.alpha * sD[level_of(i, j, L)] * p;
-        if (DST == LDST_APPLY) {
-            a.out[pos] = q;
-            dot.add(p, q);
-        } else {
-            const T rr = x - q;
-            const T z = jv * rr;
-            a.vr[pos] = rr;
-            a.vz[pos] = z;
-            a.vp[pos] = z;
-            a.vbprev[pos] = x;
-            drz.add(rr, z);
-        }
+        a.out[pos] = q;
+        dot.add(p, q);
     };
     if (has_band) {
         dwt_pass<T, false>(cbuf, rb, n, 1, cs);
@@ -765,7 +723,7 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
             const int k = threadIdx.x + s2 * NT;
             if (k < ecnt) {
                 const int i = row_start + (k >> lrb), jj = (k & (rb - 1));
-                epi(i, r0 + jj, off + i * n + r0 + jj, cbuf[i * cs + jj], pre_p[s2], xb[s2], jb[s2]);
+                epi(i, r0 + jj, off + i * n + r0 + jj, cbuf[i * cs + jj], pre_p[s2]);
             }
         }
     }
@@ -794,8 +752,7 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
             if (r == 0)
                 for (int k = threadIdx.x; k < h * h; k += NT) {
                     const int i = k >> lh, j = k & (h - 1);
-                    epi(i, j, off + i * n + j, lbuf[i * lsd + j], QAPPLY ? lsp[k] : T(0),
-                        NEEDB ? lsb[k] : T(0), INIT ? lsj[k] : T(0));
+                    epi(i, j, off + i * n + j, lbuf[i * lsd + j], QAPPLY ? lsp[k] : T(0));
                 }
         } else {
 #pragma unroll
@@ -803,7 +760,7 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
                 const int k = threadIdx.x + s2 * NT;
                 if (k < lcnt) {
                     const int i = lr0 + (k >> lh), j = k & (h - 1);
-                    epi(i, j, off + i * n + j, ldist ? ybuf[k] : lbuf[i * lsd + j], pl[s2], xl[s2], jl[s2]);
+                    epi(i, j, off + i * n + j, ldist ? ybuf[k] : lbuf[i * lsd + j], pl[s2]);
                 }
             }
         }
@@ -811,7 +768,7 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
     if (DST == LDST_APPLY) {
         double* slots = a.pcg.pqpart + a.iter * PQ_SLOTS;
         cta_dot_store(dot, red, slots + l * CL + r);
-        if (!a.defer_total && last_arrival(a.pcg.count + 1, ctas, &last) && threadIdx.x < 32) {
+        if (last_arrival(a.pcg.count + 1, ctas, &last) && threadIdx.x < 32) {
             // fixed order: layer-major, rank-minor over the slots of the layers present
             const double tot = warp_total(slots, d.n_layers * CL, &dot);
             if (threadIdx.x == 0) {
@@ -820,26 +777,12 @@ __device__ __forceinline__ void cl_fwd_body(const Desc<T>& d, const ClArgs<T>& a
             }
         }
     }
-    if (INIT) {
-        // r.z of the new residual into rz slot `rzslot`, fixed order over the layer CTAs
-        cta_dot_store(drz, red, a.rzp + l * CL + r);
-        if (!a.defer_total && last_arrival(a.pcg.count, ctas, &last) && threadIdx.x < 32) {
-            const double tot = warp_total(a.rzp, d.n_layers * CL, &drz);
-            if (threadIdx.x == 0) {
-                a.pcg.rztot[a.rzslot] = tot;
-                a.pcg.count[0] = 0;
-            }
-        }
-    }
 }
 
 // ---------------------------------------------------------------------------
 // Inverse layer kernel (cluster per layer): phi = W^T c, optionally advancing the CG
 // direction first (Sec. 3.3).  PUPD = 0: phi = W^T a.in.  PUPD = 1: p = z + beta p in place
-// (a.pupd), beta = rz_k / rz_(k-1), then phi = W^T p.  PUPD = 2, the augmented PCG of
-// Sec. 3.4: p_new = z + beta p_old - sum_j mu_j P_j into a.pout, mu_j = q_j.z / p_j.q_j of
-// the previous frame's directions P_j (p_old = a.pupd; none, and beta = 0, for a frame's
-// first direction), then phi = W^T p_new.  The direction update is spread over the
+// (a.pupd), beta = rz_k / rz_(k-1), then phi = W^T p.  The direction update is spread over the
 // cluster: every CTA updates its column band (below the LL quadrant when coarse) and a
 // share of the LL quadrant's rows, which it pushes to the leader for the coarse levels.
 // ---------------------------------------------------------------------------
@@ -873,14 +816,9 @@ __device__ __forceinline__ void cl_inv_body(const Desc<T>& d, const ClArgs<T>& a
     const int lr0 = coarse ? min(r * hb, h) : 0, lr1 = coarse ? min(lr0 + hb, h) : 0;
     const int lcnt = (lr1 - lr0) * h;
 
-    // beta = rz_k / rz_(k-1) and the mu_j, formed once (an FP64 division costs ~10 FP64
-    // instructions, and GB300 issues a warp's FP64 instruction in ~64 cycles) and broadcast
+    // beta = rz_k / rz_(k-1), formed once (an FP64 division costs ~10 FP64 instructions, and
+    // GB300 issues a warp's FP64 instruction in ~64 cycles) and broadcast
     __shared__ T sbeta;
-    __shared__ T smu[AUG_MAX];
-    const bool has_old = PUPD == 1 || (PUPD == 2 && a.pupd != nullptr);
-    const bool stage_src = PUPD == 0 || has_old;
-    const T* src = PUPD ? a.pupd : a.in;
-    T* pdst = PUPD == 2 ? a.pout : a.pupd;
     // the exchanges below push into peers' shared memory before the first full cluster
     // barrier: arrive now, wait before the first push, so that every CTA has started
     asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
@@ -927,70 +865,12 @@ __device__ __forceinline__ void cl_inv_body(const Desc<T>& d, const ClArgs<T>& a
     // The direction being advanced (PUPD > 0: p_old, last written by the inverse kernel of
     // the previous iteration) is staged before the dependency wait; z, the plain input (its
     // writer may be the previous kernel) and the scalars after it.
-    if (PUPD && stage_src) stage_vec(src, sp, lp);
+    if (PUPD) stage_vec(a.pupd, sp, lp);
     pdl_wait();
-    if (!PUPD && stage_src) stage_vec(src, sp, lp);
-    if (PUPD) stage_vec(a.zupd, sz, lz);
-    // beta and mu are formed while the copies are in flight; a deferred r.z total first
-    // (warp 0, fixed order: the same value in every CTA)
-    if (threadIdx.x < 32 && (PUPD || a.rz_cnt > 0)) {
-        double rz_new = 0.0;
-        if (a.rz_cnt > 0) {
-            rz_new = warp_total(a.rz_parts, a.rz_cnt, static_cast<const DotAcc<T>*>(nullptr));
-            if (threadIdx.x == 0 && l == 0 && r == 0) a.pcg.rztot[a.rz_slot] = rz_new;
-        }
-        if (PUPD && threadIdx.x == 0) {
-            double b = 0.0;
-            if (has_old) {
-                if (a.rz_cnt == 0) rz_new = a.pcg.rztot[a.iter];
-                const double rz_old = a.pcg.rztot[a.iter - 1];
-                b = rz_old != 0.0 ? rz_new / rz_old : 0.0;
-            }
-            sbeta = T(b);
-        }
-    }
-    if (PUPD == 2) {
-        if (a.aug_pcnt > 0) {
-            // deferred totals: warps 1, 2, ... each total dot j in the fixed order
-            const int warp1 = threadIdx.x >> 5, nw1 = NT >> 5;
-            for (int j = warp1 - 1; warp1 > 0 && j < a.aug_m; j += nw1 - 1) {
-                const double num = warp_total(a.aug_parts + static_cast<long long>(j) * a.aug_pcnt, a.aug_pcnt,
-                                              static_cast<const DotAcc<T>*>(nullptr));
-                if ((threadIdx.x & 31) == 0) {
-                    const double den = a.aug_pq[j];
-                    smu[j] = T(den > 0.0 ? num / den : 0.0);
-                }
-            }
-        } else if (threadIdx.x >= 32 && threadIdx.x < 32 + a.aug_m) {
-            const int j = threadIdx.x - 32;
-            const double num = a.aug_tot[AUG_MAX + j], den = a.aug_pq[j];
-            smu[j] = T(den > 0.0 ? num / den : 0.0);
-        }
-    }
-    // the augmented update's sum_j mu_j P_j at this thread's positions, its loads in flight
-    // beside the staging copies
-    T cb[PF], cl[PL];
-#pragma unroll
-    for (int s2 = 0; s2 < PF; ++s2) cb[s2] = T(0);
-#pragma unroll
-    for (int s2 = 0; s2 < PL; ++s2) cl[s2] = T(0);
-    if (PUPD == 2) {
-        __syncthreads();                                             // smu
-        for (int j = 0; j < a.aug_m; ++j) {
-            const T mu = smu[j];
-            const T* Pj = a.augP + static_cast<long long>(j) * a.aug_ld + off;
-#pragma unroll
-            for (int s2 = 0; s2 < PF; ++s2) {
-                const int k = threadIdx.x + s2 * NT;
-                if (has_band && k < nrow * rb)
-                    cb[s2] += mu * __ldg(Pj + (row_start + (k >> lrb)) * n + r0 + (k & (rb - 1)));
-            }
-#pragma unroll
-            for (int s2 = 0; s2 < PL; ++s2) {
-                const int k = threadIdx.x + s2 * NT;
-                if (k < lcnt) cl[s2] += mu * __ldg(Pj + (lr0 + (k >> lh)) * n + (k & (h - 1)));
-            }
-        }
+    stage_vec(PUPD ? a.zupd : a.in, PUPD ? sz : sp, PUPD ? lz : lp);
+    if (PUPD && threadIdx.x == 0) {
+        const double rz_new = a.pcg.rztot[a.iter], rz_old = a.pcg.rztot[a.iter - 1];
+        sbeta = T(rz_old != 0.0 ? rz_new / rz_old : 0.0);
     }
     cp_async_wait();
     __syncthreads();
@@ -1001,10 +881,9 @@ __device__ __forceinline__ void cl_inv_body(const Desc<T>& d, const ClArgs<T>& a
         const int k = threadIdx.x + s2 * NT;
         if (has_band && k < nrow * rb) {
             const int i = k >> lrb, jj = k & (rb - 1);
-            T p = stage_src ? sp[k] : T(0);
-            if (PUPD == 1) p = sz[k] + beta * p;
-            if (PUPD == 2) p = (has_old ? sz[k] + beta * p : sz[k]) - cb[s2];
-            if (PUPD) pdst[off + (row_start + i) * n + r0 + jj] = p;
+            T p = sp[k];
+            if (PUPD) p = sz[k] + beta * p;
+            if (PUPD) a.pupd[off + (row_start + i) * n + r0 + jj] = p;
             cbuf[(row_start + i) * cs + jj] = p;
         }
     }
@@ -1012,10 +891,9 @@ __device__ __forceinline__ void cl_inv_body(const Desc<T>& d, const ClArgs<T>& a
     for (int s2 = 0; s2 < PL; ++s2) {
         const int k = threadIdx.x + s2 * NT;
         if (k < lcnt) {
-            T p = stage_src ? lp[k] : T(0);
-            if (PUPD == 1) p = lz[k] + beta * p;
-            if (PUPD == 2) p = (has_old ? lz[k] + beta * p : lz[k]) - cl[s2];
-            if (PUPD) pdst[off + (lr0 + (k >> lh)) * n + (k & (h - 1))] = p;
+            T p = lp[k];
+            if (PUPD) p = lz[k] + beta * p;
+            if (PUPD) a.pupd[off + (lr0 + (k >> lh)) * n + (k & (h - 1))] = p;
             lp[k] = p;
         }
     }
@@ -1123,8 +1001,8 @@ __device__ __forceinline__ void cl_sensor_body(const Desc<T>& d, const SensorArg
     // the mask and the descriptor are set-up data, read before the dependency wait; the
     // projected layers or the slopes after it
     pdl_wait();
-    constexpr bool FROM_PHI = SRC == SSRC_PHI || SRC == SSRC_RESID;
-    bool bad = false;                          // a non-finite measured slope (SLOPES, RESID)
+    constexpr bool FROM_PHI = SRC == SSRC_PHI;
+    bool bad = false;                          // a non-finite measured slope (SLOPES)
     if (FROM_PHI && rows > 0) {
         // ---- V = P_g phi = sum_l (pair term of layer l) on node rows [s0, s1] ---------
         // a warp per node row; every lane's columns accumulate in the fixed layer order,
@@ -1165,14 +1043,6 @@ __device__ __forceinline__ void cl_sensor_body(const Desc<T>& d, const SensorArg
                 const T v10 = V[(ii + 1) * NP + j], v11 = V[(ii + 1) * NP + j + 1];
                 sx = T(0.5) * ((v01 - v00) + (v11 - v10));
                 sy = T(0.5) * ((v10 - v00) + (v11 - v01));
-                if (SRC == SSRC_RESID && W.nb == 1) {
-                    // residual of an ordinary sensor: measured minus modelled slope (a coarse
-                    // sensor's measurement enters after its block sums, below)
-                    const T mx = a.in[W.soff + id], my = a.in[W.soff + W.n_active + id];
-                    bad |= !(isfinite(mx) && isfinite(my));
-                    sx = mx - sx;
-                    sy = my - sy;
-                }
             }
             SX[k] = sx;
             SY[k] = sy;
@@ -1323,22 +1193,9 @@ __device__ __forceinline__ void cl_sensor_body(const Desc<T>& d, const SensorArg
                     sx += cps[q * 2 * MAXCOARSE + 2 * blk];
                     sy += cps[q * 2 * MAXCOARSE + 2 * blk + 1];
                 }
-                // coarse slope = sum / nb; Gamma_coarse^T spreads sigma^-2 slope / nb.  The
-                // residual form subtracts it from the block's measured slope.
-                if (SRC == SSRC_RESID) {
-                    const int K = d.cidx[W.cmask_off + blk];
-                    T mx = T(0), my = T(0);
-                    if (K >= 0) {
-                        mx = a.in[W.soff + K];
-                        my = a.in[W.soff + W.n_active + K];
-                        if (!(isfinite(mx) && isfinite(my)) && a.status) atomicOr(a.status, 1u);
-                    }
-                    cw[2 * blk] = (mx - sx * nbinv) * inv * nbinv;
-                    cw[2 * blk + 1] = (my - sy * nbinv) * inv * nbinv;
-                } else {
-                    cw[2 * blk] = sx * nbinv * inv * nbinv;
-                    cw[2 * blk + 1] = sy * nbinv * inv * nbinv;
-                }
+                // coarse slope = sum / nb; Gamma_coarse^T spreads sigma^-2 slope / nb
+                cw[2 * blk] = sx * nbinv * inv * nbinv;
+                cw[2 * blk + 1] = sy * nbinv * inv * nbinv;
             }
             __syncthreads();
             for (int ii = warp; ii < rows; ii += nwarp)

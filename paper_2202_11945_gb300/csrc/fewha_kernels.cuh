@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(BLK) k_layer(const Desc<T> d, const LayerArgs<
 // SRC / WEIGHT / DST.  Shared tiles: V (aperture nodes), SX, SY (per subaperture,
 // zero outside the active set).
 // ---------------------------------------------------------------------------
-// SSRC_RESID (cluster sensor kernel only): the measured slopes (in) minus the projected
+// SSRC_RESID (tile sensor kernel only): the measured slopes (in) minus the projected
 // layers' slopes, the initial residual's data term before the noise weighting
 // SSRC_RAW (tile sensor kernel only): slopes without their noise weights (the model's adjoint)
 enum { SSRC_PHI = 0, SSRC_NODES = 1, SSRC_SLOPES = 2, SSRC_RESID = 3, SSRC_RAW = 4 };

@@ -96,7 +96,7 @@ __device__ __noinline__ void st_sensor(const Desc<T>& d, const SensorArgs<T>& a,
 template <class T, int DST>
 __device__ __noinline__ void st_fwd(const Desc<T>& d, const ClArgs<T>& a, const ClLayout& lay, const PairBufs<T>& pb,
                                     int l, unsigned ctas) {
-    cl_fwd_body<T, LSRC_NODES, DST>(d, a, lay, pb, l, ctas);
+    cl_fwd_body<T, DST>(d, a, lay, pb, l, ctas);
 }
 template <class T>
 __device__ __noinline__ void st_proj(const Desc<T>& d, const T* phi, const PairBufs<T>& pb, int p0, int step) {
