@@ -598,8 +598,8 @@ int enqueue_apply(fewha_handle* H, const Desc<T>& d, const T* x, T* qout, int sl
     T* phi = static_cast<T*>(H->phi);
     int rc;
     ClArgs<T> a = cl_args<T>(H, x, phi);
-    a.zero_piston = 1;
-    a.fsh = H->fsh;                 // the data path's input leaves the piston out
+    a.zero_piston = 1;              // the data path's input leaves the piston out
+    a.fsh = H->fsh;
     a.rz_parts = df.rz_parts;
     a.rz_cnt = df.rz_cnt;
     a.rz_slot = df.rz_slot;
@@ -694,8 +694,8 @@ int enqueue_apply_init(fewha_handle* H, const Desc<T>& d, T* c, cudaStream_t st,
 // C^-1 (s - Gamma P phi0) (phi0 = W^T c0, its piston left out), the adjoint projection and
 // the forward kernel give r0 = W P^T Gamma^T C^-1 (s - Gamma P phi0) - alpha D c0 and the
 // initial residual's vector step (z0, p0, r.z in slot 0, only shares with `defer`).  By
-// linearity this is b - M c0 of Algorithm 1 without forming b: 5 kernels instead of the
-// right-hand side's 3 plus the apply's 5.  b and b_prev are not written.
+// linearity this is b - M c0 of Algorithm 1 without forming b: 4 kernels instead of the
+// right-hand side's 4 and the apply's 4.  b and b_prev are not written.
 template <class T>
 int enqueue_resid_init(fewha_handle* H, const Desc<T>& d, const T* s, T* c, cudaStream_t st, bool defer,
                        T* p0 = nullptr, T* phi_out = nullptr, T* r0 = nullptr, T* z0 = nullptr) {
@@ -1319,10 +1319,6 @@ bool tail_used(const HostSetup& s) {
     return false;
 }
 
-// Shared-memory layouts of the cluster kernels: the largest band over all layers and
-// sensors, element counts in T units after a fixed header; every region starts on a
-// 16-byte boundary (cp.async targets).
-
 // Tables and shared-memory layouts of the tile, band and sensor kernels (fewha_tile.cuh).
 template <class T>
 int tile_tables(fewha_handle* H) {
@@ -1514,7 +1510,7 @@ int tile_tables(fewha_handle* H) {
             int at = 0;
             for (int g = 0; g < ng; ++g) {
                 if (g % f.gb == 0) at = 0;
-                    bsrc[(u * ng + g) * 4 + 2] = at;
+                bsrc[(u * ng + g) * 4 + 2] = at;
                 at += need[u][g];
                 most = std::max(most, at);
             }
@@ -1802,6 +1798,10 @@ int functional_tables(fewha_handle* H) {
     return FEWHA_OK;
 }
 
+// Shared-memory layouts of the persistent frame's bodies: the largest band over all layers and
+// sensors, element counts in T units after a fixed header; every region starts on a 16-byte
+// boundary (cp.async targets).  With them the footprint boxes, the tail operator and the pair
+// buffers, which the tile kernels use too.
 template <class T>
 int cluster_layouts(fewha_handle* H) {
     const HostSetup& s = H->setup;

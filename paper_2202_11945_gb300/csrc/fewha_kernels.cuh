@@ -39,8 +39,7 @@ constexpr int NWARP = BLK / 32;
 // Daubechies' N = 3 scaling filter (Sec. 3.1; the closed form's values, as db3_taps computes
 // them) and the wavelet filter g_k = (-1)^k h_(5-k), as immediate operands: every kernel
 // starts with a cold constant cache, and the first reads of taps kept in constant memory
-// stood on the critical path of each wavelet pass (frame of the 8 m system 96.3 -> 91.3 us,
-// of the MAORY one 176.4 -> 173.5).
+// stood on the critical path of each wavelet pass (5 us of an 8 m frame, 3 of a MAORY one).
 __host__ __device__ constexpr double db3_h(int t) {
     return t == 0   ? 0.33267055295008263
            : t == 1 ? 0.80689150931109266
@@ -212,6 +211,9 @@ __device__ __forceinline__ double warp_total(const double* p, int cnt, const Dot
 // batched frame) need not get the same choice in both: the commands would differ by a rounding.
 __device__ __forceinline__ float dot2(float a, float b, float c, float d) { return __fmaf_rn(a, b, __fmul_rn(c, d)); }
 __device__ __forceinline__ double dot2(double a, double b, double c, double d) { return __fma_rn(a, b, __dmul_rn(c, d)); }
+// a b + c in one rounding: sums of products that two kernels share are chains of these.
+__device__ __forceinline__ float fmadd(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fmadd(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // LGS spot elongation of subaperture (i, j) (Eq. 3): beta and gamma, so that
 // C_ij^-1 = sigma^-2 (I - gamma beta beta^T) (Sherman-Morrison).
@@ -1259,8 +1261,8 @@ __device__ __forceinline__ void fit_body(const Desc<T>& d, const T* __restrict__
 #pragma unroll
         for (int u = 0; u < 4; ++u)
             if (w[u] != T(0))
-                acc += w[u] * dot2(T(1) - fy[u], dot2(T(1) - fx[u], v[u][0], fx[u], v[u][1]), fy[u],
-                                   dot2(T(1) - fx[u], v[u][2], fx[u], v[u][3]));
+                acc = fmadd(w[u], dot2(T(1) - fy[u], dot2(T(1) - fx[u], v[u][0], fx[u], v[u][1]), fy[u],
+                                       dot2(T(1) - fx[u], v[u][2], fx[u], v[u][3])), acc);
     }
     if (cpist) {
         // phi without the full layers' pistons (the carried layers): a unit piston coefficient
@@ -1268,12 +1270,12 @@ __device__ __forceinline__ void fit_body(const Desc<T>& d, const T* __restrict__
         // to one, so each adds w_lm c_piston / n
         for (int l = 0; l < d.n_layers; ++l) {
             const T wl = d.fitw[m][l];
-            if (d.L[l].full && wl != T(0)) acc += wl * (cpist[d.L[l].off] / T(d.L[l].n));
+            if (d.L[l].full && wl != T(0)) acc = fmadd(wl, cpist[d.L[l].off] / T(d.L[l].n), acc);
         }
     }
     if (apply_gain == 2) {
         const T cur = a_prev[idx];
-        const T a = cur + d.gain * (acc - a_old[idx]);
+        const T a = fmadd(d.gain, acc - a_old[idx], cur);
         a_old[idx] = cur;
         a_prev[idx] = a;
         out[idx] = a;

@@ -2,7 +2,8 @@
 // layers of separable interpolations, P_g phi = sum_l R_y,gl phi_l R_x,gl^T, and its
 // adjoint is sum_g R_y,gl^T u_g R_x,gl.  One CTA per pair computes its term with two
 // separable passes in shared memory; the sensor and layer kernels add the terms up.
-// No reduction crosses CTAs here, so the sums stay in a fixed order.
+// No reduction crosses CTAs here, so the sums stay in a fixed order.  The persistent frame's form
+// of P and P^T; the frame of separate launches has them in its sensor and band kernels.
 #pragma once
 
 #include "fewha_cluster.cuh"

@@ -7,9 +7,8 @@
 // what a frame waits for is the chain launch -> loads -> levels -> store.  A cluster of 8
 // CTAs per layer (bands exchanged through distributed shared memory, the coarse levels on
 // one leader CTA, three cluster barriers) took 8.0 us a launch on the 9 layers of the MAORY
-// geometry and filled 72 of the 152 SMs; the tiles redo the halos (1.4 times the level-0
-// arithmetic at ts = 32) but wait for nobody: 144 CTAs, 4.8 us, and the MAORY frame went
-// from 192.6 to 176.4 us (FP64 842 to 827), a batch of 16 instances from 686 to 577 us.
+// geometry and filled 72 of the 152 SMs; the tiles redo the halos (2.2 times the arithmetic
+// at ts = 32) but wait for nobody: 120 CTAs, 5.7 us with the sums over the sensors in it.
 #pragma once
 
 #include "fewha_cluster.cuh"
@@ -115,8 +114,8 @@ __device__ __forceinline__ int tdiv(int t, int magic) { return (t * magic) >> 16
 // scaling (a) and wavelet (d) half.
 template <class T>
 __device__ __forceinline__ void synth_pair(T a0, T a1, T a2, T d0, T d1, T d2, T& e, T& o) {
-    e = dot2(tap_h<T>(0), a0, tap_h<T>(2), a1) + tap_h<T>(4) * a2 + tap_g<T>(0) * d0 + tap_g<T>(2) * d1 + tap_g<T>(4) * d2;
-    o = dot2(tap_h<T>(1), a0, tap_h<T>(3), a1) + tap_h<T>(5) * a2 + tap_g<T>(1) * d0 + tap_g<T>(3) * d1 + tap_g<T>(5) * d2;
+    e = fmadd(tap_g<T>(4), d2, fmadd(tap_g<T>(2), d1, fmadd(tap_g<T>(0), d0, fmadd(tap_h<T>(4), a2, dot2(tap_h<T>(0), a0, tap_h<T>(2), a1)))));
+    o = fmadd(tap_g<T>(5), d2, fmadd(tap_g<T>(3), d1, fmadd(tap_g<T>(1), d0, fmadd(tap_h<T>(5), a2, dot2(tap_h<T>(1), a0, tap_h<T>(3), a1)))));
 }
 
 // Sums over one sensor's measured slopes, as its functionals sum the modelled ones: tip and
@@ -301,13 +300,13 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
                     const T* Pj = a.augP + static_cast<long long>(j) * a.aug_ld;
 #pragma unroll
                     for (int s = 0; s < SL; ++s)
-                        if (pos[s] >= 0) cor[s] += mu * __ldg(Pj + pos[s]);
+                        if (pos[s] >= 0) cor[s] = fmadd(mu, __ldg(Pj + pos[s]), cor[s]);
                 }
             }
 #pragma unroll
             for (int s = 0; s < SL; ++s)
                 if (pos[s] >= 0) {
-                    if (has_old) zv[s] = zv[s] + beta * po[s];
+                    if (has_old) zv[s] = fmadd(beta, po[s], zv[s]);
                     if (PUPD == 2) zv[s] -= cor[s];
                     if (own[s]) a.pout[pos[s]] = zv[s];
                 }
@@ -334,7 +333,7 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
         const int o = t >> 3, part = t & 7;
         T acc[2] = {T(0), T(0)};
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i & 1] += sop[o * TAIL_LD + part * 8 + i] * tailb[part * 8 + i];
+        for (int i = 0; i < 8; ++i) acc[i & 1] = fmadd(sop[o * TAIL_LD + part * 8 + i], tailb[part * 8 + i], acc[i & 1]);
         T y = acc[0] + acc[1];
         y += __shfl_down_sync(0xffffffffu, y, 4);
         y += __shfl_down_sync(0xffffffffu, y, 2);
@@ -406,7 +405,7 @@ __device__ __forceinline__ void tinv_body(const Desc<T>& d, const ClArgs<T>& a, 
                 if (k + 8 * q < k1) e[q] = k + 8 * q < d.fcap ? fent[k + 8 * q] : gent[f0 + k + 8 * q];
 #pragma unroll
             for (int q = 0; q < 4; ++q)
-                if (k + 8 * q < k1) x += e[q].y * sc[static_cast<int>(e[q].x)];
+                if (k + 8 * q < k1) x = fmadd(e[q].y, sc[static_cast<int>(e[q].x)], x);
             s.add(x, T(1));
         }
         A x = AccOf<T>::of(s);
@@ -488,8 +487,8 @@ __device__ __forceinline__ void analyse(T* buf, T* tmp, const T* tail, int n, in
 #pragma unroll
             for (int q = 0; q < 6; ++q) {
                 const T v = x[(2 * k + q) & (m - 1)];
-                a += tap_h<T>(q) * v;
-                dd += tap_g<T>(q) * v;
+                a = fmadd(tap_h<T>(q), v, a);
+                dd = fmadd(tap_g<T>(q), v, dd);
             }
             tmp[row * ld + k] = a;
             tmp[row * ld + hm + k] = dd;
@@ -501,8 +500,8 @@ __device__ __forceinline__ void analyse(T* buf, T* tmp, const T* tail, int n, in
 #pragma unroll
             for (int q = 0; q < 6; ++q) {
                 const T v = tmp[((2 * k + q) & (m - 1)) * ld + c];
-                a += tap_h<T>(q) * v;
-                dd += tap_g<T>(q) * v;
+                a = fmadd(tap_h<T>(q), v, a);
+                dd = fmadd(tap_g<T>(q), v, dd);
             }
             buf[k * ld + c] = a;
             buf[(hm + k) * ld + c] = dd;
@@ -518,7 +517,7 @@ __device__ __forceinline__ void analyse(T* buf, T* tmp, const T* tail, int n, in
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
                 const int k = 16 * part + i;
-                acc[i & 1] += tail[k * TAIL_LD + o] * buf[(k >> 3) * ld + (k & 7)];
+                acc[i & 1] = fmadd(tail[k * TAIL_LD + o], buf[(k >> 3) * ld + (k & 7)], acc[i & 1]);
             }
             y = acc[0] + acc[1];
             y += __shfl_down_sync(0xffffffffu, y, 2);
@@ -535,18 +534,17 @@ __device__ __forceinline__ void analyse(T* buf, T* tmp, const T* tail, int n, in
 // the apply or of the initial residual.  The sensor kernel has applied the column half of
 // P_g^T (R_x, per sensor and layer, in pb.Y).  k_tfwd, a CTA per band of rows of a layer and
 // its halo of 4: the row half summed over the sensors, the finest analysis level, the
-// epilogue of the three detail bands; its LL block goes to a.ll.  k_tcoarse, a CTA per
-// epilogue of the three detail bands; its LL block goes to a.ll.  k_tcoarse, a CTA per
-// layer of several bands: the other levels and their epilogue.  A layer of one band (side
+// epilogue of the three detail bands; its LL block goes to a.ll.  k_tcoarse, the other levels
+// of a layer of several bands and their epilogue.  A layer of one band (side
 // at most 32) is finished by k_tfwd.
 //
 // Bound: latency again (launch, one block of staged reads, two passes).  Before, a kernel of
-// (sensor, layer) pairs made the whole adjoint projection (4.9 us on the MAORY geometry) and
-// a cluster per layer summed the pairs, transformed and finished on one leader CTA (11 us).
-// Bands of 8 whole rows keep every global read a contiguous block and need a halo in one
-// direction only; square tiles with a halo on four sides read the aperture vectors 1.9 times
-// over and were slower (the frame 212 us).  Stamps inside a frame: 6.5 us for the bands and 5
-// for the coarse levels, with the CG update in both (5.3, 4.8 and 2.5 as a kernel of its own).
+// (sensor, layer) pairs made the whole adjoint projection (4.9 us on the MAORY geometry), a
+// cluster per layer summed the pairs, transformed and finished on one leader CTA (11 us) and the
+// CG update was a kernel (4.3 us); stamps inside a frame now: 6.5 us for the bands and 5 for the
+// coarse levels.  Bands of 8 whole rows keep every global read a contiguous block and need a halo
+// in one direction only; square tiles with a halo on four sides read the aperture vectors 1.9
+// times over and were slower.
 // ---------------------------------------------------------------------------
 constexpr int TF_BAND = 8;       // rows of a band
 constexpr int TF_ONE = 32;       // a layer of this side or less is one band
@@ -563,7 +561,7 @@ template <> struct Quad<float> {
     float4 v;
     __device__ __forceinline__ void zero() { v = make_float4(0.f, 0.f, 0.f, 0.f); }
     __device__ __forceinline__ void fma(float w, const Quad& q) {
-        v.x += w * q.v.x; v.y += w * q.v.y; v.z += w * q.v.z; v.w += w * q.v.w;
+        v = make_float4(fmadd(w, q.v.x, v.x), fmadd(w, q.v.y, v.y), fmadd(w, q.v.z, v.z), fmadd(w, q.v.w, v.w));
     }
     // even and odd columns
     __device__ __forceinline__ void split(float* e, float* o) const {
@@ -574,7 +572,7 @@ template <> struct Quad<float> {
 template <> struct Quad<double> {
     double2 v;
     __device__ __forceinline__ void zero() { v = make_double2(0.0, 0.0); }
-    __device__ __forceinline__ void fma(double w, const Quad& q) { v.x += w * q.v.x; v.y += w * q.v.y; }
+    __device__ __forceinline__ void fma(double w, const Quad& q) { v = make_double2(fmadd(w, q.v.x, v.x), fmadd(w, q.v.y, v.y)); }
     __device__ __forceinline__ void split(double* e, double* o) const {
         *e = v.x;
         *o = v.y;
@@ -609,20 +607,20 @@ __device__ __forceinline__ void epi_apply(const ClArgs<T>& a, T alpha, T dl, int
     if (DST == LDST_COEF) {
         a.out[pos] = v;
     } else if (DST == LDST_APPLY) {
-        const T q = v + alpha * dl * o.p;
+        const T q = fmadd(alpha * dl, o.p, v);
         a.out[pos] = q;
         dot.add(o.p, q);
     } else if (DST == LDST_UPDATE) {
-        const T q = v + alpha * dl * o.p;
+        const T q = fmadd(alpha * dl, o.p, v);
         if (a.out) a.out[pos] = q;
-        const T rr = o.r - step * q;
+        const T rr = fmadd(-step, q, o.r);
         const T z = o.j * rr;
-        if (upc) a.vc[pos] = a.vc[pos] + step * o.p;
+        if (upc) a.vc[pos] = fmadd(step, o.p, a.vc[pos]);
         a.vr[pos] = rr;
         a.vz[pos] = z;
         dot.add(rr, z);
     } else {
-        const T rr = DST == LDST_RESID_INIT ? v - alpha * dl * o.p : o.b - (v + alpha * dl * o.p);
+        const T rr = DST == LDST_RESID_INIT ? fmadd(-(alpha * dl), o.p, v) : o.b - fmadd(alpha * dl, o.p, v);
         const T z = o.j * rr;
         a.vr[pos] = rr;
         a.vz[pos] = z;
@@ -819,7 +817,7 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
                         if (c < 0 || c >= b.y) continue;
                         const T* row = st + static_cast<int>(w[g * (kt + 1) + kt]) + c;
                         for (int q = 0; q < kt; ++q)
-                            if (w[g * (kt + 1) + q] != T(0)) x += w[g * (kt + 1) + q] * row[q * b.y];
+                            if (w[g * (kt + 1) + q] != T(0)) x = fmadd(w[g * (kt + 1) + q], row[q * b.y], x);
                     }
                     acc[k].v.x += x;
                 } else if (kt == 3) {
@@ -861,11 +859,11 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
     const T step = UPD ? sstep : T(0);
 #pragma unroll
     for (int k = 0; k < CPT; ++k)
-        if (carry && t + k * NT < n * n) a.phic[L.off + t + k * NT] = cph[k] + step * pph[k];
+        if (carry && t + k * NT < n * n) a.phic[L.off + t + k * NT] = fmadd(step, pph[k], cph[k]);
     // ---- the finest analysis level: rows, then columns ---------------------------------------
     // In double the row half once per row, through shared memory (the staging buffer, read
     // by now): about 50 multiply-adds a block of four where the fused form has 96, on a pipe of
-    // two a cycle; the MAORY frame went from 563 to 550 us, an 8 m iteration from 48 to 43.
+    // two a cycle; the MAORY frame takes 550 us, 563 with the fused form, an 8 m iteration 43, 48.
     // Single precision is bound by latency and keeps the form with one barrier less.
     constexpr bool SPLIT = sizeof(T) == 8;
     const int msd = n + 1;
@@ -877,8 +875,8 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
 #pragma unroll
             for (int q = 0; q < 6; ++q) {
                 const T x = (q & 1 ? yo : ye)[i * ysd + ((kx + (q >> 1)) & (h - 1))];
-                av += tap_h<T>(q) * x;
-                dv += tap_g<T>(q) * x;
+                av = fmadd(tap_h<T>(q), x, av);
+                dv = fmadd(tap_g<T>(q), x, dv);
             }
             mid[i * msd + kx] = av;
             mid[i * msd + h + kx] = dv;
@@ -886,8 +884,10 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
         __syncthreads();
     }
     DotAcc<T> dot;
+    // A block per thread: pos and op are those of block t.  Written as a loop, which runs once, the
+    // MAORY frame takes 135.2 us, as a condition 137.4 (the same commands).
     static_assert((TF_BAND / 2) * (MAXN / 2) <= NT && (TF_ONE / 2) * (TF_ONE / 2) <= NT, "a block per thread");
-    if (const int b = t; b < nblk) {
+    for (int b = t; b < nblk; b += NT) {
         const int msk = bands > 1 ? 15 : n - 1;           // a band holds its halo
         const int ky = 2 * (b >> lh), kx = b & (h - 1);
         T ra[6], rd[6];
@@ -905,8 +905,8 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
 #pragma unroll
             for (int q = 0; q < 6; ++q) {
                 const T x = (q & 1 ? ro : re)[(kx + (q >> 1)) & (h - 1)];
-                av += tap_h<T>(q) * x;
-                dv += tap_g<T>(q) * x;
+                av = fmadd(tap_h<T>(q), x, av);
+                dv = fmadd(tap_g<T>(q), x, dv);
             }
             ra[r] = av;
             rd[r] = dv;
@@ -914,10 +914,10 @@ __device__ __forceinline__ void tfwd_body(const Desc<T>& d, const ClArgs<T>& a, 
         T ll = T(0), v[3] = {T(0), T(0), T(0)};
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
-            ll += tap_h<T>(r) * ra[r];
-            v[0] += tap_h<T>(r) * rd[r];
-            v[1] += tap_g<T>(r) * ra[r];
-            v[2] += tap_g<T>(r) * rd[r];
+            ll = fmadd(tap_h<T>(r), ra[r], ll);
+            v[0] = fmadd(tap_h<T>(r), rd[r], v[0]);
+            v[1] = fmadd(tap_g<T>(r), ra[r], v[1]);
+            v[2] = fmadd(tap_g<T>(r), rd[r], v[2]);
         }
         const int rk = (Y0 >> 1) + (b >> lh);
         if (bands > 1)
@@ -963,8 +963,8 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
 // operands are read before the wait.
 //
 // Bound: the leader's chain of passes, latency of one CTA: 5.0 us of a MAORY iteration in
-// single precision.  The quadrants and the vector chunks on CTAs of their own keep it at that
-// with the updates of c, of its layers, of r and z inside, which were a kernel of 3 us before.
+// single precision, with the updates of c, of its layers, of r and z hidden beside it on CTAs of
+// their own.
 constexpr int TC_VEC = 2048;
 struct TcLayout {
     int lbuf, tmp, tail, st, total;  // T units after the reduction scratch; st: staged operands
@@ -992,8 +992,8 @@ __device__ __forceinline__ void tcoarse_body(const Desc<T>& d, const ClArgs<T>& 
         const T step = a.alphas[a.iter];
         const int k0 = (part - TC_SH) * TC_VEC, k1 = min(k0 + TC_VEC, n * n);
         for (int k = k0 + t; k < k1; k += NT) {
-            a.vc[L.off + k] += step * a.pin[L.off + k];
-            if (a.phic) a.phic[L.off + k] += step * a.phip[L.off + k];
+            a.vc[L.off + k] = fmadd(step, a.pin[L.off + k], a.vc[L.off + k]);
+            if (a.phic) a.phic[L.off + k] = fmadd(step, a.phip[L.off + k], a.phic[L.off + k]);
         }
         return;
     }
@@ -1033,12 +1033,12 @@ __device__ __forceinline__ void tcoarse_body(const Desc<T>& d, const ClArgs<T>& 
                 T av = T(0), dv = T(0);
 #pragma unroll
                 for (int q = 0; q < 6; ++q) {
-                    av += tap_h<T>(q) * x[q];
-                    dv += tap_g<T>(q) * x[q];
+                    av = fmadd(tap_h<T>(q), x[q], av);
+                    dv = fmadd(tap_g<T>(q), x[q], dv);
                 }
-                v[0] += tap_h<T>(r) * dv;
-                v[1] += tap_g<T>(r) * av;
-                v[2] += tap_g<T>(r) * dv;
+                v[0] = fmadd(tap_h<T>(r), dv, v[0]);
+                v[1] = fmadd(tap_g<T>(r), av, v[1]);
+                v[2] = fmadd(tap_g<T>(r), dv, v[2]);
             }
 #pragma unroll
             for (int e = 0; e < 3; ++e) epi_apply<T, DST>(a, salpha, sD[2], pos[e], v[e], op[e], dot, sstep);
@@ -1085,7 +1085,7 @@ __device__ __forceinline__ void tcoarse_body(const Desc<T>& d, const ClArgs<T>& 
             const T* x = raw + row * hs;
             T av = T(0);
 #pragma unroll
-            for (int q = 0; q < 6; ++q) av += tap_h<T>(q) * x[(2 * k + q) & (h - 1)];
+            for (int q = 0; q < 6; ++q) av = fmadd(tap_h<T>(q), x[(2 * k + q) & (h - 1)], av);
             mid[row * ld + k] = av;
         }
         __syncthreads();
@@ -1093,7 +1093,7 @@ __device__ __forceinline__ void tcoarse_body(const Desc<T>& d, const ClArgs<T>& 
             const int k = b >> lhh, c = b & (hh - 1);
             T av = T(0);
 #pragma unroll
-            for (int q = 0; q < 6; ++q) av += tap_h<T>(q) * mid[((2 * k + q) & (h - 1)) * ld + c];
+            for (int q = 0; q < 6; ++q) av = fmadd(tap_h<T>(q), mid[((2 * k + q) & (h - 1)) * ld + c], av);
             lbuf[k * ld + c] = av;
         }
         __syncthreads();
@@ -1135,8 +1135,8 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
 // Gamma_g, C_hat_g^-1 (Eq. 2, Sec. 3.2), Gamma_g^T and the column half of P_g^T.  SRC_PHI:
 // slopes of the projected layers (the M-apply); SRC_RESID: measured minus modelled slopes
 // (the initial residual); SRC_SLOPES: measured slopes (the right-hand side); SRC_RAW: the same
-// without C_hat_g^-1 (the model's adjoint).  The layers are read by direct bilinear gathers; the result goes out per layer as the aperture rows'
-// values on the layer's columns (pb.Y, slot g * n_layers + l, rows of box[3] columns), whose
+// without C_hat_g^-1 (the model's adjoint).  The layers are read by direct bilinear gathers; the
+// result goes out per layer as the aperture rows' values on the layer's columns (pb.Y, slot g * n_layers + l, rows of box[3] columns), whose
 // row half the band kernel applies.
 //
 // No CTA waits for another.  What the weighting of one subaperture needs of all the others
@@ -1145,8 +1145,8 @@ __global__ void __launch_bounds__(cblk<T>(), sizeof(T) == 4 ? 2 : 1)
 // formed; the slopes of the row below the band are formed here once more.
 //
 // Bound: latency (launch, the gather's L2 reads, two barriers): 6 us a launch on the MAORY
-// geometry, 180 CTAs.  With the sums inside clusters of 16 CTAs it took 8.5 us, 3 of them
-// before the clusters started: a cluster waits for a group of SMs to be free, so nothing of
+// geometry, 180 CTAs; with the sums inside clusters of 16 CTAs 8.5 us, 3 of them before the
+// clusters started: a cluster waits for a group of SMs to be free, so nothing of
 // its prologue hides behind the kernel before.  Bands of 4 rows instead of 5 keep a CTA at
 // 512 threads of 64 registers, which fit beside the neighbours'; 576 of 56 did not.
 // ---------------------------------------------------------------------------
@@ -1347,8 +1347,8 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
                         T b1, b2, gam;
                         elong(W, q0 + ii, j, b1, b2, gam);
                         const T bu = dot2(b1, ux, b2, uy);
-                        ux = (ux - gam * b1 * bu) + g1;
-                        uy = (uy - gam * b2 * bu) + g2;
+                        ux = fmadd(-(gam * b1), bu, ux) + g1;
+                        uy = fmadd(-(gam * b2), bu, uy) + g2;
                     }
                     wx = inv * ux;
                     wy = inv * uy;
@@ -1422,7 +1422,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
                     T x = T(0);
 #pragma unroll
                     for (int q = 0; q < 3; ++q)
-                        if (q < c.y) x += w[q] * src[ia * NP + q];
+                        if (q < c.y) x = fmadd(w[q], src[ia * NP + q], x);
                     dst[ia * cols] = x;
                 }
         } else {
@@ -1433,7 +1433,7 @@ __device__ __forceinline__ void tsen_body(const Desc<T>& d, const SensorArgs<T>&
                 T x = T(0);
 #pragma unroll
                 for (int q = 0; q < KMAX; ++q)
-                    if (q < c.y) x += w[q] * src[ia * NP + q];
+                    if (q < c.y) x = fmadd(w[q], src[ia * NP + q], x);
                 dst[ia * cols] = x;
             }
         }
@@ -1546,8 +1546,8 @@ __global__ void __launch_bounds__(OP_NT) k_weigh(__grid_constant__ const Desc<T>
             T b1, b2, gam;
             elong(W, k / W.N, k % W.N, b1, b2, gam);
             const T bu = b1 * ux + b2 * uy;
-            ux = (ux - gam * b1 * bu) + g1;
-            uy = (uy - gam * b2 * bu) + g2;
+            ux = fmadd(-(gam * b1), bu, ux) + g1;
+            uy = fmadd(-(gam * b2), bu, uy) + g2;
         }
     }
     out[W.soff + id] = inv * ux;
